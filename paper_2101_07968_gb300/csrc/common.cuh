@@ -18,7 +18,6 @@ constexpr int kMidLMax = 256;        // looped thread-per-instance kernel: 17 <=
 constexpr int kSmemTableLMax = 64;   // group kernel keeps its DP table on chip up to here
 constexpr int64_t kMidSlots = 152 * 16 * 32;  // traceback slots of the looped kernel (L <= 64)
 constexpr int64_t kRangeLimit = int64_t(1) << 52;
-constexpr uint64_t kNarrowLimit = 0xFFFFFFFEull;  // bound that lets a DP run in 32 bits
 // capped bound under which the shifted form of a DP runs in signed 32 bits
 constexpr uint64_t kShiftedLimit = 0x7FFFFFFFull;
 
