@@ -1,7 +1,7 @@
 // One instance of the DynaComm DP (Eq. 8 / Algorithm 3 and Eq. 9 / Algorithm 4)
-// solved by a CTA in O(L log L) per segment count, in 64-bit arithmetic: the
-// device code shared by the deep-chain pass (dp_deep.cu) and the work-list pass
-// (dp_group.cu).
+// solved by a warp or a CTA in O(L log L) per segment count: the device code shared
+// by the warp-per-instance pass (dp_mid.cu), the CTA-per-instance pass (dp_deep.cu)
+// and the work-list pass (dp_group.cu).
 //
 // With the layers in processing order, P the prefix of the transfer costs and C
 // that of the compute costs, put
@@ -38,7 +38,10 @@
 //    H[L][n]. The fill stops after the first column without one (on the deep
 //    chain after 6.2 columns on average, where the optimum has 5.6 segments), or
 //    when c_n + a[L] - b[L-1], which bounds every later T, reaches the optimum.
-// Values stay below 2^53 (the range check), so 64 bits hold every sum.
+// Only cells that their column lowered are ever visited by the traceback (an
+// unchanged one would be a decision with fewer segments), so only those are kept.
+// Values stay below 2^53 (the range check), so 64 bits hold every sum; an instance
+// with a[L] + b[L] + (L + 1) dt < 2^31 runs in 32 bits.
 #pragma once
 
 #include "common.cuh"
@@ -46,65 +49,52 @@
 namespace dc {
 namespace {
 
-constexpr int kChainPairs = 4;             // row pairs per thread, at most
-constexpr int kChainThreads = 512;         // threads per instance, at most
-constexpr int kChainRows = 2 * kChainPairs;  // rows per thread, at most
-
-// Shared memory of a CTA: two key buffers (H + e + b of a column, rows 1..L at
-// 0..L-1) and b, then the decision words, the scan's partial sums and a few
-// words that one thread publishes.
+// Arrays of the solver, in the caller's shared memory: K (the newest column's keys
+// H + e + b) and b of rows 1..L at 0..L-1, an even number of 64-bit places each
+// (the 32-bit form uses half of them).
 __host__ __device__ inline size_t chain_row_bytes(int L) { return size_t((L + 1) / 2) * 16; }
-__host__ __device__ inline size_t chain_bits_bytes(int L)
-{
-    return (size_t(words_for(L)) * 4 + 15) / 16 * 16;
-}
-constexpr size_t kChainScratch = (2 * kChainPairs * (kChainThreads / 32) + 8 + 4) * 8;
-__host__ __device__ inline size_t chain_smem_bytes(int L)
-{
-    return 3 * chain_row_bytes(L) + chain_bits_bytes(L) + kChainScratch;
-}
 
-// Threads per instance: the fewest warps that hold the rows (8 per thread), and
-// more, down to one row pair per thread, while `count` instances leave the GPU's
-// SMs with fewer than 16 warps each.
-inline int chain_threads(int64_t count, int L, int sms)
-{
-    int nt = 32 * ((L + 32 * kChainRows - 1) / (32 * kChainRows));
-    while (nt * 2 <= kChainThreads && nt * 2 < L && count * (nt / 32) < int64_t(sms) * 16) nt *= 2;
-    return nt;
-}
-
-// Where H of column n >= 2 goes for the traceback. Offsets from H[1][1], which no
-// value is below, in 32 bits (the caller has checked the range), or whole values.
+// The columns kept for the traceback, 2..last: offsets from `base` (no value of the
+// instance is below it) in 32 bits, columns 2..shared in shared memory and the rest
+// in a slot of the workspace.
 struct KeptOffsets {
-    uint32_t *at;
-    int L, last;  // columns 2..last
+    uint32_t *sm, *gm;
+    int L, shared, last;
     int64_t base;
-    __device__ bool holds(int n) const { return n <= last; }
-    __device__ void put(int n, int m, int64_t v) const
+    __device__ __forceinline__ bool holds(int n) const { return n <= last; }
+    template <typename T>
+    __device__ __forceinline__ void put(int n, int m, T v) const
     {
-        const int64_t j = int64_t(n - 2) * L + (m - 1);
-        if (DC_CHECK(n >= 2 && n <= last && m >= 1 && m <= L))
-            at[j] = uint32_t(min(uint64_t(v - base), uint64_t(0xffffffffu)));
+        const uint32_t off = uint32_t(v - T(base));
+        if (!DC_CHECK(n >= 2 && m >= 1 && m <= L)) return;
+        if (n <= shared)
+            sm[(n - 2) * L + (m - 1)] = off;
+        else if (n <= last)
+            gm[int64_t(n - 1 - shared) * L + (m - 1)] = off;
     }
-    __device__ int64_t get(int n, int m) const
+    template <typename T>
+    __device__ __forceinline__ T get(int n, int m) const
     {
-        if (!DC_CHECK(n >= 2 && n <= last && m >= 1 && m <= L)) return 0;
-        return base + int64_t(at[int64_t(n - 2) * L + (m - 1)]);
+        if (!DC_CHECK(n >= 2 && n <= last && m >= 1 && m <= L)) return T(0);
+        return T(base) + T(n <= shared ? sm[(n - 2) * L + (m - 1)]
+                                       : gm[int64_t(n - 1 - shared) * L + (m - 1)]);
     }
 };
-struct KeptValues {  // the triangle of cells m >= n, every column
+// whole values, every column: the triangle of cells m >= n
+struct KeptValues {
     int64_t *at;
     int L;
-    __device__ bool holds(int) const { return true; }
-    __device__ void put(int n, int m, int64_t v) const
+    __device__ __forceinline__ bool holds(int) const { return true; }
+    template <typename T>
+    __device__ __forceinline__ void put(int n, int m, T v) const
     {
-        if (m >= n && DC_CHECK(n >= 1 && m <= L)) at[tri_index(L, m, n)] = v;
+        if (m >= n && DC_CHECK(n >= 1 && m <= L)) at[tri_index(L, m, n)] = int64_t(v);
     }
-    __device__ int64_t get(int n, int m) const
+    template <typename T>
+    __device__ __forceinline__ T get(int n, int m) const
     {
-        if (!DC_CHECK(n >= 1 && m >= n && m <= L)) return 0;
-        return at[tri_index(L, m, n)];
+        if (!DC_CHECK(n >= 1 && m >= n && m <= L)) return T(0);
+        return T(at[tri_index(L, m, n)]);
     }
 };
 
@@ -114,229 +104,181 @@ struct ChainOut {
     int32_t *nseg, *status;
 };
 
-// Number of keys below t among key[1..N] (key[k] at K[k-1], sorted), P the largest
-// power of two <= N: the first probe splits [0, N] into two ranges of at most P
-// values, the rest halve it. Two searches at once (independent load chains).
-__device__ __forceinline__ void count_below2(const int64_t *K, int N, int P, int64_t t0,
-                                             int64_t t1, int &p0, int &p1)
+template <typename T>
+struct Pair;
+template <>
+struct Pair<int32_t> {
+    using type = int2;
+    static __device__ __forceinline__ int2 make(int32_t x, int32_t y) { return make_int2(x, y); }
+};
+template <>
+struct Pair<int64_t> {
+    using type = longlong2;
+    static __device__ __forceinline__ longlong2 make(int64_t x, int64_t y) { return make_longlong2(x, y); }
+};
+
+// One halving of two searches at once; `top` is the largest power of two that the
+// search range needs (uniform), so the steps above it are skipped.
+template <typename T, int STEP>
+__device__ __forceinline__ void halve2(const T *K, int top, T t0, T t1, int &p0, int &p1)
 {
-    const int64_t kp = K[P - 1];
-    p0 = kp < t0 ? N - P + 1 : 0;
-    p1 = kp < t1 ? N - P + 1 : 0;
-    for (int st = P >> 1; st > 0; st >>= 1) {
-        const int64_t k0 = K[p0 + st - 1], k1 = K[p1 + st - 1];
-        if (k0 < t0) p0 += st;
-        if (k1 < t1) p1 += st;
+    if (STEP < top) {
+        const T k0 = K[p0 + STEP - 1], k1 = K[p1 + STEP - 1];
+        if (k0 < t0) p0 += STEP;
+        if (k1 < t1) p1 += STEP;
     }
 }
-
-// Solves instance i (rows crow, xrow of L costs) with the whole CTA. make_kept(base,
-// range) gives the store of kept columns, or refuses by returning false; returns
-// false, having written nothing, when the instance needs columns the store does not
-// hold. `vec`: the rows are 16-byte aligned and L is even.
-template <bool FWD, typename Kept, typename MakeKept>
-__device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const int64_t *crow,
-                            const int64_t *xrow, int64_t dt, bool vec, const ChainOut &o,
-                            MakeKept make_kept)
+// Number of keys below t among the sorted key[1..N] (key[k] at K[k-1]), P the largest
+// power of two <= N: the first probe splits [0, N] into two ranges of at most P
+// values, the rest halve it.
+template <typename T, int TOP>
+__device__ __forceinline__ void count_below2(const T *K, int N, int P, T t0, T t1, int &p0, int &p1)
 {
-    const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = NT >> 5;
-    const int W = words_for(L);
-    const size_t rb = chain_row_bytes(L);
-    int64_t *K0 = reinterpret_cast<int64_t *>(smem), *K1 = reinterpret_cast<int64_t *>(smem + rb);
-    int64_t *B = reinterpret_cast<int64_t *>(smem + 2 * rb);
-    uint32_t *bitsw = reinterpret_cast<uint32_t *>(smem + 3 * rb);
-    uint64_t *tot = reinterpret_cast<uint64_t *>(smem + 3 * rb + chain_bits_bytes(L));
-    uint32_t *orw = reinterpret_cast<uint32_t *>(tot + 2 * kChainPairs * (kChainThreads / 32));
-    int64_t *s_aL = reinterpret_cast<int64_t *>(orw + 16);
-    const int NJ = (L + 2 * NT - 1) / (2 * NT);  // row pairs per thread
+    const T kp = K[P - 1];
+    p0 = kp < t0 ? N - P + 1 : 0;
+    p1 = kp < t1 ? N - P + 1 : 0;
+    if constexpr (TOP > 1024) halve2<T, 1024>(K, P, t0, t1, p0, p1);
+    if constexpr (TOP > 512) halve2<T, 512>(K, P, t0, t1, p0, p1);
+    if constexpr (TOP > 256) halve2<T, 256>(K, P, t0, t1, p0, p1);
+    if constexpr (TOP > 128) halve2<T, 128>(K, P, t0, t1, p0, p1);
+    if constexpr (TOP > 64) halve2<T, 64>(K, P, t0, t1, p0, p1);
+    if constexpr (TOP > 32) halve2<T, 32>(K, P, t0, t1, p0, p1);
+    halve2<T, 16>(K, P, t0, t1, p0, p1);
+    halve2<T, 8>(K, P, t0, t1, p0, p1);
+    halve2<T, 4>(K, P, t0, t1, p0, p1);
+    halve2<T, 2>(K, P, t0, t1, p0, p1);
+    halve2<T, 1>(K, P, t0, t1, p0, p1);
+}
 
-    // ---- rows: pair j of this thread holds rows r, r+1 with r = 2 (j NT + tid) + 1
-    uint64_t a[kChainPairs][2], b[kChainPairs][2];
-    uint64_t any = uint64_t(dt);
+// Columns 2.., the traceback and the outputs of instance i, from its prefixes:
+// thread tid of NT holds rows r, r+1 with r = 2 (j NT + tid) + 1 as a[j], b[j] (rows
+// past L hold the totals). WARP: one warp solves it (NT = 32), else the CTA. word:
+// shared memory, W decision words (CTA only); pub: two values that the CTA's last row
+// publishes. TOP: a power of two >= L - 1's largest. Returns false, having written
+// nothing, when the optimum needs columns that `kept` does not hold.
+template <bool FWD, typename T, int NJ, bool WARP, int TOP, typename Kept>
+__device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub, int tid, int NT,
+                                              int64_t i, int L, T dt, const T (&a)[NJ][2],
+                                              const T (&b)[NJ][2], T aL, T bL, const Kept &kept,
+                                              const ChainOut &o)
+{
+    using P2 = Pair<T>;
+    using Two = typename P2::type;
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = tid & 31, W = words_for(L);
+    const T e = FWD ? T(0) : dt, h1 = FWD ? dt : T(0);  // H[m][1] = h1 + a[m]
+    T h[NJ][2];
 #pragma unroll
-    for (int j = 0; j < kChainPairs; ++j) {
-        if (j < NJ) {
-            const int r = 2 * (j * NT + tid) + 1;
-            uint64_t c0 = 0, c1 = 0, x0 = 0, x1 = 0;
-            if (r < L && vec) {
-                const int at = FWD ? r - 1 : L - r - 1;
-                const ulonglong2 c = *reinterpret_cast<const ulonglong2 *>(crow + at);
-                const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(xrow + at);
-                c0 = FWD ? c.x : c.y;
-                c1 = FWD ? c.y : c.x;
-                x0 = FWD ? x.x : x.y;
-                x1 = FWD ? x.y : x.x;
-            } else if (r <= L) {
-                const int at = FWD ? r - 1 : L - r;
-                c0 = uint64_t(__ldg(crow + at));
-                x0 = uint64_t(__ldg(xrow + at));
-                if (r < L) {
-                    c1 = uint64_t(__ldg(crow + (FWD ? at + 1 : at - 1)));
-                    x1 = uint64_t(__ldg(xrow + (FWD ? at + 1 : at - 1)));
-                }
-            }
-            any |= c0 | c1 | x0 | x1;
-            uint64_t sa = FWD ? x0 + x1 : c0 + c1, sb = FWD ? c0 + c1 : x0 + x1;
-            const uint64_t ta = sa, tb = sb;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint64_t ua = __shfl_up_sync(0xffffffffu, sa, d);
-                const uint64_t ub = __shfl_up_sync(0xffffffffu, sb, d);
-                if (lane >= d) {
-                    sa += ua;
-                    sb += ub;
-                }
-            }
-            if (lane == 31) {
-                tot[j * NW + warp] = sa;
-                tot[(NJ + j) * NW + warp] = sb;
-            }
-            a[j][0] = sa - ta + (FWD ? x0 : c0);
-            a[j][1] = sa;
-            b[j][0] = sb - tb + (FWD ? c0 : x0);
-            b[j][1] = sb;
-        }
-    }
-    const uint32_t hi = __reduce_or_sync(0xffffffffu, uint32_t(any >> 32));
-    if (lane == 0) orw[warp] = hi;
-    for (int w = tid; w < W; w += NT) bitsw[w] = 0u;
-    __syncthreads();
-    uint32_t all = 0;
-    for (int w = 0; w < NW; ++w) all |= orw[w];
-    uint64_t accA = 0, accB = 0;
-    {
-        int next = warp;
-        int j = 0;
-        uint64_t offA[kChainPairs] = {}, offB[kChainPairs] = {};
-        for (int q = 0; q < NJ * NW; ++q) {
-            if (q == next) {
-#pragma unroll
-                for (int u = 0; u < kChainPairs; ++u)
-                    if (u == j) {
-                        offA[u] = accA;
-                        offB[u] = accB;
-                    }
-                ++j;
-                next += NW;
-            }
-            accA += tot[q];
-            accB += tot[NJ * NW + q];
-        }
-#pragma unroll
-        for (int u = 0; u < kChainPairs; ++u) {
-            a[u][0] += offA[u];
-            a[u][1] += offA[u];
-            b[u][0] += offB[u];
-            b[u][1] += offB[u];
-        }
-    }
-    // accA = a[L], accB = b[L]: the totals
-    int st = DC_OK;
-    if (all >> 31)
-        st = DC_ERR_NEGATIVE;
-    else if (all >> 20 || exceeds_range(L, dt, FWD ? accB : accA, FWD ? accA : accB))
-        st = DC_ERR_RANGE;
-    if (st != DC_OK) {
-        if (tid == 0) {
-            o.makespan[i] = -int64_t(st);
-            if (o.nseg) o.nseg[i] = 0;
-            if (o.status) o.status[i] = st;
-        }
-        for (int w = tid; w < W; w += NT) o.bits[i * W + w] = 0u;
-        return true;
-    }
-    const int64_t e = FWD ? 0 : dt, h1 = FWD ? dt : 0;  // H[m][1] = h1 + a[m]
-    const int64_t aL = int64_t(accA), bL = int64_t(accB);
-#pragma unroll
-    for (int j = 0; j < kChainPairs; ++j) {
+    for (int j = 0; j < NJ; ++j) {
         const int r = 2 * (j * NT + tid) + 1;
-        if (j < NJ && r <= L) {  // row L + 1 of an odd L's last pair is padding
-            *reinterpret_cast<ulonglong2 *>(B + r - 1) = make_ulonglong2(b[j][0], b[j][1]);
-            *reinterpret_cast<ulonglong2 *>(K0 + r - 1) =
-                make_ulonglong2(a[j][0] + b[j][0] + uint64_t(h1 + e), a[j][1] + b[j][1] + uint64_t(h1 + e));
-            if (r == 1) *s_aL = int64_t(a[j][0]);
+        h[j][0] = h1 + a[j][0];
+        h[j][1] = h1 + a[j][1];
+        if (r <= L) {  // row L + 1 of an odd L's last pair is padding
+            *reinterpret_cast<Two *>(B + r - 1) = P2::make(b[j][0], b[j][1]);
+            *reinterpret_cast<Two *>(K + r - 1) = P2::make(h[j][0] + e + b[j][0], h[j][1] + e + b[j][1]);
         }
     }
-    __syncthreads();
-    int64_t hL = h1 + aL;  // H[L][n] of the newest column
-    const int64_t base = h1 + *s_aL;
-    Kept kept;
-    if (!make_kept(kept, base, uint64_t(hL - base))) return false;
+    if (WARP) __syncwarp(); else __syncthreads();
+    T hL = h1 + aL;  // H[L] of the newest column
     int s = 1;
     bool deep = false;  // the optimum lies beyond the kept columns
-
-    // ---- columns 2..
     const int N = L - 1;
-    int P = 1;
-    while (P * 2 <= N) P *= 2;
-    int64_t *K = K0, *Kn = K1;
-    const int64_t bL1 = L > 1 ? B[L - 2] : 0;
+    const int P = 1 << (31 - __clz(N | 1));
+    const T bL1 = N > 0 ? B[N - 1] : T(0);
+    T c = FWD ? dt : T(0);
     for (int n = 2; n <= L; ++n) {
-        const int64_t c = FWD ? int64_t(n) * dt : 0;
+        if (FWD) c += dt;
         if (c + aL - bL1 >= hL) break;
-        int64_t least = INT64_MAX;  // lowest H that this column lowered
+        T v[NJ][2];
+        bool low[NJ][2];
 #pragma unroll
-        for (int j = 0; j < kChainPairs; ++j) {
+        for (int j = 0; j < NJ; ++j) {
             const int r = 2 * (j * NT + tid) + 1;
-            if (j < NJ && r <= L) {
-                const int64_t t0 = c + int64_t(a[j][0]), t1 = c + int64_t(a[j][1]);
-                int p0, p1;
-                count_below2(K, N, P, t0, t1, p0, p1);
-                // k = p + 1 is the first with H + e + b >= t (row L when there is
-                // none: H[L] lowers nothing), k = p the last below it (p = 0 gives
-                // t, which lowers nothing)
-                const longlong2 bb = *reinterpret_cast<const longlong2 *>(B + r - 1);
-                const longlong2 kk = *reinterpret_cast<const longlong2 *>(K + r - 1);
-                const int64_t o0 = kk.x - bb.x - e, o1 = kk.y - bb.y - e;
-                const int64_t u0 = min(K[p0] - B[p0], t0 - (p0 > 0 ? B[p0 - 1] : 0));
-                const int64_t u1 = min(K[p1] - B[p1], t1 - (p1 > 0 ? B[p1 - 1] : 0));
-                const int64_t v0 = min(o0, u0), v1 = min(o1, u1);
-                *reinterpret_cast<longlong2 *>(Kn + r - 1) = make_longlong2(v0 + e + bb.x, v1 + e + bb.y);
-                if (v0 < o0) least = min(least, v0);
-                if (r < L && v1 < o1) least = min(least, v1);
-                if (kept.holds(n)) {
-                    kept.put(n, r, v0);
-                    if (r < L) kept.put(n, r + 1, v1);
-                }
+            const T t0 = c + a[j][0], t1 = c + a[j][1];
+            int p0, p1;
+            count_below2<T, TOP>(K, N, P, t0, t1, p0, p1);
+            // k = p + 1 is the first with H + e + b >= t (row L when there is none:
+            // H[L] lowers nothing), k = p the last below it (p = 0 gives t, which
+            // lowers nothing)
+            const T u0 = min(K[p0] - B[p0], p0 > 0 ? t0 - B[p0 - 1] : t0);
+            const T u1 = min(K[p1] - B[p1], p1 > 0 ? t1 - B[p1 - 1] : t1);
+            v[j][0] = min(h[j][0], u0);
+            v[j][1] = min(h[j][1], u1);
+            low[j][0] = r <= L && u0 < h[j][0];
+            low[j][1] = r < L && u1 < h[j][1];
+            if (low[j][0]) kept.put(n, r, v[j][0]);
+            if (low[j][1]) kept.put(n, r + 1, v[j][1]);
+            if (!WARP && (r == L || r + 1 == L)) pub[n & 1] = r == L ? v[j][0] : v[j][1];
+        }
+        T hn;
+        if (WARP) {
+            const int q = (L - 1) / 2;  // row L's pair
+            T mine = v[0][0];
+#pragma unroll
+            for (int j = 0; j < NJ; ++j)
+                if (j == q / 32) mine = (L & 1) ? v[j][0] : v[j][1];
+            hn = __shfl_sync(kAll, mine, q % 32);  // every lane has read column n-1
+        } else {
+            __syncthreads();
+            hn = pub[n & 1];
+        }
+        // another column only while a lowered H may still lower H[L]
+        bool more = false;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            const int r = 2 * (j * NT + tid) + 1;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (low[j][u]) K[r - 1 + u] = v[j][u] + e + b[j][u];
+                more |= low[j][u] && v[j][u] + e < hn;
+                h[j][u] = v[j][u];
             }
         }
-        __syncthreads();
-        const int64_t h = Kn[L - 1] - bL - e;
-        if (h < hL) {
-            hL = h;
+        if (hn < hL) {
+            hL = hn;
             s = n;
             if (n > 2 && !kept.holds(n - 1)) deep = true;
         }
-        // another column only while a lowered H may still lower H[L]; e >= 0, so the
-        // sentinel stays above every sum
-        const bool more = least != INT64_MAX && least + e < hL;
-        int64_t *sw = K;
-        K = Kn;
-        Kn = sw;
-        if (!__syncthreads_or(more) || deep) break;
+        if (WARP) {
+            __syncwarp();
+            if (!__any_sync(kAll, more) || deep) break;
+        } else {
+            if (!__syncthreads_or(more) || deep) break;
+        }
     }
     if (deep) return false;
 
-    // ---- traceback by warp 0: Path[m][n] = the first k with b[k] >= c_n + a[m] - v.
-    // a goes to the idle key buffer first.
+    // ---- traceback by one warp: Path[m][n] = the first k with b[k] >= c_n + a[m] - v;
+    // a goes to the key array first
+    if (!WARP || s > 1) {
 #pragma unroll
-    for (int j = 0; j < kChainPairs; ++j) {
-        const int r = 2 * (j * NT + tid) + 1;
-        if (j < NJ && r <= L)
-            *reinterpret_cast<ulonglong2 *>(Kn + r - 1) = make_ulonglong2(a[j][0], a[j][1]);
+        for (int j = 0; j < NJ; ++j) {
+            const int r = 2 * (j * NT + tid) + 1;
+            if (r <= L) *reinterpret_cast<Two *>(K + r - 1) = P2::make(a[j][0], a[j][1]);
+        }
     }
-    __syncthreads();
-    if (warp == 0) {
-        int err = 0, m = L, n = s;
-        int64_t v = hL;
-        while (n > 1) {
-            const int64_t thr = (FWD ? int64_t(n) * dt : 0) + Kn[m - 1] - v;
-            int lo = 1, len = N;  // the answer lies in [lo, lo + len], lo + len: none
+    if (WARP) __syncwarp(); else __syncthreads();
+    if (!WARP && tid >= 32) return true;
+    int err = 0, m = L, n = s;
+    T v = hL;
+    uint32_t mine = 0u;  // WARP: lane w's decision word w
+    T cn = FWD ? T(n) * dt : T(0);
+    while (n > 1) {
+        const T thr = cn + K[m - 1] - v;
+        int k;
+        if (WARP) {
+            int below = 0;  // rows past L hold b[L] >= thr, or there is no such k
+#pragma unroll
+            for (int j = 0; j < NJ; ++j)
+                below += __popc(__ballot_sync(kAll, b[j][0] < thr)) + __popc(__ballot_sync(kAll, b[j][1] < thr));
+            k = below + 1;
+        } else {
+            int lo = 1, len = N;  // the answer lies in [lo, lo + len]
             while (len > 0) {
                 const int step = (len + 31) / 32;
-                const int k = lo + (lane + 1) * step - 1;  // last k of this lane's piece
-                const bool hit = k >= lo + len || B[k - 1] >= thr;
-                const unsigned bal = __ballot_sync(0xffffffffu, hit);
+                const int probe = lo + (lane + 1) * step - 1;  // last k of this lane's piece
+                const bool hit = probe >= lo + len || B[probe - 1] >= thr;
+                const unsigned bal = __ballot_sync(kAll, hit);
                 if (bal == 0u) {  // the last piece ends the range, and none reaches thr
                     lo += len;
                     break;
@@ -346,30 +288,203 @@ __device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const int64_t
                 lo += q * step;
                 len = min(step - 1, end - lo);
             }
-            const int k = lo;
-            if (k < n - 1 || k >= m) {
-                err = 1;
-                break;
-            }
-            const int64_t hk = n == 2 ? h1 + Kn[k - 1] : kept.get(n - 1, k);
-            if (hk + e > v) {
-                err = 1;
-                break;
-            }
-            if (lane == 0) bitsw[(k - 1) >> 5] |= 1u << ((k - 1) & 31);
-            v = hk;
-            m = k;
-            n -= 1;
+            k = lo;
         }
-        __syncwarp();
-        if (lane == 0) {
-            o.makespan[i] = err ? -int64_t(DC_ERR_INTERNAL) : hL + e + bL;
-            if (o.nseg) o.nseg[i] = err ? 0 : s;
-            if (o.status) o.status[i] = err ? DC_ERR_INTERNAL : DC_OK;
+        if (k < n - 1 || k >= m) {
+            err = 1;
+            break;
         }
-        for (int w = lane; w < W; w += 32) o.bits[i * W + w] = err ? 0u : bitsw[w];
+        const T hk = n == 2 ? h1 + K[k - 1] : kept.template get<T>(n - 1, k);
+        if (hk + e > v) {
+            err = 1;
+            break;
+        }
+        const uint32_t bit = 1u << ((k - 1) & 31);
+        if (WARP)
+            mine |= lane == ((k - 1) >> 5) ? bit : 0u;
+        else if (lane == 0)
+            word[(k - 1) >> 5] |= bit;
+        v = hk;
+        m = k;
+        n -= 1;
+        if (FWD) cn -= dt;
+    }
+    if (!WARP) __syncwarp();
+    if (lane == 0) {
+        o.makespan[i] = err ? -int64_t(DC_ERR_INTERNAL) : int64_t(hL + e) + int64_t(bL);
+        if (o.nseg) o.nseg[i] = err ? 0 : s;
+        if (o.status) o.status[i] = err ? DC_ERR_INTERNAL : DC_OK;
+    }
+    if (WARP) {
+        if (lane < W) o.bits[i * W + lane] = err ? 0u : mine;
+    } else {
+        for (int w = lane; w < W; w += 32) o.bits[i * W + w] = err ? 0u : word[w];
     }
     return true;
+}
+
+__device__ __forceinline__ void chain_failure(int st, int64_t i, int W, int tid, int NT, const ChainOut &o)
+{
+    if (tid == 0) {
+        o.makespan[i] = -int64_t(st);
+        if (o.nseg) o.nseg[i] = 0;
+        if (o.status) o.status[i] = st;
+    }
+    for (int w = tid; w < W; w += NT) o.bits[i * W + w] = 0u;
+}
+
+// The costs of rows r, r+1 (r odd; zero past L) of an instance's rows in processing
+// order. vec: the rows are 16-byte aligned and L is even.
+template <bool FWD>
+__device__ __forceinline__ void load_pair(const int64_t *row, int L, int r, bool vec, uint64_t &v0,
+                                          uint64_t &v1)
+{
+    v0 = 0;
+    v1 = 0;
+    if (r > L) return;
+    if (vec) {
+        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(row + (FWD ? r - 1 : L - r - 1)));
+        v0 = FWD ? v.x : v.y;
+        v1 = FWD ? v.y : v.x;
+    } else {
+        const int at = FWD ? r - 1 : L - r;
+        v0 = uint64_t(__ldg(row + at));
+        if (r < L) v1 = uint64_t(__ldg(row + (FWD ? at + 1 : at - 1)));
+    }
+}
+
+// Inclusive prefixes over a warp's lanes of two values at once.
+template <typename U>
+__device__ __forceinline__ void scan2(U &sa, U &sb, int lane)
+{
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const U ua = __shfl_up_sync(0xffffffffu, sa, d), ub = __shfl_up_sync(0xffffffffu, sb, d);
+        if (lane >= d) {
+            sa += ua;
+            sb += ub;
+        }
+    }
+}
+
+// ---------------------------------------------------------------- CTA per instance
+constexpr int kChainThreads = 1024;  // threads per instance, at most
+constexpr int kChainPairs = 2;       // row pairs per thread, at most
+
+__host__ __device__ inline size_t chain_word_bytes(int L)
+{
+    return (size_t(words_for(L)) * 4 + 15) / 16 * 16;
+}
+// K and b, the decision words, then the scan's partial sums, the warps' flags and two
+// published values
+__host__ __device__ inline size_t chain_smem_bytes(int L)
+{
+    return 2 * chain_row_bytes(L) + chain_word_bytes(L) +
+           size_t(2 * kChainPairs * (kChainThreads / 32)) * 8 + 32 * 4 + 16;
+}
+
+// Solves instance i with the whole CTA, NJ row pairs per thread. make_kept(base,
+// range) returns the store of kept columns for values from base to base + range, with
+// `ok` false when it cannot hold them. Returns false, having written nothing, when
+// the instance is left to the work list.
+template <bool FWD, int NJ, typename MakeKept>
+__device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const int64_t *crow,
+                            const int64_t *xrow, int64_t dt, bool vec, const ChainOut &o,
+                            MakeKept make_kept)
+{
+    const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = NT >> 5;
+    const int W = words_for(L);
+    const size_t rb = chain_row_bytes(L);
+    uint32_t *word = reinterpret_cast<uint32_t *>(smem + 2 * rb);
+    uint64_t *tot = reinterpret_cast<uint64_t *>(smem + 2 * rb + chain_word_bytes(L));
+    uint32_t *orw = reinterpret_cast<uint32_t *>(tot + 2 * kChainPairs * (kChainThreads / 32));
+    unsigned char *pub = reinterpret_cast<unsigned char *>(orw + 32);
+
+    uint64_t a[NJ][2], b[NJ][2];
+    uint64_t any = uint64_t(dt);
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        const int r = 2 * (j * NT + tid) + 1;
+        uint64_t a0, a1, b0, b1;
+        load_pair<FWD>(FWD ? xrow : crow, L, r, vec, a0, a1);
+        load_pair<FWD>(FWD ? crow : xrow, L, r, vec, b0, b1);
+        any |= a0 | a1 | b0 | b1;
+        uint64_t sa = a0 + a1, sb = b0 + b1;
+        scan2(sa, sb, lane);
+        if (lane == 31) {
+            tot[j * NW + warp] = sa;
+            tot[(NJ + j) * NW + warp] = sb;
+        }
+        a[j][0] = sa - a1;
+        a[j][1] = sa;
+        b[j][0] = sb - b1;
+        b[j][1] = sb;
+    }
+    const uint32_t hi = __reduce_or_sync(0xffffffffu, uint32_t(any >> 32));
+    if (lane == 0) orw[warp] = hi;
+    for (int w = tid; w < W; w += NT) word[w] = 0u;
+    __syncthreads();
+    // every warp scans the partial sums: lane q holds those of warp q
+    const uint32_t all = __reduce_or_sync(0xffffffffu, lane < NW ? orw[lane] : 0u);
+    uint64_t aL = 0, bL = 0;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        uint64_t sa = lane < NW ? tot[j * NW + lane] : 0u, sb = lane < NW ? tot[(NJ + j) * NW + lane] : 0u;
+        const uint64_t xa = sa, xb = sb;
+        scan2(sa, sb, lane);
+        const uint64_t oa = aL + __shfl_sync(0xffffffffu, sa - xa, warp);
+        const uint64_t ob = bL + __shfl_sync(0xffffffffu, sb - xb, warp);
+        a[j][0] += oa;
+        a[j][1] += oa;
+        b[j][0] += ob;
+        b[j][1] += ob;
+        aL += __shfl_sync(0xffffffffu, sa, 31);
+        bL += __shfl_sync(0xffffffffu, sb, 31);
+    }
+    int st = DC_OK;
+    if (all >> 31)
+        st = DC_ERR_NEGATIVE;
+    else if (all >> 20 || exceeds_range(L, dt, FWD ? bL : aL, FWD ? aL : bL))
+        st = DC_ERR_RANGE;
+    if (st != DC_OK) {
+        chain_failure(st, i, W, tid, NT, o);
+        return true;
+    }
+    constexpr int kTop = 4096;
+    if (aL + bL + uint64_t(L + 1) * uint64_t(dt) < (uint64_t(1) << 31)) {
+        int32_t a32[NJ][2], b32[NJ][2];
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                a32[j][u] = int32_t(a[j][u]);
+                b32[j][u] = int32_t(b[j][u]);
+            }
+        bool ok = true;
+        const auto kept = make_kept(int64_t(0), uint64_t(0), ok);
+        return chain_columns<FWD, int32_t, NJ, false, kTop>(
+            reinterpret_cast<int32_t *>(smem), reinterpret_cast<int32_t *>(smem + rb), word,
+            reinterpret_cast<int32_t *>(pub), tid, NT, i, L, int32_t(dt), a32, b32, int32_t(aL),
+            int32_t(bL), kept, o);
+    }
+    int64_t a64[NJ][2], b64[NJ][2];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            a64[j][u] = int64_t(a[j][u]);
+            b64[j][u] = int64_t(b[j][u]);
+        }
+    // H lies between H[1][1] and H[L][1]; the first row's a is the smallest cost
+    const int64_t h1 = FWD ? dt : 0;
+    const int64_t a1 = __ldg((FWD ? xrow : crow) + (FWD ? 0 : L - 1));
+    bool ok = true;
+    const auto kept = make_kept(h1 + a1, aL - uint64_t(a1), ok);
+    if (!ok) return false;
+    return chain_columns<FWD, int64_t, NJ, false, kTop>(
+        reinterpret_cast<int64_t *>(smem), reinterpret_cast<int64_t *>(smem + rb), word,
+        reinterpret_cast<int64_t *>(pub), tid, NT, i, L, dt, a64, b64, int64_t(aL), int64_t(bL),
+        kept, o);
 }
 
 }  // namespace

@@ -1,31 +1,35 @@
-// CTA-per-instance DynaComm DP for 257 <= L <= 4096 (Eq. 8 / Algorithm 3 and
+// CTA-per-instance DynaComm DP for 129 <= L <= 4096 (Eq. 8 / Algorithm 3 and
 // Eq. 9 / Algorithm 4): the first pass over a deep batch. The method is in
 // chain.cuh: O(L log L) per column, and no more columns than the optimum has
 // segments, plus about one.
 //
 // Design (GB300):
-//  * an instance per CTA of 1 to 16 warps, up to 8 rows per thread (chain_threads):
-//    a column is one independent binary search per row in shared memory, so every
-//    thread works in every column; two searches run at once in a thread to overlap
-//    their shared-memory latency, and the other CTAs of the SM (8 at L = 1024, 32
-//    warps) hide the rest;
-//  * what bounds it: integer issue in the searches (L log2 L steps of 5 instructions
-//    a column), then the rows' 64-bit scans; the profiles are read once (16 L bytes
-//    per instance and direction) and the columns kept for the traceback stay in L2;
-//  * 64-bit values throughout: every valid instance fits, there is no choice of
-//    arithmetic and no cap on transfers. A column keeps 32-bit offsets for the
-//    traceback, columns 2..64 in a slot of the workspace per resident CTA; optima
-//    deeper than 65 segments, and instances whose useful values span 2^32, go to
-//    the work list (dp_group.cu, whole values, every column);
-//  * persistent CTAs take instances from a per-launch ticket, and a long batch is
-//    split into launches of four resident waves, so that kernels of other streams
-//    get their turn on the GPU between them. The launches are chained by
+//  * an instance per CTA of up to 32 warps, two or four rows per thread
+//    (deep_threads): a column is one independent binary search per row in shared
+//    memory, so every thread works in every column; a thread's searches run two at
+//    a time to overlap their shared-memory latency, and the other CTAs of the SM
+//    hide the rest;
+//  * what bounds it: integer issue in the searches (L log2 L steps of 3 to 4
+//    instructions a column) and the two CTA barriers of a column; the profiles are
+//    read once (16 L bytes per instance and direction) and the columns kept for the
+//    traceback stay in L2;
+//  * a column is updated in place: every thread's results wait in registers for a
+//    barrier, then only the lowered cells are written;
+//  * 32-bit values where the instance's sums fit, otherwise 64-bit (two in five
+//    instances of the deep chain), chosen per instance. Columns 2..64 are kept as
+//    32-bit offsets in a slot of the workspace per resident CTA; optima deeper than
+//    65 segments, and instances whose useful values span 2^32, go to the work list
+//    (dp_group.cu, whole values, every column);
+//  * persistent CTAs take instances from a per-launch ticket, and a long batch of
+//    L > 256 is split into launches of four resident waves, so that kernels of other
+//    streams get their turn on the GPU between them. The launches are chained by
 //    programmatic dependent launch: each may fill the SMs as the one before drains.
 //    A CTA claims a free slot from a bitmap for as long as it lives.
 //
-// Measured, both directions together: 16,384 instances of L = 1024 in 1.65 ms, and
-// 383 of L = 1023 in 0.21 ms (532 ms and 20.5 ms for the fill of all L columns over
-// every candidate that this kernel replaced).
+// Measured, both directions together: 16,384 instances of L = 1024 in 1.08 ms, and
+// 383 of L = 1023 in 0.16 ms (1.65 and 0.21 ms with 64-bit values only, eight rows
+// per thread and two key buffers; 532 and 20.5 ms for the fill of all L columns over
+// every candidate).
 #include "chain.cuh"
 
 namespace dc {
@@ -34,6 +38,7 @@ int sm_count();  // SMs of the current device (dp_small.cu)
 
 namespace {
 
+constexpr int kSplitLMin = 256;  // longer batches are split into launches above this depth
 constexpr int kKeep = 64;  // columns 2..kKeep kept for the traceback
 
 __host__ __device__ inline size_t slot_bytes(int L)
@@ -77,8 +82,8 @@ __device__ int claim_slot(uint32_t *busy, int nslots)
     return -1;
 }
 
-template <bool FWD>
-__global__ void __launch_bounds__(kChainThreads, 2) deep_kernel(DeepArgs a)
+template <bool FWD, int NJ>
+__global__ void __launch_bounds__(kChainThreads, 1) deep_kernel(DeepArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_slot;
@@ -102,11 +107,11 @@ __global__ void __launch_bounds__(kChainThreads, 2) deep_kernel(DeepArgs a)
         const uint32_t taken = s_taken;
         if (int64_t(taken) >= a.count) break;
         const int64_t i = a.lo + int64_t(taken);
-        const bool solved = chain_solve<FWD, KeptOffsets>(
+        const bool solved = chain_solve<FWD, NJ>(
             smem, i, L, a.comp + i * L, a.xfer + i * L, __ldg(a.dt + i), a.vec, a.out,
-            [&](KeptOffsets &k, int64_t base, uint64_t range) {
-                k = KeptOffsets{at, L, last, base};
-                return range < 0xffffffffull;
+            [&](int64_t base, uint64_t range, bool &ok) {
+                ok = range < (uint64_t(1) << 32);
+                return KeptOffsets{nullptr, at, L, 1, last, base};
             });
         if (!solved && tid == 0) {
             const uint32_t p = atomicAdd(a.list_count, 1u);
@@ -140,22 +145,30 @@ int64_t deep_slots_bound(int L)
 
 namespace {
 
-template <bool FWD>
-cudaError_t launch_deep_dir(const DeepArgs &a, bool pdl, cudaStream_t stream)
+// Threads per instance: four rows per thread (two row pairs, whose searches hide
+// each other's latency) in a full GPU; two per thread, for a shorter column, while
+// `count` instances of twice the warps leave the SMs with no more than 32 warps
+// each (383 x 1,023: see the figures above).
+int deep_threads(int64_t count, int L, int sms)
+{
+    const int nt2 = 32 * ((L + 127) / 128), nt1 = 32 * ((L + 63) / 64);
+    return nt1 <= kChainThreads && count * (nt1 / 32) <= int64_t(sms) * 32 ? nt1 : nt2;
+}
+
+template <bool FWD, int NJ>
+cudaError_t launch_deep_nj(const DeepArgs &a, int nt, bool pdl, cudaStream_t stream)
 {
     static DeviceCache attr;
     int done = 0;
     cudaError_t e = attr.get(done, [](int &v) {
         v = 1;
-        return cudaFuncSetAttribute(deep_kernel<FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        return cudaFuncSetAttribute(deep_kernel<FWD, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     int(chain_smem_bytes(DC_L_MAX)));
     });
     if (e != cudaSuccess) return e;
-    int nt = chain_threads(a.count, a.L, sm_count());
-    if (const int f = forced_warps(); f && a.L <= 32 * kChainRows * f) nt = 32 * f;
     const size_t smem = chain_smem_bytes(a.L);
     int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, deep_kernel<FWD>, nt, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, deep_kernel<FWD, NJ>, nt, smem);
     if (e != cudaSuccess) return e;
     int64_t grid = int64_t(nb < 1 ? 1 : nb) * sm_count();
     if (grid > a.nslots) grid = a.nslots;
@@ -170,12 +183,23 @@ cudaError_t launch_deep_dir(const DeepArgs &a, bool pdl, cudaStream_t stream)
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
     lc.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&lc, deep_kernel<FWD>, a);
+    return cudaLaunchKernelEx(&lc, deep_kernel<FWD, NJ>, a);
 }
 
-// Instances per launch: four resident waves.
+template <bool FWD>
+cudaError_t launch_deep_dir(const DeepArgs &a, bool pdl, cudaStream_t stream)
+{
+    int nt = deep_threads(a.count, a.L, sm_count());
+    // the test hook's warps, where four rows per thread cover the instance
+    if (const int f = forced_warps(); f && a.L <= 128 * f) nt = 32 * f;
+    return a.L <= 2 * nt ? launch_deep_nj<FWD, 1>(a, nt, pdl, stream)
+                         : launch_deep_nj<FWD, 2>(a, nt, pdl, stream);
+}
+
+// Instances per launch: four resident waves above L = 256, the whole batch below.
 int64_t deep_per_launch(int64_t batch, int L)
 {
+    if (L <= kSplitLMin) return batch;
     const int64_t per = 4 * deep_slots_bound(L);
     if (per >= batch) return batch;
     const int64_t n = (batch + per - 1) / per;  // equal shares

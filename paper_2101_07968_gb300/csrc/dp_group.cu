@@ -1,6 +1,6 @@
 // CTA-per-instance DynaComm DP for any 1 <= L <= 4096 (Eq. 8 / Algorithm 3 and
-// Eq. 9 / Algorithm 4): the pass over the work lists of the looped kernel
-// (dp_mid.cu) and the deep-chain kernel (dp_deep.cu), whose instances have values
+// Eq. 9 / Algorithm 4): the pass over the work lists of the looped and
+// warp-per-instance kernels (dp_mid.cu) and the deep-chain kernel (dp_deep.cu), whose instances have values
 // beyond the first pass's range or an optimum deeper than its kept columns. The
 // method is in chain.cuh; this pass takes every value (64 bits) and keeps every
 // column, in shared memory up to L = 64, otherwise in a per-CTA table of the
@@ -30,8 +30,8 @@ inline size_t group_smem_bytes(int L, bool table_in_smem)
     return group_table_offset(L) + (table_in_smem ? size_t(tri_cells(L)) * 8 : 0);
 }
 
-template <bool FWD>
-__global__ void __launch_bounds__(kChainThreads, 2) group_kernel(GroupArgs a)
+template <bool FWD, int NJ>
+__global__ void __launch_bounds__(kChainThreads, 1) group_kernel(GroupArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int L = a.L;
@@ -42,38 +42,37 @@ __global__ void __launch_bounds__(kChainThreads, 2) group_kernel(GroupArgs a)
     for (int64_t j = blockIdx.x; j < count; j += gridDim.x) {
         const int64_t i = int64_t(a.list[j]);
         if (!DC_CHECK(i >= 0 && i < a.batch)) continue;
-        chain_solve<FWD, KeptValues>(smem, i, L, a.comp + i * L, a.xfer + i * L, __ldg(a.dt + i),
-                                     a.vec, a.out, [&](KeptValues &k, int64_t, uint64_t) {
-                                         k = KeptValues{table, L};
-                                         return true;
-                                     });
+        chain_solve<FWD, NJ>(smem, i, L, a.comp + i * L, a.xfer + i * L, __ldg(a.dt + i), a.vec,
+                             a.out, [&](int64_t, uint64_t, bool &) { return KeptValues{table, L}; });
         __syncthreads();  // shared memory is read
     }
 }
 
-// Threads per instance: lists are short, so up to one row pair per thread.
-int group_threads(int L)
-{
-    int nt = 32;
-    while (nt < kChainThreads && 2 * nt < L) nt *= 2;
-    return nt;
-}
-
-template <bool FWD>
-cudaError_t launch_group_dir(const GroupArgs &a, int64_t grid, cudaStream_t stream)
+template <bool FWD, int NJ>
+cudaError_t launch_group_nj(const GroupArgs &a, int nt, int64_t grid, cudaStream_t stream)
 {
     static DeviceCache attr;  // the kernel's shared-memory limit, raised once per device
     int done = 0;
     const cudaError_t e = attr.get(done, [](int &v) {
         v = 1;
-        return cudaFuncSetAttribute(group_kernel<FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        return cudaFuncSetAttribute(group_kernel<FWD, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     int(group_smem_bytes(DC_L_MAX, false)));
     });
     if (e != cudaSuccess) return e;
-    int nt = group_threads(a.L);
-    if (const int f = forced_warps(); f && a.L <= 32 * kChainRows * f) nt = 32 * f;
-    group_kernel<FWD><<<unsigned(grid), nt, group_smem_bytes(a.L, a.tables == nullptr), stream>>>(a);
+    group_kernel<FWD, NJ><<<unsigned(grid), nt, group_smem_bytes(a.L, a.tables == nullptr), stream>>>(a);
     return cudaGetLastError();
+}
+
+template <bool FWD>
+cudaError_t launch_group_dir(const GroupArgs &a, int64_t grid, cudaStream_t stream)
+{
+    // lists are short: two rows per thread, for the shortest column
+    int nt = 32 * ((a.L + 63) / 64);
+    if (nt > kChainThreads) nt = 32 * ((a.L + 127) / 128);
+    // the test hook's warps, where four rows per thread cover the instance
+    if (const int f = forced_warps(); f && a.L <= 128 * f) nt = 32 * f;
+    return a.L <= 2 * nt ? launch_group_nj<FWD, 1>(a, nt, grid, stream)
+                         : launch_group_nj<FWD, 2>(a, nt, grid, stream);
 }
 
 }  // namespace
