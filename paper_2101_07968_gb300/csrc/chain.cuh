@@ -367,6 +367,106 @@ __device__ __forceinline__ void scan2(U &sa, U &sb, int lane)
     }
 }
 
+// --------------------------------------------------------------- warp per instance
+// The same with a flag that gathers bit 31 of every partial sum: clear for all lanes
+// when no sum of the prefix reached 2^31 (the operands of the first that does are
+// below it, so it does not wrap).
+__device__ __forceinline__ void scan2_flag(uint32_t &sa, uint32_t &sb, uint32_t &flag, int lane)
+{
+    flag |= sa | sb;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t ua = __shfl_up_sync(0xffffffffu, sa, d), ub = __shfl_up_sync(0xffffffffu, sb, d);
+        if (lane >= d) {
+            sa += ua;
+            sb += ub;
+        }
+        flag |= sa | sb;
+    }
+}
+
+// Solves instance i with one warp, NJ row pairs per lane (L <= 64 NJ). smem: the
+// warp's K and b. make_kept as in chain_solve. Returns false, having written nothing,
+// when the instance is left to the work list.
+template <bool FWD, int NJ, typename MakeKept>
+__device__ __forceinline__ bool chain_solve_warp(unsigned char *smem, int64_t i, int L,
+                                                 const int64_t *crow, const int64_t *xrow,
+                                                 int64_t dt, bool vec, const ChainOut &o,
+                                                 MakeKept make_kept)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kTop = 64 * NJ;
+    const int lane = threadIdx.x & 31;
+    const size_t rb = chain_row_bytes(L);
+    uint64_t a[NJ][2], b[NJ][2];
+    uint32_t hi = uint32_t(uint64_t(dt) >> 32), flag = uint32_t(dt);
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        const int r = 2 * (32 * j + lane) + 1;
+        load_pair<FWD>(FWD ? xrow : crow, L, r, vec, a[j][0], a[j][1]);
+        load_pair<FWD>(FWD ? crow : xrow, L, r, vec, b[j][0], b[j][1]);
+        hi |= uint32_t((a[j][0] | a[j][1] | b[j][0] | b[j][1]) >> 32);
+        flag |= uint32_t(a[j][0] | a[j][1] | b[j][0] | b[j][1]);
+    }
+    int32_t a32[NJ][2], b32[NJ][2];
+    uint32_t aL32 = 0, bL32 = 0;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        uint32_t sa = uint32_t(a[j][0]) + uint32_t(a[j][1]), sb = uint32_t(b[j][0]) + uint32_t(b[j][1]);
+        scan2_flag(sa, sb, flag, lane);
+        a32[j][0] = int32_t(aL32 + sa - uint32_t(a[j][1]));
+        a32[j][1] = int32_t(aL32 + sa);
+        b32[j][0] = int32_t(bL32 + sb - uint32_t(b[j][1]));
+        b32[j][1] = int32_t(bL32 + sb);
+        aL32 += __shfl_sync(kAll, sa, 31);  // below 2^31 + 2^31 where it matters
+        bL32 += __shfl_sync(kAll, sb, 31);
+        flag |= aL32 | bL32;
+    }
+    const bool narrow = !__any_sync(kAll, (hi | (flag >> 31)) != 0u) &&
+                        uint64_t(aL32) + bL32 + uint64_t(L + 1) * uint64_t(dt) < (uint64_t(1) << 31);
+    if (narrow) {
+        bool ok = true;
+        const auto kept = make_kept(int64_t(0), uint64_t(0), ok);
+        return chain_columns<FWD, int32_t, NJ, true, kTop>(
+            reinterpret_cast<int32_t *>(smem), reinterpret_cast<int32_t *>(smem + rb),
+            static_cast<uint32_t *>(nullptr), static_cast<int32_t *>(nullptr), lane, 32, i, L,
+            int32_t(dt), a32, b32, int32_t(aL32), int32_t(bL32), kept, o);
+    }
+    // any other instance: 64-bit sums, the input checks, 64-bit values
+    uint64_t any = uint64_t(dt), aL = 0, bL = 0;
+    int64_t a64[NJ][2], b64[NJ][2];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        any |= a[j][0] | a[j][1] | b[j][0] | b[j][1];
+        uint64_t sa = a[j][0] + a[j][1], sb = b[j][0] + b[j][1];
+        scan2(sa, sb, lane);
+        a64[j][0] = int64_t(aL + sa - a[j][1]);
+        a64[j][1] = int64_t(aL + sa);
+        b64[j][0] = int64_t(bL + sb - b[j][1]);
+        b64[j][1] = int64_t(bL + sb);
+        aL += __shfl_sync(kAll, sa, 31);
+        bL += __shfl_sync(kAll, sb, 31);
+    }
+    const uint32_t all = __reduce_or_sync(kAll, uint32_t(any >> 32));
+    int st = DC_OK;
+    if (all >> 31)
+        st = DC_ERR_NEGATIVE;
+    else if (all >> 20 || exceeds_range(L, dt, FWD ? bL : aL, FWD ? aL : bL))
+        st = DC_ERR_RANGE;
+    if (st != DC_OK) {
+        chain_failure(st, i, words_for(L), lane, 32, o);
+        return true;
+    }
+    const int64_t a1 = __shfl_sync(kAll, a64[0][0], 0);  // H lies between H[1][1] and H[L][1]
+    bool ok = true;
+    const auto kept = make_kept((FWD ? dt : 0) + a1, aL - uint64_t(a1), ok);
+    if (!ok) return false;
+    return chain_columns<FWD, int64_t, NJ, true, kTop>(
+        reinterpret_cast<int64_t *>(smem), reinterpret_cast<int64_t *>(smem + rb),
+        static_cast<uint32_t *>(nullptr), static_cast<int64_t *>(nullptr), lane, 32, i, L, dt, a64,
+        b64, int64_t(aL), int64_t(bL), kept, o);
+}
+
 // ---------------------------------------------------------------- CTA per instance
 constexpr int kChainThreads = 1024;  // threads per instance, at most
 constexpr int kChainPairs = 2;       // row pairs per thread, at most

@@ -14,9 +14,9 @@
 namespace dc {
 
 constexpr int kSmallLMax = 16;       // unrolled thread-per-instance kernel: 1 <= L <= 16
-constexpr int kMidLMax = 256;        // looped thread-per-instance kernel: 17 <= L <= 256
+constexpr int kMidLMax = 192;        // looped and warp-per-instance kernels: 17 <= L <= 192
 constexpr int kSmemTableLMax = 64;   // group kernel keeps its DP table on chip up to here
-constexpr int64_t kMidSlots = 152 * 16 * 32;  // traceback slots of the looped kernel (L <= 64)
+constexpr int64_t kMidSlots = 152 * 16 * 32;  // traceback slots of the looped kernel
 constexpr int64_t kRangeLimit = int64_t(1) << 52;
 // capped bound under which the shifted form of a DP runs in signed 32 bits
 constexpr uint64_t kShiftedLimit = 0x7FFFFFFFull;
@@ -43,7 +43,8 @@ inline int64_t table_slots(int L)
     return s;
 }
 
-size_t mid_scratch_bytes(int64_t batch, int L);  // dp_mid.cu
+size_t mid_scratch_bytes(int64_t batch, int L);   // dp_mid.cu
+size_t warp_scratch_bytes(int64_t batch, int L);  // dp_warp.cu
 size_t deep_slot_bytes(int L);                   // dp_deep.cu
 int64_t deep_slots_bound(int L);                 // dp_deep.cu
 
@@ -147,7 +148,7 @@ struct NvtxRange {
 };
 
 // Test hook for the barrier discipline: DC_BLOCK_WARPS=1|2|4|8 in the
-// environment makes the looped, deep-chain and CTA-per-instance kernels run with
+// environment makes the warp- and CTA-per-instance kernels run with
 // that many warps per CTA where the kernel allows it (results must not change);
 // unset or any other value keeps each kernel's own choice. Read on every launch.
 inline int forced_warps()
@@ -243,6 +244,10 @@ cudaError_t launch_mid(bool forward, int64_t batch, int L, const int64_t *comp,
                        const int64_t *xfer, const int64_t *dt, int64_t *makespan,
                        uint32_t *bits, int32_t *nseg, int32_t *status, uint32_t *ticket,
                        uint32_t *list_count, uint32_t *list, uint32_t *tb, cudaStream_t stream);
+cudaError_t launch_warp(bool forward, int64_t batch, int L, const int64_t *comp,
+                        const int64_t *xfer, const int64_t *dt, int64_t *makespan, uint32_t *bits,
+                        int32_t *nseg, int32_t *status, uint32_t *ticket, uint32_t *list_count,
+                        uint32_t *list, uint32_t *slots, cudaStream_t stream);
 cudaError_t launch_deep(bool forward, int64_t batch, int L, const int64_t *comp,
                         const int64_t *xfer, const int64_t *dt, int64_t *makespan,
                         uint32_t *bits, int32_t *nseg, int32_t *status, uint32_t *tickets,

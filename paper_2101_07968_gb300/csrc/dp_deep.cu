@@ -1,4 +1,4 @@
-// CTA-per-instance DynaComm DP for 129 <= L <= 4096 (Eq. 8 / Algorithm 3 and
+// CTA-per-instance DynaComm DP for 193 <= L <= 4096 (Eq. 8 / Algorithm 3 and
 // Eq. 9 / Algorithm 4): the first pass over a deep batch. The method is in
 // chain.cuh: O(L log L) per column, and no more columns than the optimum has
 // segments, plus about one.

@@ -1,5 +1,6 @@
-// Thread-per-instance DynaComm DP for 17 <= L <= 256 (Eq. 8 / Algorithm 3 and
-// Eq. 9 / Algorithm 4), 32-bit arithmetic, runtime loops.
+// Thread-per-instance DynaComm DP for large batches of 17 <= L <= 19 (Eq. 8 /
+// Algorithm 3 and Eq. 9 / Algorithm 4), 32-bit arithmetic, runtime loops; other
+// 17 <= L <= 192 take the warp-per-instance kernel (dp_warp.cu), see launch_mid.
 //
 // Same processing-order template as the other kernels:
 //   X[m][n] = min_{k in [n-1, m-1]} max(X[k][n-1], R(m,n)) - S[k] + S[m] + c,
@@ -33,20 +34,13 @@
 //    kernel); the shifted values fit in signed 32 bits whenever the capped bound
 //    L*dt + sum(comp) + sum(capped xfer) is below 2^31;
 //  * value-only fill with deferred argmin, as in the short-L kernel: columns
-//    2..8 (L <= 64) or 2..16 are written to a per-thread slot of the caller's
+//    2..8 are written to a per-thread slot of the caller's
 //    workspace (coalesced across the warp) and the traceback re-derives each
 //    Path[m][n] as the lowest k whose candidate equals the cell. Instances whose
 //    optimum needs a deeper column, or whose values need more than 31 bits, are
 //    put on a work list that the CTA-per-instance kernel solves afterwards;
-//  * persistent CTAs claim 32-instance tiles from an atomic ticket, so the
-//    long, uneven per-tile work balances across the GPU. The lane slices take
-//    3*(L+1) words per lane and limit the resident warps, so for long rows 2, 4
-//    or 8 warps share a tile (same slices, less shared memory per warp): the
-//    column's row blocks are dealt to them in a snake, each warp keeps its
-//    results in registers until all have read column n-1 (a CTA barrier), then
-//    all write column n and meet at a second barrier. The tile's instances are
-//    dealt to the warps (32/NW each) for the row reads and the tracebacks, so
-//    no warp waits while another does them alone;
+//  * persistent single-warp CTAs claim 32-instance tiles from an atomic ticket, so
+//    the long, uneven per-tile work balances across the GPU;
 //  * the traceback skips the candidates that cannot match: U[m] + V[k] is
 //    non-increasing in k and bounds the candidate from below, so a binary
 //    search over V finds the first k with U[m] + V[k] <= the cell, and the scan
@@ -57,20 +51,11 @@ namespace dc {
 namespace {
 
 constexpr int kB = 8;  // rows per register block
-constexpr int kQ = 4;  // row blocks of a column per warp, at most (L <= 32 * warps)
+constexpr int kLoopedLMax = 19;
+constexpr int64_t kLoopedMinBatch = 160000;
 
-// warps sharing a tile: the lane slices take 3*(L+1) words per lane and limit
-// the resident warps, so longer rows spread a tile over more warps (measured
-// faster from L = 41 on)
-__host__ __device__ inline int mid_warps(int L) { return L <= 40 ? 1 : L <= 64 ? 2 : L <= 128 ? 4 : 8; }
-
-// last column kept for the traceback (a traceback of s segments reads columns
-// 1..s-1): 8 up to L = 64, 16 beyond (deeper optima are more common there)
-__host__ __device__ inline int mid_keep_last(int L)
-{
-    const int keep = L <= 64 ? 8 : 16;
-    return L - 1 < keep ? L - 1 : keep;
-}
+// last column kept for the traceback (a traceback of s segments reads columns 1..s-1)
+__host__ __device__ inline int mid_keep_last(int L) { return L - 1 < 8 ? L - 1 : 8; }
 // stored cell (m, n), 2 <= n <= keep_last
 __host__ __device__ inline int mid_cell(int L, int m, int n)
 {
@@ -81,15 +66,14 @@ __host__ __device__ inline int mid_cells(int L)
     const int c = mid_keep_last(L);
     return c >= 2 ? mid_cell(L, L, c) + 1 : 0;
 }
-// traceback slots (one per lane of a launched CTA): about one resident wave of
-// CTAs (kMidSlots up to L = 64), and no more than the batch's tiles need
-__host__ __device__ inline int64_t mid_slots(int64_t batch, int L)
+// traceback slots (one per lane of a launched CTA): about one resident wave of CTAs,
+// and no more than the batch's tiles need
+__host__ __device__ inline int64_t mid_slots(int64_t batch)
 {
-    const int nw = mid_warps(L);
-    const int64_t wave = nw <= 2 ? kMidSlots : int64_t(152) * 32 * (nw == 4 ? 4 : 2);
     const int64_t need = (batch + 31) / 32 * 32;
-    return need < wave ? need : wave;
+    return need < kMidSlots ? need : kMidSlots;
 }
+inline bool use_looped(int64_t batch, int L) { return L <= kLoopedLMax && batch >= kLoopedMinBatch; }
 
 // Rows -> the lane slices: U (Q forward, BC - dt backward) at 32*v, and the
 // (column, V) pairs with column 1 in .x and V (G forward, NGT backward) in .y.
@@ -142,10 +126,8 @@ __device__ __forceinline__ bool mid_prefix(int64_t batch, int64_t i, int L, cons
                                int32_t(FWD ? tcu - uint32_t(pc) : 0u - uint32_t(pxc)));
     }
     if (pc + pxc + uint64_t(L) * uint64_t(dti) > kShiftedLimit) {
-        {
-            const uint32_t at = atomicAdd(list_count, 1u);
-            if (DC_CHECK(int64_t(at) < batch)) list[at] = uint32_t(i);
-        }
+        const uint32_t at = atomicAdd(list_count, 1u);
+        if (DC_CHECK(int64_t(at) < batch)) list[at] = uint32_t(i);
         return false;
     }
     fcL = int32_t(tcu);
@@ -249,25 +231,8 @@ __device__ __forceinline__ void mid_write(int2 *pv, uint32_t *myslot, int64_t ns
     }
 }
 
-// Block b of a column (b = 0 holds row L): rows bot..top.
-__device__ __forceinline__ void mid_rows(int L, int n, int b, int &top, int &bot)
-{
-    top = L - kB * b;
-    bot = top - kB + 1 > n ? top - kB + 1 : n;
-}
-
-// Block of warp w for its q-th slot when NW warps share a column: a snake over
-// the blocks (0, 3, 4, 7 to warp 0 and 1, 2, 5, 6 to warp 1 for NW = 2; rows
-// 0..NW-1 left to right, the next NW right to left, and so on), which evens out
-// the work of the upper (longer) and lower blocks.
-template <int NW>
-__device__ __forceinline__ int mid_block_of(int q, int w)
-{
-    return (q % 2 == 0) ? NW * q + w : NW * q + NW - 1 - w;
-}
-
-template <bool FWD, int NW>
-__global__ void __launch_bounds__(32 * NW)
+template <bool FWD>
+__global__ void __launch_bounds__(32)
     mid_kernel(int64_t batch, int L, const int64_t *__restrict__ comp,
                const int64_t *__restrict__ xfer, const int64_t *__restrict__ dt,
                int64_t *__restrict__ makespan, uint32_t *__restrict__ bits,
@@ -276,11 +241,7 @@ __global__ void __launch_bounds__(32 * NW)
                uint32_t *__restrict__ list, uint32_t *__restrict__ tb, int64_t nslots)
 {
     extern __shared__ uint32_t smem[];
-    __shared__ uint32_t s_tile;
-    __shared__ int32_t s_dt[32], s_fcL[32], s_go[32], s_best[32], s_s[32];
-    __shared__ uint64_t s_px[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int W = words_for(L);
+    const int lane = threadIdx.x;
     // lane slices: U[v] at word 32*v + lane (v in [0, L]), then the current column
     // and V as (C[v], V[v]) pairs at 64-bit word 32*v + lane
     uint32_t *lw = smem + lane;
@@ -292,107 +253,50 @@ __global__ void __launch_bounds__(32 * NW)
     const int64_t tiles = (batch + 31) / 32;
 
     for (;;) {
-        if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
-        __syncthreads();
-        const uint32_t tile = s_tile;
+        uint32_t tile = 0;
+        if (lane == 0) tile = atomicAdd(ticket, 1u);
+        tile = __shfl_sync(0xffffffffu, tile, 0);
         if (int64_t(tile) >= tiles) break;
         const int64_t i = int64_t(tile) * 32 + lane;
 
-        // ---- rows -> lane slices: the tile's instances dealt to the warps, 32/NW
-        // each (a lane's slice is the same in every warp)
-        const bool mine = lane / (32 / NW) == warp;
-        if (mine) {
-            const int64_t dti = i < batch ? __ldg(dt + i) : 0;
-            uint64_t px = 0;
-            int32_t fcL = 0;
-            const bool go = i < batch && mid_prefix<FWD>(batch, i, L, comp, xfer, dti, lw, pv, makespan,
-                                                         bits, nseg, status, list_count, list, px,
-                                                         fcL);
-            s_dt[lane] = int32_t(dti);
-            s_go[lane] = go;
-            s_px[lane] = px;
-            s_fcL[lane] = fcL;
-        }
-        if (NW > 1) __syncthreads(); else __syncwarp();
-        // every lane runs the fill (lanes without an instance on stale slices:
-        // all accesses stay in the lane's own slice and slot), so that the
-        // barriers of the split fill are reached by all threads
-        const int32_t dt32 = s_dt[lane];
-        const int32_t fcL = s_fcL[lane];
+        // ---- rows -> lane slices (each lane's own: no synchronisation)
+        if (i >= batch) continue;
+        const int64_t dti = __ldg(dt + i);
+        uint64_t px = 0;
+        int32_t fcL = 0;
+        if (!mid_prefix<FWD>(batch, i, L, comp, xfer, dti, lw, pv, makespan, bits, nseg, status,
+                             list_count, list, px, fcL))
+            continue;
+        const int32_t dt32 = int32_t(dti);
 
         // ---- fill
-        int32_t bestV = 0;
+        int32_t bestV = FWD ? fcL + dt32 : U[32 * L] + 2 * dt32;
         int s = 1;
-        if (warp == 0) bestV = FWD ? fcL + dt32 : U[32 * L] + 2 * dt32;
         for (int n = 2; n <= L; ++n) {
             int32_t last = 0;  // row L's minimum: B[L][n] + Q[L] (forward) or F[L][n] - dt
-            if constexpr (NW == 1) {
-                // rows top-down, so column n overwrites column n-1 in place: a
-                // block reads only rows below its own top, which still hold n-1
-                for (int top = L; top >= n; top -= kB) {
-                    const int bot = top - kB + 1 > n ? top - kB + 1 : n;
-                    int32_t best[kB];
-                    mid_block<FWD>(pv, U, n, top, bot, best);
-                    mid_write<FWD>(pv, myslot, nslots, L, n, keep, top, bot, best, dt32, last);
-                }
-            } else {
-                // NW warps share the column's blocks; a block's rows are read by
-                // the blocks above it, so every result waits in registers until
-                // all warps have read column n-1
-                const int nb = (L - n + kB) / kB;
-                int32_t res[kQ][kB];
-#pragma unroll
-                for (int q = 0; q < kQ; ++q) {
-                    const int b = mid_block_of<NW>(q, warp);
-                    if (b < nb) {
-                        int top, bot;
-                        mid_rows(L, n, b, top, bot);
-                        mid_block<FWD>(pv, U, n, top, bot, res[q]);
-                    }
-                }
-                __syncthreads();
-#pragma unroll
-                for (int q = 0; q < kQ; ++q) {
-                    const int b = mid_block_of<NW>(q, warp);
-                    if (b < nb) {
-                        int top, bot;
-                        mid_rows(L, n, b, top, bot);
-                        mid_write<FWD>(pv, myslot, nslots, L, n, keep, top, bot, res[q], dt32, last);
-                    }
-                }
-                __syncthreads();
+            // rows top-down, so column n overwrites column n-1 in place: a block reads
+            // only rows below its own top, which still hold n-1
+            for (int top = L; top >= n; top -= kB) {
+                const int bot = top - kB + 1 > n ? top - kB + 1 : n;
+                int32_t best[kB];
+                mid_block<FWD>(pv, U, n, top, bot, best);
+                mid_write<FWD>(pv, myslot, nslots, L, n, keep, top, bot, best, dt32, last);
             }
-            if (warp == 0) {  // row L is in block 0, which warp 0 holds
-                // X[L][n] less P[L] (forward: B[L][n] + n dt) or S[L] (backward: F[L][n] + dt)
-                const int32_t v = FWD ? last - U[32 * L] + n * dt32 : last + 2 * dt32;
-                if (v < bestV) {  // strict: the lowest n wins ties
-                    bestV = v;
-                    s = n;
-                }
+            // X[L][n] less P[L] (forward: B[L][n] + n dt) or S[L] (backward: F[L][n] + dt)
+            const int32_t v = FWD ? last - U[32 * L] + n * dt32 : last + 2 * dt32;
+            if (v < bestV) {  // strict: the lowest n wins ties
+                bestV = v;
+                s = n;
             }
         }
-        // the tracebacks, dealt to the warps like the rows
-        if (warp == 0) {
-            s_best[lane] = bestV;
-            s_s[lane] = s;
-        }
-        if (NW > 1) __syncthreads(); else __syncwarp();
-        if (!mine || !s_go[lane]) continue;
-        bestV = s_best[lane];
-        s = s_s[lane];
-        const uint64_t px = s_px[lane];
         if (s - 1 > keep && s - 1 >= 2) {  // traceback would need an unkept column
-            {
             const uint32_t at = atomicAdd(list_count, 1u);
             if (DC_CHECK(int64_t(at) < batch)) list[at] = uint32_t(i);
-        }
             continue;
         }
 
         // ---- traceback: lowest k whose candidate equals the cell
-        // decision words 0 and 1 in registers; words 2.. (L > 65) set in place
-        uint32_t word0 = 0u, word1 = 0u;
-        for (int w = 2; w < W; ++w) bits[i * W + w] = 0u;
+        uint32_t word = 0u;  // W = 1 up to L = 33
         int err = 0, m = L, n = s;
         int32_t target = FWD ? bestV - s * dt32 + U[32 * L] : bestV - 2 * dt32;  // B[L][s] + Q[L] or F[L][s] - dt
         while (n > 1) {
@@ -437,12 +341,7 @@ __global__ void __launch_bounds__(32 * NW)
                 err = 1;
                 break;
             }
-            if (k - 1 < 32)
-                word0 |= 1u << (k - 1);
-            else if (k - 1 < 64)
-                word1 |= 1u << (k - 33);
-            else
-                bits[i * W + ((k - 1) >> 5)] |= 1u << ((k - 1) & 31);
+            word |= 1u << (k - 1);
             target = FWD ? fk + dt32 : fk - dt32;  // the cell (k, n-1): B + Q[k] = A + dt, or F - dt
             m = k;
             n -= 1;
@@ -450,32 +349,20 @@ __global__ void __launch_bounds__(32 * NW)
         makespan[i] = int64_t(uint64_t(uint32_t(bestV)) + px);
         if (nseg) nseg[i] = s;
         if (status) status[i] = err ? DC_ERR_INTERNAL : DC_OK;
-        bits[i * W] = word0;
-        if (W > 1) bits[i * W + 1] = word1;
+        bits[i] = word;
     }
 }
 
-template <bool FWD, int NW>
-cudaError_t launch_mid_nw(int64_t batch, int L, const int64_t *comp, const int64_t *xfer,
+template <bool FWD>
+cudaError_t launch_looped(int64_t batch, int L, const int64_t *comp, const int64_t *xfer,
                           const int64_t *dt, int64_t *makespan, uint32_t *bits, int32_t *nseg,
-                          int32_t *status, uint32_t *ticket, uint32_t *list_count,
-                          uint32_t *list, uint32_t *tb, cudaStream_t stream)
+                          int32_t *status, uint32_t *ticket, uint32_t *list_count, uint32_t *list,
+                          uint32_t *tb, cudaStream_t stream)
 {
     const size_t smem = size_t(3) * (L + 1) * 32 * 4;
-    static DeviceCache attr;  // the kernel's shared-memory limit, raised once per device
-    int done = 0;
-    const cudaError_t ae = attr.get(done, [](int &v) {
-        const int most = 3 * (kMidLMax + 1) * 32 * 4;
-        v = 1;
-        return cudaFuncSetAttribute(mid_kernel<FWD, NW>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    });
-    if (ae != cudaSuccess) return ae;
-    const int64_t slots = mid_slots(batch, L);
-    const int64_t grid = slots / 32;
-    mid_kernel<FWD, NW><<<unsigned(grid), 32 * NW, smem, stream>>>(
-        batch, L, comp, xfer, dt, makespan, bits, nseg, status, ticket, list_count, list, tb,
-        slots);
+    const int64_t slots = mid_slots(batch);
+    mid_kernel<FWD><<<unsigned(slots / 32), 32, smem, stream>>>(
+        batch, L, comp, xfer, dt, makespan, bits, nseg, status, ticket, list_count, list, tb, slots);
     return cudaGetLastError();
 }
 
@@ -483,31 +370,25 @@ cudaError_t launch_mid_nw(int64_t batch, int L, const int64_t *comp, const int64
 
 size_t mid_scratch_bytes(int64_t batch, int L)
 {
-    return size_t(mid_slots(batch, L)) * size_t(mid_cells(L)) * 4;
+    return use_looped(batch, L) ? size_t(mid_slots(batch)) * size_t(mid_cells(L)) * 4
+                                : warp_scratch_bytes(batch, L);
 }
 
+// One instance per thread while its lanes are better used than a warp's on one short
+// row: 400,000 x 17 in 188 us against 238 by the warp kernel, but 100,000 x 17 and
+// 400,000 x 20 are equal, and 400,000 x 24 takes 312 us against 253.
 cudaError_t launch_mid(bool forward, int64_t batch, int L, const int64_t *comp,
                        const int64_t *xfer, const int64_t *dt, int64_t *makespan,
                        uint32_t *bits, int32_t *nseg, int32_t *status, uint32_t *ticket,
                        uint32_t *list_count, uint32_t *list, uint32_t *tb, cudaStream_t stream)
 {
-#define DC_MID_LAUNCH(NW)                                                                        \
-    return forward ? launch_mid_nw<true, NW>(batch, L, comp, xfer, dt, makespan, bits, nseg,    \
-                                             status, ticket, list_count, list, tb, stream)       \
-                   : launch_mid_nw<false, NW>(batch, L, comp, xfer, dt, makespan, bits, nseg,   \
-                                              status, ticket, list_count, list, tb, stream);
-    // warps per tile: the kernel's choice, or the test hook's when its blocks
-    // (4 per warp and column) still cover a column's rows
-    int nw = mid_warps(L);
-    const int f = forced_warps();
-    if (f == 1 || (f > 1 && (L + 6) / 8 <= 4 * f)) nw = f;
-    switch (nw) {
-        case 1: DC_MID_LAUNCH(1)
-        case 2: DC_MID_LAUNCH(2)
-        case 4: DC_MID_LAUNCH(4)
-        default: DC_MID_LAUNCH(8)
-    }
-#undef DC_MID_LAUNCH
+    if (!use_looped(batch, L))
+        return launch_warp(forward, batch, L, comp, xfer, dt, makespan, bits, nseg, status, ticket,
+                           list_count, list, tb, stream);
+    return forward ? launch_looped<true>(batch, L, comp, xfer, dt, makespan, bits, nseg, status,
+                                         ticket, list_count, list, tb, stream)
+                   : launch_looped<false>(batch, L, comp, xfer, dt, makespan, bits, nseg, status,
+                                          ticket, list_count, list, tb, stream);
 }
 
 }  // namespace dc

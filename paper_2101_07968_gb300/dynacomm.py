@@ -21,7 +21,7 @@ _PKG = os.path.dirname(os.path.abspath(__file__))
 # instead of trapping; build it with `python -m paper_2101_07968_gb300.build --checked`)
 LIB_PATH = os.path.join(_PKG, "libdynacomm_checked.so" if os.environ.get("DC_CHECKED") == "1"
                         else "libdynacomm.so")
-CHECKED_UNITS = ("dp_deep", "dp_mid", "dp_small", "dp_group", "dp_fused")
+CHECKED_UNITS = ("dp_deep", "dp_mid", "dp_warp", "dp_small", "dp_group", "dp_fused")
 
 DC_OK, DC_ERR_NULL, DC_ERR_BAD_SHAPE, DC_ERR_NEGATIVE, DC_ERR_RANGE = 0, 1, 2, 3, 4
 DC_ERR_WORKSPACE, DC_ERR_CUDA, DC_ERR_BAD_CONFIG, DC_ERR_INTERNAL = 5, 6, 7, 8
