@@ -150,6 +150,26 @@ __device__ __forceinline__ void count_below2(const T *K, int N, int P, T t0, T t
     halve2<T, 1>(K, P, t0, t1, p0, p1);
 }
 
+// First k in [lo, lo + len] for which pred holds, given that it holds from some k on
+// and at lo + len (which is not asked); one warp, 32 probes a round.
+template <typename Pred>
+__device__ __forceinline__ int warp_first(int lo, int len, Pred pred)
+{
+    const int lane = threadIdx.x & 31;
+    while (len > 0) {
+        const int step = (len + 31) / 32;
+        const int probe = lo + (lane + 1) * step - 1;  // last k of this lane's piece
+        const bool hit = probe >= lo + len || pred(probe);
+        const unsigned bal = __ballot_sync(0xffffffffu, hit);
+        if (bal == 0u) return lo + len;  // the last piece ends the range
+        const int q = __ffs(int(bal)) - 1;
+        const int end = lo + len;
+        lo += q * step;
+        len = min(step - 1, end - lo);
+    }
+    return lo;
+}
+
 // Columns 2.., the traceback and the outputs of instance i, from its prefixes:
 // thread tid of NT holds rows r, r+1 with r = 2 (j NT + tid) + 1 as a[j], b[j] (rows
 // past L hold the totals). WARP: one warp solves it (NT = 32), else the CTA. word:
@@ -273,22 +293,7 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
                 below += __popc(__ballot_sync(kAll, b[j][0] < thr)) + __popc(__ballot_sync(kAll, b[j][1] < thr));
             k = below + 1;
         } else {
-            int lo = 1, len = N;  // the answer lies in [lo, lo + len]
-            while (len > 0) {
-                const int step = (len + 31) / 32;
-                const int probe = lo + (lane + 1) * step - 1;  // last k of this lane's piece
-                const bool hit = probe >= lo + len || B[probe - 1] >= thr;
-                const unsigned bal = __ballot_sync(kAll, hit);
-                if (bal == 0u) {  // the last piece ends the range, and none reaches thr
-                    lo += len;
-                    break;
-                }
-                const int q = __ffs(int(bal)) - 1;
-                const int end = lo + len;
-                lo += q * step;
-                len = min(step - 1, end - lo);
-            }
-            k = lo;
+            k = warp_first(1, N, [&](int q) { return B[q - 1] >= thr; });
         }
         if (k < n - 1 || k >= m) {
             err = 1;
@@ -483,24 +488,17 @@ __host__ __device__ inline size_t chain_smem_bytes(int L)
            size_t(2 * kChainPairs * (kChainThreads / 32)) * 8 + 32 * 4 + 16;
 }
 
-// Solves instance i with the whole CTA, NJ row pairs per thread. make_kept(base,
-// range) returns the store of kept columns for values from base to base + range, with
-// `ok` false when it cannot hold them. Returns false, having written nothing, when
-// the instance is left to the work list.
-template <bool FWD, int NJ, typename MakeKept>
-__device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const int64_t *crow,
-                            const int64_t *xrow, int64_t dt, bool vec, const ChainOut &o,
-                            MakeKept make_kept)
+// The prefixes of an instance's rows over the whole CTA, in processing order (a, b and
+// the row layout of chain_columns; 64-bit). tot, orw: scratch. One CTA barrier, which
+// also publishes what the threads wrote to shared memory before. Returns the
+// instance's status: DC_OK or its input error.
+template <bool FWD, int NJ>
+__device__ __forceinline__ int cta_prefix(uint64_t *tot, uint32_t *orw, int L, const int64_t *crow,
+                                          const int64_t *xrow, int64_t dt, bool vec,
+                                          uint64_t (&a)[NJ][2], uint64_t (&b)[NJ][2], uint64_t &aL,
+                                          uint64_t &bL)
 {
     const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = NT >> 5;
-    const int W = words_for(L);
-    const size_t rb = chain_row_bytes(L);
-    uint32_t *word = reinterpret_cast<uint32_t *>(smem + 2 * rb);
-    uint64_t *tot = reinterpret_cast<uint64_t *>(smem + 2 * rb + chain_word_bytes(L));
-    uint32_t *orw = reinterpret_cast<uint32_t *>(tot + 2 * kChainPairs * (kChainThreads / 32));
-    unsigned char *pub = reinterpret_cast<unsigned char *>(orw + 32);
-
-    uint64_t a[NJ][2], b[NJ][2];
     uint64_t any = uint64_t(dt);
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
@@ -522,11 +520,11 @@ __device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const int64_t
     }
     const uint32_t hi = __reduce_or_sync(0xffffffffu, uint32_t(any >> 32));
     if (lane == 0) orw[warp] = hi;
-    for (int w = tid; w < W; w += NT) word[w] = 0u;
     __syncthreads();
     // every warp scans the partial sums: lane q holds those of warp q
     const uint32_t all = __reduce_or_sync(0xffffffffu, lane < NW ? orw[lane] : 0u);
-    uint64_t aL = 0, bL = 0;
+    aL = 0;
+    bL = 0;
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
         uint64_t sa = lane < NW ? tot[j * NW + lane] : 0u, sb = lane < NW ? tot[(NJ + j) * NW + lane] : 0u;
@@ -541,11 +539,31 @@ __device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const int64_t
         aL += __shfl_sync(0xffffffffu, sa, 31);
         bL += __shfl_sync(0xffffffffu, sb, 31);
     }
-    int st = DC_OK;
-    if (all >> 31)
-        st = DC_ERR_NEGATIVE;
-    else if (all >> 20 || exceeds_range(L, dt, FWD ? bL : aL, FWD ? aL : bL))
-        st = DC_ERR_RANGE;
+    if (all >> 31) return DC_ERR_NEGATIVE;
+    if (all >> 20 || exceeds_range(L, dt, FWD ? bL : aL, FWD ? aL : bL)) return DC_ERR_RANGE;
+    return DC_OK;
+}
+
+// Solves instance i with the whole CTA, NJ row pairs per thread. make_kept(base,
+// range) returns the store of kept columns for values from base to base + range, with
+// `ok` false when it cannot hold them. Returns false, having written nothing, when
+// the instance is left to the work list.
+template <bool FWD, int NJ, typename MakeKept>
+__device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const int64_t *crow,
+                            const int64_t *xrow, int64_t dt, bool vec, const ChainOut &o,
+                            MakeKept make_kept)
+{
+    const int NT = blockDim.x, tid = threadIdx.x;
+    const int W = words_for(L);
+    const size_t rb = chain_row_bytes(L);
+    uint32_t *word = reinterpret_cast<uint32_t *>(smem + 2 * rb);
+    uint64_t *tot = reinterpret_cast<uint64_t *>(smem + 2 * rb + chain_word_bytes(L));
+    uint32_t *orw = reinterpret_cast<uint32_t *>(tot + 2 * kChainPairs * (kChainThreads / 32));
+    unsigned char *pub = reinterpret_cast<unsigned char *>(orw + 32);
+
+    for (int w = tid; w < W; w += NT) word[w] = 0u;
+    uint64_t a[NJ][2], b[NJ][2], aL, bL;
+    const int st = cta_prefix<FWD, NJ>(tot, orw, L, crow, xrow, dt, vec, a, b, aL, bL);
     if (st != DC_OK) {
         chain_failure(st, i, W, tid, NT, o);
         return true;

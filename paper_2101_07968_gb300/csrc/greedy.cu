@@ -12,23 +12,33 @@
 //    slack; with none meeting it, the largest slack; the loop runs while m < L;
 //  * Algorithm 2's "estimated total execution time" is f_m, the backward replay.
 //
-// Prefix sums are non-decreasing, which makes each choice a short monotone scan
-// instead of the listings' enumerations:
+// Prefix sums are non-decreasing, which makes each choice a search instead of the
+// listings' enumerations:
 //  * forward: D1 is valid iff dt + P[L] - P[D1] >= FC[D1] (take D2 = L), a prefix
 //    of [1, L-1]; its largest FC is at the last valid D1 and the smallest P among
 //    equal FC at the first D1 of that plateau (a lower D1 never has a larger
 //    minimum slack). D2, and every later step, is the first x whose transfer
 //    covers the compute (minimum slack), else the first x reaching P[L];
 //  * backward: the positions x meeting k*dt + GT[m..L] >= BC[x..m-1] form a
-//    suffix [x*, m-1]; the minimum slack is at x*, found by one downward scan;
-//    with none, the largest slack is at m-1, extended down over zero-compute
-//    layers (ties keep the lowest x).
+//    suffix [x*, m-1]; the minimum slack is at x*; with none, the largest slack is
+//    at m-1, extended down over zero-compute layers (ties keep the lowest x).
 // Segment boundaries come in time order, so f_m is accumulated on the fly
 // (forward: end_s = max(end_{s-1}, s*dt + P[b_s]) + FC[b_s] - FC[b_{s-1}];
 // backward: link = max(link, BC[q..L]) + dt + GT of the segment).
-#include "common.cuh"
+//
+// Two kernels, chosen in per_thread. One instance per thread scans its own rows: O(L) for
+// Algorithm 1, O(L^2) for Algorithm 2, bound by the latency of its uncoalesced reads.
+// One instance per CTA (a single warp up to L = 64) has its prefix sums in shared
+// memory: Algorithm 1's one chain takes a 32-way search per step, and Algorithm 2's
+// L - 1 chains, one per second position, run one per thread with a binary search per
+// step; it is bound by integer issue and by the longest chain of the warp.
+// 65,537 x 54 (ResNet-50): backward 142 us, 1,554 one instance per thread.
+#include "chain.cuh"
 
 namespace dc {
+
+int sm_count();  // SMs of the current device (dp_small.cu)
+
 namespace {
 
 __device__ __forceinline__ int instance_check(int L, const int64_t *c, const int64_t *x, int64_t dt,
@@ -108,7 +118,6 @@ __device__ void greedy_fwd(int L, const int64_t *fc, const int64_t *pt, int64_t 
     end = max(end, 2 * dt + Pm) + (FCm - FC1);
     int s = 2;
     set_bit(bits, d1);
-    int n = d1;
     int64_t FCn = FC1;
     while (m < L) {
         set_bit(bits, m);
@@ -139,13 +148,11 @@ __device__ void greedy_fwd(int L, const int64_t *fc, const int64_t *pt, int64_t 
         }
         ++s;
         end = max(end, int64_t(s) * dt + Px) + (FCx - FCm);
-        n = m;
         FCn = FCm;
         m = j;
         Pm = Px;
         FCm = FCx;
     }
-    (void)n;
     *makespan = end;
 }
 
@@ -248,6 +255,246 @@ __global__ void __launch_bounds__(128) greedy_kernel(int64_t batch, int L,
         greedy_bwd(L, c, x, dti, int64_t(sc), int64_t(sx), w, makespan + i);
 }
 
+struct GreedyArgs {
+    int64_t batch;
+    int L;
+    const int64_t *comp, *xfer, *dt;
+    int64_t *makespan;
+    uint32_t *bits;
+    int vec;  // the cost rows are 16-byte aligned
+};
+
+// Prefixes A, B of rows 0..L (chain.cuh's a and b), then the decision words, the
+// scan's partial sums and flags, and the warps' best chains.
+__host__ __device__ inline size_t greedy_row_bytes(int L) { return (size_t(L + 2) * 8 + 15) / 16 * 16; }
+constexpr size_t kGreedyScratch = size_t(2 * kChainPairs * (kChainThreads / 32)) * 8 + 32 * 4 + 32 * 16;
+__host__ __device__ inline size_t greedy_smem_bytes(int L)
+{
+    return 2 * greedy_row_bytes(L) + chain_word_bytes(L) + kGreedyScratch;
+}
+
+// Algorithm 1 by one warp.
+template <typename T>
+__device__ T greedy_forward_warp(const T *A, const T *B, int L, T dt, uint32_t *word)
+{
+    const T aL = A[L];
+    auto mark = [&](int l) {
+        if ((threadIdx.x & 31) == 0) set_bit(word, l);
+    };
+    const int last = warp_first(1, L - 1, [&](int d) { return A[d] + B[d] > dt + aL; }) - 1;
+    int n = 1, m;
+    if (last >= 1) {
+        n = warp_first(1, last - 1, [&](int d) { return B[d] >= B[last]; });
+        const T thr = A[n] + B[n] - dt;
+        m = warp_first(n + 1, L - n - 1, [&](int x) { return A[x] >= thr; });
+    } else {
+        m = warp_first(2, L - 2, [&](int x) { return A[x] >= aL; });
+    }
+    mark(n);
+    T pull = dt + dt, end = dt + A[n] + B[n];
+    end = max(end, pull + A[m]) + (B[m] - B[n]);
+    while (m < L) {
+        mark(m);
+        // the first x that covers the segment's compute, else the first with all transfers
+        const T thr = min(A[m] + (B[m] - B[n]) - dt, aL);
+        const int x = warp_first(m + 1, L - m - 1, [&](int q) { return A[q] >= thr; });
+        pull += dt;
+        end = max(end, pull + A[x]) + (B[x] - B[m]);
+        n = m;
+        m = x;
+    }
+    return end;
+}
+
+// One chain of Algorithm 2 whose first push holds the last p layers; visit(q) for
+// every break. Returns its f_m.
+template <typename T, typename Visit>
+__device__ __forceinline__ T greedy_chain(const T *A, const T *B, int L, int P, T dt, int p, Visit visit)
+{
+    T link = A[p] + dt + B[p], sent = dt;
+    visit(p);
+    while (p < L) {
+        // the longest segment whose compute the link estimate covers, else one layer
+        // and the zero-compute layers after it
+        const T lim = max(A[p] + sent + B[p], A[p + 1]);
+        int q = p + 1;
+        for (int st = P; st > 0; st >>= 1)
+            if (q + st <= L && A[q + st] <= lim) q += st;
+        link = max(link, A[q]) + dt + (B[q] - B[p]);
+        sent += dt;
+        p = q;
+        if (p < L) visit(p);
+    }
+    return link;
+}
+
+// Algorithm 2 by the CTA; the result in thread 0.
+template <typename T>
+__device__ T greedy_backward_cta(const T *A, const T *B, int L, T dt, uint32_t *word, longlong2 *best_of)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = blockDim.x >> 5;
+    int P = 1;
+    while (2 * P < L) P *= 2;
+    T best = T(0);
+    int at = 0;  // ties keep the longest first push (the lowest second position)
+    uint64_t mask = 0;
+    for (int p = 1 + tid; p < L; p += int(blockDim.x)) {
+        uint64_t breaks = 0;
+        const T t = greedy_chain(A, B, L, P, dt, p, [&](int q) { breaks |= uint64_t(1) << ((q - 1) & 63); });
+        if (at == 0 || t <= best) {
+            best = t;
+            at = p;
+            mask = breaks;
+        }
+    }
+    int64_t key = at ? int64_t(best) : INT64_MAX;
+    int from = at;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        const int64_t k = __shfl_xor_sync(0xffffffffu, key, d);
+        const int f = __shfl_xor_sync(0xffffffffu, from, d);
+        if (k < key || (k == key && f > from)) {
+            key = k;
+            from = f;
+        }
+    }
+    if (NW > 1) {
+        if (lane == 0) best_of[warp] = make_longlong2(key, from);
+        __syncthreads();
+        for (int w = 0; w < NW; ++w) {
+            const longlong2 o = best_of[w];
+            if (o.x < key || (o.x == key && int(o.y) > from)) {
+                key = o.x;
+                from = int(o.y);
+            }
+        }
+    }
+    if (L <= 64) {  // one warp or two: the chain's own breaks
+        if (at == from) {
+            word[0] = uint32_t(mask);
+            if (L > 33) word[1] = uint32_t(mask >> 32);
+        }
+    } else if (tid == 0) {
+        greedy_chain(A, B, L, P, dt, from, [&](int q) { set_bit(word, q); });
+    }
+    __syncthreads();
+    return T(key);
+}
+
+template <bool FWD, typename T, int NJ>
+__device__ void greedy_solve(unsigned char *smem, uint32_t *word, longlong2 *best_of, int64_t i,
+                             const GreedyArgs &g, T dt, const uint64_t (&a)[NJ][2],
+                             const uint64_t (&b)[NJ][2], uint64_t aL, uint64_t bL)
+{
+    const int L = g.L, tid = threadIdx.x, NT = blockDim.x, W = words_for(L);
+    T *A = reinterpret_cast<T *>(smem), *B = reinterpret_cast<T *>(smem + greedy_row_bytes(L));
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        const int r = 2 * (j * NT + tid) + 1;
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            if (r + u <= L) {
+                A[r + u] = T(a[j][u]);
+                B[r + u] = T(b[j][u]);
+            }
+    }
+    if (tid == 0) {
+        A[0] = T(0);
+        B[0] = T(0);
+    }
+    __syncthreads();
+    T t = T(aL) + T(bL) + dt;  // L = 1: one segment
+    if (L > 1) {
+        if (!FWD)
+            t = greedy_backward_cta(A, B, L, dt, word, best_of);
+        else if (tid < 32)
+            t = greedy_forward_warp(A, B, L, dt, word);
+        if (FWD) __syncwarp();
+    }
+    if (tid < 32) {
+        if (tid == 0) g.makespan[i] = int64_t(t);
+        for (int w = tid; w < W; w += 32) g.bits[i * W + w] = word[w];
+    }
+}
+
+template <bool FWD, int NJ>
+__global__ void __launch_bounds__(kChainThreads, 1) greedy_cta_kernel(GreedyArgs g)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int L = g.L, W = words_for(L), tid = threadIdx.x, NT = blockDim.x;
+    uint32_t *word = reinterpret_cast<uint32_t *>(smem + 2 * greedy_row_bytes(L));
+    uint64_t *tot = reinterpret_cast<uint64_t *>(smem + 2 * greedy_row_bytes(L) + chain_word_bytes(L));
+    uint32_t *orw = reinterpret_cast<uint32_t *>(tot + 2 * kChainPairs * (kChainThreads / 32));
+    longlong2 *best_of = reinterpret_cast<longlong2 *>(orw + 32);
+    for (int64_t i = blockIdx.x; i < g.batch; i += gridDim.x) {
+        const int64_t dt = __ldg(g.dt + i);
+        for (int w = tid; w < W; w += NT) word[w] = 0u;
+        uint64_t a[NJ][2], b[NJ][2], aL, bL;
+        const int st = cta_prefix<FWD, NJ>(tot, orw, L, g.comp + i * L, g.xfer + i * L, dt, g.vec, a, b, aL, bL);
+        if (st != DC_OK) {
+            if (tid == 0) g.makespan[i] = -int64_t(st);
+            for (int w = tid; w < W; w += NT) g.bits[i * W + w] = 0u;
+        } else if (aL + bL + uint64_t(L + 1) * uint64_t(dt) < (uint64_t(1) << 31)) {
+            greedy_solve<FWD, int32_t, NJ>(smem, word, best_of, i, g, int32_t(dt), a, b, aL, bL);
+        } else {
+            greedy_solve<FWD, int64_t, NJ>(smem, word, best_of, i, g, dt, a, b, aL, bL);
+        }
+        __syncthreads();  // shared memory is read
+    }
+}
+
+template <bool FWD, int NJ>
+cudaError_t launch_greedy_cta(const GreedyArgs &g, int nt, cudaStream_t stream)
+{
+    static DeviceCache attr;  // the kernel's shared-memory limit, raised once per device
+    int done = 0;
+    cudaError_t e = attr.get(done, [](int &v) {
+        v = 1;
+        return cudaFuncSetAttribute(greedy_cta_kernel<FWD, NJ>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    int(greedy_smem_bytes(DC_L_MAX)));
+    });
+    if (e != cudaSuccess) return e;
+    const size_t smem = greedy_smem_bytes(g.L);
+    int nb = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, greedy_cta_kernel<FWD, NJ>, nt, smem);
+    if (e != cudaSuccess) return e;
+    // four waves of CTAs, each walking every grid-th instance: chains differ in length
+    int64_t grid = int64_t(nb < 1 ? 1 : nb) * sm_count() * 4;
+    if (grid > g.batch) grid = g.batch;
+    greedy_cta_kernel<FWD, NJ><<<unsigned(grid), nt, smem, stream>>>(g);
+    return cudaGetLastError();
+}
+
+// One instance per thread where a warp's lanes are better used on 32 instances than on
+// one short row. Forward: up to L = 32 (100,000 x 20: 41 us against 76 per CTA; equal at
+// 32), and up to 128 on large batches (100,000 x 100: 139 against 152; but 10,000 x 100:
+// 50 against 39). Backward, quadratic in L per thread: up to L = 8, and up to 12 on large
+// batches (100,000 x 12: 82 us against about 95; 100,000 x 17: 174 against 98).
+template <bool FWD>
+bool per_thread(int64_t batch, int L)
+{
+    if (FWD) return L <= 32 || (L <= 128 && batch >= 50000);
+    return L <= 8 || (L <= 12 && batch >= 50000);
+}
+
+template <bool FWD>
+cudaError_t launch_greedy(int64_t batch, int L, const int64_t *comp, const int64_t *xfer,
+                          const int64_t *dt, int64_t *makespan, uint32_t *bits, cudaStream_t stream)
+{
+    if (per_thread<FWD>(batch, L)) {
+        greedy_kernel<FWD><<<unsigned((batch + 127) / 128), 128, 0, stream>>>(batch, L, comp, xfer, dt,
+                                                                             makespan, bits);
+        return cudaGetLastError();
+    }
+    const bool vec = (L % 2 == 0) &&
+                     ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0;
+    const GreedyArgs g{batch, L, comp, xfer, dt, makespan, bits, vec ? 1 : 0};
+    const int nt = 32 * ((L + 63) / 64);
+    return nt <= kChainThreads ? launch_greedy_cta<FWD, 1>(g, nt, stream)
+                               : launch_greedy_cta<FWD, 2>(g, 32 * ((L + 127) / 128), stream);
+}
+
 }  // namespace
 }  // namespace dc
 
@@ -260,9 +507,9 @@ extern "C" dc_status dc_greedy_forward_batch(int64_t batch, int32_t L, const int
     if (batch < 0 || L < 1 || L > DC_L_MAX || batch > int64_t(0xffffffffll)) return DC_ERR_BAD_SHAPE;
     if (batch == 0) return DC_OK;
     if (!fc || !pt || !dt || !makespan || (!bits && dc::words_for(L) > 0)) return DC_ERR_NULL;
-    const unsigned grid = unsigned((batch + 127) / 128);
-    dc::greedy_kernel<true><<<grid, 128, 0, stream>>>(batch, L, fc, pt, dt, makespan, bits);
-    return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+    return dc::launch_greedy<true>(batch, L, fc, pt, dt, makespan, bits, stream) == cudaSuccess
+               ? DC_OK
+               : DC_ERR_CUDA;
 }
 
 extern "C" dc_status dc_greedy_backward_batch(int64_t batch, int32_t L, const int64_t *bc,
@@ -274,7 +521,7 @@ extern "C" dc_status dc_greedy_backward_batch(int64_t batch, int32_t L, const in
     if (batch < 0 || L < 1 || L > DC_L_MAX || batch > int64_t(0xffffffffll)) return DC_ERR_BAD_SHAPE;
     if (batch == 0) return DC_OK;
     if (!bc || !gt || !dt || !makespan || (!bits && dc::words_for(L) > 0)) return DC_ERR_NULL;
-    const unsigned grid = unsigned((batch + 127) / 128);
-    dc::greedy_kernel<false><<<grid, 128, 0, stream>>>(batch, L, bc, gt, dt, makespan, bits);
-    return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+    return dc::launch_greedy<false>(batch, L, bc, gt, dt, makespan, bits, stream) == cudaSuccess
+               ? DC_OK
+               : DC_ERR_CUDA;
 }

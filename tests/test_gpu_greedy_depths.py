@@ -1,0 +1,89 @@
+"""The CTA-per-instance greedy schedulers at depths around their warp, row-pair and
+search boundaries, in 32 and in 64 bits, against the oracle; above L = 600, where the
+oracle's backward enumeration is too slow, against the same rule by bisection."""
+import bisect
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2101_07968_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dc():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2101_07968_gb300 import build, dynacomm
+    build.build()
+    dynacomm.lib()
+    return dynacomm
+
+
+def _run(dc, d, comp, xfer, dt):
+    import torch
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    out = dc.greedy(d, t(comp), t(xfer), t(dt))
+    return out["makespan"].cpu().numpy(), out["bits"].cpu().numpy().view(np.uint32)
+
+
+def _instances(L, B, wide):
+    comp, xfer, dt = wl.skewed_instances(91 + L, B, L)
+    comp[::4] = 0                      # no compute at all: every position ties
+    comp[1::4, L // 3:] = 0            # a zero-compute tail and head
+    if wide:
+        comp[2::4] <<= 20
+        xfer[::2] <<= 18
+    return comp, xfer, dt
+
+
+@pytest.mark.parametrize("wide", [False, True])
+@pytest.mark.parametrize("L", [17, 18, 33, 34, 63, 64, 65, 66, 127, 128, 129, 257])
+def test_depths(dc, L, wide):
+    comp, xfer, dt = _instances(L, 21, wide)
+    for d in (0, 1):
+        mk, bits = _run(dc, d, comp, xfer, dt)
+        exp = oracle.greedy_batch(d, comp, xfer, dt, nthreads=os.cpu_count() or 1)
+        assert np.array_equal(mk, exp["makespan"]) and np.array_equal(bits, exp["bits"]), (L, d)
+
+
+def _backward(bc, gt, dt):
+    """Algorithm 2 in processing order: every first push p, each next segment as long
+    as the link estimate covers, least f_m, the longest first push on ties."""
+    A, B = [0], [0]
+    for c, x in zip(bc[::-1].tolist(), gt[::-1].tolist()):
+        A.append(A[-1] + c)
+        B.append(B[-1] + x)
+    L, best = len(bc), None
+    for p0 in range(L - 1, 0, -1):
+        p, sent, link, cuts = p0, dt, A[p0] + dt + B[p0], []
+        while p < L:
+            cuts.append(p)
+            q = bisect.bisect_right(A, max(A[p] + sent + B[p], A[p + 1])) - 1
+            link = max(link, A[q]) + dt + B[q] - B[p]
+            p, sent = q, sent + dt
+        if best is None or link < best[0]:
+            best = (link, cuts)
+    return best
+
+
+@pytest.mark.parametrize("L", [600, 1025, 2049])
+def test_deep(dc, L):
+    comp, xfer, dt = _instances(L, 5, True)
+    mk, bits = _run(dc, 0, comp, xfer, dt)
+    if L <= 1025:  # the oracle enumerates every pair
+        exp = oracle.greedy_batch(0, comp, xfer, dt, nthreads=os.cpu_count() or 1)
+        assert np.array_equal(mk, exp["makespan"]) and np.array_equal(bits, exp["bits"])
+    else:
+        assert np.array_equal(mk, oracle.replay_batch(0, comp, xfer, dt, bits))
+    mk, bits = _run(dc, 1, comp, xfer, dt)
+    for i in range(len(dt)):
+        t, cuts = _backward(comp[i], xfer[i], int(dt[i]))
+        word = np.zeros(dc.words(L), np.uint32)
+        for q in cuts:
+            word[(q - 1) // 32] |= np.uint32(1 << ((q - 1) % 32))
+        assert mk[i] == t and np.array_equal(bits[i], word), (L, i)
