@@ -116,7 +116,6 @@ __global__ void __launch_bounds__(32, DC_SMALL_MINB)
                 uvb[32 * (L + 1 + m)] = Vb[m];
             }
         }
-        if (!active) return;
 #pragma unroll 1
         for (int dir = 0; dir < 2; ++dir) {
             const bool fwd = dir == 0;
@@ -127,12 +126,13 @@ __global__ void __launch_bounds__(32, DC_SMALL_MINB)
                 U[m] = uv[32 * m];
                 V[m] = uv[32 * (L + 1 + m)];
             }
-            if (st[dir] != DC_OK) {
+            const bool run = active && st[dir] == DC_OK && !wide[dir];
+            const bool done = solve_uv<L>(fwd, run, U, V, int32_t(dti), xraw[dir], lw, i,
+                                          o.makespan[dir], o.bits[dir], o.nseg[dir], o.status[dir]);
+            if (active && st[dir] != DC_OK) {
                 write_failure(st[dir], i, W, o.makespan[dir], o.bits[dir], o.nseg[dir],
                               o.status[dir]);
-            } else if (wide[dir] || !solve_uv<L>(fwd, U, V, int32_t(dti), xraw[dir], lw, i,
-                                                 o.makespan[dir], o.bits[dir], o.nseg[dir],
-                                                 o.status[dir])) {
+            } else if (active && (wide[dir] || !done)) {
                 const uint32_t at = atomicAdd(o.wide_count[dir], 1u);
                 if (DC_CHECK(int64_t(at) < g.batch)) o.wide_list[dir][at] = uint32_t(i);
             }

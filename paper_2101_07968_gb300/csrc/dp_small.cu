@@ -14,13 +14,13 @@
 //  * the 32-bit pass solves the shifted form (see the block before fill_e in
 //    dp_small.cuh): a transition is one add-then-max and two candidates fold
 //    into one 3-input min, 1.5 integer-ALU instructions on GB300;
+//  * the columns end early, when no lane's optimum can fall any more (see fill_e);
 //  * the fill keeps only the minimum VALUE per cell; the traceback recovers
-//    Path[m][n] as the lowest k whose candidate equals the cell, which is the k
-//    Algorithm 3/4 keeps with its strict-improvement test. A step compares all
-//    of its candidates at once (bit mask, lowest set bit), and every step runs
-//    the same code (column 1 is read as U less a constant, the other kept
-//    columns from the table), so the lanes of a warp at different depths do not
-//    split into separate paths. The pass keeps only columns 1..kKeepCols: the
+//    Path[m][n], the lowest k that attains the cell, as the first k with U[m] + V[k]
+//    at most the cell: a binary search over V in registers and one load of the cell
+//    (k, n-1). Every step runs the same code (column 1 is read as U plus a constant,
+//    the other kept columns from the table), so the lanes of a warp at different
+//    depths do not split into separate paths. The pass keeps only columns 1..kKeepCols: the
 //    traceback of an s-segment optimum reads columns 1..s-1 only, and s is small
 //    in practice (2-5 on CNN-shaped profiles); an instance whose s needs a
 //    deeper column is re-solved by the 64-bit pass, which keeps every column;
@@ -92,13 +92,15 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
         if (lane == 0) v = atomicAdd(ticket, 1u);
         return v;
     };
-    // the solve of one tile's rows, held by each lane in U, V
-    auto finish = [&](int64_t i, const int32_t (&U)[L + 1], const int32_t (&V)[L + 1],
+    // the solve of one tile's rows, held by each lane in U, V; every lane takes part
+    auto finish = [&](int64_t i, bool active, const int32_t (&U)[L + 1], const int32_t (&V)[L + 1],
                       int64_t dti, uint64_t xraw, bool wide, int st) {
-        if (st != DC_OK) {
+        const bool run = active && st == DC_OK && !wide;
+        const bool done = solve_uv<L>(FWD, run, U, V, int32_t(dti), xraw, lw, i, makespan, bits,
+                                      nseg, status);
+        if (active && st != DC_OK) {
             write_failure(st, i, W, makespan, bits, nseg, status);
-        } else if (wide ||
-                   !solve_uv<L>(FWD, U, V, int32_t(dti), xraw, lw, i, makespan, bits, nseg, status)) {
+        } else if (active && (wide || !done)) {
             // 64-bit values, or a traceback deeper than the kept columns: work list
             const uint32_t at = atomicAdd(wide_count, 1u);
             if (DC_CHECK(int64_t(at) < batch)) wide_list[at] = uint32_t(i);
@@ -135,7 +137,7 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
                 next_raw = claim();
             }
             tile = next;
-            if (active) finish(i, U, V, dti, xraw, wide, st);
+            finish(i, active, U, V, dti, xraw, wide, st);
         }
     } else {
         int64_t tile = blockIdx.x;
@@ -164,7 +166,7 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
             row_uv<L, FWD>(stC + lane * K::kStride, stX + lane * K::kStride, dti, U, V, xraw,
                            wide, st);
             __syncwarp();  // rows read: the lanes' table slices may be written
-            if (active) finish(i, U, V, dti, xraw, wide, st);
+            finish(i, active, U, V, dti, xraw, wide, st);
         }
     }
 }
