@@ -124,8 +124,9 @@ size_t dc_schedule_workspace_bytes(int64_t batch, int32_t L);
 /* ------------------------------------------------------------------------
  * dc_schedule_kernel_launches -- how many kernels one dc_schedule_forward_batch
  * or dc_schedule_backward_batch call with (batch, L) launches: a first pass and
- * a second pass over its work list; for L > 256 the first pass is split into
- * launches of about 90 ms of work each (at least two resident waves), chained
+ * a second pass over its work list, or a single pass for small batches of L <= 64
+ * (some ten thousand instances); for L > 256 the first pass is split into
+ * launches of four resident waves each, chained
  * so that each may start while the one before drains. For counting only (the
  * calls need no caller action per launch). Returns 0 for batch <= 0 or L out of
  * range. Pure host function, no CUDA call.

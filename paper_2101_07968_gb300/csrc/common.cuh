@@ -248,6 +248,10 @@ cudaError_t launch_warp(bool forward, int64_t batch, int L, const int64_t *comp,
                         const int64_t *xfer, const int64_t *dt, int64_t *makespan, uint32_t *bits,
                         int32_t *nseg, int32_t *status, uint32_t *ticket, uint32_t *list_count,
                         uint32_t *list, uint32_t *slots, cudaStream_t stream);
+bool use_solo(int64_t batch, int L);  // one launch solves the batch (dp_warp.cu)
+cudaError_t launch_solo(bool forward, int64_t batch, int L, const int64_t *comp,
+                        const int64_t *xfer, const int64_t *dt, int64_t *makespan, uint32_t *bits,
+                        int32_t *nseg, int32_t *status, uint32_t *list_count, cudaStream_t stream);
 cudaError_t launch_deep(bool forward, int64_t batch, int L, const int64_t *comp,
                         const int64_t *xfer, const int64_t *dt, int64_t *makespan,
                         uint32_t *bits, int32_t *nseg, int32_t *status, uint32_t *tickets,

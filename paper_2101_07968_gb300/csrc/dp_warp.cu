@@ -14,6 +14,9 @@
 //    ballot over the lanes' b;
 //  * persistent warps take runs of instances from an atomic ticket, the next run
 //    claimed while one is solved.
+// Small batches of L <= 64 (use_solo) take one launch without tickets, work list or
+// memset: solo_kernel keeps every column, in whole values, in shared memory, so one
+// warp solves any instance to the end.
 // Bound by integer issue: the searches, the scans and the per-column bookkeeping.
 // Measured per direction against the looped thread-per-instance kernel that took
 // L <= 256 before (every candidate of every column): 262,144 x 54 (ResNet-50) 185 us
@@ -86,6 +89,20 @@ __global__ void __launch_bounds__(256, NJ == 1 ? 4 : NJ == 2 ? 3 : 2) warp_kerne
     }
 }
 
+template <bool FWD>
+__global__ void __launch_bounds__(32) solo_kernel(WarpArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int L = a.L;
+    const int64_t i = blockIdx.x;
+    int64_t *table = reinterpret_cast<int64_t *>(smem + 2 * chain_row_bytes(L));
+    if (i == 0 && threadIdx.x == 0) *a.list_count = 0u;  // nothing is left to a second pass
+    chain_solve_warp<FWD, 1>(smem, i, L, a.comp + i * L, a.xfer + i * L, __ldg(a.dt + i), a.vec,
+                             a.out, [&](int64_t, uint64_t, bool &) { return KeptValues{table, L}; });
+}
+
+inline size_t solo_smem_bytes(int L) { return 2 * chain_row_bytes(L) + size_t(tri_cells(L)) * 8; }
+
 template <bool FWD, int NJ>
 cudaError_t launch_warp_nj(WarpArgs a, cudaStream_t stream)
 {
@@ -119,6 +136,35 @@ cudaError_t launch_warp_nj(WarpArgs a, cudaStream_t stream)
 }
 
 }  // namespace
+
+// Whether one launch of solo_kernel solves the batch. It saves the memset and the list
+// pass (about 4 us on the GPU, more on the host), and a warp per instance starts sooner
+// than a thread per instance finishes (per direction, from a graph: one instance of
+// L = 16 2.2 us against 6.5, of L = 54 2.3 against 8.2; 4,000 x 16 4.8 us against 27 with
+// optima on the work list), but from a wave on it costs about 0.6 us per 1,000 instances:
+// 16,000 x 8 10.4 us against 7.6-10.3; 32,000 x 16 19.4 against 30.5 and 32,000 x 32
+// 21.9 against 35.7; 32,000 x 64, with 17.7 KB of shared memory a warp, 40.6 against 38.8.
+bool use_solo(int64_t batch, int L)
+{
+    const int64_t most = L <= 8 ? 8000 : L <= 16 ? 24000 : L <= 48 ? 40000 : L <= 64 ? 20000 : 0;
+    return batch <= most;
+}
+
+cudaError_t launch_solo(bool forward, int64_t batch, int L, const int64_t *comp,
+                        const int64_t *xfer, const int64_t *dt, int64_t *makespan, uint32_t *bits,
+                        int32_t *nseg, int32_t *status, uint32_t *list_count, cudaStream_t stream)
+{
+    const bool vec = (L % 2 == 0) &&
+                     ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0;
+    const WarpArgs a{batch, L, comp, xfer, dt, ChainOut{makespan, bits, nseg, status},
+                     nullptr, list_count, nullptr, nullptr, 1, vec ? 1 : 0};
+    const size_t smem = solo_smem_bytes(L);  // 17.7 KB at L = 64
+    if (forward)
+        solo_kernel<true><<<unsigned(batch), 32, smem, stream>>>(a);
+    else
+        solo_kernel<false><<<unsigned(batch), 32, smem, stream>>>(a);
+    return cudaGetLastError();
+}
 
 // Slots of the kept columns past shared memory: one per warp of the largest grid, and
 // no more than the batch has instances (rounded up to whole CTAs of 8).

@@ -30,6 +30,13 @@ cudaError_t launch_schedule(bool forward, int64_t batch, int L, const int64_t *c
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     // events around the first pass of a looped or deep-chain solve
     auto mark = [&](cudaEvent_t ev) { return ev ? cudaEventRecord(ev, stream) : cudaSuccess; };
+    if (use_solo(batch, L)) {  // one pass, nothing listed
+        cudaError_t e = mark(pe.start);
+        if (e != cudaSuccess) return e;
+        e = launch_solo(forward, batch, L, comp, xfer, dt, makespan, bits, nseg, status,
+                        reinterpret_cast<uint32_t *>(ws), stream);
+        return e != cudaSuccess ? e : mark(pe.stop);
+    }
     if (L <= kSmallLMax) {
         // header: work-list counter, then the dense pass's tile ticket
         uint32_t *count = reinterpret_cast<uint32_t *>(ws);
@@ -152,6 +159,7 @@ dc_status dc_schedule_generated_batch(const dc_profile_cfg *cfg, int64_t *makesp
 int32_t dc_schedule_kernel_launches(int64_t batch, int32_t L)
 {
     if (batch <= 0 || L < 1 || L > DC_L_MAX) return 0;
+    if (dc::use_solo(batch, L)) return 1;
     if (L <= dc::kMidLMax) return 2;
     return int32_t(dc::deep_launches(batch, L) + 1);
 }
