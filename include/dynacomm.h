@@ -224,6 +224,22 @@ dc_status dc_eval_timeline_batch(int64_t batch, int32_t L, int32_t dir, const in
                                  int64_t *makespan, cudaStream_t stream);
 
 /* ------------------------------------------------------------------------
+ * dc_schedule_replay_batch -- dc_schedule_forward_batch (dir 0) or
+ * dc_schedule_backward_batch (dir 1) and, for each instance, the cost measurement
+ * f_m of the decision it writes, evaluated while the instance's prefix sums are on
+ * chip: replay [batch] holds what dc_eval_timeline_batch gives for the same rows
+ * and bits (-(status) for a failed instance). comp, xfer: fc, pt or bc, gt; the
+ * other arguments, the workspace and the errors as for the schedule calls (replay
+ * NULL: DC_ERR_NULL; dir not 0/1: DC_ERR_BAD_SHAPE). A dc_time_next_pass request
+ * is used up here too.
+ * ---------------------------------------------------------------------- */
+dc_status dc_schedule_replay_batch(int32_t dir, int64_t batch, int32_t L, const int64_t *comp,
+                                   const int64_t *xfer, const int64_t *dt, int64_t *makespan,
+                                   uint32_t *bits, int32_t *nseg, int32_t *status,
+                                   int64_t *replay, void *workspace, size_t workspace_bytes,
+                                   cudaStream_t stream);
+
+/* ------------------------------------------------------------------------
  * dc_schedule_batch_static -- the paper has no counterpart: this is a
  * deployment variant of the two schedule calls above for callers that cannot
  * allocate device memory where they schedule (a scheduler embedded in a

@@ -98,12 +98,6 @@ struct KeptValues {
     }
 };
 
-struct ChainOut {
-    int64_t *makespan;
-    uint32_t *bits;
-    int32_t *nseg, *status;
-};
-
 template <typename T>
 struct Pair;
 template <>
@@ -180,7 +174,7 @@ template <bool FWD, typename T, int NJ, bool WARP, int TOP, typename Kept>
 __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub, int tid, int NT,
                                               int64_t i, int L, T dt, const T (&a)[NJ][2],
                                               const T (&b)[NJ][2], T aL, T bL, const Kept &kept,
-                                              const ChainOut &o)
+                                              const SolveOut &o)
 {
     using P2 = Pair<T>;
     using Two = typename P2::type;
@@ -282,6 +276,9 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
     int err = 0, m = L, n = s;
     T v = hL;
     uint32_t mine = 0u;  // WARP: lane w's decision word w
+    // f_m of the decision, from its own segments: the largest over its segments j of
+    // c_j + a[end] - b[start] + (s - j) e, then the same e + b[L] as T
+    T span = T(0), later = T(0);
     T cn = FWD ? T(n) * dt : T(0);
     while (n > 1) {
         const T thr = cn + K[m - 1] - v;
@@ -304,6 +301,11 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
             err = 1;
             break;
         }
+        if (o.replay) {
+            const T w = cn + K[m - 1] - B[k - 1] + later;
+            span = n == s ? w : max(span, w);
+            later += e;
+        }
         const uint32_t bit = 1u << ((k - 1) & 31);
         if (WARP)
             mine |= lane == ((k - 1) >> 5) ? bit : 0u;
@@ -314,8 +316,13 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
         n -= 1;
         if (FWD) cn -= dt;
     }
+    if (o.replay) {
+        const T first = h1 + later + (s > 1 ? K[m - 1] : aL);  // the first segment
+        span = s > 1 ? max(span, first) : first;
+    }
     if (!WARP) __syncwarp();
     if (lane == 0) {
+        if (o.replay) o.replay[i] = err ? -int64_t(DC_ERR_INTERNAL) : int64_t(span + e) + int64_t(bL);
         o.makespan[i] = err ? -int64_t(DC_ERR_INTERNAL) : int64_t(hL + e) + int64_t(bL);
         if (o.nseg) o.nseg[i] = err ? 0 : s;
         if (o.status) o.status[i] = err ? DC_ERR_INTERNAL : DC_OK;
@@ -328,35 +335,49 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
     return true;
 }
 
-__device__ __forceinline__ void chain_failure(int st, int64_t i, int W, int tid, int NT, const ChainOut &o)
+__device__ __forceinline__ void chain_failure(int st, int64_t i, int W, int tid, int NT, const SolveOut &o)
 {
     if (tid == 0) {
         o.makespan[i] = -int64_t(st);
         if (o.nseg) o.nseg[i] = 0;
         if (o.status) o.status[i] = st;
+        if (o.replay) o.replay[i] = -int64_t(st);
     }
     for (int w = tid; w < W; w += NT) o.bits[i * W + w] = 0u;
 }
 
-// The costs of rows r, r+1 (r odd; zero past L) of an instance's rows in processing
-// order. vec: the rows are 16-byte aligned and L is even.
+// Where an instance's costs come from: operator()(r, c0, c1, x0, x1) gives the compute
+// and transfer costs of rows r, r+1 (r odd) in processing order, zero past L. This one
+// reads its rows; vec: they are 16-byte aligned and L is even.
 template <bool FWD>
-__device__ __forceinline__ void load_pair(const int64_t *row, int L, int r, bool vec, uint64_t &v0,
-                                          uint64_t &v1)
-{
-    v0 = 0;
-    v1 = 0;
-    if (r > L) return;
-    if (vec) {
-        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(row + (FWD ? r - 1 : L - r - 1)));
-        v0 = FWD ? v.x : v.y;
-        v1 = FWD ? v.y : v.x;
-    } else {
-        const int at = FWD ? r - 1 : L - r;
-        v0 = uint64_t(__ldg(row + at));
-        if (r < L) v1 = uint64_t(__ldg(row + (FWD ? at + 1 : at - 1)));
+struct RowLoader {
+    const int64_t *crow, *xrow;
+    int L;
+    bool vec;
+    __device__ __forceinline__ void operator()(int r, uint64_t &c0, uint64_t &c1, uint64_t &x0,
+                                               uint64_t &x1) const
+    {
+        c0 = c1 = x0 = x1 = 0;
+        if (r > L) return;
+        if (vec) {
+            const int at = FWD ? r - 1 : L - r - 1;
+            const ulonglong2 c = __ldg(reinterpret_cast<const ulonglong2 *>(crow + at));
+            const ulonglong2 x = __ldg(reinterpret_cast<const ulonglong2 *>(xrow + at));
+            c0 = FWD ? c.x : c.y;
+            c1 = FWD ? c.y : c.x;
+            x0 = FWD ? x.x : x.y;
+            x1 = FWD ? x.y : x.x;
+        } else {
+            const int at = FWD ? r - 1 : L - r, next = FWD ? at + 1 : at - 1;
+            c0 = uint64_t(__ldg(crow + at));
+            x0 = uint64_t(__ldg(xrow + at));
+            if (r < L) {
+                c1 = uint64_t(__ldg(crow + next));
+                x1 = uint64_t(__ldg(xrow + next));
+            }
+        }
     }
-}
+};
 
 // Inclusive prefixes over a warp's lanes of two values at once.
 template <typename U>
@@ -393,10 +414,9 @@ __device__ __forceinline__ void scan2_flag(uint32_t &sa, uint32_t &sb, uint32_t 
 // Solves instance i with one warp, NJ row pairs per lane (L <= 64 NJ). smem: the
 // warp's K and b. make_kept as in chain_solve. Returns false, having written nothing,
 // when the instance is left to the work list.
-template <bool FWD, int NJ, typename MakeKept>
+template <bool FWD, int NJ, typename Load, typename MakeKept>
 __device__ __forceinline__ bool chain_solve_warp(unsigned char *smem, int64_t i, int L,
-                                                 const int64_t *crow, const int64_t *xrow,
-                                                 int64_t dt, bool vec, const ChainOut &o,
+                                                 const Load &load, int64_t dt, const SolveOut &o,
                                                  MakeKept make_kept)
 {
     constexpr unsigned kAll = 0xffffffffu;
@@ -408,8 +428,10 @@ __device__ __forceinline__ bool chain_solve_warp(unsigned char *smem, int64_t i,
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
         const int r = 2 * (32 * j + lane) + 1;
-        load_pair<FWD>(FWD ? xrow : crow, L, r, vec, a[j][0], a[j][1]);
-        load_pair<FWD>(FWD ? crow : xrow, L, r, vec, b[j][0], b[j][1]);
+        if (FWD)
+            load(r, b[j][0], b[j][1], a[j][0], a[j][1]);
+        else
+            load(r, a[j][0], a[j][1], b[j][0], b[j][1]);
         hi |= uint32_t((a[j][0] | a[j][1] | b[j][0] | b[j][1]) >> 32);
         flag |= uint32_t(a[j][0] | a[j][1] | b[j][0] | b[j][1]);
     }
@@ -489,14 +511,13 @@ __host__ __device__ inline size_t chain_smem_bytes(int L)
 }
 
 // The prefixes of an instance's rows over the whole CTA, in processing order (a, b and
-// the row layout of chain_columns; 64-bit). tot, orw: scratch. One CTA barrier, which
-// also publishes what the threads wrote to shared memory before. Returns the
+// the row layout of chain_columns; 64-bit). tot, orw: scratch; first: a[1], published,
+// like what the threads wrote to shared memory before, by the one CTA barrier in here. Returns the
 // instance's status: DC_OK or its input error.
-template <bool FWD, int NJ>
-__device__ __forceinline__ int cta_prefix(uint64_t *tot, uint32_t *orw, int L, const int64_t *crow,
-                                          const int64_t *xrow, int64_t dt, bool vec,
-                                          uint64_t (&a)[NJ][2], uint64_t (&b)[NJ][2], uint64_t &aL,
-                                          uint64_t &bL)
+template <bool FWD, int NJ, typename Load>
+__device__ __forceinline__ int cta_prefix(uint64_t *tot, uint32_t *orw, uint64_t *first, int L,
+                                          const Load &load, int64_t dt, uint64_t (&a)[NJ][2],
+                                          uint64_t (&b)[NJ][2], uint64_t &aL, uint64_t &bL)
 {
     const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = NT >> 5;
     uint64_t any = uint64_t(dt);
@@ -504,8 +525,11 @@ __device__ __forceinline__ int cta_prefix(uint64_t *tot, uint32_t *orw, int L, c
     for (int j = 0; j < NJ; ++j) {
         const int r = 2 * (j * NT + tid) + 1;
         uint64_t a0, a1, b0, b1;
-        load_pair<FWD>(FWD ? xrow : crow, L, r, vec, a0, a1);
-        load_pair<FWD>(FWD ? crow : xrow, L, r, vec, b0, b1);
+        if (FWD)
+            load(r, b0, b1, a0, a1);
+        else
+            load(r, a0, a1, b0, b1);
+        if (j == 0 && tid == 0) *first = a0;
         any |= a0 | a1 | b0 | b1;
         uint64_t sa = a0 + a1, sb = b0 + b1;
         scan2(sa, sb, lane);
@@ -548,10 +572,9 @@ __device__ __forceinline__ int cta_prefix(uint64_t *tot, uint32_t *orw, int L, c
 // range) returns the store of kept columns for values from base to base + range, with
 // `ok` false when it cannot hold them. Returns false, having written nothing, when
 // the instance is left to the work list.
-template <bool FWD, int NJ, typename MakeKept>
-__device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const int64_t *crow,
-                            const int64_t *xrow, int64_t dt, bool vec, const ChainOut &o,
-                            MakeKept make_kept)
+template <bool FWD, int NJ, typename Load, typename MakeKept>
+__device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const Load &load, int64_t dt,
+                            const SolveOut &o, MakeKept make_kept)
 {
     const int NT = blockDim.x, tid = threadIdx.x;
     const int W = words_for(L);
@@ -563,7 +586,8 @@ __device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const int64_t
 
     for (int w = tid; w < W; w += NT) word[w] = 0u;
     uint64_t a[NJ][2], b[NJ][2], aL, bL;
-    const int st = cta_prefix<FWD, NJ>(tot, orw, L, crow, xrow, dt, vec, a, b, aL, bL);
+    const int st = cta_prefix<FWD, NJ>(tot, orw, reinterpret_cast<uint64_t *>(pub), L, load, dt, a,
+                                       b, aL, bL);
     if (st != DC_OK) {
         chain_failure(st, i, W, tid, NT, o);
         return true;
@@ -593,9 +617,9 @@ __device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const int64_t
             a64[j][u] = int64_t(a[j][u]);
             b64[j][u] = int64_t(b[j][u]);
         }
-    // H lies between H[1][1] and H[L][1]; the first row's a is the smallest cost
+    // H lies between H[1][1] and H[L][1]
     const int64_t h1 = FWD ? dt : 0;
-    const int64_t a1 = __ldg((FWD ? xrow : crow) + (FWD ? 0 : L - 1));
+    const int64_t a1 = *reinterpret_cast<const int64_t *>(pub);
     bool ok = true;
     const auto kept = make_kept(h1 + a1, aL - uint64_t(a1), ok);
     if (!ok) return false;

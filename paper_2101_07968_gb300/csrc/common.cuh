@@ -225,38 +225,53 @@ struct PassEvents {
 };
 PassEvents take_pass_events();  // this thread's request, cleared (dynacomm_abi.cu)
 
+// Outputs of a solve; nseg, status and replay (f_m of the written decision) may be
+// null.
+struct SolveOut {
+    int64_t *makespan;
+    uint32_t *bits;
+    int32_t *nseg, *status;
+    int64_t *replay;
+};
+
+// Outputs of an instance with an input error: -(status) as its makespan and replay.
+__device__ __forceinline__ void write_failure(int st, int64_t i, int W, const SolveOut &o)
+{
+    o.makespan[i] = -int64_t(st);
+    if (o.nseg) o.nseg[i] = 0;
+    if (o.status) o.status[i] = st;
+    if (o.replay) o.replay[i] = -int64_t(st);
+    for (int w = 0; w < W; ++w) o.bits[i * W + w] = 0u;
+}
+
 // Kernel launchers implemented in the .cu files.
 cudaError_t launch_schedule(bool forward, int64_t batch, int L, const int64_t *comp,
-                            const int64_t *xfer, const int64_t *dt, int64_t *makespan,
-                            uint32_t *bits, int32_t *nseg, int32_t *status, void *workspace,
-                            const PassEvents &pe, cudaStream_t stream);
+                            const int64_t *xfer, const int64_t *dt, const SolveOut &out,
+                            void *workspace, const PassEvents &pe, cudaStream_t stream);
 cudaError_t launch_small(bool forward, int64_t batch, int L, const int64_t *comp,
-                         const int64_t *xfer, const int64_t *dt, int64_t *makespan,
-                         uint32_t *bits, int32_t *nseg, int32_t *status,
+                         const int64_t *xfer, const int64_t *dt, const SolveOut &out,
                          uint32_t *wide_count, uint32_t *wide_list, const PassEvents &pe,
                          cudaStream_t stream);
 cudaError_t launch_group(bool forward, int64_t batch, int L, const int64_t *comp,
-                         const int64_t *xfer, const int64_t *dt, int64_t *makespan,
-                         uint32_t *bits, int32_t *nseg, int32_t *status,
+                         const int64_t *xfer, const int64_t *dt, const SolveOut &out,
                          const uint32_t *list_count, const uint32_t *list, void *tables,
                          int64_t grid, cudaStream_t stream);
 cudaError_t launch_mid(bool forward, int64_t batch, int L, const int64_t *comp,
-                       const int64_t *xfer, const int64_t *dt, int64_t *makespan,
-                       uint32_t *bits, int32_t *nseg, int32_t *status, uint32_t *ticket,
-                       uint32_t *list_count, uint32_t *list, uint32_t *tb, cudaStream_t stream);
+                       const int64_t *xfer, const int64_t *dt, const SolveOut &out,
+                       uint32_t *ticket, uint32_t *list_count, uint32_t *list, uint32_t *tb,
+                       cudaStream_t stream);
 cudaError_t launch_warp(bool forward, int64_t batch, int L, const int64_t *comp,
-                        const int64_t *xfer, const int64_t *dt, int64_t *makespan, uint32_t *bits,
-                        int32_t *nseg, int32_t *status, uint32_t *ticket, uint32_t *list_count,
-                        uint32_t *list, uint32_t *slots, cudaStream_t stream);
+                        const int64_t *xfer, const int64_t *dt, const SolveOut &out,
+                        uint32_t *ticket, uint32_t *list_count, uint32_t *list, uint32_t *slots,
+                        cudaStream_t stream);
 bool use_solo(int64_t batch, int L);  // one launch solves the batch (dp_warp.cu)
 cudaError_t launch_solo(bool forward, int64_t batch, int L, const int64_t *comp,
-                        const int64_t *xfer, const int64_t *dt, int64_t *makespan, uint32_t *bits,
-                        int32_t *nseg, int32_t *status, uint32_t *list_count, cudaStream_t stream);
+                        const int64_t *xfer, const int64_t *dt, const SolveOut &out,
+                        uint32_t *list_count, cudaStream_t stream);
 cudaError_t launch_deep(bool forward, int64_t batch, int L, const int64_t *comp,
-                        const int64_t *xfer, const int64_t *dt, int64_t *makespan,
-                        uint32_t *bits, int32_t *nseg, int32_t *status, uint32_t *tickets,
-                        uint32_t *busy, uint32_t *list_count, uint32_t *list, void *slots,
-                        int64_t nslots, cudaStream_t stream);
+                        const int64_t *xfer, const int64_t *dt, const SolveOut &out,
+                        uint32_t *tickets, uint32_t *busy, uint32_t *list_count, uint32_t *list,
+                        void *slots, int64_t nslots, cudaStream_t stream);
 int64_t deep_launches(int64_t batch, int L);  // launches of one deep-chain pass (dp_deep.cu)
 cudaError_t launch_eval(bool forward, int64_t batch, int L, const int64_t *comp,
                         const int64_t *xfer, const int64_t *dt, const uint32_t *bits,

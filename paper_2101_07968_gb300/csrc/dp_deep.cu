@@ -51,7 +51,7 @@ struct DeepArgs {
     int64_t lo, count;  // this launch solves instances lo .. lo + count - 1
     int L;
     const int64_t *comp, *xfer, *dt;
-    ChainOut out;
+    SolveOut out;
     uint32_t *ticket;             // instances taken so far (zero before the launch)
     uint32_t *list_count, *list;  // instances left to the work-list pass
     uint32_t *busy;               // slot bitmap: bit set while a CTA holds the slot (zero before the first launch)
@@ -108,7 +108,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) deep_kernel(DeepArgs a)
         if (int64_t(taken) >= a.count) break;
         const int64_t i = a.lo + int64_t(taken);
         const bool solved = chain_solve<FWD, NJ>(
-            smem, i, L, a.comp + i * L, a.xfer + i * L, __ldg(a.dt + i), a.vec, a.out,
+            smem, i, L, RowLoader<FWD>{a.comp + i * L, a.xfer + i * L, L, a.vec != 0},
+            __ldg(a.dt + i), a.out,
             [&](int64_t base, uint64_t range, bool &ok) {
                 ok = range < (uint64_t(1) << 32);
                 return KeptOffsets{nullptr, at, L, 1, last, base};
@@ -216,8 +217,7 @@ int64_t deep_launches(int64_t batch, int L)
 }
 
 cudaError_t launch_deep(bool forward, int64_t batch, int L, const int64_t *comp,
-                        const int64_t *xfer, const int64_t *dt, int64_t *makespan,
-                        uint32_t *bits, int32_t *nseg, int32_t *status, uint32_t *tickets,
+                        const int64_t *xfer, const int64_t *dt, const SolveOut &out, uint32_t *tickets,
                         uint32_t *busy, uint32_t *list_count, uint32_t *list, void *slots,
                         int64_t nslots, cudaStream_t stream)
 {
@@ -234,7 +234,7 @@ cudaError_t launch_deep(bool forward, int64_t batch, int L, const int64_t *comp,
     int64_t k = 0;
     for (int64_t lo = 0; lo < batch; lo += per, ++k) {
         const int64_t count = batch - lo < per ? batch - lo : per;
-        DeepArgs a{lo, count, L, comp, xfer, dt, ChainOut{makespan, bits, nseg, status},
+        DeepArgs a{lo, count, L, comp, xfer, dt, out,
                    tickets + k, list_count, list, busy, static_cast<unsigned char *>(slots),
                    slot_bytes(L), int(nslots), vec ? 1 : 0};
         // the first launch waits for the memsets in stream order; later ones may

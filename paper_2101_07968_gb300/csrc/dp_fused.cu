@@ -1,6 +1,7 @@
 // Generate-and-solve for 1 <= L <= 16 (dc_schedule_generated_batch): the short-L
 // passes of dp_small.cu with each tile's rows drawn inside the kernel by the
 // profile generator's device functions instead of being read from memory.
+#include "chain.cuh"
 #include "dp_small.cuh"
 
 namespace dc {
@@ -21,9 +22,7 @@ namespace {
 inline size_t fused_tables_offset(int64_t batch) { return (256 + 8 * size_t(batch) + 255) / 256 * 256; }
 
 struct FusedOut {
-    int64_t *makespan[2];
-    uint32_t *bits[2];
-    int32_t *nseg[2], *status[2];
+    SolveOut out[2];
     uint32_t *wide_count[2], *wide_list[2];
     uint32_t *ticket;  // tiles handed out (zero before the launch)
 };
@@ -126,15 +125,20 @@ __global__ void __launch_bounds__(32, DC_SMALL_MINB)
                 U[m] = uv[32 * m];
                 V[m] = uv[32 * (L + 1 + m)];
             }
-            const bool run = active && st[dir] == DC_OK && !wide[dir];
-            const bool done = solve_uv<L>(fwd, run, U, V, int32_t(dti), xraw[dir], lw, i,
-                                          o.makespan[dir], o.bits[dir], o.nseg[dir], o.status[dir]);
-            if (active && st[dir] != DC_OK) {
-                write_failure(st[dir], i, W, o.makespan[dir], o.bits[dir], o.nseg[dir],
-                              o.status[dir]);
-            } else if (active && (wide[dir] || !done)) {
-                const uint32_t at = atomicAdd(o.wide_count[dir], 1u);
-                if (DC_CHECK(int64_t(at) < g.batch)) o.wide_list[dir][at] = uint32_t(i);
+            // selected, not indexed by `dir`: an index would put the pairs on the stack
+            const int std = fwd ? st[0] : st[1];
+            const bool wd = fwd ? wide[0] : wide[1];
+            const uint64_t xd = fwd ? xraw[0] : xraw[1];
+            const SolveOut od = fwd ? o.out[0] : o.out[1];
+            const bool done = solve_uv<L, false>(fwd, active && std == DC_OK && !wd, U, V, int32_t(dti),
+                                                 xd, lw, i, od);
+            if (active && std != DC_OK) {
+                write_failure(std, i, W, od);
+            } else if (active && (wd || !done)) {
+                uint32_t *count = fwd ? o.wide_count[0] : o.wide_count[1];
+                uint32_t *list = fwd ? o.wide_list[0] : o.wide_list[1];
+                const uint32_t at = atomicAdd(count, 1u);
+                if (DC_CHECK(int64_t(at) < g.batch)) list[at] = uint32_t(i);
             }
         }
     };
@@ -156,64 +160,70 @@ __global__ void __launch_bounds__(32, DC_SMALL_MINB)
     }
 }
 
-// 64-bit pass over one direction's list, rows regenerated.
-template <int L, bool FWD>
+// The costs of one instance's rows in processing order, drawn (see RowLoader).
+template <bool FWD>
+struct DrawLoader {
+    const GenParams &g;
+    const GenTables *t;
+    const InstanceDraws &d;
+    int64_t gi;
+    __device__ __forceinline__ void row(int r, uint64_t &c, uint64_t &x) const
+    {
+        c = x = 0;
+        if (r > g.L) return;
+        int64_t params, flops, f, b, v;
+        layer_draws(g, t->l0, t->l1, gi, FWD ? r - 1 : g.L - r, params, flops);
+        layer_costs(g, d, params, flops, f, b, v);
+        c = uint64_t(FWD ? f : b);
+        x = uint64_t(v);
+    }
+    __device__ __forceinline__ void operator()(int r, uint64_t &c0, uint64_t &c1, uint64_t &x0,
+                                               uint64_t &x1) const
+    {
+        row(r, c0, x0);
+        row(r + 1, c1, x1);
+    }
+};
+
+// Pass over one direction's list, rows regenerated: one warp per instance, every value
+// and every column (chain.cuh).
+template <bool FWD>
 __global__ void __launch_bounds__(32)
     fused_list_kernel(const __grid_constant__ GenParams g, const GenTables *t, const FusedOut o)
 {
     constexpr int dir = FWD ? 0 : 1;
     extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x;
-    uint64_t *lw = reinterpret_cast<uint64_t *>(smem) + lane;
+    int64_t *table = reinterpret_cast<int64_t *>(smem + 2 * chain_row_bytes(g.L));
     pdl_wait();  // the passes ahead of this one have finished
     const int64_t count = int64_t(*o.wide_count[dir]);
-    for (int64_t j = int64_t(blockIdx.x) * 32 + lane; j - lane < count; j += int64_t(gridDim.x) * 32) {
-        if (j >= count) continue;
+    for (int64_t j = blockIdx.x; j < count; j += gridDim.x) {
         const int64_t i = int64_t(o.wide_list[dir][j]);
+        if (!DC_CHECK(i < g.batch)) continue;
         const int64_t gi = g.inst0 + i;
         const InstanceDraws d = instance_draws(g, t->rate, t->bw, gi);
-        uint64_t Pc[L + 1], Px[L + 1], xraw;
-        bool neg = false, big = false;  // checked by the dense pass
-        row_prefix<L, FWD>(
-            [&](int col, int64_t &cv, int64_t &xv) {
-                int64_t params, flops, f, b, x;
-                layer_draws(g, t->l0, t->l1, gi, col, params, flops);
-                layer_costs(g, d, params, flops, f, b, x);
-                cv = FWD ? f : b;
-                xv = x;
-            },
-            Pc, Px, xraw, neg, big);
-        solve<L, FWD, uint64_t, L>(Pc, Px, d.dt, xraw - Px[L], lw, i, o.makespan[dir],
-                                   o.bits[dir], o.nseg[dir], o.status[dir]);
+        const int L = g.L;
+        chain_solve_warp<FWD, 1>(smem, i, L, DrawLoader<FWD>{g, t, d, gi}, d.dt, o.out[dir],
+                                 [&](int64_t, uint64_t, bool &) { return KeptValues{table, L}; });
+        __syncwarp();  // shared memory is read
     }
 }
 
-template <int L, bool FWD>
+template <bool FWD>
 cudaError_t launch_fused_list(const GenParams &g, const GenTables *t, const FusedOut &o,
                               cudaStream_t stream)
 {
-    using K64 = Small<L, uint64_t, L>;
-    static DeviceCache attr;  // the list kernel's shared-memory limit, raised once per device
-    int done = 0;
-    cudaError_t ae = attr.get(done, [](int &v) {
-        v = 1;
-        return cudaFuncSetAttribute(fused_list_kernel<L, FWD>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, K64::kTableBytes);
-    });
-    if (ae != cudaSuccess) return ae;
-    int64_t lgrid = (g.batch + 31) / 32;
-    if (lgrid > int64_t(sm_count()) * 4) lgrid = int64_t(sm_count()) * 4;
+    const int64_t lgrid = g.batch < int64_t(sm_count()) * 16 ? g.batch : int64_t(sm_count()) * 16;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(unsigned(lgrid));
     lc.blockDim = dim3(32);
-    lc.dynamicSmemBytes = K64::kTableBytes;
+    lc.dynamicSmemBytes = 2 * chain_row_bytes(g.L) + size_t(tri_cells(g.L)) * 8;
     lc.stream = stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, fused_list_kernel<L, FWD>, g, t, o);
+    return cudaLaunchKernelEx(&lc, fused_list_kernel<FWD>, g, t, o);
 }
 
 template <int L>
@@ -237,9 +247,9 @@ cudaError_t launch_fused_L(const GenParams &g, const GenTables *t, const FusedOu
     fused_pair_kernel<L><<<unsigned(grid), 32, Pair32<L>::kBytes, stream>>>(g, t, o);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = launch_fused_list<L, true>(g, t, o, stream);
+    e = launch_fused_list<true>(g, t, o, stream);
     if (e != cudaSuccess) return e;
-    return launch_fused_list<L, false>(g, t, o, stream);
+    return launch_fused_list<false>(g, t, o, stream);
 }
 
 }  // namespace
@@ -255,10 +265,8 @@ cudaError_t launch_fused(const GenParams &g, int64_t *makespan, uint32_t *bits, 
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     FusedOut o;
     for (int d = 0; d < 2; ++d) {
-        o.makespan[d] = makespan + d * B;
-        o.bits[d] = bits + d * B * W;
-        o.nseg[d] = nseg ? nseg + d * B : nullptr;
-        o.status[d] = status ? status + d * B : nullptr;
+        o.out[d] = SolveOut{makespan + d * B, bits + d * B * W, nseg ? nseg + d * B : nullptr,
+                            status ? status + d * B : nullptr, nullptr};
         o.wide_count[d] = reinterpret_cast<uint32_t *>(ws) + d;
         o.wide_list[d] = reinterpret_cast<uint32_t *>(ws + 256) + d * B;
     }

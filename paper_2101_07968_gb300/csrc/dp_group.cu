@@ -1,6 +1,6 @@
 // CTA-per-instance DynaComm DP for any 1 <= L <= 4096 (Eq. 8 / Algorithm 3 and
-// Eq. 9 / Algorithm 4): the pass over the work lists of the looped and
-// warp-per-instance kernels (dp_mid.cu) and the deep-chain kernel (dp_deep.cu), whose instances have values
+// Eq. 9 / Algorithm 4): the pass over the first passes' work lists (dp_small.cu,
+// dp_mid.cu, dp_warp.cu, dp_deep.cu), whose instances have values
 // beyond the first pass's range or an optimum deeper than its kept columns. The
 // method is in chain.cuh; this pass takes every value (64 bits) and keeps every
 // column, in shared memory up to L = 64, otherwise in a per-CTA table of the
@@ -15,7 +15,7 @@ struct GroupArgs {
     int64_t batch;
     int L;
     const int64_t *comp, *xfer, *dt;
-    ChainOut out;
+    SolveOut out;
     const uint32_t *list_count, *list;
     unsigned char *tables;  // nullptr: the table in shared memory
     int vec;                // the cost rows are 16-byte aligned
@@ -38,12 +38,15 @@ __global__ void __launch_bounds__(kChainThreads, 1) group_kernel(GroupArgs a)
     int64_t *table = reinterpret_cast<int64_t *>(
         a.tables ? a.tables + size_t(blockIdx.x) * size_t(tri_cells(L)) * 8
                  : smem + group_table_offset(L));
+    pdl_wait();  // the first pass has finished its list
     const int64_t count = int64_t(*a.list_count);
     for (int64_t j = blockIdx.x; j < count; j += gridDim.x) {
         const int64_t i = int64_t(a.list[j]);
         if (!DC_CHECK(i >= 0 && i < a.batch)) continue;
-        chain_solve<FWD, NJ>(smem, i, L, a.comp + i * L, a.xfer + i * L, __ldg(a.dt + i), a.vec,
-                             a.out, [&](int64_t, uint64_t, bool &) { return KeptValues{table, L}; });
+        chain_solve<FWD, NJ>(smem, i, L,
+                             RowLoader<FWD>{a.comp + i * L, a.xfer + i * L, L, a.vec != 0},
+                             __ldg(a.dt + i), a.out,
+                             [&](int64_t, uint64_t, bool &) { return KeptValues{table, L}; });
         __syncthreads();  // shared memory is read
     }
 }
@@ -59,8 +62,19 @@ cudaError_t launch_group_nj(const GroupArgs &a, int nt, int64_t grid, cudaStream
                                     int(group_smem_bytes(DC_L_MAX, false)));
     });
     if (e != cudaSuccess) return e;
-    group_kernel<FWD, NJ><<<unsigned(grid), nt, group_smem_bytes(a.L, a.tables == nullptr), stream>>>(a);
-    return cudaGetLastError();
+    // launched early (programmatic dependent launch): its CTAs wait in hardware until
+    // the first pass completes, so the launch overlaps that pass's tail
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(unsigned(grid));
+    lc.blockDim = dim3(unsigned(nt));
+    lc.dynamicSmemBytes = group_smem_bytes(a.L, a.tables == nullptr);
+    lc.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, group_kernel<FWD, NJ>, a);
 }
 
 template <bool FWD>
@@ -78,15 +92,13 @@ cudaError_t launch_group_dir(const GroupArgs &a, int64_t grid, cudaStream_t stre
 }  // namespace
 
 cudaError_t launch_group(bool forward, int64_t batch, int L, const int64_t *comp,
-                         const int64_t *xfer, const int64_t *dt, int64_t *makespan,
-                         uint32_t *bits, int32_t *nseg, int32_t *status,
-                         const uint32_t *list_count, const uint32_t *list, void *tables,
+                         const int64_t *xfer, const int64_t *dt, const SolveOut &out, const uint32_t *list_count, const uint32_t *list, void *tables,
                          int64_t grid, cudaStream_t stream)
 {
     if (grid <= 0) return cudaSuccess;
     const bool vec = (L % 2 == 0) &&
                      ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0;
-    const GroupArgs a{batch, L, comp, xfer, dt, ChainOut{makespan, bits, nseg, status},
+    const GroupArgs a{batch, L, comp, xfer, dt, out,
                       list_count, list, static_cast<unsigned char *>(tables), vec ? 1 : 0};
     return forward ? launch_group_dir<true>(a, grid, stream) : launch_group_dir<false>(a, grid, stream);
 }

@@ -83,12 +83,10 @@ inline bool use_looped(int64_t batch, int L) { return L <= kLoopedLMax && batch 
 template <bool FWD>
 __device__ __forceinline__ bool mid_prefix(int64_t batch, int64_t i, int L, const int64_t *__restrict__ comp,
                                            const int64_t *__restrict__ xfer, int64_t dti,
-                                           uint32_t *lw, int2 *pv, int64_t *makespan,
-                                           uint32_t *bits, int32_t *nseg, int32_t *status,
+                                           uint32_t *lw, int2 *pv, const SolveOut &o,
                                            uint32_t *list_count, uint32_t *list, uint64_t &px,
                                            int32_t &fcL)
 {
-    const int W = words_for(L);
     // transfer costs capped at the total compute (exact: same decisions, makespan
     // lower by sum(xfer) - sum(capped xfer), added back at the end)
     const int64_t *crow = comp + i * L, *xrow = xfer + i * L;
@@ -103,11 +101,7 @@ __device__ __forceinline__ bool mid_prefix(int64_t batch, int64_t i, int L, cons
         px += uint64_t(xv);
     }
     if (neg || big || exceeds_range(L, dti, tc, px)) {
-        const int st = neg ? DC_ERR_NEGATIVE : DC_ERR_RANGE;
-        makespan[i] = -int64_t(st);
-        if (nseg) nseg[i] = 0;
-        if (status) status[i] = st;
-        for (int w = 0; w < W; ++w) bits[i * W + w] = 0u;
+        write_failure(neg ? DC_ERR_NEGATIVE : DC_ERR_RANGE, i, words_for(L), o);
         return false;
     }
     // wrapping 32-bit arithmetic: the values are used only when the range check passes
@@ -235,9 +229,7 @@ template <bool FWD>
 __global__ void __launch_bounds__(32)
     mid_kernel(int64_t batch, int L, const int64_t *__restrict__ comp,
                const int64_t *__restrict__ xfer, const int64_t *__restrict__ dt,
-               int64_t *__restrict__ makespan, uint32_t *__restrict__ bits,
-               int32_t *__restrict__ nseg, int32_t *__restrict__ status,
-               uint32_t *__restrict__ ticket, uint32_t *__restrict__ list_count,
+               const SolveOut o, uint32_t *__restrict__ ticket, uint32_t *__restrict__ list_count,
                uint32_t *__restrict__ list, uint32_t *__restrict__ tb, int64_t nslots)
 {
     extern __shared__ uint32_t smem[];
@@ -264,8 +256,8 @@ __global__ void __launch_bounds__(32)
         const int64_t dti = __ldg(dt + i);
         uint64_t px = 0;
         int32_t fcL = 0;
-        if (!mid_prefix<FWD>(batch, i, L, comp, xfer, dti, lw, pv, makespan, bits, nseg, status,
-                             list_count, list, px, fcL))
+        if (!mid_prefix<FWD>(batch, i, L, comp, xfer, dti, lw, pv, o, list_count, list, px,
+                             fcL))
             continue;
         const int32_t dt32 = int32_t(dti);
 
@@ -297,6 +289,8 @@ __global__ void __launch_bounds__(32)
 
         // ---- traceback: lowest k whose candidate equals the cell
         uint32_t word = 0u;  // W = 1 up to L = 33
+        // f_m of the decision from its own segments, in the cells' shifted terms
+        int32_t span = INT32_MIN, later = 0;
         int err = 0, m = L, n = s;
         int32_t target = FWD ? bestV - s * dt32 + U[32 * L] : bestV - 2 * dt32;  // B[L][s] + Q[L] or F[L][s] - dt
         while (n > 1) {
@@ -342,27 +336,37 @@ __global__ void __launch_bounds__(32)
                 break;
             }
             word |= 1u << (k - 1);
+            span = max(span, uu + pv[32 * k].y + later);
+            later += FWD ? -dt32 : dt32;
             target = FWD ? fk + dt32 : fk - dt32;  // the cell (k, n-1): B + Q[k] = A + dt, or F - dt
             m = k;
             n -= 1;
         }
-        makespan[i] = int64_t(uint64_t(uint32_t(bestV)) + px);
-        if (nseg) nseg[i] = s;
-        if (status) status[i] = err ? DC_ERR_INTERNAL : DC_OK;
-        bits[i] = word;
+        if (o.replay) {
+            int32_t f = bestV;  // s = 1: the one segment
+            if (s > 1) {
+                const int32_t c1 = FWD ? fcL - dt32 : dt32;  // column 1 is U + c1
+                span = max(span, U[32 * m] + c1 + later - (FWD ? -dt32 : dt32));
+                f = FWD ? span - U[32 * L] + s * dt32 : span + 2 * dt32;
+            }
+            o.replay[i] = err ? -int64_t(DC_ERR_INTERNAL) : int64_t(uint64_t(uint32_t(f)) + px);
+        }
+        o.makespan[i] = int64_t(uint64_t(uint32_t(bestV)) + px);
+        if (o.nseg) o.nseg[i] = s;
+        if (o.status) o.status[i] = err ? DC_ERR_INTERNAL : DC_OK;
+        o.bits[i] = word;
     }
 }
 
 template <bool FWD>
 cudaError_t launch_looped(int64_t batch, int L, const int64_t *comp, const int64_t *xfer,
-                          const int64_t *dt, int64_t *makespan, uint32_t *bits, int32_t *nseg,
-                          int32_t *status, uint32_t *ticket, uint32_t *list_count, uint32_t *list,
+                          const int64_t *dt, const SolveOut &out, uint32_t *ticket, uint32_t *list_count, uint32_t *list,
                           uint32_t *tb, cudaStream_t stream)
 {
     const size_t smem = size_t(3) * (L + 1) * 32 * 4;
     const int64_t slots = mid_slots(batch);
     mid_kernel<FWD><<<unsigned(slots / 32), 32, smem, stream>>>(
-        batch, L, comp, xfer, dt, makespan, bits, nseg, status, ticket, list_count, list, tb, slots);
+        batch, L, comp, xfer, dt, out, ticket, list_count, list, tb, slots);
     return cudaGetLastError();
 }
 
@@ -378,17 +382,14 @@ size_t mid_scratch_bytes(int64_t batch, int L)
 // row: 400,000 x 17 in 188 us against 238 by the warp kernel, but 100,000 x 17 and
 // 400,000 x 20 are equal, and 400,000 x 24 takes 312 us against 253.
 cudaError_t launch_mid(bool forward, int64_t batch, int L, const int64_t *comp,
-                       const int64_t *xfer, const int64_t *dt, int64_t *makespan,
-                       uint32_t *bits, int32_t *nseg, int32_t *status, uint32_t *ticket,
+                       const int64_t *xfer, const int64_t *dt, const SolveOut &out, uint32_t *ticket,
                        uint32_t *list_count, uint32_t *list, uint32_t *tb, cudaStream_t stream)
 {
     if (!use_looped(batch, L))
-        return launch_warp(forward, batch, L, comp, xfer, dt, makespan, bits, nseg, status, ticket,
+        return launch_warp(forward, batch, L, comp, xfer, dt, out, ticket,
                            list_count, list, tb, stream);
-    return forward ? launch_looped<true>(batch, L, comp, xfer, dt, makespan, bits, nseg, status,
-                                         ticket, list_count, list, tb, stream)
-                   : launch_looped<false>(batch, L, comp, xfer, dt, makespan, bits, nseg, status,
-                                          ticket, list_count, list, tb, stream);
+    return forward ? launch_looped<true>(batch, L, comp, xfer, dt, out, ticket, list_count, list, tb, stream)
+                   : launch_looped<false>(batch, L, comp, xfer, dt, out, ticket, list_count, list, tb, stream);
 }
 
 }  // namespace dc

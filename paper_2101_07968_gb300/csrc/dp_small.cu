@@ -23,7 +23,7 @@
 //    depths do not split into separate paths. The pass keeps only columns 1..kKeepCols: the
 //    traceback of an s-segment optimum reads columns 1..s-1 only, and s is small
 //    in practice (2-5 on CNN-shaped profiles); an instance whose s needs a
-//    deeper column is re-solved by the 64-bit pass, which keeps every column;
+//    deeper column goes to the work list;
 //  * a row whose costs all fit 32 bits (compute below 2^31 / L) gets its prefix
 //    sums in 32-bit arithmetic (fast_uv); other rows take the 64-bit prefix,
 //    which also classifies bad input;
@@ -31,9 +31,11 @@
 //    changes no decision (see row_prefix); the shifted 32-bit form is exact
 //    whenever the capped bound L*dt + sum(capped xfer) + sum(comp) is below
 //    2^31. Other instances (and the deep ones above) are appended to a work list
-//    that a 64-bit instantiation of the literal template solves afterwards; that
-//    pass is launched early and waits in hardware for this one (programmatic
-//    dependent launch);
+//    that the CTA-per-instance pass solves afterwards (dp_group.cu); it is launched
+//    early and waits in hardware for this one (programmatic dependent launch);
+//  * with REPLAY the traceback also evaluates f_m of the decision, segment by segment
+//    (a select chain and two instructions a step), in place of a kernel that reads the
+//    rows again: the 1,000,000-instance VGG-16 step takes 208 us instead of 291;
 //  * persistent single-warp CTAs walk 32-instance tiles. A tile's rows arrive by
 //    cp.async (coalesced 16-byte copies of cost pairs for even L) at a row
 //    stride at which every lane reads its own row without bank conflicts
@@ -64,14 +66,12 @@ __host__ __device__ constexpr int dense_min_ctas(int L) { return L >= kSplitMinL
 //    atomic ticket, claimed one tile ahead: warps on a crowded sub-partition
 //    progress more slowly than others, and a static deal would leave the SMs
 //    emptying out behind the slowest warps.
-template <int L, bool FWD>
+template <int L, bool FWD, bool REPLAY>
 __global__ void __launch_bounds__(32, dense_min_ctas(L))
     small_dense_kernel(int64_t batch, const int64_t *__restrict__ comp,
                        const int64_t *__restrict__ xfer, const int64_t *__restrict__ dt,
-                       int64_t *__restrict__ makespan, uint32_t *__restrict__ bits,
-                       int32_t *__restrict__ nseg, int32_t *__restrict__ status,
-                       uint32_t *__restrict__ wide_count, uint32_t *__restrict__ wide_list,
-                       bool pairs)
+                       const SolveOut o, uint32_t *__restrict__ wide_count,
+                       uint32_t *__restrict__ wide_list, bool pairs)
 {
     using K = Tab32<L>;
     constexpr int W = (L - 1 + 31) / 32;
@@ -96,10 +96,9 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
     auto finish = [&](int64_t i, bool active, const int32_t (&U)[L + 1], const int32_t (&V)[L + 1],
                       int64_t dti, uint64_t xraw, bool wide, int st) {
         const bool run = active && st == DC_OK && !wide;
-        const bool done = solve_uv<L>(FWD, run, U, V, int32_t(dti), xraw, lw, i, makespan, bits,
-                                      nseg, status);
+        const bool done = solve_uv<L, REPLAY>(FWD, run, U, V, int32_t(dti), xraw, lw, i, o);
         if (active && st != DC_OK) {
-            write_failure(st, i, W, makespan, bits, nseg, status);
+            write_failure(st, i, W, o);
         } else if (active && (wide || !done)) {
             // 64-bit values, or a traceback deeper than the kept columns: work list
             const uint32_t at = atomicAdd(wide_count, 1u);
@@ -171,39 +170,6 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
     }
 }
 
-// 64-bit pass over the work list, every column kept.
-template <int L, bool FWD>
-__global__ void __launch_bounds__(32)
-    small_list_kernel(const int64_t *__restrict__ comp, const int64_t *__restrict__ xfer,
-                      const int64_t *__restrict__ dt, int64_t *__restrict__ makespan,
-                      uint32_t *__restrict__ bits, int32_t *__restrict__ nseg,
-                      int32_t *__restrict__ status, const uint32_t *__restrict__ wide_count,
-                      const uint32_t *__restrict__ wide_list)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x;
-    uint64_t *lw = reinterpret_cast<uint64_t *>(smem) + lane;
-    pdl_wait();  // the dense pass has finished its list
-    const int64_t count = int64_t(*wide_count);
-    for (int64_t j = int64_t(blockIdx.x) * 32 + lane; j - lane < count; j += int64_t(gridDim.x) * 32) {
-        if (j >= count) continue;
-        const int64_t i = int64_t(wide_list[j]);
-        const int64_t *crow = comp + i * L;
-        const int64_t *xrow = xfer + i * L;
-        const int64_t dti = __ldg(dt + i);
-        uint64_t Pc[L + 1], Px[L + 1], xraw;
-        bool neg = false, big = false;  // checked by the dense pass
-        row_prefix<L, FWD>(
-            [&](int col, int64_t &cv, int64_t &xv) {
-                cv = __ldg(crow + col);
-                xv = __ldg(xrow + col);
-            },
-            Pc, Px, xraw, neg, big);
-        solve<L, FWD, uint64_t, L>(Pc, Px, dti, xraw - Px[L], lw, i, makespan, bits, nseg,
-                                   status);
-    }
-}
-
 }  // namespace
 
 int sm_count()
@@ -221,24 +187,19 @@ int sm_count()
 
 namespace {
 
-template <int L, bool FWD>
+template <int L, bool FWD, bool REPLAY>
 cudaError_t launch_dir(int64_t batch, const int64_t *comp, const int64_t *xfer,
-                       const int64_t *dt, int64_t *makespan, uint32_t *bits, int32_t *nseg,
-                       int32_t *status, uint32_t *wide_count, uint32_t *wide_list,
-                       const PassEvents &pe, cudaStream_t stream)
+                       const int64_t *dt, const SolveOut &o, uint32_t *wide_count,
+                       uint32_t *wide_list, const PassEvents &pe, cudaStream_t stream)
 {
-    using K64 = Small<L, uint64_t, L>;
     constexpr int kSmem = L >= kSplitMinL ? Tab32<L>::kSplitBytes : Tab32<L>::kSharedBytes;
     static DeviceCache resident;  // single-warp CTAs of the dense kernel per SM
     int per_sm = 0;
     cudaError_t le = resident.get(per_sm, [](int &n) {
-        cudaError_t e = cudaFuncSetAttribute(small_dense_kernel<L, FWD>,
+        cudaError_t e = cudaFuncSetAttribute(small_dense_kernel<L, FWD, REPLAY>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(small_list_kernel<L, FWD>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, K64::kTableBytes);
-        if (e != cudaSuccess) return e;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, small_dense_kernel<L, FWD>, 32,
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, small_dense_kernel<L, FWD, REPLAY>, 32,
                                                              kSmem);
     });
     if (le != cudaSuccess) return le;
@@ -249,8 +210,8 @@ cudaError_t launch_dir(int64_t batch, const int64_t *comp, const int64_t *xfer,
         const cudaError_t re = cudaEventRecord(pe.start, stream);
         if (re != cudaSuccess) return re;
     }
-    small_dense_kernel<L, FWD><<<unsigned(grid), 32, kSmem, stream>>>(
-        batch, comp, xfer, dt, makespan, bits, nseg, status, wide_count, wide_list,
+    small_dense_kernel<L, FWD, REPLAY><<<unsigned(grid), 32, kSmem, stream>>>(
+        batch, comp, xfer, dt, o, wide_count, wide_list,
         ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -258,41 +219,35 @@ cudaError_t launch_dir(int64_t batch, const int64_t *comp, const int64_t *xfer,
         e = cudaEventRecord(pe.stop, stream);
         if (e != cudaSuccess) return e;
     }
-    // the list length is known on the device only: persistent warps (4 per SM)
-    // walk it, and the surplus exits at once
-    int64_t lgrid = (batch + 31) / 32;
-    if (lgrid > int64_t(sm_count()) * 4) lgrid = int64_t(sm_count()) * 4;
-    // launched early (programmatic dependent launch): its CTAs wait in hardware
-    // until the dense pass completes, so the launch overlaps that pass's tail
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(unsigned(lgrid));
-    lc.blockDim = dim3(32);
-    lc.dynamicSmemBytes = K64::kTableBytes;
-    lc.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, small_list_kernel<L, FWD>, comp, xfer, dt, makespan, bits,
-                              nseg, status, static_cast<const uint32_t *>(wide_count),
-                              static_cast<const uint32_t *>(wide_list));
+    // the list length is known on the device only: one-warp CTAs (up to 4 per SM) walk
+    // it, and the surplus exits at once
+    const int64_t lgrid = batch < int64_t(sm_count()) * 4 ? batch : int64_t(sm_count()) * 4;
+    return launch_group(FWD, batch, L, comp, xfer, dt, o, wide_count, wide_list, nullptr, lgrid,
+                        stream);
+}
+
+template <int L, bool REPLAY>
+cudaError_t launch_both(bool forward, int64_t batch, const int64_t *comp, const int64_t *xfer,
+                        const int64_t *dt, const SolveOut &o, uint32_t *wide_count,
+                        uint32_t *wide_list, const PassEvents &pe, cudaStream_t stream)
+{
+    return forward ? launch_dir<L, true, REPLAY>(batch, comp, xfer, dt, o, wide_count, wide_list, pe, stream)
+                   : launch_dir<L, false, REPLAY>(batch, comp, xfer, dt, o, wide_count, wide_list, pe, stream);
 }
 
 }  // namespace
 
 cudaError_t launch_small(bool forward, int64_t batch, int L, const int64_t *comp,
-                         const int64_t *xfer, const int64_t *dt, int64_t *makespan,
-                         uint32_t *bits, int32_t *nseg, int32_t *status,
+                         const int64_t *xfer, const int64_t *dt, const SolveOut &out,
                          uint32_t *wide_count, uint32_t *wide_list, const PassEvents &pe,
                          cudaStream_t stream)
 {
 #define DC_SMALL_CASE(LL)                                                                     \
     case LL:                                                                                  \
-        return forward ? launch_dir<LL, true>(batch, comp, xfer, dt, makespan, bits, nseg,   \
-                                              status, wide_count, wide_list, pe, stream)     \
-                       : launch_dir<LL, false>(batch, comp, xfer, dt, makespan, bits, nseg,  \
-                                               status, wide_count, wide_list, pe, stream);
+        return out.replay ? launch_both<LL, true>(forward, batch, comp, xfer, dt, out,       \
+                                                  wide_count, wide_list, pe, stream)          \
+                          : launch_both<LL, false>(forward, batch, comp, xfer, dt, out,      \
+                                                   wide_count, wide_list, pe, stream);
     switch (L) {
         DC_SMALL_CASE(1) DC_SMALL_CASE(2) DC_SMALL_CASE(3) DC_SMALL_CASE(4)
         DC_SMALL_CASE(5) DC_SMALL_CASE(6) DC_SMALL_CASE(7) DC_SMALL_CASE(8)

@@ -18,10 +18,6 @@ namespace {
 #ifndef DC_SMALL_MINB
 #define DC_SMALL_MINB 16  // resident single-warp CTAs per SM the registers must allow
 #endif
-#ifndef DC_TREE_MIN
-#define DC_TREE_MIN 1
-#endif
-constexpr int kTbGroup = 4;  // traceback candidates loaded per round
 // From this L on the dense and fused passes take their tiles from an atomic
 // ticket (and the dense pass stages each tile beside its table); shorter rows
 // take every grid-th tile, for which one atomic per tile costs more than the
@@ -44,18 +40,6 @@ __host__ __device__ constexpr int stage_stride(int L)
 {
     return (L % 2 == 1) ? L : (L % 4 == 2 ? L : L + 2);
 }
-
-// Table of the 64-bit pass: stored columns 2..C with C = min(keep, L-1) (KEEP = L
-// keeps them all), then S[0..L] and R[0..L].
-template <int L, typename T, int KEEP>
-struct Small {
-    static constexpr int kLast = KEEP < L - 1 ? KEEP : L - 1;  // last stored column
-    static constexpr int kCells = kLast >= 2 ? cell2(L, L, kLast) + 1 : 0;
-    static constexpr int kOffS = kCells;          // S[0..L]
-    static constexpr int kOffR = kCells + L + 1;  // R[0..L]
-    static constexpr int kLaneVals = kCells + 2 * (L + 1);
-    static constexpr int kTableBytes = 32 * kLaneVals * int(sizeof(T));
-};
 
 // Shared memory of a warp of the 32-bit pass. Its table, per lane (32-bit words,
 // lane-interleaved): word 0 unused, the kept cells of columns 2..kLast at
@@ -80,133 +64,6 @@ struct Tab32 {
 template <typename T>
 __device__ __forceinline__ T lds(const T *lane_base, int v) { return lane_base[32 * v]; }
 
-// The fill. lw = this lane's values in shared memory (value v at lw[32*v]).
-template <int L, bool FWD, typename T, int KEEP>
-__device__ __forceinline__ void fill(const T (&S)[L + 1], const T (&Rb)[L + 1], T dtv, T c,
-                                     T *lw, T &best_T, int &best_s)
-{
-    T col[L + 1];
-#pragma unroll
-    for (int m = 1; m <= L; ++m) col[m] = T((FWD ? T(dtv + Rb[m]) : Rb[m]) + S[m] + c);
-    best_T = col[L];
-    best_s = 1;
-#pragma unroll
-    for (int n = 2; n <= L; ++n) {
-        // rows in descending order so column n overwrites column n-1 in place:
-        // row m reads rows k < m, which still hold column n-1.
-#pragma unroll
-        for (int m = L; m >= n; --m) {
-            const T R = FWD ? T(T(n) * dtv + Rb[m]) : Rb[m];
-            constexpr int kMax = L;
-            T cand[kMax];
-            const int cnt = m - n + 1;  // k = n-1 .. m-1
-#pragma unroll
-            for (int j = 0; j < cnt; ++j) cand[j] = T(dmax(col[n - 1 + j], R) - S[n - 1 + j]);
-            if (DC_TREE_MIN) {  // balanced tree: log-depth chains
-#pragma unroll
-                for (int w = 1; w < cnt; w *= 2) {
-#pragma unroll
-                    for (int j = 0; j + w < cnt; j += 2 * w) cand[j] = dmin(cand[j], cand[j + w]);
-                }
-            } else {
-#pragma unroll
-                for (int j = 1; j < cnt; ++j) cand[0] = dmin(cand[0], cand[j]);
-            }
-            col[m] = T(cand[0] + S[m] + c);
-            if (n <= Small<L, T, KEEP>::kLast) lw[32 * cell2(L, m, n)] = col[m];
-        }
-        if (col[L] < best_T) {  // strict: the lowest n wins ties
-            best_T = col[L];
-            best_s = n;
-        }
-    }
-}
-
-// X[k][n-1] during the traceback: column 1 from S and R, others from the table.
-template <int L, bool FWD, typename T, int KEEP>
-__device__ __forceinline__ T prev_cell(const T *lw, int k, int nm1, T dtv, T c)
-{
-    using K = Small<L, T, KEEP>;
-    if (nm1 == 1) {
-        const T r = lds(lw, K::kOffR + k);
-        return T((FWD ? T(dtv + r) : r) + lds(lw, K::kOffS + k) + c);
-    }
-    return lds(lw, cell2(L, k, nm1));
-}
-
-// Solve one instance (row data already reduced to 64-bit prefix sums in
-// processing order) and write its outputs.
-// Returns false (writing nothing) when the optimum's traceback needs a column the
-// pass did not keep; the caller then lists the instance for the full pass.
-template <int L, bool FWD, typename T, int KEEP>
-__device__ __forceinline__ bool solve(const uint64_t (&Pc)[L + 1], const uint64_t (&Px)[L + 1],
-                                      int64_t dti, uint64_t shift, T *lw, int64_t i,
-                                      int64_t *makespan, uint32_t *bits, int32_t *nseg,
-                                      int32_t *status)
-{
-    using K = Small<L, T, KEEP>;
-    constexpr int W = (L - 1 + 31) / 32;
-    T S[L + 1], Rb[L + 1];
-#pragma unroll
-    for (int m = 0; m <= L; ++m) {
-        S[m] = T(FWD ? Pc[m] : Px[m]);
-        Rb[m] = T(FWD ? Px[m] : Pc[m]);
-        lw[32 * (K::kOffS + m)] = S[m];
-        lw[32 * (K::kOffR + m)] = Rb[m];
-    }
-    const T dtv = T(dti);
-    const T c = FWD ? T(0) : dtv;
-    T Tbest;
-    int s;
-    fill<L, FWD, T, KEEP>(S, Rb, dtv, c, lw, Tbest, s);
-    if (s - 1 > K::kLast && s - 1 >= 2) return false;
-
-    // traceback: from (L, s) step to the lowest k whose candidate equals the
-    // cell, set p_k / g_k, continue at (k, n-1)
-    uint32_t word = 0;
-    int err = 0;
-    int m = L, n = s;
-    T cell = Tbest;
-    while (n > 1) {
-        const T rm = lds(lw, K::kOffR + m);
-        const T R = FWD ? T(T(n) * dtv + rm) : rm;
-        const T target = T(cell - lds(lw, K::kOffS + m) - c);
-        // candidates in groups of kTbGroup: the loads issue back to back, then the
-        // compares run from the highest k down so that the lowest match wins
-        int k = -1;
-        T fk = T(0);
-        for (int k0 = n - 1; k0 < m && k < 0; k0 += kTbGroup) {
-            T f[kTbGroup], sk[kTbGroup];
-#pragma unroll
-            for (int u = 0; u < kTbGroup; ++u) {
-                const int kk = k0 + u < m ? k0 + u : m - 1;  // stay inside column n-1
-                f[u] = prev_cell<L, FWD, T, KEEP>(lw, kk, n - 1, dtv, c);
-                sk[u] = lds(lw, K::kOffS + kk);
-            }
-#pragma unroll
-            for (int u = kTbGroup - 1; u >= 0; --u) {
-                if (k0 + u < m && T(dmax(f[u], R) - sk[u]) == target) {
-                    k = k0 + u;
-                    fk = f[u];
-                }
-            }
-        }
-        if (k < 0) {  // cannot happen: the fill and this check use the same arithmetic
-            err = 1;
-            break;
-        }
-        word |= 1u << ((k - 1) & 31);
-        m = k;
-        n -= 1;
-        cell = fk;
-    }
-    makespan[i] = int64_t(uint64_t(Tbest) + shift);
-    if (nseg) nseg[i] = s;
-    if (status) status[i] = err ? DC_ERR_INTERNAL : DC_OK;
-    if (W > 0) bits[i * W] = word;
-    return true;
-}
-
 // ---------------------------------------------------------------------------
 // The 32-bit pass in shifted form. Every value is taken relative to the time
 // the last pull (forward) or push (backward) of its cell can start, which turns
@@ -229,7 +86,7 @@ __device__ __forceinline__ bool solve(const uint64_t (&Pc)[L + 1], const uint64_
 // column, and the previous column C in the max operand. Each candidate differs from Eq. 8/9's by a
 // constant of its row, so every argmin is the same. All values and sums lie in
 // [-2^31, 2^31) when the capped bound L*dt + sum(comp) + sum(capped xfer) is
-// below 2^31; other instances take the 64-bit pass. The table stores A (forward)
+// below 2^31; other instances take the work-list pass. The table stores A (forward)
 // or F (backward) for columns 1..kKeepCols and the row U (Q forward, BC - dt
 // backward); V (G forward, NGT backward) stays in registers.
 
@@ -317,10 +174,12 @@ __device__ __forceinline__ void fill_e(const bool fwd, const bool run, const int
 }
 
 // Number of v[0..N-1] (non-increasing) above t: N a power of two, halved by selects.
+// next: the first value that is not above, if any.
 template <int N>
-__device__ __forceinline__ int count_above(const int32_t (&v)[N], int32_t t)
+__device__ __forceinline__ int count_above(const int32_t (&v)[N], int32_t t, int32_t &next)
 {
     if constexpr (N == 1) {
+        if (v[0] <= t) next = v[0];
         return v[0] > t ? 1 : 0;
     } else {
         constexpr int H = N / 2;
@@ -328,7 +187,8 @@ __device__ __forceinline__ int count_above(const int32_t (&v)[N], int32_t t)
         int32_t w[H];
 #pragma unroll
         for (int j = 0; j < H; ++j) w[j] = up ? v[H + j] : v[j];
-        return (up ? H : 0) + count_above<H>(w, t);
+        if (!up) next = v[H - 1];
+        return (up ? H : 0) + count_above<H>(w, t, next);
     }
 }
 
@@ -338,13 +198,12 @@ __host__ __device__ constexpr int ceil_log2(int x) { return x <= 1 ? 0 : 1 + cei
 // from its U and V rows (forward: U = dt + capped transfer prefix, V = FC[L] - compute
 // prefix; backward: U = compute prefix - dt, V = -capped transfer prefix) and the raw
 // transfer sum. Every lane of the warp calls it; lanes with `run` false write nothing
-// but their slice. Returns false (having written nothing) when the traceback needs a
-// column the pass did not keep.
-template <int L>
+// but their slice. REPLAY: o.replay takes f_m of the decision. Returns false (having
+// written nothing) when the traceback needs a column the pass did not keep.
+template <int L, bool REPLAY>
 __device__ __forceinline__ bool solve_uv(const bool fwd, const bool run, const int32_t (&U)[L + 1],
                                          const int32_t (&V)[L + 1], int32_t dt, uint64_t xraw,
-                                         int32_t *lw, int64_t i, int64_t *makespan,
-                                         uint32_t *bits, int32_t *nseg, int32_t *status)
+                                         int32_t *lw, int64_t i, const SolveOut &o)
 {
     using K = Tab32<L>;
     constexpr int W = (L - 1 + 31) / 32;
@@ -369,9 +228,15 @@ __device__ __forceinline__ bool solve_uv(const bool fwd, const bool run, const i
     int m = L, n = s;
     int32_t target = fwd ? bestV - s * dt + U[L] : bestV - 2 * dt;  // B[L][s] + Q[L] or F[L][s] - dt
     const int32_t off1 = fwd ? fcL - dt : dt;  // column 1 is U + off1 (not stored)
+    // f_m of the decision from its own segments, in the cells' shifted terms: the
+    // largest over its segments of U[end] + V[start] and the shift since, then the
+    // first segment's U
+    int32_t span = INT32_MIN, later = 0;
     while (n > 1) {
         const int nm1 = n - 1;
-        const int k = 1 + count_above<kPad>(vs, target - lds(lw, K::kOffU + m));
+        const int32_t u = lds(lw, K::kOffU + m);
+        int32_t vk = INT32_MIN;
+        const int k = 1 + count_above<kPad>(vs, target - u, vk);
         // cell (k, n-1) of a kept column is word base + k
         const int base = nm1 == 1 ? K::kOffU : 1 + cell2(L, 0, nm1);
         const int at = k < m ? k : m;  // inside the column
@@ -381,14 +246,26 @@ __device__ __forceinline__ bool solve_uv(const bool fwd, const bool run, const i
             break;
         }
         word |= 1u << ((k - 1) & 31);
+        if constexpr (REPLAY) {
+            span = max(span, u + vk + later);
+            later += fwd ? -dt : dt;
+        }
         target = fwd ? fk + dt : fk - dt;  // the cell (k, n-1): B + Q[k] = A + dt, or F - dt
         m = k;
         n = nm1;
     }
-    makespan[i] = int64_t(uint64_t(uint32_t(bestV)) + xraw);
-    if (nseg) nseg[i] = s;
-    if (status) status[i] = err ? DC_ERR_INTERNAL : DC_OK;
-    if (W > 0) bits[i * W] = word;
+    o.makespan[i] = int64_t(uint64_t(uint32_t(bestV)) + xraw);
+    if (o.nseg) o.nseg[i] = s;
+    if (o.status) o.status[i] = err ? DC_ERR_INTERNAL : DC_OK;
+    if constexpr (REPLAY) {
+        int32_t f = bestV;  // s = 1: the one segment, dt + FC[L] or dt + BC[L]
+        if (s > 1) {
+            span = max(span, lds(lw, K::kOffU + m) + off1 + later - (fwd ? -dt : dt));
+            f = fwd ? span - U[L] + s * dt : span + 2 * dt;
+        }
+        o.replay[i] = err ? -int64_t(DC_ERR_INTERNAL) : int64_t(uint64_t(uint32_t(f)) + xraw);
+    }
+    if (W > 0) o.bits[i * W] = word;
     return true;
 }
 
@@ -576,15 +453,6 @@ __device__ __forceinline__ void row_uv(const int64_t *rc, const int64_t *rx, int
         st = DC_ERR_RANGE;
     wide = uint64_t(L) * uint64_t(dti) + Pc[L] + Px[L] > kShiftedLimit;  // capped bound
     shifted_uv<L, FWD>(Pc, Px, dti, U, V);
-}
-
-__device__ __forceinline__ void write_failure(int st, int64_t i, int W, int64_t *makespan,
-                                              uint32_t *bits, int32_t *nseg, int32_t *status)
-{
-    makespan[i] = -int64_t(st);
-    if (nseg) nseg[i] = 0;
-    if (status) status[i] = st;
-    for (int w = 0; w < W; ++w) bits[i * W + w] = 0u;
 }
 
 }  // namespace

@@ -39,7 +39,7 @@ struct WarpArgs {
     int64_t batch;
     int L;
     const int64_t *comp, *xfer, *dt;
-    ChainOut out;
+    SolveOut out;
     uint32_t *ticket;  // runs of instances taken so far (zero before the launch)
     uint32_t *list_count, *list;
     uint32_t *slots;  // columns 9..16, one slot per warp of the grid
@@ -74,7 +74,8 @@ __global__ void __launch_bounds__(256, NJ == 1 ? 4 : NJ == 2 ? 3 : 2) warp_kerne
         const int64_t end = at + a.run < a.batch ? at + a.run : a.batch;
         for (int64_t i = at; i < end; ++i) {
             const bool solved = chain_solve_warp<FWD, NJ>(
-                mine, i, L, a.comp + i * L, a.xfer + i * L, __ldg(a.dt + i), a.vec, a.out,
+                mine, i, L, RowLoader<FWD>{a.comp + i * L, a.xfer + i * L, L, a.vec != 0},
+                __ldg(a.dt + i), a.out,
                 [&](int64_t base, uint64_t range, bool &ok) {
                     ok = range < (uint64_t(1) << 32);
                     return KeptOffsets{cols, slot, L, kShared, last, base};
@@ -97,8 +98,10 @@ __global__ void __launch_bounds__(32) solo_kernel(WarpArgs a)
     const int64_t i = blockIdx.x;
     int64_t *table = reinterpret_cast<int64_t *>(smem + 2 * chain_row_bytes(L));
     if (i == 0 && threadIdx.x == 0) *a.list_count = 0u;  // nothing is left to a second pass
-    chain_solve_warp<FWD, 1>(smem, i, L, a.comp + i * L, a.xfer + i * L, __ldg(a.dt + i), a.vec,
-                             a.out, [&](int64_t, uint64_t, bool &) { return KeptValues{table, L}; });
+    chain_solve_warp<FWD, 1>(smem, i, L,
+                             RowLoader<FWD>{a.comp + i * L, a.xfer + i * L, L, a.vec != 0},
+                             __ldg(a.dt + i), a.out,
+                             [&](int64_t, uint64_t, bool &) { return KeptValues{table, L}; });
 }
 
 inline size_t solo_smem_bytes(int L) { return 2 * chain_row_bytes(L) + size_t(tri_cells(L)) * 8; }
@@ -151,12 +154,11 @@ bool use_solo(int64_t batch, int L)
 }
 
 cudaError_t launch_solo(bool forward, int64_t batch, int L, const int64_t *comp,
-                        const int64_t *xfer, const int64_t *dt, int64_t *makespan, uint32_t *bits,
-                        int32_t *nseg, int32_t *status, uint32_t *list_count, cudaStream_t stream)
+                        const int64_t *xfer, const int64_t *dt, const SolveOut &out, uint32_t *list_count, cudaStream_t stream)
 {
     const bool vec = (L % 2 == 0) &&
                      ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0;
-    const WarpArgs a{batch, L, comp, xfer, dt, ChainOut{makespan, bits, nseg, status},
+    const WarpArgs a{batch, L, comp, xfer, dt, out,
                      nullptr, list_count, nullptr, nullptr, 1, vec ? 1 : 0};
     const size_t smem = solo_smem_bytes(L);  // 17.7 KB at L = 64
     if (forward)
@@ -177,13 +179,12 @@ size_t warp_scratch_bytes(int64_t batch, int L)
 }
 
 cudaError_t launch_warp(bool forward, int64_t batch, int L, const int64_t *comp,
-                        const int64_t *xfer, const int64_t *dt, int64_t *makespan, uint32_t *bits,
-                        int32_t *nseg, int32_t *status, uint32_t *ticket, uint32_t *list_count,
+                        const int64_t *xfer, const int64_t *dt, const SolveOut &out, uint32_t *ticket, uint32_t *list_count,
                         uint32_t *list, uint32_t *slots, cudaStream_t stream)
 {
     const bool vec = (L % 2 == 0) &&
                      ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0;
-    const WarpArgs a{batch, L, comp, xfer, dt, ChainOut{makespan, bits, nseg, status},
+    const WarpArgs a{batch, L, comp, xfer, dt, out,
                      ticket, list_count, list, slots, 1, vec ? 1 : 0};
     if (L <= 64) return forward ? launch_warp_nj<true, 1>(a, stream) : launch_warp_nj<false, 1>(a, stream);
     if (L <= 128) return forward ? launch_warp_nj<true, 2>(a, stream) : launch_warp_nj<false, 2>(a, stream);

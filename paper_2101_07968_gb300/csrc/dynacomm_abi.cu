@@ -23,9 +23,8 @@ PassEvents take_pass_events()
 // Forward and backward solves share one path after the layers are put in
 // processing order (done inside the kernels).
 cudaError_t launch_schedule(bool forward, int64_t batch, int L, const int64_t *comp,
-                            const int64_t *xfer, const int64_t *dt, int64_t *makespan,
-                            uint32_t *bits, int32_t *nseg, int32_t *status, void *workspace,
-                            const PassEvents &pe, cudaStream_t stream)
+                            const int64_t *xfer, const int64_t *dt, const SolveOut &out,
+                            void *workspace, const PassEvents &pe, cudaStream_t stream)
 {
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     // events around the first pass of a looped or deep-chain solve
@@ -33,7 +32,7 @@ cudaError_t launch_schedule(bool forward, int64_t batch, int L, const int64_t *c
     if (use_solo(batch, L)) {  // one pass, nothing listed
         cudaError_t e = mark(pe.start);
         if (e != cudaSuccess) return e;
-        e = launch_solo(forward, batch, L, comp, xfer, dt, makespan, bits, nseg, status,
+        e = launch_solo(forward, batch, L, comp, xfer, dt, out,
                         reinterpret_cast<uint32_t *>(ws), stream);
         return e != cudaSuccess ? e : mark(pe.stop);
     }
@@ -44,7 +43,7 @@ cudaError_t launch_schedule(bool forward, int64_t batch, int L, const int64_t *c
         cudaError_t e = cudaMemsetAsync(count, 0, 2 * sizeof(uint32_t), stream);
         if (e != cudaSuccess) return e;
         // 32-bit pass over the batch, then a 64-bit pass over the instances it listed
-        return launch_small(forward, batch, L, comp, xfer, dt, makespan, bits, nseg, status,
+        return launch_small(forward, batch, L, comp, xfer, dt, out,
                             count, list, pe, stream);
     }
     if (L <= kMidLMax) {
@@ -58,17 +57,17 @@ cudaError_t launch_schedule(bool forward, int64_t batch, int L, const int64_t *c
         if (e != cudaSuccess) return e;
         e = mark(pe.start);
         if (e != cudaSuccess) return e;
-        e = launch_mid(forward, batch, L, comp, xfer, dt, makespan, bits, nseg, status, ticket,
+        e = launch_mid(forward, batch, L, comp, xfer, dt, out, ticket,
                        count, list, tb, stream);
         if (e != cudaSuccess) return e;
         e = mark(pe.stop);
         if (e != cudaSuccess) return e;
         if (L <= kSmemTableLMax) {  // tables of the listed instances in shared memory
             const int64_t grid = batch < 152 * 8 ? batch : 152 * 8;
-            return launch_group(forward, batch, L, comp, xfer, dt, makespan, bits, nseg, status,
+            return launch_group(forward, batch, L, comp, xfer, dt, out,
                                 count, list, nullptr, grid, stream);
         }
-        return launch_group(forward, batch, L, comp, xfer, dt, makespan, bits, nseg, status,
+        return launch_group(forward, batch, L, comp, xfer, dt, out,
                             count, list, ws + Workspace::group_tables_offset(batch, L),
                             int64_t(Workspace::slots(batch, L)), stream);
     }
@@ -83,13 +82,13 @@ cudaError_t launch_schedule(bool forward, int64_t batch, int L, const int64_t *c
     if (e != cudaSuccess) return e;
     e = mark(pe.start);
     if (e != cudaSuccess) return e;
-    e = launch_deep(forward, batch, L, comp, xfer, dt, makespan, bits, nseg, status, tickets,
+    e = launch_deep(forward, batch, L, comp, xfer, dt, out, tickets,
                     busy, count, list, ws + Workspace::deep_slots_offset(batch, L), nslots,
                     stream);
     if (e != cudaSuccess) return e;
     e = mark(pe.stop);
     if (e != cudaSuccess) return e;
-    return launch_group(forward, batch, L, comp, xfer, dt, makespan, bits, nseg, status, count,
+    return launch_group(forward, batch, L, comp, xfer, dt, out, count,
                         list, ws + Workspace::group_tables_offset(batch, L),
                         int64_t(Workspace::slots(batch, L)), stream);
 }
@@ -97,18 +96,17 @@ cudaError_t launch_schedule(bool forward, int64_t batch, int L, const int64_t *c
 namespace {
 
 dc_status schedule(bool forward, int64_t batch, int32_t L, const int64_t *comp,
-                   const int64_t *xfer, const int64_t *dt, int64_t *makespan, uint32_t *bits,
-                   int32_t *nseg, int32_t *status, void *workspace, size_t workspace_bytes,
-                   cudaStream_t stream)
+                   const int64_t *xfer, const int64_t *dt, const SolveOut &out, void *workspace,
+                   size_t workspace_bytes, cudaStream_t stream)
 {
     const PassEvents pe = take_pass_events();  // used up by this call, whatever it returns
     if (batch < 0 || L < 1 || L > DC_L_MAX || batch > int64_t(0xffffffffll))
         return DC_ERR_BAD_SHAPE;
     if (batch == 0) return DC_OK;
-    if (!comp || !xfer || !dt || !makespan || (!bits && words_for(L) > 0)) return DC_ERR_NULL;
+    if (!comp || !xfer || !dt || !out.makespan || (!out.bits && words_for(L) > 0)) return DC_ERR_NULL;
     if (!workspace || workspace_bytes < Workspace::bytes(batch, L)) return DC_ERR_WORKSPACE;
-    const cudaError_t e = launch_schedule(forward, batch, L, comp, xfer, dt, makespan, bits,
-                                          nseg, status, workspace, pe, stream);
+    const cudaError_t e = launch_schedule(forward, batch, L, comp, xfer, dt, out, workspace, pe,
+                                          stream);
     return e == cudaSuccess ? DC_OK : DC_ERR_CUDA;
 }
 
@@ -176,8 +174,8 @@ dc_status dc_schedule_forward_batch(int64_t batch, int32_t L, const int64_t *fc,
                                     void *workspace, size_t workspace_bytes, cudaStream_t stream)
 {
     const dc::NvtxRange nvtx("dc_schedule_forward_batch");
-    return dc::schedule(true, batch, L, fc, pt, dt, makespan, bits, nseg, status, workspace,
-                        workspace_bytes, stream);
+    return dc::schedule(true, batch, L, fc, pt, dt, {makespan, bits, nseg, status, nullptr},
+                        workspace, workspace_bytes, stream);
 }
 
 dc_status dc_schedule_backward_batch(int64_t batch, int32_t L, const int64_t *bc,
@@ -187,8 +185,27 @@ dc_status dc_schedule_backward_batch(int64_t batch, int32_t L, const int64_t *bc
                                      cudaStream_t stream)
 {
     const dc::NvtxRange nvtx("dc_schedule_backward_batch");
-    return dc::schedule(false, batch, L, bc, gt, dt, makespan, bits, nseg, status, workspace,
-                        workspace_bytes, stream);
+    return dc::schedule(false, batch, L, bc, gt, dt, {makespan, bits, nseg, status, nullptr},
+                        workspace, workspace_bytes, stream);
+}
+
+dc_status dc_schedule_replay_batch(int32_t dir, int64_t batch, int32_t L, const int64_t *comp,
+                                   const int64_t *xfer, const int64_t *dt, int64_t *makespan,
+                                   uint32_t *bits, int32_t *nseg, int32_t *status,
+                                   int64_t *replay, void *workspace, size_t workspace_bytes,
+                                   cudaStream_t stream)
+{
+    const dc::NvtxRange nvtx("dc_schedule_replay_batch");
+    if (dir != 0 && dir != 1) {
+        dc::take_pass_events();
+        return DC_ERR_BAD_SHAPE;
+    }
+    if (!replay && batch > 0) {
+        dc::take_pass_events();
+        return DC_ERR_NULL;
+    }
+    return dc::schedule(dir == 0, batch, L, comp, xfer, dt, {makespan, bits, nseg, status, replay},
+                        workspace, workspace_bytes, stream);
 }
 
 dc_status dc_eval_timeline_batch(int64_t batch, int32_t L, int32_t dir, const int64_t *comp,

@@ -430,7 +430,9 @@ __global__ void __launch_bounds__(kChainThreads, 1) greedy_cta_kernel(GreedyArgs
         const int64_t dt = __ldg(g.dt + i);
         for (int w = tid; w < W; w += NT) word[w] = 0u;
         uint64_t a[NJ][2], b[NJ][2], aL, bL;
-        const int st = cta_prefix<FWD, NJ>(tot, orw, L, g.comp + i * L, g.xfer + i * L, dt, g.vec, a, b, aL, bL);
+        const int st = cta_prefix<FWD, NJ>(
+            tot, orw, reinterpret_cast<uint64_t *>(best_of), L,
+            RowLoader<FWD>{g.comp + i * L, g.xfer + i * L, L, g.vec != 0}, dt, a, b, aL, bL);
         if (st != DC_OK) {
             if (tid == 0) g.makespan[i] = -int64_t(st);
             for (int w = tid; w < W; w += NT) g.bits[i * W + w] = 0u;

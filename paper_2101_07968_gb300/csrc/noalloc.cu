@@ -61,7 +61,8 @@ extern "C" dc_status dc_schedule_batch_static(int32_t dir, int64_t batch, int32_
         return DC_ERR_NULL;
     void *scratch = nullptr;
     if (dc::static_scratch(&scratch) != cudaSuccess) return DC_ERR_CUDA;
-    const cudaError_t e = dc::launch_schedule(dir == 0, batch, L, comp, xfer, dt, makespan,
-                                              bits, nseg, status, scratch, pe, stream);
+    const cudaError_t e = dc::launch_schedule(dir == 0, batch, L, comp, xfer, dt,
+                                              {makespan, bits, nseg, status, nullptr}, scratch, pe,
+                                              stream);
     return e == cudaSuccess ? DC_OK : DC_ERR_CUDA;
 }

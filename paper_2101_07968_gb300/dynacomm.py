@@ -64,6 +64,8 @@ _SIGNATURES = {
                                          _SZ, _VP]),
     "dc_schedule_backward_batch": (_I32, [_I64, _I32, _VP, _VP, _VP, _VP, _VP, _VP, _VP, _VP,
                                           _SZ, _VP]),
+    "dc_schedule_replay_batch": (_I32, [_I32, _I64, _I32, _VP, _VP, _VP, _VP, _VP, _VP, _VP,
+                                        _VP, _VP, _SZ, _VP]),
     "dc_eval_timeline_batch": (_I32, [_I64, _I32, _I32, _VP, _VP, _VP, _VP, _VP, _VP]),
     "dc_schedule_batch_static": (_I32, [_I32, _I64, _I32, _VP, _VP, _VP, _VP, _VP, _VP, _VP,
                                         _VP]),
@@ -215,6 +217,14 @@ def dc_schedule_backward_batch(batch, L, bc, gt, dt, makespan, bits, nseg, statu
     return int(lib().dc_schedule_backward_batch(
         int(batch), int(L), _ptr(bc), _ptr(gt), _ptr(dt), _ptr(makespan), _ptr(bits),
         _ptr(nseg), _ptr(status), _ptr(workspace), int(workspace_bytes), _stream(stream)))
+
+
+def dc_schedule_replay_batch(direction, batch, L, comp, xfer, dt, makespan, bits, nseg, status,
+                             replay, workspace, workspace_bytes, stream=None) -> int:
+    return int(lib().dc_schedule_replay_batch(
+        int(direction), int(batch), int(L), _ptr(comp), _ptr(xfer), _ptr(dt), _ptr(makespan),
+        _ptr(bits), _ptr(nseg), _ptr(status), _ptr(replay), _ptr(workspace),
+        int(workspace_bytes), _stream(stream)))
 
 
 def dc_schedule_batch_static(direction, batch, L, comp, xfer, dt, makespan, bits, nseg, status,
@@ -383,8 +393,9 @@ class StepGraph:
     kernels' own time; replay() issues them as one graph launch. The two
     directions are independent, so after the generator they run on two branches
     of the graph (each with its own workspace): one direction's kernels start on
-    the SMs the other's tail leaves free, and a replay kernel (memory-bound) can
-    run beside the other direction's DP (integer-ALU-bound). After each replay():
+    the SMs the other's tail leaves free. Each DP pass evaluates f_m itself
+    (dc_schedule_replay_batch), so the profiles are read once per direction. After
+    each replay():
     prof (fc, pt, bc, gt, dt), sched.out[d] and replay_out[d] for d in (FWD, BWD)
     hold that step's results."""
 
@@ -418,9 +429,11 @@ class StepGraph:
     def _direction(self, d, sched):
         p = self.prof
         c, x = ("fc", "pt") if d == FWD else ("bc", "gt")
-        o = sched.run(d, p[c], p[x], p["dt"])
-        _check(dc_eval_timeline_batch(self.B, self.L, d, p[c], p[x], p["dt"], o["bits"],
-                                      self.replay_out[d]), "dc_eval_timeline_batch")
+        o = sched.out[d]
+        _check(dc_schedule_replay_batch(d, self.B, self.L, p[c], p[x], p["dt"], o["makespan"],
+                                        o["bits"], o["nseg"], o["status"], self.replay_out[d],
+                                        sched.workspace, sched.ws_bytes),
+               "dc_schedule_replay_batch")
 
     def _step(self):
         import torch
@@ -533,13 +546,10 @@ class HostPipeline:
             d = {k: v + lo * 8 * (1 if k == "dt" else L) for k, v in dev.items()}
             o = {k: at + lo * row for k, (at, row) in out.items()}
             for dr, (ck, xk) in ((FWD, ("fc", "pt")), (BWD, ("bc", "gt"))):
-                fn = dc_schedule_forward_batch if dr == FWD else dc_schedule_backward_batch
-                _check(fn(hi - lo, L, d[ck], d[xk], d["dt"], o[(dr, "makespan")],
-                          o[(dr, "bits")], o[(dr, "nseg")], None, ws, self.ws_bytes, sr),
-                       "schedule (host pipeline)")
-                _check(dc_eval_timeline_batch(hi - lo, L, dr, d[ck], d[xk], d["dt"],
-                                              o[(dr, "bits")], o[(dr, "replay")], sr),
-                       "dc_eval_timeline_batch (host pipeline)")
+                _check(dc_schedule_replay_batch(
+                    dr, hi - lo, L, d[ck], d[xk], d["dt"], o[(dr, "makespan")], o[(dr, "bits")],
+                    o[(dr, "nseg")], None, o[(dr, "replay")], ws, self.ws_bytes, sr),
+                    "dc_schedule_replay_batch (host pipeline)")
             self.ev_run[c].record(self.s_run)
         last = pieces[-1]
         groups = ([(pieces[-2][0], 0, last[1])] if len(pieces) > 1 else []) + [last]
