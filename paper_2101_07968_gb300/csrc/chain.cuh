@@ -38,8 +38,6 @@
 //    H[L][n]. The fill stops after the first column without one (on the deep
 //    chain after 6.2 columns on average, where the optimum has 5.6 segments), or
 //    when c_n + a[L] - b[L-1], which bounds every later T, reaches the optimum.
-// Only cells that their column lowered are ever visited by the traceback (an
-// unchanged one would be a decision with fewer segments), so only those are kept.
 // Values stay below 2^53 (the range check), so 64 bits hold every sum; an instance
 // with a[L] + b[L] + (L + 1) dt < 2^31 runs in 32 bits.
 #pragma once
@@ -49,46 +47,64 @@
 namespace dc {
 namespace {
 
-// Arrays of the solver, in the caller's shared memory: K (the newest column's keys
-// H + e + b) and b of rows 1..L at 0..L-1, an even number of 64-bit places each
-// (the 32-bit form uses half of them).
-__host__ __device__ inline size_t chain_row_bytes(int L) { return size_t((L + 1) / 2) * 16; }
+// Shared memory is addressed by byte offsets from the CTA's dynamic shared memory, so
+// that a load needs no address arithmetic beyond the search's own offset.
+template <typename T>
+__device__ __forceinline__ T &sh(int off)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    return *reinterpret_cast<T *>(smem + off);
+}
 
-// The columns kept for the traceback, 2..last: offsets from `base` (no value of the
-// instance is below it) in 32 bits, columns 2..shared in shared memory and the rest
-// in a slot of the workspace.
-struct KeptOffsets {
-    uint32_t *sm, *gm;
-    int L, shared, last;
-    int64_t base;
+// Arrays of the solver: K (the newest column's keys H + e + b) and b of rows 1, 2, ..,
+// 8 bytes a row (the 32-bit form uses the first half of each array), with 16 bytes
+// between them whose last 8 are zero: b of row 0.
+__host__ __device__ inline int chain_rows_bytes(int rows) { return rows * 8; }
+__host__ __device__ inline int chain_pair_bytes(int rows) { return 2 * chain_rows_bytes(rows) + 16; }
+
+// The columns kept for the traceback, 1..last, as 32-bit words at a stride of
+// chain_stride(L) cells; columns 1..shared in shared memory (from byte `sm`) and the
+// rest in a slot of the workspace. A word is the value itself where values have 32
+// bits, otherwise H[m][1] - H[m][n], which lies between 0 and min(a[L], b[L] + h1):
+// H[m][n] is at least H[1][1], and at least c_n + a[m] - b[L].
+__host__ __device__ inline int chain_stride(int L) { return (L + 1) & ~1; }
+struct KeptWords {
+    int sm;
+    uint32_t *gm;
+    int stride, shared, last;
+    static constexpr bool kWhole = false;
     __device__ __forceinline__ bool holds(int n) const { return n <= last; }
+    // cells (m, n), (m + 1, n), m odd; the second may be padding past an odd L
     template <typename T>
-    __device__ __forceinline__ void put(int n, int m, T v) const
+    __device__ __forceinline__ void put2(int n, int m, T v0, T v1) const
     {
-        const uint32_t off = uint32_t(v - T(base));
-        if (!DC_CHECK(n >= 2 && m >= 1 && m <= L)) return;
+        if (!DC_CHECK(n >= 1 && m >= 1 && m < stride)) return;
+        const uint2 x = make_uint2(uint32_t(v0), uint32_t(v1));
         if (n <= shared)
-            sm[(n - 2) * L + (m - 1)] = off;
+            sh<uint2>(sm + 4 * ((n - 1) * stride + (m - 1))) = x;
         else if (n <= last)
-            gm[int64_t(n - 1 - shared) * L + (m - 1)] = off;
+            *reinterpret_cast<uint2 *>(gm + int64_t(n - 1 - shared) * stride + (m - 1)) = x;
     }
     template <typename T>
     __device__ __forceinline__ T get(int n, int m) const
     {
-        if (!DC_CHECK(n >= 2 && n <= last && m >= 1 && m <= L)) return T(0);
-        return T(base) + T(n <= shared ? sm[(n - 2) * L + (m - 1)]
-                                       : gm[int64_t(n - 1 - shared) * L + (m - 1)]);
+        if (!DC_CHECK(n >= 1 && n <= last && m >= 1 && m <= stride)) return T(0);
+        return T(n <= shared ? sh<uint32_t>(sm + 4 * ((n - 1) * stride + (m - 1)))
+                             : gm[int64_t(n - 1 - shared) * stride + (m - 1)]);
     }
 };
 // whole values, every column: the triangle of cells m >= n
 struct KeptValues {
     int64_t *at;
     int L;
+    static constexpr bool kWhole = true;
     __device__ __forceinline__ bool holds(int) const { return true; }
     template <typename T>
-    __device__ __forceinline__ void put(int n, int m, T v) const
+    __device__ __forceinline__ void put2(int n, int m, T v0, T v1) const
     {
-        if (m >= n && DC_CHECK(n >= 1 && m <= L)) at[tri_index(L, m, n)] = int64_t(v);
+        if (!DC_CHECK(n >= 1 && m >= 1 && m <= L)) return;
+        if (m >= n) at[tri_index(L, m, n)] = int64_t(v0);
+        if (m + 1 >= n && m + 1 <= L) at[tri_index(L, m + 1, n)] = int64_t(v1);
     }
     template <typename T>
     __device__ __forceinline__ T get(int n, int m) const
@@ -97,51 +113,64 @@ struct KeptValues {
         return T(at[tri_index(L, m, n)]);
     }
 };
+// whether KeptWords can hold the values of an instance in 64 bits
+__device__ __forceinline__ bool words_hold(uint64_t aL, uint64_t bL, uint64_t h1)
+{
+    return min(aL, bL + h1) < (uint64_t(1) << 32);
+}
 
 template <typename T>
 struct Pair;
 template <>
 struct Pair<int32_t> {
     using type = int2;
+    static constexpr int32_t kMax = INT32_MAX;
     static __device__ __forceinline__ int2 make(int32_t x, int32_t y) { return make_int2(x, y); }
 };
 template <>
 struct Pair<int64_t> {
     using type = longlong2;
+    static constexpr int64_t kMax = INT64_MAX;
     static __device__ __forceinline__ longlong2 make(int64_t x, int64_t y) { return make_longlong2(x, y); }
 };
 
-// One halving of two searches at once; `top` is the largest power of two that the
-// search range needs (uniform), so the steps above it are skipped.
+// Searches for the sorted keys below t0 and t1, two at once (independent load chains):
+// q = the byte offset of key p + 1, with p the number of keys below t.
+//
+// halve_from<STEP>: the count lies in [0, 2 STEP - 1] past q; keys that the caller
+// padded with the largest value end it earlier.
 template <typename T, int STEP>
-__device__ __forceinline__ void halve2(const T *K, int top, T t0, T t1, int &p0, int &p1)
+__device__ __forceinline__ void halve_from(T t0, T t1, int &q0, int &q1)
 {
-    if (STEP < top) {
-        const T k0 = K[p0 + STEP - 1], k1 = K[p1 + STEP - 1];
-        if (k0 < t0) p0 += STEP;
-        if (k1 < t1) p1 += STEP;
-    }
+    constexpr int S = int(sizeof(T));
+    const T k0 = sh<T>(q0 + (STEP - 1) * S), k1 = sh<T>(q1 + (STEP - 1) * S);
+    if (k0 < t0) q0 += STEP * S;
+    if (k1 < t1) q1 += STEP * S;
+    if constexpr (STEP > 1) halve_from<T, STEP / 2>(t0, t1, q0, q1);
 }
-// Number of keys below t among the sorted key[1..N] (key[k] at K[k-1]), P the largest
-// power of two <= N: the first probe splits [0, N] into two ranges of at most P
-// values, the rest halve it.
-template <typename T, int TOP>
-__device__ __forceinline__ void count_below2(const T *K, int N, int P, T t0, T t1, int &p0, int &p1)
+// search_below: N keys from byte kb, P the largest power of two <= N: the first probe
+// splits [0, N] into two ranges of at most P values, the rest halve it.
+template <typename T>
+__device__ __forceinline__ void search_below(int kb, int N, int P, T t0, T t1, int &q0, int &q1)
 {
-    const T kp = K[P - 1];
-    p0 = kp < t0 ? N - P + 1 : 0;
-    p1 = kp < t1 ? N - P + 1 : 0;
-    if constexpr (TOP > 1024) halve2<T, 1024>(K, P, t0, t1, p0, p1);
-    if constexpr (TOP > 512) halve2<T, 512>(K, P, t0, t1, p0, p1);
-    if constexpr (TOP > 256) halve2<T, 256>(K, P, t0, t1, p0, p1);
-    if constexpr (TOP > 128) halve2<T, 128>(K, P, t0, t1, p0, p1);
-    if constexpr (TOP > 64) halve2<T, 64>(K, P, t0, t1, p0, p1);
-    if constexpr (TOP > 32) halve2<T, 32>(K, P, t0, t1, p0, p1);
-    halve2<T, 16>(K, P, t0, t1, p0, p1);
-    halve2<T, 8>(K, P, t0, t1, p0, p1);
-    halve2<T, 4>(K, P, t0, t1, p0, p1);
-    halve2<T, 2>(K, P, t0, t1, p0, p1);
-    halve2<T, 1>(K, P, t0, t1, p0, p1);
+    constexpr int S = int(sizeof(T));
+    const T kp = sh<T>(kb + (P - 1) * S);
+    const int far = kb + (N - P + 1) * S;
+    q0 = kp < t0 ? far : kb;
+    q1 = kp < t1 ? far : kb;
+    switch (P) {  // uniform
+        case 2048: halve_from<T, 1024>(t0, t1, q0, q1); break;
+        case 1024: halve_from<T, 512>(t0, t1, q0, q1); break;
+        case 512: halve_from<T, 256>(t0, t1, q0, q1); break;
+        case 256: halve_from<T, 128>(t0, t1, q0, q1); break;
+        case 128: halve_from<T, 64>(t0, t1, q0, q1); break;
+        default:
+            for (int st = P >> 1; st > 0; st >>= 1) {
+                const T k0 = sh<T>(q0 + (st - 1) * S), k1 = sh<T>(q1 + (st - 1) * S);
+                if (k0 < t0) q0 += st * S;
+                if (k1 < t1) q1 += st * S;
+            }
+    }
 }
 
 // First k in [lo, lo + len] for which pred holds, given that it holds from some k on
@@ -166,12 +195,13 @@ __device__ __forceinline__ int warp_first(int lo, int len, Pred pred)
 
 // Columns 2.., the traceback and the outputs of instance i, from its prefixes:
 // thread tid of NT holds rows r, r+1 with r = 2 (j NT + tid) + 1 as a[j], b[j] (rows
-// past L hold the totals). WARP: one warp solves it (NT = 32), else the CTA. word:
-// shared memory, W decision words (CTA only); pub: two values that the CTA's last row
-// publishes. TOP: a power of two >= L - 1's largest. Returns false, having written
-// nothing, when the optimum needs columns that `kept` does not hold.
-template <bool FWD, typename T, int NJ, bool WARP, int TOP, typename Kept>
-__device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub, int tid, int NT,
+// past L hold the totals). WARP: one warp solves it (NT = 32), else the CTA. kb: byte
+// of K; D: bytes from K to b, both arrays with room for 2 NJ NT rows. word: shared
+// memory, W decision words, pub: two values that the CTA's last row publishes (both
+// CTA only). Returns false, having written nothing, when the optimum needs columns
+// that `kept` does not hold.
+template <bool FWD, typename T, int NJ, bool WARP, typename Kept>
+__device__ __forceinline__ bool chain_columns(int kb, int D, uint32_t *word, T *pub, int tid, int NT,
                                               int64_t i, int L, T dt, const T (&a)[NJ][2],
                                               const T (&b)[NJ][2], T aL, T bL, const Kept &kept,
                                               const SolveOut &o)
@@ -179,18 +209,24 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
     using P2 = Pair<T>;
     using Two = typename P2::type;
     constexpr unsigned kAll = 0xffffffffu;
+    constexpr int S = int(sizeof(T));
+    constexpr bool kDrop = S == 8 && !Kept::kWhole;  // kept words are H[m][1] - H[m][n]
     const int lane = tid & 31, W = words_for(L);
     const T e = FWD ? T(0) : dt, h1 = FWD ? dt : T(0);  // H[m][1] = h1 + a[m]
     T h[NJ][2];
+    bool in[NJ][2];  // rows 1..L-1: the k of a step
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
         const int r = 2 * (j * NT + tid) + 1;
+        in[j][0] = r < L;
+        in[j][1] = r + 1 < L;
         h[j][0] = h1 + a[j][0];
         h[j][1] = h1 + a[j][1];
-        if (r <= L) {  // row L + 1 of an odd L's last pair is padding
-            *reinterpret_cast<Two *>(B + r - 1) = P2::make(b[j][0], b[j][1]);
-            *reinterpret_cast<Two *>(K + r - 1) = P2::make(h[j][0] + e + b[j][0], h[j][1] + e + b[j][1]);
-        }
+        // keys from row L on end every search: they lower nothing
+        sh<Two>(kb + D + (r - 1) * S) = P2::make(b[j][0], b[j][1]);
+        sh<Two>(kb + (r - 1) * S) = P2::make(in[j][0] ? h[j][0] + e + b[j][0] : P2::kMax,
+                                             in[j][1] ? h[j][1] + e + b[j][1] : P2::kMax);
+        if (r <= L) kept.put2(1, r, kDrop ? T(0) : h[j][0], kDrop ? T(0) : h[j][1]);
     }
     if (WARP) __syncwarp(); else __syncthreads();
     T hL = h1 + aL;  // H[L] of the newest column
@@ -198,55 +234,51 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
     bool deep = false;  // the optimum lies beyond the kept columns
     const int N = L - 1;
     const int P = 1 << (31 - __clz(N | 1));
-    const T bL1 = N > 0 ? B[N - 1] : T(0);
+    const T tail = N > 0 ? aL - sh<T>(kb + D + (N - 1) * S) : aL;  // a[L] - b[L-1]
     T c = FWD ? dt : T(0);
     for (int n = 2; n <= L; ++n) {
         if (FWD) c += dt;
-        if (c + aL - bL1 >= hL) break;
+        if (c + tail >= hL) break;
         T v[NJ][2];
-        bool low[NJ][2];
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
             const int r = 2 * (j * NT + tid) + 1;
             const T t0 = c + a[j][0], t1 = c + a[j][1];
-            int p0, p1;
-            count_below2<T, TOP>(K, N, P, t0, t1, p0, p1);
-            // k = p + 1 is the first with H + e + b >= t (row L when there is none:
-            // H[L] lowers nothing), k = p the last below it (p = 0 gives t, which
-            // lowers nothing)
-            const T u0 = min(K[p0] - B[p0], p0 > 0 ? t0 - B[p0 - 1] : t0);
-            const T u1 = min(K[p1] - B[p1], p1 > 0 ? t1 - B[p1 - 1] : t1);
-            v[j][0] = min(h[j][0], u0);
-            v[j][1] = min(h[j][1], u1);
-            low[j][0] = r <= L && u0 < h[j][0];
-            low[j][1] = r < L && u1 < h[j][1];
-            if (low[j][0]) kept.put(n, r, v[j][0]);
-            if (low[j][1]) kept.put(n, r + 1, v[j][1]);
+            int q0 = kb, q1 = kb;
+            if constexpr (WARP)
+                halve_from<T, NJ == 1 ? 32 : NJ == 2 ? 64 : 128>(t0, t1, q0, q1);
+            else
+                search_below<T>(kb, N, P, t0, t1, q0, q1);
+            // k = p + 1, at q, is the first with H + e + b >= t, k = p the last below it
+            // (p = 0 gives t, which lowers nothing)
+            v[j][0] = min(min(h[j][0], sh<T>(q0) - sh<T>(q0 + D)), t0 - sh<T>(q0 + D - S));
+            v[j][1] = min(min(h[j][1], sh<T>(q1) - sh<T>(q1 + D)), t1 - sh<T>(q1 + D - S));
+            if (r <= L)
+                kept.put2(n, r, kDrop ? h1 + a[j][0] - v[j][0] : v[j][0],
+                          kDrop ? h1 + a[j][1] - v[j][1] : v[j][1]);
             if (!WARP && (r == L || r + 1 == L)) pub[n & 1] = r == L ? v[j][0] : v[j][1];
         }
         T hn;
         if (WARP) {
-            const int q = (L - 1) / 2;  // row L's pair
-            T mine = v[0][0];
-#pragma unroll
-            for (int j = 0; j < NJ; ++j)
-                if (j == q / 32) mine = (L & 1) ? v[j][0] : v[j][1];
-            hn = __shfl_sync(kAll, mine, q % 32);  // every lane has read column n-1
+            // the last row that a lane holds is row L or past it (then it has row L's a, and
+            // comes out the same); every lane has read column n-1 here
+            hn = __shfl_sync(kAll, v[NJ - 1][1], 31);
         } else {
             __syncthreads();
             hn = pub[n & 1];
         }
-        // another column only while a lowered H may still lower H[L]
+        // another column only while a lowered H may still lower H[L] (rows from L on
+        // never pass: their H is H[L])
         bool more = false;
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
             const int r = 2 * (j * NT + tid) + 1;
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                if (low[j][u]) K[r - 1 + u] = v[j][u] + e + b[j][u];
-                more |= low[j][u] && v[j][u] + e < hn;
-                h[j][u] = v[j][u];
-            }
+            more |= v[j][0] < h[j][0] && v[j][0] + e < hn;
+            more |= v[j][1] < h[j][1] && v[j][1] + e < hn;
+            h[j][0] = v[j][0];
+            h[j][1] = v[j][1];
+            sh<Two>(kb + (r - 1) * S) = P2::make(in[j][0] ? v[j][0] + e + b[j][0] : P2::kMax,
+                                                 in[j][1] ? v[j][1] + e + b[j][1] : P2::kMax);
         }
         if (hn < hL) {
             hL = hn;
@@ -266,10 +298,8 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
     // a goes to the key array first
     if (!WARP || s > 1) {
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            const int r = 2 * (j * NT + tid) + 1;
-            if (r <= L) *reinterpret_cast<Two *>(K + r - 1) = P2::make(a[j][0], a[j][1]);
-        }
+        for (int j = 0; j < NJ; ++j)
+            sh<Two>(kb + 2 * (j * NT + tid) * S) = P2::make(a[j][0], a[j][1]);
     }
     if (WARP) __syncwarp(); else __syncthreads();
     if (!WARP && tid >= 32) return true;
@@ -281,7 +311,8 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
     T span = T(0), later = T(0);
     T cn = FWD ? T(n) * dt : T(0);
     while (n > 1) {
-        const T thr = cn + K[m - 1] - v;
+        const T am = cn + sh<T>(kb + (m - 1) * S);
+        const T thr = am - v;
         int k;
         if (WARP) {
             int below = 0;  // rows past L hold b[L] >= thr, or there is no such k
@@ -290,19 +321,20 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
                 below += __popc(__ballot_sync(kAll, b[j][0] < thr)) + __popc(__ballot_sync(kAll, b[j][1] < thr));
             k = below + 1;
         } else {
-            k = warp_first(1, N, [&](int q) { return B[q - 1] >= thr; });
+            k = warp_first(1, N, [&](int q) { return sh<T>(kb + D + (q - 1) * S) >= thr; });
         }
         if (k < n - 1 || k >= m) {
             err = 1;
             break;
         }
-        const T hk = n == 2 ? h1 + K[k - 1] : kept.template get<T>(n - 1, k);
+        T hk = kept.template get<T>(n - 1, k);
+        if (kDrop) hk = h1 + sh<T>(kb + (k - 1) * S) - hk;
         if (hk + e > v) {
             err = 1;
             break;
         }
         if (o.replay) {
-            const T w = cn + K[m - 1] - B[k - 1] + later;
+            const T w = am - sh<T>(kb + D + (k - 1) * S) + later;
             span = n == s ? w : max(span, w);
             later += e;
         }
@@ -317,7 +349,7 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
         if (FWD) cn -= dt;
     }
     if (o.replay) {
-        const T first = h1 + later + (s > 1 ? K[m - 1] : aL);  // the first segment
+        const T first = h1 + later + (s > 1 ? sh<T>(kb + (m - 1) * S) : aL);  // the first segment
         span = s > 1 ? max(span, first) : first;
     }
     if (!WARP) __syncwarp();
@@ -329,6 +361,7 @@ __device__ __forceinline__ bool chain_columns(T *K, T *B, uint32_t *word, T *pub
     }
     if (WARP) {
         if (lane < W) o.bits[i * W + lane] = err ? 0u : mine;
+        __syncwarp();  // lane 0 rejoins here and not somewhere in the next instance
     } else {
         for (int w = lane; w < W; w += 32) o.bits[i * W + w] = err ? 0u : word[w];
     }
@@ -393,6 +426,12 @@ __device__ __forceinline__ void scan2(U &sa, U &sb, int lane)
     }
 }
 
+// b's row 0, for arrays with room for `rows` rows at byte kb.
+__device__ __forceinline__ void zero_row(int kb, int rows)
+{
+    sh<int64_t>(kb + chain_rows_bytes(rows) + 8) = 0;
+}
+
 // --------------------------------------------------------------- warp per instance
 // The same with a flag that gathers bit 31 of every partial sum: clear for all lanes
 // when no sum of the prefix reached 2^31 (the operands of the first that does are
@@ -411,18 +450,17 @@ __device__ __forceinline__ void scan2_flag(uint32_t &sa, uint32_t &sb, uint32_t 
     }
 }
 
-// Solves instance i with one warp, NJ row pairs per lane (L <= 64 NJ). smem: the
-// warp's K and b. make_kept as in chain_solve. Returns false, having written nothing,
-// when the instance is left to the work list.
-template <bool FWD, int NJ, typename Load, typename MakeKept>
-__device__ __forceinline__ bool chain_solve_warp(unsigned char *smem, int64_t i, int L,
-                                                 const Load &load, int64_t dt, const SolveOut &o,
-                                                 MakeKept make_kept)
+// Solves instance i with one warp, NJ row pairs per lane (L <= 64 NJ). kb: byte of the
+// warp's K, b beside it (chain_pair_bytes(64 NJ); the caller zeroes b's row 0 once with
+// zero_row). Returns false, having written nothing, when the instance is left to the
+// work list, as chain_solve does.
+template <bool FWD, int NJ, typename Load, typename Kept>
+__device__ __forceinline__ bool chain_solve_warp(int kb, int64_t i, int L, const Load &load,
+                                                 int64_t dt, const SolveOut &o, const Kept &kept)
 {
     constexpr unsigned kAll = 0xffffffffu;
-    constexpr int kTop = 64 * NJ;
+    constexpr int D = 64 * NJ * 8 + 16;
     const int lane = threadIdx.x & 31;
-    const size_t rb = chain_row_bytes(L);
     uint64_t a[NJ][2], b[NJ][2];
     uint32_t hi = uint32_t(uint64_t(dt) >> 32), flag = uint32_t(dt);
 #pragma unroll
@@ -452,11 +490,8 @@ __device__ __forceinline__ bool chain_solve_warp(unsigned char *smem, int64_t i,
     const bool narrow = !__any_sync(kAll, (hi | (flag >> 31)) != 0u) &&
                         uint64_t(aL32) + bL32 + uint64_t(L + 1) * uint64_t(dt) < (uint64_t(1) << 31);
     if (narrow) {
-        bool ok = true;
-        const auto kept = make_kept(int64_t(0), uint64_t(0), ok);
-        return chain_columns<FWD, int32_t, NJ, true, kTop>(
-            reinterpret_cast<int32_t *>(smem), reinterpret_cast<int32_t *>(smem + rb),
-            static_cast<uint32_t *>(nullptr), static_cast<int32_t *>(nullptr), lane, 32, i, L,
+        return chain_columns<FWD, int32_t, NJ, true>(
+            kb, D, static_cast<uint32_t *>(nullptr), static_cast<int32_t *>(nullptr), lane, 32, i, L,
             int32_t(dt), a32, b32, int32_t(aL32), int32_t(bL32), kept, o);
     }
     // any other instance: 64-bit sums, the input checks, 64-bit values
@@ -484,14 +519,10 @@ __device__ __forceinline__ bool chain_solve_warp(unsigned char *smem, int64_t i,
         chain_failure(st, i, words_for(L), lane, 32, o);
         return true;
     }
-    const int64_t a1 = __shfl_sync(kAll, a64[0][0], 0);  // H lies between H[1][1] and H[L][1]
-    bool ok = true;
-    const auto kept = make_kept((FWD ? dt : 0) + a1, aL - uint64_t(a1), ok);
-    if (!ok) return false;
-    return chain_columns<FWD, int64_t, NJ, true, kTop>(
-        reinterpret_cast<int64_t *>(smem), reinterpret_cast<int64_t *>(smem + rb),
-        static_cast<uint32_t *>(nullptr), static_cast<int64_t *>(nullptr), lane, 32, i, L, dt, a64,
-        b64, int64_t(aL), int64_t(bL), kept, o);
+    if (!Kept::kWhole && !words_hold(aL, bL, uint64_t(FWD ? dt : 0))) return false;
+    return chain_columns<FWD, int64_t, NJ, true>(
+        kb, D, static_cast<uint32_t *>(nullptr), static_cast<int64_t *>(nullptr), lane, 32, i, L, dt,
+        a64, b64, int64_t(aL), int64_t(bL), kept, o);
 }
 
 // ---------------------------------------------------------------- CTA per instance
@@ -502,22 +533,24 @@ __host__ __device__ inline size_t chain_word_bytes(int L)
 {
     return (size_t(words_for(L)) * 4 + 15) / 16 * 16;
 }
-// K and b, the decision words, then the scan's partial sums, the warps' flags and two
-// published values
-__host__ __device__ inline size_t chain_smem_bytes(int L)
+// K and b with room for `rows` rows (2 NJ times the threads), the decision words, then the
+// scan's partial sums, the warps' flags and two published values
+constexpr size_t kChainScratch = size_t(2 * kChainPairs * (kChainThreads / 32)) * 8 + 32 * 4 + 16;
+__host__ __device__ inline size_t chain_smem_bytes(int L, int rows)
 {
-    return 2 * chain_row_bytes(L) + chain_word_bytes(L) +
-           size_t(2 * kChainPairs * (kChainThreads / 32)) * 8 + 32 * 4 + 16;
+    return chain_pair_bytes(rows) + chain_word_bytes(L) + kChainScratch;
 }
+// the most that any choice of threads takes at depth L: whole warps of one row pair
+__host__ __device__ inline size_t chain_smem_most(int L) { return chain_smem_bytes(L, (L + 127) / 128 * 128); }
 
 // The prefixes of an instance's rows over the whole CTA, in processing order (a, b and
-// the row layout of chain_columns; 64-bit). tot, orw: scratch; first: a[1], published,
-// like what the threads wrote to shared memory before, by the one CTA barrier in here. Returns the
+// the row layout of chain_columns; 64-bit). tot, orw: scratch. One CTA barrier, which
+// also publishes what the threads wrote to shared memory before. Returns the
 // instance's status: DC_OK or its input error.
 template <bool FWD, int NJ, typename Load>
-__device__ __forceinline__ int cta_prefix(uint64_t *tot, uint32_t *orw, uint64_t *first, int L,
-                                          const Load &load, int64_t dt, uint64_t (&a)[NJ][2],
-                                          uint64_t (&b)[NJ][2], uint64_t &aL, uint64_t &bL)
+__device__ __forceinline__ int cta_prefix(uint64_t *tot, uint32_t *orw, int L, const Load &load,
+                                          int64_t dt, uint64_t (&a)[NJ][2], uint64_t (&b)[NJ][2],
+                                          uint64_t &aL, uint64_t &bL)
 {
     const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = NT >> 5;
     uint64_t any = uint64_t(dt);
@@ -529,7 +562,6 @@ __device__ __forceinline__ int cta_prefix(uint64_t *tot, uint32_t *orw, uint64_t
             load(r, b0, b1, a0, a1);
         else
             load(r, a0, a1, b0, b1);
-        if (j == 0 && tid == 0) *first = a0;
         any |= a0 | a1 | b0 | b1;
         uint64_t sa = a0 + a1, sb = b0 + b1;
         scan2(sa, sb, lane);
@@ -568,31 +600,28 @@ __device__ __forceinline__ int cta_prefix(uint64_t *tot, uint32_t *orw, uint64_t
     return DC_OK;
 }
 
-// Solves instance i with the whole CTA, NJ row pairs per thread. make_kept(base,
-// range) returns the store of kept columns for values from base to base + range, with
-// `ok` false when it cannot hold them. Returns false, having written nothing, when
-// the instance is left to the work list.
-template <bool FWD, int NJ, typename Load, typename MakeKept>
-__device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const Load &load, int64_t dt,
-                            const SolveOut &o, MakeKept make_kept)
+// Solves instance i with the whole CTA, NJ row pairs per thread, keeping columns in
+// `kept`. Returns false, having written nothing, when the instance is left to the work
+// list: its values do not fit there, or its optimum needs a column it does not hold.
+template <bool FWD, int NJ, typename Load, typename Kept>
+__device__ bool chain_solve(int64_t i, int L, const Load &load, int64_t dt, const SolveOut &o,
+                            const Kept &kept)
 {
     const int NT = blockDim.x, tid = threadIdx.x;
-    const int W = words_for(L);
-    const size_t rb = chain_row_bytes(L);
-    uint32_t *word = reinterpret_cast<uint32_t *>(smem + 2 * rb);
-    uint64_t *tot = reinterpret_cast<uint64_t *>(smem + 2 * rb + chain_word_bytes(L));
+    const int W = words_for(L), rows = 2 * NJ * NT, D = chain_rows_bytes(rows) + 16;
+    uint32_t *word = &sh<uint32_t>(chain_pair_bytes(rows));
+    uint64_t *tot = &sh<uint64_t>(chain_pair_bytes(rows) + int(chain_word_bytes(L)));
     uint32_t *orw = reinterpret_cast<uint32_t *>(tot + 2 * kChainPairs * (kChainThreads / 32));
     unsigned char *pub = reinterpret_cast<unsigned char *>(orw + 32);
 
+    if (tid == 0) zero_row(0, rows);
     for (int w = tid; w < W; w += NT) word[w] = 0u;
     uint64_t a[NJ][2], b[NJ][2], aL, bL;
-    const int st = cta_prefix<FWD, NJ>(tot, orw, reinterpret_cast<uint64_t *>(pub), L, load, dt, a,
-                                       b, aL, bL);
+    const int st = cta_prefix<FWD, NJ>(tot, orw, L, load, dt, a, b, aL, bL);
     if (st != DC_OK) {
         chain_failure(st, i, W, tid, NT, o);
         return true;
     }
-    constexpr int kTop = 4096;
     if (aL + bL + uint64_t(L + 1) * uint64_t(dt) < (uint64_t(1) << 31)) {
         int32_t a32[NJ][2], b32[NJ][2];
 #pragma unroll
@@ -602,12 +631,9 @@ __device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const Load &l
                 a32[j][u] = int32_t(a[j][u]);
                 b32[j][u] = int32_t(b[j][u]);
             }
-        bool ok = true;
-        const auto kept = make_kept(int64_t(0), uint64_t(0), ok);
-        return chain_columns<FWD, int32_t, NJ, false, kTop>(
-            reinterpret_cast<int32_t *>(smem), reinterpret_cast<int32_t *>(smem + rb), word,
-            reinterpret_cast<int32_t *>(pub), tid, NT, i, L, int32_t(dt), a32, b32, int32_t(aL),
-            int32_t(bL), kept, o);
+        return chain_columns<FWD, int32_t, NJ, false>(0, D, word, reinterpret_cast<int32_t *>(pub), tid,
+                                                      NT, i, L, int32_t(dt), a32, b32, int32_t(aL),
+                                                      int32_t(bL), kept, o);
     }
     int64_t a64[NJ][2], b64[NJ][2];
 #pragma unroll
@@ -617,16 +643,9 @@ __device__ bool chain_solve(unsigned char *smem, int64_t i, int L, const Load &l
             a64[j][u] = int64_t(a[j][u]);
             b64[j][u] = int64_t(b[j][u]);
         }
-    // H lies between H[1][1] and H[L][1]
-    const int64_t h1 = FWD ? dt : 0;
-    const int64_t a1 = *reinterpret_cast<const int64_t *>(pub);
-    bool ok = true;
-    const auto kept = make_kept(h1 + a1, aL - uint64_t(a1), ok);
-    if (!ok) return false;
-    return chain_columns<FWD, int64_t, NJ, false, kTop>(
-        reinterpret_cast<int64_t *>(smem), reinterpret_cast<int64_t *>(smem + rb), word,
-        reinterpret_cast<int64_t *>(pub), tid, NT, i, L, dt, a64, b64, int64_t(aL), int64_t(bL),
-        kept, o);
+    if (!Kept::kWhole && !words_hold(aL, bL, uint64_t(FWD ? dt : 0))) return false;
+    return chain_columns<FWD, int64_t, NJ, false>(0, D, word, reinterpret_cast<int64_t *>(pub), tid, NT,
+                                                  i, L, dt, a64, b64, int64_t(aL), int64_t(bL), kept, o);
 }
 
 }  // namespace

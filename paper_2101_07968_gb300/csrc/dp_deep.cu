@@ -14,12 +14,13 @@
 //    read once (16 L bytes per instance and direction) and the columns kept for the
 //    traceback stay in L2;
 //  * a column is updated in place: every thread's results wait in registers for a
-//    barrier, then only the lowered cells are written;
+//    barrier, then they are written;
 //  * 32-bit values where the instance's sums fit, otherwise 64-bit (two in five
-//    instances of the deep chain), chosen per instance. Columns 2..64 are kept as
-//    32-bit offsets in a slot of the workspace per resident CTA; optima deeper than
-//    65 segments, and instances whose useful values span 2^32, go to the work list
-//    (dp_group.cu, whole values, every column);
+//    instances of the deep chain), chosen per instance. Columns 1..64 are kept as
+//    32-bit words, the first in shared memory, the rest in a slot of the workspace per
+//    resident CTA; optima deeper than 65
+//    segments, and the rare instances whose values do not fit (see KeptWords), go to
+//    the work list (dp_group.cu, whole values, every column);
 //  * persistent CTAs take instances from a per-launch ticket, and a long batch of
 //    L > 256 is split into launches of four resident waves, so that kernels of other
 //    streams get their turn on the GPU between them. The launches are chained by
@@ -39,12 +40,13 @@ int sm_count();  // SMs of the current device (dp_small.cu)
 namespace {
 
 constexpr int kSplitLMin = 256;  // longer batches are split into launches above this depth
-constexpr int kKeep = 64;  // columns 2..kKeep kept for the traceback
+constexpr int kSmemPerSm = 227 * 1024;
+constexpr int kKeep = 64;  // columns 1..kKeep kept for the traceback
 
 __host__ __device__ inline size_t slot_bytes(int L)
 {
     const int last = L - 1 < kKeep ? L - 1 : kKeep;
-    return (size_t(last > 1 ? last - 1 : 0) * L * 4 + 255) / 256 * 256;
+    return (size_t(last) * chain_stride(L) * 4 + 255) / 256 * 256;
 }
 
 struct DeepArgs {
@@ -58,7 +60,8 @@ struct DeepArgs {
     unsigned char *slots;
     size_t slot_bytes;
     int nslots;
-    int vec;  // the cost rows are 16-byte aligned
+    int vec;     // the cost rows are 16-byte aligned
+    int shared;  // kept columns in shared memory, the rest in the slot
 };
 
 // A free slot, or -1: at most one resident wave of CTAs lives at a time, over this
@@ -85,7 +88,6 @@ __device__ int claim_slot(uint32_t *busy, int nslots)
 template <bool FWD, int NJ>
 __global__ void __launch_bounds__(kChainThreads, 1) deep_kernel(DeepArgs a)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_slot;
     __shared__ uint32_t s_taken;
     const int L = a.L, tid = threadIdx.x;
@@ -100,7 +102,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) deep_kernel(DeepArgs a)
         return;
     }
     uint32_t *at = reinterpret_cast<uint32_t *>(a.slots + size_t(slot) * a.slot_bytes);
-    const int last = L - 1 < kKeep ? L - 1 : kKeep;
+    const int cols = int((chain_smem_bytes(L, 2 * NJ * int(blockDim.x)) + 15) / 16 * 16);
+    const KeptWords kept{cols, at, chain_stride(L), a.shared, L - 1 < kKeep ? L - 1 : kKeep};
     for (;;) {
         if (tid == 0) s_taken = atomicAdd(a.ticket, 1u);
         __syncthreads();
@@ -108,12 +111,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) deep_kernel(DeepArgs a)
         if (int64_t(taken) >= a.count) break;
         const int64_t i = a.lo + int64_t(taken);
         const bool solved = chain_solve<FWD, NJ>(
-            smem, i, L, RowLoader<FWD>{a.comp + i * L, a.xfer + i * L, L, a.vec != 0},
-            __ldg(a.dt + i), a.out,
-            [&](int64_t base, uint64_t range, bool &ok) {
-                ok = range < (uint64_t(1) << 32);
-                return KeptOffsets{nullptr, at, L, 1, last, base};
-            });
+            i, L, RowLoader<FWD>{a.comp + i * L, a.xfer + i * L, L, a.vec != 0}, __ldg(a.dt + i),
+            a.out, kept);
         if (!solved && tid == 0) {
             const uint32_t p = atomicAdd(a.list_count, 1u);
             if (DC_CHECK(int64_t(p) < a.lo + a.count)) a.list[p] = uint32_t(i);
@@ -137,7 +136,7 @@ size_t deep_slot_bytes(int L) { return slot_bytes(L); }
 // is sized from it on the host, without a device query).
 int64_t deep_slots_bound(int L)
 {
-    const size_t per = chain_smem_bytes(L) + 1024;  // the runtime reserves 1 KB per CTA
+    const size_t per = chain_smem_bytes(L, L) + 1024;  // the runtime reserves 1 KB per CTA
     int64_t n = int64_t((228 * 1024) / per);
     if (n > 32) n = 32;
     if (n < 1) n = 1;
@@ -157,17 +156,26 @@ int deep_threads(int64_t count, int L, int sms)
 }
 
 template <bool FWD, int NJ>
-cudaError_t launch_deep_nj(const DeepArgs &a, int nt, bool pdl, cudaStream_t stream)
+cudaError_t launch_deep_nj(DeepArgs a, int nt, bool pdl, cudaStream_t stream)
 {
     static DeviceCache attr;
     int done = 0;
     cudaError_t e = attr.get(done, [](int &v) {
         v = 1;
         return cudaFuncSetAttribute(deep_kernel<FWD, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    int(chain_smem_bytes(DC_L_MAX)));
+                                    kSmemPerSm - 1024);
     });
     if (e != cudaSuccess) return e;
-    const size_t smem = chain_smem_bytes(a.L);
+    // The kernel's 64 registers allow 1,024 threads on an SM; the shared memory that
+    // leaves a CTA holds its first columns (9 at L = 1024), so that the traceback of
+    // most instances does not wait for L2 at every step
+    const size_t fixed = (chain_smem_bytes(a.L, 2 * NJ * nt) + 15) / 16 * 16;
+    const int ctas = 1024 / nt > 32 ? 32 : 1024 / nt < 1 ? 1 : 1024 / nt;
+    const size_t room = size_t(kSmemPerSm) / ctas - 1024, col = size_t(chain_stride(a.L)) * 4;
+    a.shared = room > fixed ? int((room - fixed) / col) : 0;
+    if (a.shared > a.L - 1) a.shared = a.L - 1;
+    if (a.shared > kKeep) a.shared = kKeep;
+    const size_t smem = fixed + a.shared * col;
     int nb = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, deep_kernel<FWD, NJ>, nt, smem);
     if (e != cudaSuccess) return e;
@@ -236,7 +244,7 @@ cudaError_t launch_deep(bool forward, int64_t batch, int L, const int64_t *comp,
         const int64_t count = batch - lo < per ? batch - lo : per;
         DeepArgs a{lo, count, L, comp, xfer, dt, out,
                    tickets + k, list_count, list, busy, static_cast<unsigned char *>(slots),
-                   slot_bytes(L), int(nslots), vec ? 1 : 0};
+                   slot_bytes(L), int(nslots), vec ? 1 : 0, 0};
         // the first launch waits for the memsets in stream order; later ones may
         // overlap the tail of the one before
         e = forward ? launch_deep_dir<true>(a, k > 0, stream)

@@ -192,8 +192,8 @@ __global__ void __launch_bounds__(32)
     fused_list_kernel(const __grid_constant__ GenParams g, const GenTables *t, const FusedOut o)
 {
     constexpr int dir = FWD ? 0 : 1;
-    extern __shared__ __align__(16) unsigned char smem[];
-    int64_t *table = reinterpret_cast<int64_t *>(smem + 2 * chain_row_bytes(g.L));
+    int64_t *table = &sh<int64_t>(chain_pair_bytes(64));
+    if (threadIdx.x == 0) zero_row(0, 64);
     pdl_wait();  // the passes ahead of this one have finished
     const int64_t count = int64_t(*o.wide_count[dir]);
     for (int64_t j = blockIdx.x; j < count; j += gridDim.x) {
@@ -202,8 +202,8 @@ __global__ void __launch_bounds__(32)
         const int64_t gi = g.inst0 + i;
         const InstanceDraws d = instance_draws(g, t->rate, t->bw, gi);
         const int L = g.L;
-        chain_solve_warp<FWD, 1>(smem, i, L, DrawLoader<FWD>{g, t, d, gi}, d.dt, o.out[dir],
-                                 [&](int64_t, uint64_t, bool &) { return KeptValues{table, L}; });
+        chain_solve_warp<FWD, 1>(0, i, L, DrawLoader<FWD>{g, t, d, gi}, d.dt, o.out[dir],
+                                 KeptValues{table, L});
         __syncwarp();  // shared memory is read
     }
 }
@@ -216,7 +216,7 @@ cudaError_t launch_fused_list(const GenParams &g, const GenTables *t, const Fuse
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(unsigned(lgrid));
     lc.blockDim = dim3(32);
-    lc.dynamicSmemBytes = 2 * chain_row_bytes(g.L) + size_t(tri_cells(g.L)) * 8;
+    lc.dynamicSmemBytes = chain_pair_bytes(64) + size_t(tri_cells(g.L)) * 8;
     lc.stream = stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

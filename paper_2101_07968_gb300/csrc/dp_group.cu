@@ -21,32 +21,26 @@ struct GroupArgs {
     int vec;                // the cost rows are 16-byte aligned
 };
 
-__host__ __device__ inline size_t group_table_offset(int L)
+__host__ __device__ inline int group_table_offset(int L, int rows)
 {
-    return (chain_smem_bytes(L) + 15) / 16 * 16;
-}
-inline size_t group_smem_bytes(int L, bool table_in_smem)
-{
-    return group_table_offset(L) + (table_in_smem ? size_t(tri_cells(L)) * 8 : 0);
+    return int((chain_smem_bytes(L, rows) + 15) / 16 * 16);
 }
 
 template <bool FWD, int NJ>
 __global__ void __launch_bounds__(kChainThreads, 1) group_kernel(GroupArgs a)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
     const int L = a.L;
-    int64_t *table = reinterpret_cast<int64_t *>(
-        a.tables ? a.tables + size_t(blockIdx.x) * size_t(tri_cells(L)) * 8
-                 : smem + group_table_offset(L));
+    int64_t *table = a.tables ? reinterpret_cast<int64_t *>(
+                                    a.tables + size_t(blockIdx.x) * size_t(tri_cells(L)) * 8)
+                              : &sh<int64_t>(group_table_offset(L, 2 * NJ * int(blockDim.x)));
     pdl_wait();  // the first pass has finished its list
     const int64_t count = int64_t(*a.list_count);
     for (int64_t j = blockIdx.x; j < count; j += gridDim.x) {
         const int64_t i = int64_t(a.list[j]);
         if (!DC_CHECK(i >= 0 && i < a.batch)) continue;
-        chain_solve<FWD, NJ>(smem, i, L,
+        chain_solve<FWD, NJ>(i, L,
                              RowLoader<FWD>{a.comp + i * L, a.xfer + i * L, L, a.vec != 0},
-                             __ldg(a.dt + i), a.out,
-                             [&](int64_t, uint64_t, bool &) { return KeptValues{table, L}; });
+                             __ldg(a.dt + i), a.out, KeptValues{table, L});
         __syncthreads();  // shared memory is read
     }
 }
@@ -59,7 +53,7 @@ cudaError_t launch_group_nj(const GroupArgs &a, int nt, int64_t grid, cudaStream
     const cudaError_t e = attr.get(done, [](int &v) {
         v = 1;
         return cudaFuncSetAttribute(group_kernel<FWD, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    int(group_smem_bytes(DC_L_MAX, false)));
+                                    int(chain_smem_most(DC_L_MAX)) + 1024);
     });
     if (e != cudaSuccess) return e;
     // launched early (programmatic dependent launch): its CTAs wait in hardware until
@@ -67,7 +61,7 @@ cudaError_t launch_group_nj(const GroupArgs &a, int nt, int64_t grid, cudaStream
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(unsigned(grid));
     lc.blockDim = dim3(unsigned(nt));
-    lc.dynamicSmemBytes = group_smem_bytes(a.L, a.tables == nullptr);
+    lc.dynamicSmemBytes = group_table_offset(a.L, 2 * NJ * nt) + (a.tables ? 0 : size_t(tri_cells(a.L)) * 8);
     lc.stream = stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

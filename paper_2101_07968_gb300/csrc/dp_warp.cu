@@ -7,22 +7,22 @@
 //    into registers and scanned by shuffles, in 32 bits with a flag for sums past
 //    2^31; the instances it marks run in 64 bits. A column's keys and b sit in the
 //    warp's slice of shared memory; there are no CTA barriers;
-//  * columns 2..8 are kept for the traceback in shared memory, 9..16 in a slot of the
-//    workspace per resident warp; optima deeper than 17 segments, and instances whose
-//    useful values span 2^32, go to the work list (dp_group.cu);
+//  * columns 1..8 are kept for the traceback in shared memory, 9..24 in a slot of the
+//    workspace per resident warp; optima deeper than 25 segments, and instances whose
+//    useful values span 2^32 (see KeptWords), go to the work list (dp_group.cu);
 //  * the traceback finds Path[m][n], the first k with b[k] at least a bound, by one
 //    ballot over the lanes' b;
-//  * persistent warps take runs of instances from an atomic ticket, the next run
-//    claimed while one is solved.
+//  * persistent warps solve an equal share of the batch each, then runs of instances
+//    from an atomic ticket, the next run claimed while one is solved.
 // Small batches of L <= 64 (use_solo) take one launch without tickets, work list or
 // memset: solo_kernel keeps every column, in whole values, in shared memory, so one
 // warp solves any instance to the end.
-// Bound by integer issue: the searches, the scans and the per-column bookkeeping.
-// Measured per direction against the looped thread-per-instance kernel that took
-// L <= 256 before (every candidate of every column): 262,144 x 54 (ResNet-50) 185 us
-// against 945; 20,000 x 128 80 us against 955; one instance of L = 54 23 us, launches
-// included, against 88. Above L = 192 (eight rows per lane) the CTA-per-instance pass
-// is as fast on large batches and faster on small ones: 3,000 x 200 66 us against 81.
+// Bound by integer issue (0.7 of the slots while all warps run) and, on small batches, by
+// the deepest instances at the end. Measured per direction against the looped
+// thread-per-instance kernel that took L <= 256 before (every candidate of every
+// column): 262,144 x 54 (ResNet-50) 155 us against 945; 20,000 x 128 45 us against 955.
+// Above L = 192 (eight rows per lane) the CTA-per-instance pass is as fast on large
+// batches and faster on small ones: 3,000 x 200 66 us against 81.
 #include "chain.cuh"
 
 namespace dc {
@@ -31,7 +31,7 @@ int sm_count();  // SMs of the current device (dp_small.cu)
 
 namespace {
 
-constexpr int kShared = 8, kLast = 16;  // columns kept in shared memory, and in all
+constexpr int kShared = 8, kLast = 24;  // columns kept in shared memory, and in all
 constexpr int kMaxWarpsPerSm = 64;
 constexpr int64_t kSlotWarps = 152 * kMaxWarpsPerSm;  // slots of the workspace, at most
 
@@ -42,69 +42,71 @@ struct WarpArgs {
     SolveOut out;
     uint32_t *ticket;  // runs of instances taken so far (zero before the launch)
     uint32_t *list_count, *list;
-    uint32_t *slots;  // columns 9..16, one slot per warp of the grid
-    int run;          // instances per run
+    uint32_t *slots;  // columns 9..24, one slot per warp of the grid
+    int own;          // instances of each warp's own, before the ticket's
+    int run;          // instances per run of the ticket
     int vec;          // the cost rows are 16-byte aligned
 };
 
-__host__ __device__ inline size_t warp_smem_bytes(int L)
+// K and b of 64 NJ rows, then the kept columns
+__host__ __device__ inline int warp_smem_bytes(int L, int nj)
 {
-    return (2 * chain_row_bytes(L) + size_t(kShared - 1) * L * 4 + 15) / 16 * 16;
+    return (chain_pair_bytes(64 * nj) + kShared * chain_stride(L) * 4 + 15) / 16 * 16;
 }
-__host__ __device__ inline int64_t warp_slot_words(int L) { return int64_t(kLast - kShared) * L; }
+__host__ __device__ inline int64_t warp_slot_words(int L) { return int64_t(kLast - kShared) * chain_stride(L); }
 
 template <bool FWD, int NJ>
 __global__ void __launch_bounds__(256, NJ == 1 ? 4 : NJ == 2 ? 3 : 2) warp_kernel(WarpArgs a)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
     const int L = a.L, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    unsigned char *mine = smem + size_t(warp) * warp_smem_bytes(L);
-    uint32_t *cols = reinterpret_cast<uint32_t *>(mine + 2 * chain_row_bytes(L));
+    const int kb = warp * warp_smem_bytes(L, NJ), cols = kb + chain_pair_bytes(64 * NJ);
+    if (lane == 0) zero_row(kb, 64 * NJ);
     uint32_t *slot = a.slots + (int64_t(blockIdx.x) * nw + warp) * warp_slot_words(L);
-    const int last = L - 1 < kLast ? L - 1 : kLast;
+    const KeptWords kept{cols, slot, chain_stride(L), kShared, L - 1 < kLast ? L - 1 : kLast};
     pdl_trigger();
     auto claim = [&]() {
         uint32_t v = 0;
         if (lane == 0) v = atomicAdd(a.ticket, 1u);
+        __syncwarp();  // see the end of chain_columns
         return v;
     };
-    int64_t at = int64_t(__shfl_sync(0xffffffffu, claim(), 0)) * a.run;
-    while (at < a.batch) {
-        const uint32_t next = claim();
-        const int64_t end = at + a.run < a.batch ? at + a.run : a.batch;
-        for (int64_t i = at; i < end; ++i) {
+    // first this warp's own share, then runs from the ticket (claimed one ahead)
+    const int64_t gw = int64_t(blockIdx.x) * nw + warp;
+    const int64_t shared_from = a.own * int64_t(gridDim.x) * nw;
+    uint32_t next = claim();
+    int64_t at = gw * a.own, end = at + a.own;
+    for (;;) {
+        const int64_t *crow = a.comp + at * L, *xrow = a.xfer + at * L;
+        for (int64_t i = at; i < end; ++i, crow += L, xrow += L) {
             const bool solved = chain_solve_warp<FWD, NJ>(
-                mine, i, L, RowLoader<FWD>{a.comp + i * L, a.xfer + i * L, L, a.vec != 0},
-                __ldg(a.dt + i), a.out,
-                [&](int64_t base, uint64_t range, bool &ok) {
-                    ok = range < (uint64_t(1) << 32);
-                    return KeptOffsets{cols, slot, L, kShared, last, base};
-                });
+                kb, i, L, RowLoader<FWD>{crow, xrow, L, a.vec != 0}, __ldg(a.dt + i), a.out, kept);
             if (!solved && lane == 0) {
                 const uint32_t p = atomicAdd(a.list_count, 1u);
                 if (DC_CHECK(int64_t(p) < a.batch)) a.list[p] = uint32_t(i);
             }
             __syncwarp();  // the slice is read
         }
-        at = int64_t(__shfl_sync(0xffffffffu, next, 0)) * a.run;
+        at = shared_from + int64_t(__shfl_sync(0xffffffffu, next, 0)) * a.run;
+        if (at >= a.batch) break;
+        end = at + a.run < a.batch ? at + a.run : a.batch;
+        next = claim();
     }
 }
 
 template <bool FWD>
 __global__ void __launch_bounds__(32) solo_kernel(WarpArgs a)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
     const int L = a.L;
     const int64_t i = blockIdx.x;
-    int64_t *table = reinterpret_cast<int64_t *>(smem + 2 * chain_row_bytes(L));
+    int64_t *table = &sh<int64_t>(chain_pair_bytes(64));
+    if (threadIdx.x == 0) zero_row(0, 64);
     if (i == 0 && threadIdx.x == 0) *a.list_count = 0u;  // nothing is left to a second pass
-    chain_solve_warp<FWD, 1>(smem, i, L,
+    chain_solve_warp<FWD, 1>(0, i, L,
                              RowLoader<FWD>{a.comp + i * L, a.xfer + i * L, L, a.vec != 0},
-                             __ldg(a.dt + i), a.out,
-                             [&](int64_t, uint64_t, bool &) { return KeptValues{table, L}; });
+                             __ldg(a.dt + i), a.out, KeptValues{table, L});
 }
 
-inline size_t solo_smem_bytes(int L) { return 2 * chain_row_bytes(L) + size_t(tri_cells(L)) * 8; }
+inline size_t solo_smem_bytes(int L) { return chain_pair_bytes(64) + size_t(tri_cells(L)) * 8; }
 
 template <bool FWD, int NJ>
 cudaError_t launch_warp_nj(WarpArgs a, cudaStream_t stream)
@@ -112,12 +114,12 @@ cudaError_t launch_warp_nj(WarpArgs a, cudaStream_t stream)
     static DeviceCache attr;  // the shared-memory limit, raised once per device
     int nw = 4;  // warps per CTA (any number works: the warps are independent)
     if (const int f = forced_warps()) nw = f;
-    const size_t smem = size_t(nw) * warp_smem_bytes(a.L);
+    const size_t smem = size_t(nw) * warp_smem_bytes(a.L, NJ);
     int done = 0;
     cudaError_t e = attr.get(done, [](int &v) {
         v = 1;
         return cudaFuncSetAttribute(warp_kernel<FWD, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    int(8 * warp_smem_bytes(64 * NJ)));
+                                    8 * warp_smem_bytes(64 * NJ, NJ));
     });
     if (e != cudaSuccess) return e;
     int nb = 0;
@@ -125,15 +127,18 @@ cudaError_t launch_warp_nj(WarpArgs a, cudaStream_t stream)
     if (e != cudaSuccess) return e;
     if (nb < 1) nb = 1;
     if (nb * nw > kMaxWarpsPerSm) nb = kMaxWarpsPerSm / nw;
-    const int64_t warps = int64_t(sm_count()) * nb * nw;
-    // runs of up to 16 instances, at least 8 per warp: one atomic per instance would
-    // queue at the ticket (about 0.7 claims per ns), longer runs unbalance the end
-    int64_t run = a.batch / (warps * 8);
-    a.run = int(run < 1 ? 1 : run > 16 ? 16 : run);
-    const int64_t runs = (a.batch + a.run - 1) / a.run;
-    int64_t grid = (runs + nw - 1) / nw;
+    int64_t grid = (a.batch + nw - 1) / nw;
     if (grid > int64_t(sm_count()) * nb) grid = int64_t(sm_count()) * nb;
     if (grid > kSlotWarps / nw) grid = kSlotWarps / nw;
+    // The ticket takes about 1.2 claims per ns: with one claim per instance it alone took
+    // 55 us for 65,536 instances of L = 54. So each warp starts with three quarters of an
+    // equal share of its own, and only the rest comes from the ticket, in runs of up to 8,
+    // for the balance at the end (without shares, single instances from the ticket: 20,011
+    // x 129 113 us a direction against 107, 60,000 x 100 119 against 109).
+    const int64_t warps = grid * nw, share = a.batch / warps;
+    a.own = int(share >= 4 ? share * 3 / 4 : 0);
+    const int64_t run = (a.batch - a.own * warps) / (warps * 2);
+    a.run = int(run < 1 ? 1 : run > 8 ? 8 : run);
     warp_kernel<FWD, NJ><<<unsigned(grid), 32 * nw, smem, stream>>>(a);
     return cudaGetLastError();
 }
@@ -159,7 +164,7 @@ cudaError_t launch_solo(bool forward, int64_t batch, int L, const int64_t *comp,
     const bool vec = (L % 2 == 0) &&
                      ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0;
     const WarpArgs a{batch, L, comp, xfer, dt, out,
-                     nullptr, list_count, nullptr, nullptr, 1, vec ? 1 : 0};
+                     nullptr, list_count, nullptr, nullptr, 0, 1, vec ? 1 : 0};
     const size_t smem = solo_smem_bytes(L);  // 17.7 KB at L = 64
     if (forward)
         solo_kernel<true><<<unsigned(batch), 32, smem, stream>>>(a);
@@ -185,7 +190,7 @@ cudaError_t launch_warp(bool forward, int64_t batch, int L, const int64_t *comp,
     const bool vec = (L % 2 == 0) &&
                      ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0;
     const WarpArgs a{batch, L, comp, xfer, dt, out,
-                     ticket, list_count, list, slots, 1, vec ? 1 : 0};
+                     ticket, list_count, list, slots, 0, 1, vec ? 1 : 0};
     if (L <= 64) return forward ? launch_warp_nj<true, 1>(a, stream) : launch_warp_nj<false, 1>(a, stream);
     if (L <= 128) return forward ? launch_warp_nj<true, 2>(a, stream) : launch_warp_nj<false, 2>(a, stream);
     return forward ? launch_warp_nj<true, 3>(a, stream) : launch_warp_nj<false, 3>(a, stream);

@@ -431,8 +431,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) greedy_cta_kernel(GreedyArgs
         for (int w = tid; w < W; w += NT) word[w] = 0u;
         uint64_t a[NJ][2], b[NJ][2], aL, bL;
         const int st = cta_prefix<FWD, NJ>(
-            tot, orw, reinterpret_cast<uint64_t *>(best_of), L,
-            RowLoader<FWD>{g.comp + i * L, g.xfer + i * L, L, g.vec != 0}, dt, a, b, aL, bL);
+            tot, orw, L, RowLoader<FWD>{g.comp + i * L, g.xfer + i * L, L, g.vec != 0}, dt, a, b, aL, bL);
         if (st != DC_OK) {
             if (tid == 0) g.makespan[i] = -int64_t(st);
             for (int w = tid; w < W; w += NT) g.bits[i * W + w] = 0u;
