@@ -145,14 +145,16 @@ int64_t deep_slots_bound(int L)
 
 namespace {
 
-// Threads per instance: four rows per thread (two row pairs, whose searches hide
-// each other's latency) in a full GPU; two per thread, for a shorter column, while
-// `count` instances of twice the warps leave the SMs with no more than 32 warps
-// each (383 x 1,023: see the figures above).
+// Threads per instance: four rows per thread (two row pairs, whose searches hide each
+// other's latency) for long rows on a full GPU, two per thread otherwise, for shorter
+// columns and tracebacks. Measured per direction, two rows against four: 40,000 x 300
+// 296 us against 323, 383 x 1023 56 against 70, 2,432 x 1024 (256 warps per SM in all)
+// 108 against 109, 4,864 x 1024 179 against 165, 24,000 x 512 299 against 275.
 int deep_threads(int64_t count, int L, int sms)
 {
     const int nt2 = 32 * ((L + 127) / 128), nt1 = 32 * ((L + 63) / 64);
-    return nt1 <= kChainThreads && count * (nt1 / 32) <= int64_t(sms) * 32 ? nt1 : nt2;
+    if (nt1 > kChainThreads) return nt2;
+    return L <= 384 || count * (nt1 / 32) <= int64_t(sms) * 256 ? nt1 : nt2;
 }
 
 template <bool FWD, int NJ>

@@ -31,20 +31,20 @@ struct FusedOut {
 // into the workspace: lanes index them with their own draws, which global loads
 // serve in parallel where the parameter (constant) path serialises them.
 struct GenTables {
-    int64_t rate[kKnots + 1], bw[kKnots + 1], l0[kFixedMax], l1[kFixedMax];
+    int64_t rate[kKnots + 1], bw[kKnots + 1];
+    LayerRow layer[kFixedMax];
 };
 
 __global__ void __launch_bounds__(256) copy_tables_kernel(const __grid_constant__ GenParams g,
                                                           GenTables *t)
 {
-    for (int j = threadIdx.x; j <= kKnots; j += blockDim.x) {
-        t->rate[j] = g.rate_knots[j];
-        t->bw[j] = g.bw_knots[j];
-    }
-    for (int j = threadIdx.x; j < kFixedMax; j += blockDim.x) {
-        t->l0[j] = g.layer0[j];
-        t->l1[j] = g.layer1[j];
-    }
+    const int nl = g.layer_mode == DC_LAYERS_FIXED ? g.L
+                   : (g.layer_mode == DC_LAYERS_LOGUNIFORM ? kKnots + 1 : 0);
+    if (g.rate_dist == DC_DIST_LOGUNIFORM)
+        for (int j = threadIdx.x; j <= kKnots; j += blockDim.x) t->rate[j] = g.rate_knots[j];
+    if (g.bw_dist == DC_DIST_LOGUNIFORM)
+        for (int j = threadIdx.x; j <= kKnots; j += blockDim.x) t->bw[j] = g.bw_knots[j];
+    for (int j = threadIdx.x; j < nl; j += blockDim.x) t->layer[j] = g.layer[j];
 }
 
 // Shared memory of a warp of the pair pass, per lane (lane-interleaved words):
@@ -82,23 +82,37 @@ __global__ void __launch_bounds__(32, DC_SMALL_MINB)
         const int64_t i = tile * 32 + lane;
         const bool active = i < g.batch;
         const int64_t gi = g.inst0 + i;
-        InstanceDraws d = {};
-        if (active) d = instance_draws(g, t->rate, t->bw, gi);
+        int64_t dti = 0;
         __syncwarp();  // every lane is done with the area (the previous tile's table)
-        if (active) {
-            // rolled from kSplitMinL on: unrolled, the generator's divisions and the
-            // DP overflow the instruction cache
-#pragma unroll (L >= kSplitMinL ? 1 : L)
+        if (active && g.words) {
+            // rolled: unrolled, the generator's divisions and the DP overflow the
+            // instruction cache
+            const WordDraws d = word_draws(g, t->rate, t->bw, gi);
+            dti = d.dt;
+#pragma unroll 1
             for (int l = 0; l < L; ++l) {
-                int64_t params, flops, f, b, x;
-                layer_draws(g, t->l0, t->l1, gi, l, params, flops);
-                layer_costs(g, d, params, flops, f, b, x);
+                int64_t wire, flops;
+                uint32_t f, x;
+                uint64_t b;
+                layer_numerators(g, t->layer, gi, l, wire, flops);
+                word_costs(g, d.rate, d.bw, uint64_t(wire), uint64_t(flops), f, b, x);
+                stF[l] = int64_t(uint64_t(f));
+                stB[l] = int64_t(b);
+                stX[l] = int64_t(uint64_t(x));
+            }
+        } else if (active) {
+            const InstanceDraws d = instance_draws(g, t->rate, t->bw, gi);
+            dti = d.dt;
+#pragma unroll 1
+            for (int l = 0; l < L; ++l) {
+                int64_t wire, flops, f, b, x;
+                layer_numerators(g, t->layer, gi, l, wire, flops);
+                wire_costs(g, d, uint64_t(wire), uint64_t(flops), f, b, x);
                 stF[l] = f;
                 stB[l] = b;
                 stX[l] = x;
             }
         }
-        const int64_t dti = active ? d.dt : 0;
         uint64_t xraw[2];
         bool wide[2];
         int st[2];
@@ -171,9 +185,9 @@ struct DrawLoader {
     {
         c = x = 0;
         if (r > g.L) return;
-        int64_t params, flops, f, b, v;
-        layer_draws(g, t->l0, t->l1, gi, FWD ? r - 1 : g.L - r, params, flops);
-        layer_costs(g, d, params, flops, f, b, v);
+        int64_t wire, flops, f, b, v;
+        layer_numerators(g, t->layer, gi, FWD ? r - 1 : g.L - r, wire, flops);
+        wire_costs(g, d, uint64_t(wire), uint64_t(flops), f, b, v);
         c = uint64_t(FWD ? f : b);
         x = uint64_t(v);
     }

@@ -6,6 +6,7 @@
 // device: SplitMix64 draws, multiply-high uniform integers, piecewise-linear
 // log-uniform knots built on the host in double precision, and exact ceiling
 // divisions by multiply-high with a per-instance reciprocal.
+#include <algorithm>
 #include <cmath>
 
 #include "gen_device.cuh"
@@ -13,68 +14,105 @@
 namespace dc {
 namespace {
 
-// Warp-level tiles of 32 consecutive instances. Phase 1: lane j draws rate,
-// bandwidth and latency of instance j and forms the two division magic numbers
-// (32 instances' 64-bit divisions run side by side). Phase 2: the warp walks the
-// tile's 32*L (instance, layer) elements 32 at a time, so the four output rows
-// are written coalesced. Only __syncwarp between the phases.
+// Warp-level tiles of `ti` consecutive instances (32; fewer in small batches, so that
+// the elements spread over more warps). Phase 1: lane j draws rate, bandwidth and
+// latency of instance j and forms the two reciprocals (the instances' divisions run
+// side by side). Phase 2: the warp walks the tile's ti * L (instance, layer) elements 32
+// at a time, so the output rows are written coalesced. Only __syncwarp between the
+// phases.
+//
+// WORDS: every quotient is below 2^32 (all configurations here): divisions in 32-bit
+// steps (WordDiv), an instance's divisors in one 16-byte and one 4-byte load, a layer's
+// numerators in one 16-byte load. SHARED: the knots and layer tables in shared memory;
+// without it (small batches) lanes read the few entries they need from the parameters,
+// which beats copying the tables in every CTA. Bound by the HBM writes on large batches
+// (1,000,000 x 16, 520 MB: 84 us, 6.2 TB/s, with either division), by integer issue on
+// short rows (1,000,000 x 8: 48 us, 53 with 64-bit divisions) and on log-uniform layers
+// (16,384 x 1,024: 127 us, 376 with 64-bit divisions in tiles of 32).
 constexpr int kGenWarps = 8;
 
-__global__ void __launch_bounds__(32 * kGenWarps)
-    gen_kernel(const __grid_constant__ GenParams g, int64_t *__restrict__ fc,
+template <bool SHARED, bool WORDS>
+__global__ void __launch_bounds__(32 * kGenWarps, SHARED ? 5 : 1)
+    gen_kernel(const __grid_constant__ GenParams g, int ti, int tw, int64_t *__restrict__ fc,
                int64_t *__restrict__ pt, int64_t *__restrict__ bc, int64_t *__restrict__ gt,
                int64_t *__restrict__ dt)
 {
-    __shared__ int64_t s_rate[kKnots + 1], s_bw[kKnots + 1];
-    __shared__ int64_t s_l0[kFixedMax], s_l1[kFixedMax];
-    __shared__ uint64_t s_inst[kGenWarps][4][32];  // rate, magic(rate), bw, magic(bw)
-    const int L = g.L, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int nl = g.layer_mode == DC_LAYERS_FIXED ? L
-                   : (g.layer_mode == DC_LAYERS_LOGUNIFORM ? kKnots + 1 : 0);
-    for (int j = t; j <= kKnots; j += blockDim.x) {
-        s_rate[j] = g.rate_knots[j];
-        s_bw[j] = g.bw_knots[j];
+    extern __shared__ __align__(16) unsigned char dyn[];  // rate and bw knots, layer table
+    __shared__ uint4 s_div[kGenWarps][32];     // WORDS: rate.dn, rate.v, bw.dn, bw.v; else rate, its reciprocal
+    __shared__ uint4 s_div2[WORDS ? 1 : kGenWarps][32];  // else: bw, its reciprocal
+    __shared__ uint32_t s_shift[WORDS ? kGenWarps : 1][32];
+    const int L = g.L, t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = blockDim.x >> 5;
+    int64_t *s_rate = reinterpret_cast<int64_t *>(dyn), *s_bw = s_rate + kKnots + 1;
+    LayerRow *s_layer = reinterpret_cast<LayerRow *>(s_bw + kKnots + 1);
+    if (SHARED) {
+        const int nl = g.layer_mode == DC_LAYERS_FIXED ? L
+                       : (g.layer_mode == DC_LAYERS_LOGUNIFORM ? kKnots + 1 : 0);
+        if (g.rate_dist == DC_DIST_LOGUNIFORM)
+            for (int j = t; j <= kKnots; j += blockDim.x) s_rate[j] = g.rate_knots[j];
+        if (g.bw_dist == DC_DIST_LOGUNIFORM)
+            for (int j = t; j <= kKnots; j += blockDim.x) s_bw[j] = g.bw_knots[j];
+        for (int j = t; j < nl; j += blockDim.x) s_layer[j] = g.layer[j];
+        __syncthreads();
     }
-    for (int j = t; j < nl; j += blockDim.x) {
-        s_l0[j] = g.layer0[j];
-        s_l1[j] = g.layer1[j];
-    }
-    __syncthreads();
-    uint64_t(*si)[32] = s_inst[warp];
-    const int step_i = 32 / L, step_l = 32 % L;  // advance of (instance, layer) per 32 elements
-    const int64_t tiles = (g.batch + 31) / 32;
-    for (int64_t tile = int64_t(blockIdx.x) * kGenWarps + warp; tile < tiles;
-         tile += int64_t(gridDim.x) * kGenWarps) {
-        const int64_t i0 = tile * 32;
-        const int n_inst = int(g.batch - i0 < 32 ? g.batch - i0 : 32);
-        __syncwarp();  // previous tile done with si
+    // warp `sub` of the tw that share a tile takes every tw-th run of 32 elements
+    const int sub = warp % tw, stride = 32 * tw;
+    const int step_i = stride / L, step_l = stride % L;  // advance of (instance, layer) a step
+    const int64_t tiles = (g.batch + ti - 1) / ti;
+    for (int64_t tile = (int64_t(blockIdx.x) * nw + warp) / tw; tile < tiles;
+         tile += int64_t(gridDim.x) * nw / tw) {
+        const int64_t i0 = tile * ti;
+        const int n_inst = int(g.batch - i0 < ti ? g.batch - i0 : ti);
+        __syncwarp();  // previous tile done with the divisors
         if (lane < n_inst) {
             const int64_t i = i0 + lane;
-            const InstanceDraws d = instance_draws(g, s_rate, s_bw, g.inst0 + i);
-            si[0][lane] = d.rate;
-            si[1][lane] = d.mrate;
-            si[2][lane] = d.bw;
-            si[3][lane] = d.mbw;
-            dt[i] = d.dt;
+            const int64_t *kr = SHARED ? s_rate : g.rate_knots, *kw = SHARED ? s_bw : g.bw_knots;
+            if (WORDS) {
+                const WordDraws d = word_draws(g, kr, kw, g.inst0 + i);
+                s_div[warp][lane] = make_uint4(d.rate.dn, d.rate.v, d.bw.dn, d.bw.v);
+                s_shift[warp][lane] = d.rate.s | (d.bw.s << 8);
+                if (sub == 0) dt[i] = d.dt;
+            } else {
+                const InstanceDraws d = instance_draws(g, kr, kw, g.inst0 + i);
+                *reinterpret_cast<ulonglong2 *>(&s_div[warp][lane]) = make_ulonglong2(d.rate, d.mrate);
+                *reinterpret_cast<ulonglong2 *>(&s_div2[warp][lane]) = make_ulonglong2(d.bw, d.mbw);
+                if (sub == 0) dt[i] = d.dt;
+            }
         }
         __syncwarp();
         const int total = n_inst * L;
-        int il = lane / L, l = lane - (lane / L) * L;
-        for (int e = lane; e < total; e += 32) {
-            int64_t params, flops;
-            layer_draws(g, s_l0, s_l1, g.inst0 + i0 + il, l, params, flops);
-            InstanceDraws d;
-            d.rate = si[0][il];
-            d.mrate = si[1][il];
-            d.bw = si[2][il];
-            d.mbw = si[3][il];
-            int64_t f, b, x;
-            layer_costs(g, d, params, flops, f, b, x);
-            const int64_t o = i0 * L + e;
-            fc[o] = f;
-            bc[o] = b;
-            pt[o] = x;
-            gt[o] = x;
+        const int e0 = 32 * sub + lane;
+        int il = e0 / L, l = e0 - il * L;
+        const int64_t o0 = i0 * L + e0;
+        int64_t *pf = fc + o0, *pb = bc + o0, *px = pt + o0, *pg = gt + o0;
+        for (int e = e0; e < total; e += stride) {
+            int64_t wire, flops;
+            layer_numerators(g, SHARED ? s_layer : g.layer, g.inst0 + i0 + il, l, wire, flops);
+            if (WORDS) {
+                const uint4 d = s_div[warp][il];
+                const uint32_t s = s_shift[warp][il];
+                uint32_t f, x;
+                uint64_t b;
+                word_costs(g, WordDiv{d.x, d.y, s & 0xffu}, WordDiv{d.z, d.w, s >> 8}, uint64_t(wire),
+                           uint64_t(flops), f, b, x);
+                *pf = int64_t(uint64_t(f));
+                *pb = int64_t(b);
+                *px = int64_t(uint64_t(x));
+                *pg = int64_t(uint64_t(x));
+            } else {
+                const ulonglong2 r = *reinterpret_cast<const ulonglong2 *>(&s_div[warp][il]);
+                const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(&s_div2[warp][il]);
+                const InstanceDraws d{r.x, r.y, w.x, w.y, 0};
+                int64_t f, b, x;
+                wire_costs(g, d, uint64_t(wire), uint64_t(flops), f, b, x);
+                *pf = f;
+                *pb = b;
+                *px = x;
+                *pg = x;
+            }
+            pf += stride;
+            pb += stride;
+            px += stride;
+            pg += stride;
             il += step_i;
             l += step_l;
             if (l >= L) {
@@ -127,16 +165,28 @@ void fill_gen_params(const dc_profile_cfg *c, GenParams &g)
     g.params_hi = c->params_hi;
     g.flops_lo = c->flops_lo;
     g.flops_hi = c->flops_hi;
+    // the largest numerators, and whether their quotients all fit 32 bits
+    int64_t most_p = c->params_hi, most_f = c->flops_hi;
+    if (c->layer_mode == DC_LAYERS_FIXED) {
+        most_p = most_f = 0;
+        for (int l = 0; l < c->L; ++l) {
+            most_p = std::max(most_p, c->fixed_params[l]);
+            most_f = std::max(most_f, c->fixed_flops[l]);
+        }
+    }
+    auto fits = [](int64_t num, int64_t d) { return num / d < (int64_t(1) << 32); };
+    g.words = fits(int64_t(c->bits_per_param) * 1000 * most_p, c->bw_lo) &&
+              fits(int64_t(c->bwd_flops_mult == 2 ? 1 : c->bwd_flops_mult) * most_f, c->rate_lo);
     if (c->rate_dist == DC_DIST_LOGUNIFORM) knots(c->rate_lo, c->rate_hi, g.rate_knots);
     if (c->bw_dist == DC_DIST_LOGUNIFORM) knots(c->bw_lo, c->bw_hi, g.bw_knots);
     if (c->layer_mode == DC_LAYERS_FIXED) {
         for (int l = 0; l < c->L; ++l) {
-            g.layer0[l] = c->fixed_params[l];
-            g.layer1[l] = c->fixed_flops[l];
+            g.layer[l] = LayerRow{c->fixed_params[l] * (int64_t(c->bits_per_param) * 1000),
+                                  c->fixed_flops[l]};
         }
     } else if (c->layer_mode == DC_LAYERS_LOGUNIFORM) {
-        knots(c->params_lo, c->params_hi, g.layer0);
-        knots(c->flops_lo, c->flops_hi, g.layer1);
+        for (int j = 0; j <= kKnots; ++j)
+            g.layer[j] = LayerRow{knot(c->params_lo, c->params_hi, j), knot(c->flops_lo, c->flops_hi, j)};
     }
 }
 
@@ -175,10 +225,35 @@ cudaError_t launch_gen(const dc_profile_cfg *c, int64_t *fc, int64_t *pt, int64_
 {
     static thread_local GenParams g;  // 25 KB: kept off the caller's stack
     fill_gen_params(c, g);
-    const int64_t tiles = (c->batch + 31) / 32;
-    int64_t blocks = (tiles + kGenWarps - 1) / kGenWarps;
+    // tiles of 32 instances once they fill the GPU (8 warps per SM; 32 where a tile is long),
+    // else smaller ones, down to 32 elements, and for long rows several warps to an instance
+    int ti = 32, tw = 1;
+    auto tiles_of = [&](int n) { return (c->batch + n - 1) / n; };
+    while (ti > 1 && tiles_of(ti) < 152 * (ti * c->L >= 4096 ? 32 : 8) && ti / 2 * c->L >= 32) ti /= 2;
+    while (ti == 1 && tw < 4 && c->batch * tw < 152 * 32 && c->L >= 128 * tw) tw *= 2;
+    const int64_t warps = tiles_of(ti) * tw;
+    // few elements, and tables that lanes read at a few places only: no copy of them
+    // (4,096 x 8: 3.4 us from a graph, 7.2 with the copy and tiles of 32; but the
+    // log-uniform layer tables, read at 64 places a step, serialise: 11 times slower on
+    // 16,384 x 1,024)
+    if (c->batch * c->L <= (int64_t(1) << 18) && c->layer_mode != DC_LAYERS_LOGUNIFORM) {
+        const unsigned blocks = unsigned((warps + 3) / 4);
+        if (g.words)
+            gen_kernel<false, true><<<blocks, 128, 0, stream>>>(g, ti, tw, fc, pt, bc, gt, dt);
+        else
+            gen_kernel<false, false><<<blocks, 128, 0, stream>>>(g, ti, tw, fc, pt, bc, gt, dt);
+        return cudaGetLastError();
+    }
+    const size_t rows = c->layer_mode == DC_LAYERS_FIXED        ? size_t(c->L)
+                        : c->layer_mode == DC_LAYERS_LOGUNIFORM ? size_t(kKnots + 1)
+                                                                : 0;
+    const size_t smem = 2 * (kKnots + 1) * 8 + rows * sizeof(LayerRow);  // at most 24.6 KB
+    int64_t blocks = (warps + kGenWarps - 1) / kGenWarps;
     if (blocks > 152 * 8) blocks = 152 * 8;
-    gen_kernel<<<unsigned(blocks), 32 * kGenWarps, 0, stream>>>(g, fc, pt, bc, gt, dt);
+    if (g.words)
+        gen_kernel<true, true><<<unsigned(blocks), 32 * kGenWarps, smem, stream>>>(g, ti, tw, fc, pt, bc, gt, dt);
+    else
+        gen_kernel<true, false><<<unsigned(blocks), 32 * kGenWarps, smem, stream>>>(g, ti, tw, fc, pt, bc, gt, dt);
     return cudaGetLastError();
 }
 
