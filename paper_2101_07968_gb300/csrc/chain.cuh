@@ -450,16 +450,14 @@ __device__ __forceinline__ void scan2_flag(uint32_t &sa, uint32_t &sb, uint32_t 
     }
 }
 
-// Solves instance i with one warp, NJ row pairs per lane (L <= 64 NJ). kb: byte of the
-// warp's K, b beside it (chain_pair_bytes(64 NJ); the caller zeroes b's row 0 once with
-// zero_row). Returns false, having written nothing, when the instance is left to the
-// work list, as chain_solve does.
-template <bool FWD, int NJ, typename Load, typename Kept>
-__device__ __forceinline__ bool chain_solve_warp(int kb, int64_t i, int L, const Load &load,
-                                                 int64_t dt, const SolveOut &o, const Kept &kept)
+// The prefixes of an instance's rows over a warp, NJ row pairs per lane (L <= 64 NJ, the
+// row layout of chain_columns): go(a, b, aL, bL) gets them in int32_t where
+// a[L] + b[L] + (L + 1) dt < 2^31, otherwise in int64_t, and its value is returned; bad(st)
+// gets an input error's status.
+template <bool FWD, int NJ, typename Load, typename Go, typename Bad>
+__device__ __forceinline__ bool with_warp_prefix(int L, const Load &load, int64_t dt, Go go, Bad bad)
 {
     constexpr unsigned kAll = 0xffffffffu;
-    constexpr int D = 64 * NJ * 8 + 16;
     const int lane = threadIdx.x & 31;
     uint64_t a[NJ][2], b[NJ][2];
     uint32_t hi = uint32_t(uint64_t(dt) >> 32), flag = uint32_t(dt);
@@ -487,14 +485,10 @@ __device__ __forceinline__ bool chain_solve_warp(int kb, int64_t i, int L, const
         bL32 += __shfl_sync(kAll, sb, 31);
         flag |= aL32 | bL32;
     }
-    const bool narrow = !__any_sync(kAll, (hi | (flag >> 31)) != 0u) &&
-                        uint64_t(aL32) + bL32 + uint64_t(L + 1) * uint64_t(dt) < (uint64_t(1) << 31);
-    if (narrow) {
-        return chain_columns<FWD, int32_t, NJ, true>(
-            kb, D, static_cast<uint32_t *>(nullptr), static_cast<int32_t *>(nullptr), lane, 32, i, L,
-            int32_t(dt), a32, b32, int32_t(aL32), int32_t(bL32), kept, o);
-    }
-    // any other instance: 64-bit sums, the input checks, 64-bit values
+    if (!__any_sync(kAll, (hi | (flag >> 31)) != 0u) &&
+        uint64_t(aL32) + bL32 + uint64_t(L + 1) * uint64_t(dt) < (uint64_t(1) << 31))
+        return go(a32, b32, int32_t(aL32), int32_t(bL32));
+    // any other instance: 64-bit sums and the input checks
     uint64_t any = uint64_t(dt), aL = 0, bL = 0;
     int64_t a64[NJ][2], b64[NJ][2];
 #pragma unroll
@@ -510,19 +504,36 @@ __device__ __forceinline__ bool chain_solve_warp(int kb, int64_t i, int L, const
         bL += __shfl_sync(kAll, sb, 31);
     }
     const uint32_t all = __reduce_or_sync(kAll, uint32_t(any >> 32));
-    int st = DC_OK;
-    if (all >> 31)
-        st = DC_ERR_NEGATIVE;
-    else if (all >> 20 || exceeds_range(L, dt, FWD ? bL : aL, FWD ? aL : bL))
-        st = DC_ERR_RANGE;
-    if (st != DC_OK) {
-        chain_failure(st, i, words_for(L), lane, 32, o);
-        return true;
-    }
-    if (!Kept::kWhole && !words_hold(aL, bL, uint64_t(FWD ? dt : 0))) return false;
-    return chain_columns<FWD, int64_t, NJ, true>(
-        kb, D, static_cast<uint32_t *>(nullptr), static_cast<int64_t *>(nullptr), lane, 32, i, L, dt,
-        a64, b64, int64_t(aL), int64_t(bL), kept, o);
+    if (all >> 31) return bad(DC_ERR_NEGATIVE);
+    if (all >> 20 || exceeds_range(L, dt, FWD ? bL : aL, FWD ? aL : bL)) return bad(DC_ERR_RANGE);
+    return go(a64, b64, int64_t(aL), int64_t(bL));
+}
+
+// Solves instance i with one warp, NJ row pairs per lane (L <= 64 NJ). kb: byte of the
+// warp's K, b beside it (chain_pair_bytes(64 NJ); the caller zeroes b's row 0 once with
+// zero_row). Returns false, having written nothing, when the instance is left to the
+// work list, as chain_solve does.
+template <bool FWD, int NJ, typename Load, typename Kept>
+__device__ __forceinline__ bool chain_solve_warp(int kb, int64_t i, int L, const Load &load,
+                                                 int64_t dt, const SolveOut &o, const Kept &kept)
+{
+    constexpr int D = 64 * NJ * 8 + 16;
+    const int lane = threadIdx.x & 31;
+    return with_warp_prefix<FWD, NJ>(
+        L, load, dt,
+        [&](const auto &a, const auto &b, auto aL, auto bL) {
+            using T = decltype(aL);
+            if (sizeof(T) == 8 && !Kept::kWhole &&
+                !words_hold(uint64_t(aL), uint64_t(bL), uint64_t(FWD ? dt : 0)))
+                return false;
+            return chain_columns<FWD, T, NJ, true>(kb, D, static_cast<uint32_t *>(nullptr),
+                                                   static_cast<T *>(nullptr), lane, 32, i, L, T(dt),
+                                                   a, b, aL, bL, kept, o);
+        },
+        [&](int st) {
+            chain_failure(st, i, words_for(L), lane, 32, o);
+            return true;
+        });
 }
 
 // ---------------------------------------------------------------- CTA per instance

@@ -26,13 +26,15 @@
 // (forward: end_s = max(end_{s-1}, s*dt + P[b_s]) + FC[b_s] - FC[b_{s-1}];
 // backward: link = max(link, BC[q..L]) + dt + GT of the segment).
 //
-// Two kernels, chosen in per_thread. One instance per thread scans its own rows: O(L) for
-// Algorithm 1, O(L^2) for Algorithm 2, bound by the latency of its uncoalesced reads.
-// One instance per CTA (a single warp up to L = 64) has its prefix sums in shared
-// memory: Algorithm 1's one chain takes a 32-way search per step, and Algorithm 2's
-// L - 1 chains, one per second position, run one per thread with a binary search per
-// step; it is bound by integer issue and by the longest chain of the warp.
-// 65,537 x 54 (ResNet-50): backward 142 us, 1,554 one instance per thread.
+// Three kernels, chosen in launch_greedy. One instance per thread scans its own rows: O(L)
+// for Algorithm 1, O(L^2) for Algorithm 2, bound by the latency of its uncoalesced reads.
+// One instance per warp (L <= 64) or per CTA has its prefix sums in registers and
+// shared memory: Algorithm 1's one chain takes a search over all rows at once per step (a
+// ballot, or 32 probes), and Algorithm 2's L - 1 chains, one per second position, run
+// side by side with a binary search per step; both are bound by integer issue and by
+// the longest chain of the warp.
+// 65,537 x 54 (ResNet-50): forward 18 us and backward 80 us of kernel time (45 and 1,540
+// one instance per thread, 127 backward with 64-bit prefixes, one chain per lane at a time).
 #include "chain.cuh"
 
 namespace dc {
@@ -293,7 +295,7 @@ __device__ T greedy_forward_warp(const T *A, const T *B, int L, T dt, uint32_t *
     mark(n);
     T pull = dt + dt, end = dt + A[n] + B[n];
     end = max(end, pull + A[m]) + (B[m] - B[n]);
-    while (m < L) {
+    for (int step = 2; m < L && step <= L; ++step) {  // m grows every time
         mark(m);
         // the first x that covers the segment's compute, else the first with all transfers
         const T thr = min(A[m] + (B[m] - B[n]) - dt, aL);
@@ -313,7 +315,7 @@ __device__ __forceinline__ T greedy_chain(const T *A, const T *B, int L, int P, 
 {
     T link = A[p] + dt + B[p], sent = dt;
     visit(p);
-    while (p < L) {
+    for (int step = p; p < L && step < L; ++step) {  // p grows every time
         // the longest segment whose compute the link estimate covers, else one layer
         // and the zero-compute layers after it
         const T lim = max(A[p] + sent + B[p], A[p + 1]);
@@ -417,6 +419,176 @@ __device__ void greedy_solve(unsigned char *smem, uint32_t *word, longlong2 *bes
     }
 }
 
+// Algorithm 1 by one warp, two rows per lane (rows past L hold the totals). mine: lane
+// w's decision word w. Returns f_m.
+template <typename T>
+__device__ __forceinline__ T greedy_forward_rows(int kb, int D, int L, T dt, const T (&a)[1][2],
+                                                 const T (&b)[1][2], T aL, uint32_t &mine)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int S = int(sizeof(T));
+    const int lane = threadIdx.x & 31, r = 2 * lane + 1;
+    auto A = [&](int m) { return sh<T>(kb + (m - 1) * S); };
+    auto B = [&](int m) { return sh<T>(kb + D + (m - 1) * S); };
+    // the first row x past `from` with A[x] >= thr (thr <= A[L])
+    auto first = [&](T thr, int from) {
+        const int below = __popc(__ballot_sync(kAll, a[0][0] < thr)) + __popc(__ballot_sync(kAll, a[0][1] < thr));
+        return max(below, from) + 1;
+    };
+    auto mark = [&](int l) { mine |= lane == ((l - 1) >> 5) ? 1u << ((l - 1) & 31) : 0u; };
+    const T lim = dt + aL;
+    const int last = __popc(__ballot_sync(kAll, r < L && a[0][0] + b[0][0] <= lim)) +
+                     __popc(__ballot_sync(kAll, r + 1 < L && a[0][1] + b[0][1] <= lim));
+    int n = 1, m;
+    if (last >= 1) {
+        const T bl = B(last);
+        n = 1 + __popc(__ballot_sync(kAll, b[0][0] < bl)) + __popc(__ballot_sync(kAll, b[0][1] < bl));
+        m = first(A(n) + B(n) - dt, n);
+    } else {
+        m = first(aL, 1);
+    }
+    mark(n);
+    T pull = dt + dt, Bm = B(m), Am = A(m), Bn = B(n);
+    T end = dt + A(n) + Bn;
+    end = max(end, pull + Am) + (Bm - Bn);
+    for (int step = 2; m < L && step <= L; ++step) {  // m grows every time
+        mark(m);
+        const int x = first(min(Am + (Bm - Bn) - dt, aL), m);
+        pull += dt;
+        Bn = Bm;
+        Am = A(x);
+        Bm = B(x);
+        end = max(end, pull + Am) + (Bm - Bn);
+        m = x;
+    }
+    return end;
+}
+
+// Algorithm 2 by one warp (L <= 64): lane l runs the chains whose first push holds the
+// last l + 1 and l + 33 layers, both at once. The best chain's breaks go to its lane's
+// `breaks`; returns f_m and that lane.
+template <typename T>
+__device__ __forceinline__ T greedy_backward_rows(int kb, int D, int L, T dt, T aL,
+                                                  uint64_t &breaks, int &owner)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int S = int(sizeof(T));
+    const int lane = threadIdx.x & 31;
+    const int end = kb + L * S;  // where row L + 1 would be
+    // chain u stands at row p; q: byte of row p + 1
+    int q[2];
+    T A[2], B[2], next[2], link[2];
+    uint64_t mask[2] = {0, 0};
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int p = min(lane + 32 * u + 1, L);
+        q[u] = kb + p * S;
+        A[u] = sh<T>(q[u] - S);
+        B[u] = sh<T>(q[u] + D - S);
+        next[u] = sh<T>(q[u]);
+        link[u] = A[u] + dt + B[u];
+    }
+    const int own0 = q[0], own1 = q[1];
+    T sent = dt;
+    // a chain advances by a row or more each step, so L steps end them all
+    for (int step = 1; step < L && __any_sync(kAll, q[0] < end || q[1] < end); ++step) {
+        T t[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const bool on = q[u] < end;
+            const int p = (q[u] - kb) / S;  // 1..L
+            mask[u] |= on ? uint64_t(1) << (p - 1) : uint64_t(0);
+            // the longest segment whose compute the link estimate covers, else one layer
+            // and the zero-compute layers after it; a finished chain stays at L
+            t[u] = (on ? max(A[u] + sent + B[u], next[u]) : aL) + 1;
+        }
+        int n0 = kb, n1 = kb;
+        halve_from<T, 32>(t[0], t[1], n0, n1);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const bool on = q[u] < end;
+            q[u] = aL < t[u] ? end : (u == 0 ? n0 : n1);  // the search counts to 63 rows
+            const T a = sh<T>(q[u] - S), b = sh<T>(q[u] + D - S);
+            next[u] = sh<T>(q[u]);
+            link[u] = on ? max(link[u], a) + dt + (b - B[u]) : link[u];
+            A[u] = a;
+            B[u] = b;
+        }
+        sent += dt;
+    }
+    // least f_m, the longest first push on ties; chains that began at L are none
+    int64_t best = INT64_MAX;
+    int from = 0;
+    if (own0 < end) {
+        best = int64_t(link[0]);
+        from = own0;
+        breaks = mask[0];
+    }
+    if (own1 < end && int64_t(link[1]) <= best) {
+        best = int64_t(link[1]);
+        from = own1;
+        breaks = mask[1];
+    }
+    owner = lane;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        const int64_t ob = __shfl_xor_sync(kAll, best, d);
+        const int of = __shfl_xor_sync(kAll, from, d), oo = __shfl_xor_sync(kAll, owner, d);
+        if (ob < best || (ob == best && of > from)) {
+            best = ob;
+            from = of;
+            owner = oo;
+        }
+    }
+    return T(best);
+}
+
+template <bool FWD>
+__global__ void __launch_bounds__(256, 5) greedy_warp_kernel(GreedyArgs g)
+{
+    constexpr int D = 64 * 8 + 16;
+    const int L = g.L, W = words_for(L), lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int kb = int(threadIdx.x >> 5) * chain_pair_bytes(64);
+    for (int64_t i = int64_t(blockIdx.x) * nw + (threadIdx.x >> 5); i < g.batch; i += int64_t(gridDim.x) * nw) {
+        const int64_t dt = __ldg(g.dt + i);
+        with_warp_prefix<FWD, 1>(
+            L, RowLoader<FWD>{g.comp + i * L, g.xfer + i * L, L, g.vec != 0}, dt,
+            [&](const auto &a, const auto &b, auto aL, auto bL) {
+                using T = decltype(aL);
+                using P2 = Pair<T>;
+                using Two = typename P2::type;
+                constexpr int S = int(sizeof(T));
+                const int r = 2 * lane + 1;
+                sh<Two>(kb + 2 * lane * S) = P2::make(r <= L ? a[0][0] : P2::kMax, r < L ? a[0][1] : P2::kMax);
+                sh<Two>(kb + D + 2 * lane * S) = P2::make(b[0][0], b[0][1]);
+                __syncwarp();
+                uint32_t mine = 0u;
+                T t = aL + bL + T(dt);  // L = 1: one segment
+                if (L > 1) {
+                    if (FWD) {
+                        t = greedy_forward_rows<T>(kb, D, L, T(dt), a, b, aL, mine);
+                    } else {
+                        uint64_t breaks = 0;
+                        int owner = 0;
+                        t = greedy_backward_rows<T>(kb, D, L, T(dt), aL, breaks, owner);
+                        breaks = __shfl_sync(0xffffffffu, breaks, owner);
+                        mine = lane == 0 ? uint32_t(breaks) : uint32_t(breaks >> 32);
+                    }
+                }
+                if (lane == 0) g.makespan[i] = int64_t(t);
+                if (lane < W) g.bits[i * W + lane] = mine;
+                __syncwarp();
+                return true;
+            },
+            [&](int st) {
+                if (lane == 0) g.makespan[i] = -int64_t(st);
+                if (lane < W) g.bits[i * W + lane] = 0u;
+                __syncwarp();
+                return true;
+            });
+    }
+}
+
 template <bool FWD, int NJ>
 __global__ void __launch_bounds__(kChainThreads, 1) greedy_cta_kernel(GreedyArgs g)
 {
@@ -468,14 +640,15 @@ cudaError_t launch_greedy_cta(const GreedyArgs &g, int nt, cudaStream_t stream)
 }
 
 // One instance per thread where a warp's lanes are better used on 32 instances than on
-// one short row. Forward: up to L = 32 (100,000 x 20: 41 us against 76 per CTA; equal at
-// 32), and up to 128 on large batches (100,000 x 100: 139 against 152; but 10,000 x 100:
-// 50 against 39). Backward, quadratic in L per thread: up to L = 8, and up to 12 on large
-// batches (100,000 x 12: 82 us against about 95; 100,000 x 17: 174 against 98).
+// one short row. Forward: up to L = 22 (100,000 x 20: 38 us against 44 per warp, 500,000
+// x 24 equal, 100,000 x 32 72 against 45), and above the warp kernel's rows up to 128
+// on large batches (100,000 x 100: 139 against 152 per CTA; but 10,000 x 100: 50 against
+// 39). Backward, quadratic in L per thread: up to L = 8, and up to 12 on large batches
+// (500,000 x 12: 208 us against 284; 100,000 x 12 76 against 73).
 template <bool FWD>
 bool per_thread(int64_t batch, int L)
 {
-    if (FWD) return L <= 32 || (L <= 128 && batch >= 50000);
+    if (FWD) return L <= 22 || (L > 64 && L <= 128 && batch >= 50000);
     return L <= 8 || (L <= 12 && batch >= 50000);
 }
 
@@ -491,6 +664,14 @@ cudaError_t launch_greedy(int64_t batch, int L, const int64_t *comp, const int64
     const bool vec = (L % 2 == 0) &&
                      ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0;
     const GreedyArgs g{batch, L, comp, xfer, dt, makespan, bits, vec ? 1 : 0};
+    if (L <= 64) {
+        // one-warp CTAs until they fill the GPU, then four warps to a CTA in four waves
+        const int nw = batch < int64_t(sm_count()) * 32 ? 1 : 4;
+        int64_t grid = (batch + nw - 1) / nw;
+        if (nw > 1 && grid > int64_t(sm_count()) * 10 * 4) grid = int64_t(sm_count()) * 10 * 4;
+        greedy_warp_kernel<FWD><<<unsigned(grid), 32 * nw, nw * chain_pair_bytes(64), stream>>>(g);
+        return cudaGetLastError();
+    }
     const int nt = 32 * ((L + 63) / 64);
     return nt <= kChainThreads ? launch_greedy_cta<FWD, 1>(g, nt, stream)
                                : launch_greedy_cta<FWD, 2>(g, 32 * ((L + 127) / 128), stream);
