@@ -1,10 +1,10 @@
-// CTA-per-instance DynaComm DP for any 1 <= L <= 4096 (Eq. 8 / Algorithm 3 and
+// DynaComm DP of listed instances, any 1 <= L <= 4096 (Eq. 8 / Algorithm 3 and
 // Eq. 9 / Algorithm 4): the pass over the first passes' work lists (dp_small.cu,
 // dp_mid.cu, dp_warp.cu, dp_deep.cu), whose instances have values
 // beyond the first pass's range or an optimum deeper than its kept columns. The
 // method is in chain.cuh; this pass takes every value (64 bits) and keeps every
-// column, in shared memory up to L = 64, otherwise in a per-CTA table of the
-// caller's workspace.
+// column: one warp per instance with the table in shared memory up to L = 64, otherwise
+// one CTA per instance with a table in the caller's workspace.
 #include "chain.cuh"
 
 namespace dc {
@@ -17,22 +17,15 @@ struct GroupArgs {
     const int64_t *comp, *xfer, *dt;
     SolveOut out;
     const uint32_t *list_count, *list;
-    unsigned char *tables;  // nullptr: the table in shared memory
+    unsigned char *tables;  // L > 64: the tables of the CTAs
     int vec;                // the cost rows are 16-byte aligned
 };
-
-__host__ __device__ inline int group_table_offset(int L, int rows)
-{
-    return int((chain_smem_bytes(L, rows) + 15) / 16 * 16);
-}
 
 template <bool FWD, int NJ>
 __global__ void __launch_bounds__(kChainThreads, 1) group_kernel(GroupArgs a)
 {
     const int L = a.L;
-    int64_t *table = a.tables ? reinterpret_cast<int64_t *>(
-                                    a.tables + size_t(blockIdx.x) * size_t(tri_cells(L)) * 8)
-                              : &sh<int64_t>(group_table_offset(L, 2 * NJ * int(blockDim.x)));
+    int64_t *table = reinterpret_cast<int64_t *>(a.tables + size_t(blockIdx.x) * size_t(tri_cells(L)) * 8);
     pdl_wait();  // the first pass has finished its list
     const int64_t count = int64_t(*a.list_count);
     for (int64_t j = blockIdx.x; j < count; j += gridDim.x) {
@@ -45,6 +38,46 @@ __global__ void __launch_bounds__(kChainThreads, 1) group_kernel(GroupArgs a)
     }
 }
 
+// L <= 64: one warp per instance, the table in shared memory. The CTA form's barriers and
+// 64-bit scan cost it ten times the time there: 1,000,000 x 16 with some 6,000 instances
+// listed took 121 us a direction with it, 103 with this kernel (70 of it the first pass).
+template <bool FWD>
+__global__ void __launch_bounds__(32) list_warp_kernel(GroupArgs a)
+{
+    const int L = a.L;
+    int64_t *table = &sh<int64_t>(chain_pair_bytes(64));
+    if (threadIdx.x == 0) zero_row(0, 64);
+    pdl_wait();  // the first pass has finished its list
+    const int64_t count = int64_t(*a.list_count);
+    for (int64_t j = blockIdx.x; j < count; j += gridDim.x) {
+        const int64_t i = int64_t(a.list[j]);
+        if (!DC_CHECK(i >= 0 && i < a.batch)) continue;
+        chain_solve_warp<FWD, 1>(0, i, L,
+                                 RowLoader<FWD>{a.comp + i * L, a.xfer + i * L, L, a.vec != 0},
+                                 __ldg(a.dt + i), a.out, KeptValues{table, L});
+        __syncwarp();  // shared memory is read
+    }
+}
+
+// Launched early (programmatic dependent launch): the CTAs wait in hardware until the
+// first pass completes, so the launch overlaps that pass's tail.
+template <typename Kernel>
+cudaError_t launch_list(Kernel kernel, const GroupArgs &a, int64_t grid, int nt, size_t smem,
+                        cudaStream_t stream)
+{
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(unsigned(grid));
+    lc.blockDim = dim3(unsigned(nt));
+    lc.dynamicSmemBytes = smem;
+    lc.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kernel, a);
+}
+
 template <bool FWD, int NJ>
 cudaError_t launch_group_nj(const GroupArgs &a, int nt, int64_t grid, cudaStream_t stream)
 {
@@ -53,27 +86,18 @@ cudaError_t launch_group_nj(const GroupArgs &a, int nt, int64_t grid, cudaStream
     const cudaError_t e = attr.get(done, [](int &v) {
         v = 1;
         return cudaFuncSetAttribute(group_kernel<FWD, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    int(chain_smem_most(DC_L_MAX)) + 1024);
+                                    int(chain_smem_most(DC_L_MAX)));
     });
     if (e != cudaSuccess) return e;
-    // launched early (programmatic dependent launch): its CTAs wait in hardware until
-    // the first pass completes, so the launch overlaps that pass's tail
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(unsigned(grid));
-    lc.blockDim = dim3(unsigned(nt));
-    lc.dynamicSmemBytes = group_table_offset(a.L, 2 * NJ * nt) + (a.tables ? 0 : size_t(tri_cells(a.L)) * 8);
-    lc.stream = stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, group_kernel<FWD, NJ>, a);
+    return launch_list(group_kernel<FWD, NJ>, a, grid, nt, chain_smem_bytes(a.L, 2 * NJ * nt), stream);
 }
 
 template <bool FWD>
 cudaError_t launch_group_dir(const GroupArgs &a, int64_t grid, cudaStream_t stream)
 {
+    if (a.L <= kSmemTableLMax)
+        return launch_list(list_warp_kernel<FWD>, a, grid, 32,
+                           chain_pair_bytes(64) + size_t(tri_cells(a.L)) * 8, stream);
     // lists are short: two rows per thread, for the shortest column
     int nt = 32 * ((a.L + 63) / 64);
     if (nt > kChainThreads) nt = 32 * ((a.L + 127) / 128);
