@@ -184,6 +184,19 @@ dc_status dc_schedule_generated_batch(const dc_profile_cfg *cfg, int64_t *makesp
                                       size_t workspace_bytes, cudaStream_t stream);
 
 /* ------------------------------------------------------------------------
+ * dc_step_batch -- a whole step for 1 <= L <= 16 in one pass over the batch:
+ * dc_schedule_generated_batch that also writes the profiles it draws (fc, pt, bc,
+ * gt [batch][L], dt [batch], as dc_profile_gen) and f_m of each decision (replay
+ * [2][batch], as dc_eval_timeline_batch). The results are those of the separate
+ * calls, bit for bit. Workspace and errors as for dc_schedule_generated_batch; the
+ * profile arrays and replay must not be NULL.
+ * ---------------------------------------------------------------------- */
+dc_status dc_step_batch(const dc_profile_cfg *cfg, int64_t *fc, int64_t *pt, int64_t *bc,
+                        int64_t *gt, int64_t *dt, int64_t *makespan, uint32_t *bits, int32_t *nseg,
+                        int32_t *status, int64_t *replay, void *workspace, size_t workspace_bytes,
+                        cudaStream_t stream);
+
+/* ------------------------------------------------------------------------
  * dc_greedy_forward_batch, dc_greedy_backward_batch -- the paper's competing
  * schedulers (Sec. II-C), for comparison with the DP: greedy parameter
  * scheduling of iBatch (Algorithm 1, forward; inputs as

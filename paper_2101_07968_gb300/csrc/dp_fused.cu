@@ -23,6 +23,9 @@ inline size_t fused_tables_offset(int64_t batch) { return (256 + 8 * size_t(batc
 
 struct FusedOut {
     SolveOut out[2];
+    // STORE: the drawn profiles; pairs: 16-byte aligned
+    int64_t *fc, *pt, *bc, *gt, *dt;
+    int pairs;
     uint32_t *wide_count[2], *wide_list[2];
     uint32_t *ticket;  // tiles handed out (zero before the launch)
 };
@@ -61,8 +64,11 @@ struct Pair32 {
     static constexpr int kBytes = kRowsBytes > kSlotBytes ? kRowsBytes : kSlotBytes;
 };
 
-// Both directions of each instance from one draw of its rows.
-template <int L>
+// Both directions of each instance from one draw of its rows. STORE: a whole step, which
+// also writes the profiles out, coalesced from the staged rows, and f_m of the decisions:
+// the writes run under the solve (1,000,000 x 8: 99 us, 115 as a generator pass that
+// writes and two solves that read; at L = 16 the solve binds and both take 204).
+template <int L, bool STORE>
 __global__ void __launch_bounds__(32, DC_SMALL_MINB)
     fused_pair_kernel(const __grid_constant__ GenParams g, const GenTables *t, const FusedOut o)
 {
@@ -113,6 +119,33 @@ __global__ void __launch_bounds__(32, DC_SMALL_MINB)
                 stX[l] = x;
             }
         }
+        if constexpr (STORE) {
+            __syncwarp();
+            const int64_t *sf = reinterpret_cast<const int64_t *>(smem);
+            const int64_t *sb = sf + 32 * K::kStride, *sx = sb + 32 * K::kStride;
+            const int rows = int(g.batch - tile * 32 < 32 ? g.batch - tile * 32 : 32);
+            const int64_t o0 = tile * 32 * L;
+            if (L % 2 == 0 && o.pairs) {
+                constexpr int H = L / 2 > 0 ? L / 2 : 1;  // pairs per row
+                for (int p = lane; p < rows * H; p += 32) {
+                    const int r = p / H, at = r * K::kStride + 2 * (p - r * H);
+                    const longlong2 x = *reinterpret_cast<const longlong2 *>(sx + at);
+                    *reinterpret_cast<longlong2 *>(o.fc + o0 + 2 * p) = *reinterpret_cast<const longlong2 *>(sf + at);
+                    *reinterpret_cast<longlong2 *>(o.bc + o0 + 2 * p) = *reinterpret_cast<const longlong2 *>(sb + at);
+                    *reinterpret_cast<longlong2 *>(o.pt + o0 + 2 * p) = x;
+                    *reinterpret_cast<longlong2 *>(o.gt + o0 + 2 * p) = x;
+                }
+            } else {
+                for (int e = lane; e < rows * L; e += 32) {
+                    const int r = e / L, at = r * K::kStride + (e - r * L);
+                    o.fc[o0 + e] = sf[at];
+                    o.bc[o0 + e] = sb[at];
+                    o.pt[o0 + e] = sx[at];
+                    o.gt[o0 + e] = sx[at];
+                }
+            }
+            if (active) o.dt[i] = dti;
+        }
         uint64_t xraw[2];
         bool wide[2];
         int st[2];
@@ -144,7 +177,7 @@ __global__ void __launch_bounds__(32, DC_SMALL_MINB)
             const bool wd = fwd ? wide[0] : wide[1];
             const uint64_t xd = fwd ? xraw[0] : xraw[1];
             const SolveOut od = fwd ? o.out[0] : o.out[1];
-            const bool done = solve_uv<L, false>(fwd, active && std == DC_OK && !wd, U, V, int32_t(dti),
+            const bool done = solve_uv<L, STORE>(fwd, active && std == DC_OK && !wd, U, V, int32_t(dti),
                                                  xd, lw, i, od);
             if (active && std != DC_OK) {
                 write_failure(std, i, W, od);
@@ -240,25 +273,25 @@ cudaError_t launch_fused_list(const GenParams &g, const GenTables *t, const Fuse
     return cudaLaunchKernelEx(&lc, fused_list_kernel<FWD>, g, t, o);
 }
 
-template <int L>
+template <int L, bool STORE>
 cudaError_t launch_fused_L(const GenParams &g, const GenTables *t, const FusedOut &o,
                            cudaStream_t stream)
 {
     static DeviceCache resident;  // single-warp CTAs of the pair kernel per SM
     int per_sm = 0;
     cudaError_t le = resident.get(per_sm, [](int &n) {
-        cudaError_t e = cudaFuncSetAttribute(fused_pair_kernel<L>,
+        cudaError_t e = cudaFuncSetAttribute(fused_pair_kernel<L, STORE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              Pair32<L>::kBytes);
         if (e != cudaSuccess) return e;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fused_pair_kernel<L>, 32,
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fused_pair_kernel<L, STORE>, 32,
                                                              Pair32<L>::kBytes);
     });
     if (le != cudaSuccess) return le;
     const int64_t tiles = (g.batch + 31) / 32;
     int64_t grid = int64_t(sm_count()) * per_sm;
     if (grid > tiles) grid = tiles;
-    fused_pair_kernel<L><<<unsigned(grid), 32, Pair32<L>::kBytes, stream>>>(g, t, o);
+    fused_pair_kernel<L, STORE><<<unsigned(grid), 32, Pair32<L>::kBytes, stream>>>(g, t, o);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = launch_fused_list<true>(g, t, o, stream);
@@ -270,21 +303,28 @@ cudaError_t launch_fused_L(const GenParams &g, const GenTables *t, const FusedOu
 
 size_t fused_workspace_bytes(int64_t batch) { return fused_tables_offset(batch) + sizeof(GenTables); }
 
-// Generate-and-solve for 1 <= L <= 16: outputs [2][batch] (forward first).
-cudaError_t launch_fused(const GenParams &g, int64_t *makespan, uint32_t *bits, int32_t *nseg,
-                         int32_t *status, void *workspace, cudaStream_t stream)
+// Generate-and-solve for 1 <= L <= 16; rows: where the profiles go, or null.
+cudaError_t launch_fused(const GenParams &g, const SolveOut (&out)[2], const StepRows *rows,
+                         void *workspace, cudaStream_t stream)
 {
     const int64_t B = g.batch;
-    const int W = words_for(g.L);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
-    FusedOut o;
+    FusedOut o = {};
     for (int d = 0; d < 2; ++d) {
-        o.out[d] = SolveOut{makespan + d * B, bits + d * B * W, nseg ? nseg + d * B : nullptr,
-                            status ? status + d * B : nullptr, nullptr};
+        o.out[d] = out[d];
         o.wide_count[d] = reinterpret_cast<uint32_t *>(ws) + d;
         o.wide_list[d] = reinterpret_cast<uint32_t *>(ws + 256) + d * B;
     }
     o.ticket = reinterpret_cast<uint32_t *>(ws) + 2;
+    if (rows) {
+        o.fc = rows->fc;
+        o.pt = rows->pt;
+        o.bc = rows->bc;
+        o.gt = rows->gt;
+        o.dt = rows->dt;
+        o.pairs = ((reinterpret_cast<uintptr_t>(o.fc) | reinterpret_cast<uintptr_t>(o.pt) |
+                    reinterpret_cast<uintptr_t>(o.bc) | reinterpret_cast<uintptr_t>(o.gt)) & 15u) == 0;
+    }
     cudaError_t e = cudaMemsetAsync(ws, 0, 3 * sizeof(uint32_t), stream);
     if (e != cudaSuccess) return e;
     GenTables *t = reinterpret_cast<GenTables *>(ws + fused_tables_offset(B));
@@ -292,7 +332,9 @@ cudaError_t launch_fused(const GenParams &g, int64_t *makespan, uint32_t *bits, 
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
 #define DC_FUSED_CASE(LL) \
-    case LL: return launch_fused_L<LL>(g, t, o, stream);
+    case LL:                                          \
+        return rows ? launch_fused_L<LL, true>(g, t, o, stream) \
+                    : launch_fused_L<LL, false>(g, t, o, stream);
     switch (g.L) {
         DC_FUSED_CASE(1) DC_FUSED_CASE(2) DC_FUSED_CASE(3) DC_FUSED_CASE(4)
         DC_FUSED_CASE(5) DC_FUSED_CASE(6) DC_FUSED_CASE(7) DC_FUSED_CASE(8)

@@ -133,25 +133,50 @@ size_t dc_schedule_generated_workspace_bytes(int64_t batch, int32_t L)
     return dc::fused_workspace_bytes(batch);
 }
 
-dc_status dc_schedule_generated_batch(const dc_profile_cfg *cfg, int64_t *makespan,
-                                      uint32_t *bits, int32_t *nseg, int32_t *status,
-                                      void *workspace, size_t workspace_bytes,
-                                      cudaStream_t stream)
+static dc_status generated(const dc_profile_cfg *cfg, const dc::StepRows *rows, int64_t *makespan,
+                           uint32_t *bits, int32_t *nseg, int32_t *status, int64_t *replay,
+                           void *workspace, size_t workspace_bytes, cudaStream_t stream)
 {
-    const dc::NvtxRange nvtx("dc_schedule_generated_batch");
     if (!cfg) return DC_ERR_NULL;
     const dc_status st = dc::check_profile_cfg(cfg);
     if (st != DC_OK) return st;
     if (cfg->L > dc::kSmallLMax || cfg->batch > int64_t(0xffffffffll)) return DC_ERR_BAD_SHAPE;
     if (cfg->batch == 0) return DC_OK;
     if (!makespan || (!bits && dc::words_for(cfg->L) > 0)) return DC_ERR_NULL;
+    if (rows && (!rows->fc || !rows->pt || !rows->bc || !rows->gt || !rows->dt || !replay))
+        return DC_ERR_NULL;
     if (!workspace || workspace_bytes < dc::fused_workspace_bytes(cfg->batch))
         return DC_ERR_WORKSPACE;
     static thread_local dc::GenParams g;  // 25 KB: kept off the caller's stack
     dc::fill_gen_params(cfg, g);
-    return dc::launch_fused(g, makespan, bits, nseg, status, workspace, stream) == cudaSuccess
-               ? DC_OK
-               : DC_ERR_CUDA;
+    const int64_t B = cfg->batch, W = dc::words_for(cfg->L);
+    dc::SolveOut out[2];
+    for (int d = 0; d < 2; ++d)
+        out[d] = dc::SolveOut{makespan + d * B, bits ? bits + d * B * W : nullptr,
+                              nseg ? nseg + d * B : nullptr, status ? status + d * B : nullptr,
+                              replay ? replay + d * B : nullptr};
+    return dc::launch_fused(g, out, rows, workspace, stream) == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+}
+
+dc_status dc_schedule_generated_batch(const dc_profile_cfg *cfg, int64_t *makespan,
+                                      uint32_t *bits, int32_t *nseg, int32_t *status,
+                                      void *workspace, size_t workspace_bytes,
+                                      cudaStream_t stream)
+{
+    const dc::NvtxRange nvtx("dc_schedule_generated_batch");
+    return generated(cfg, nullptr, makespan, bits, nseg, status, nullptr, workspace,
+                     workspace_bytes, stream);
+}
+
+dc_status dc_step_batch(const dc_profile_cfg *cfg, int64_t *fc, int64_t *pt, int64_t *bc,
+                        int64_t *gt, int64_t *dt, int64_t *makespan, uint32_t *bits, int32_t *nseg,
+                        int32_t *status, int64_t *replay, void *workspace, size_t workspace_bytes,
+                        cudaStream_t stream)
+{
+    const dc::NvtxRange nvtx("dc_step_batch");
+    const dc::StepRows rows{fc, pt, bc, gt, dt};
+    return generated(cfg, &rows, makespan, bits, nseg, status, replay, workspace, workspace_bytes,
+                     stream);
 }
 
 int32_t dc_schedule_kernel_launches(int64_t batch, int32_t L)

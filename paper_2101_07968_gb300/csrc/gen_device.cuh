@@ -123,11 +123,14 @@ __device__ __forceinline__ void divide(uint64_t a, const WordDiv &w, uint32_t &q
 dc_status check_profile_cfg(const dc_profile_cfg *c);
 void fill_gen_params(const dc_profile_cfg *c, GenParams &g);
 
-// Generate-and-solve for 1 <= L <= 16 (dp_fused.cu): outputs [2][batch], forward
-// first; workspace: fused_workspace_bytes(batch).
+// Generate-and-solve for 1 <= L <= 16 (dp_fused.cu), forward first, the profiles to
+// `rows` unless it is null; workspace: fused_workspace_bytes(batch).
 size_t fused_workspace_bytes(int64_t batch);
-cudaError_t launch_fused(const GenParams &g, int64_t *makespan, uint32_t *bits, int32_t *nseg,
-                         int32_t *status, void *workspace, cudaStream_t stream);
+struct StepRows {
+    int64_t *fc, *pt, *bc, *gt, *dt;
+};
+cudaError_t launch_fused(const GenParams &g, const SolveOut (&out)[2], const StepRows *rows,
+                         void *workspace, cudaStream_t stream);
 
 // Rate, bandwidth and latency of global instance gi, with the reciprocals of rate and
 // bandwidth: of floor_div, or of WordDiv.

@@ -72,6 +72,8 @@ _SIGNATURES = {
     "dc_schedule_generated_workspace_bytes": (_SZ, [_I64, _I32]),
     "dc_schedule_generated_batch": (_I32, [ctypes.POINTER(dc_profile_cfg), _VP, _VP, _VP, _VP,
                                            _VP, _SZ, _VP]),
+    "dc_step_batch": (_I32, [ctypes.POINTER(dc_profile_cfg), _VP, _VP, _VP, _VP, _VP, _VP, _VP,
+                             _VP, _VP, _VP, _VP, _SZ, _VP]),
     "dc_greedy_forward_batch": (_I32, [_I64, _I32, _VP, _VP, _VP, _VP, _VP, _VP]),
     "dc_greedy_backward_batch": (_I32, [_I64, _I32, _VP, _VP, _VP, _VP, _VP, _VP]),
     "dc_status_string": (ctypes.c_char_p, [_I32]),
@@ -257,6 +259,16 @@ def dc_schedule_generated_batch(cfg, makespan, bits, nseg, status, workspace, wo
         int(workspace_bytes), _stream(stream)))
 
 
+def dc_step_batch(cfg, fc, pt, bc, gt, dt, makespan, bits, nseg, status, replay, workspace,
+                  workspace_bytes, stream=None) -> int:
+    keep: list = []
+    c = cfg if isinstance(cfg, dc_profile_cfg) else make_cfg(cfg, keep)
+    return int(lib().dc_step_batch(
+        ctypes.byref(c), _ptr(fc), _ptr(pt), _ptr(bc), _ptr(gt), _ptr(dt), _ptr(makespan),
+        _ptr(bits), _ptr(nseg), _ptr(status), _ptr(replay), _ptr(workspace),
+        int(workspace_bytes), _stream(stream)))
+
+
 def dc_greedy_forward_batch(batch, L, fc, pt, dt, makespan, bits, stream=None) -> int:
     return int(lib().dc_greedy_forward_batch(int(batch), int(L), _ptr(fc), _ptr(pt), _ptr(dt),
                                              _ptr(makespan), _ptr(bits), _stream(stream)))
@@ -386,16 +398,24 @@ def greedy(direction: int, comp, xfer, dt, stream=None) -> dict:
     return out
 
 
+def fused_step(batch: int, L: int) -> bool:
+    """Whether StepGraph takes dc_step_batch: where the step is bound by memory more than
+    by the solve. 1,000,000 x 8 (AlexNet) 99 us against 115 with separate passes, 65,536
+    x 8 22 against 23; but 1,000,000 x 16 log-uniform 324 against 307, VGG-16 equal."""
+    return L <= 11 and batch >= 65536
+
+
 class StepGraph:
     """One whole step for a fixed config -- dc_profile_gen, the forward and backward
     DPs and the f_m replay of both decisions -- captured once as a CUDA graph and
     replayed. For small batches the host cost of the step's launches exceeds the
-    kernels' own time; replay() issues them as one graph launch. The two
-    directions are independent, so after the generator they run on two branches
+    kernels' own time; replay() issues them as one graph launch. Large batches of
+    short rows (fused_step) take the one pass of dc_step_batch, which writes the
+    profiles out while it solves them. Otherwise the two directions are independent, so after the generator they run on two branches
     of the graph (each with its own workspace): one direction's kernels start on
     the SMs the other's tail leaves free. Each DP pass evaluates f_m itself
-    (dc_schedule_replay_batch), so the profiles are read once per direction. After
-    each replay():
+    (dc_schedule_replay_batch), so the profiles are read once per direction. After each
+    replay():
     prof (fc, pt, bc, gt, dt), sched.out[d] and replay_out[d] for d in (FWD, BWD)
     hold that step's results."""
 
@@ -409,10 +429,26 @@ class StepGraph:
                      for k in ("fc", "pt", "bc", "gt")}
         self.prof["dt"] = torch.empty(B, dtype=torch.int64, device=device)
         self.sched = Scheduler(B, L, device=device)
-        self.sched_b = Scheduler(B, L, device=device)  # the backward branch's workspace
-        self.sched.out[BWD] = self.sched_b.out[BWD]
-        self.replay_out = {d: torch.empty(B, dtype=torch.int64, device=device)
-                           for d in (FWD, BWD)}
+        self.fused = fused_step(B, L)
+        if self.fused:  # one [2, B] buffer per output, the directions' views of it
+            W = max(words(L), 1)
+            self.both = {
+                "makespan": torch.empty((2, B), dtype=torch.int64, device=device),
+                "bits": torch.empty((2, B, W), dtype=torch.int32, device=device),
+                "nseg": torch.empty((2, B), dtype=torch.int32, device=device),
+                "status": torch.empty((2, B), dtype=torch.int32, device=device),
+                "replay": torch.empty((2, B), dtype=torch.int64, device=device)}
+            self.sched_b = self.sched
+            self.sched.out = {d: {k: v[d] for k, v in self.both.items() if k != "replay"}
+                              for d in (FWD, BWD)}
+            self.replay_out = {d: self.both["replay"][d] for d in (FWD, BWD)}
+            self.ws_bytes = dc_schedule_generated_workspace_bytes(B, L)
+            self.ws = torch.empty(self.ws_bytes, dtype=torch.uint8, device=device)
+        else:
+            self.sched_b = Scheduler(B, L, device=device)  # the backward branch's workspace
+            self.sched.out[BWD] = self.sched_b.out[BWD]
+            self.replay_out = {d: torch.empty(B, dtype=torch.int64, device=device)
+                               for d in (FWD, BWD)}
         self._branch = torch.cuda.Stream(device=device)
         # one eager step first: one-time setup (function attributes, occupancy
         # queries) happens outside the capture
@@ -438,6 +474,12 @@ class StepGraph:
     def _step(self):
         import torch
         p = self.prof
+        if self.fused:
+            o = self.both
+            _check(dc_step_batch(self.c, p["fc"], p["pt"], p["bc"], p["gt"], p["dt"],
+                                 o["makespan"], o["bits"], o["nseg"], o["status"], o["replay"],
+                                 self.ws, self.ws_bytes), "dc_step_batch")
+            return
         _check(dc_profile_gen(self.c, p["fc"], p["pt"], p["bc"], p["gt"], p["dt"]),
                "dc_profile_gen")
         main = torch.cuda.current_stream()
