@@ -36,8 +36,10 @@ UNIT = "instances/s"
 PEAKS_PATH = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_PATH = os.path.join(ROOT, "profiles", "dp_traffic.json")
 
-# Integer-ALU roof: GB300's maximum SM clock, and the instructions one
-# transition of the 32-bit passes takes (one add-then-max, half a 3-input min).
+# The rate at which GB300 could fill the listings' tables, every candidate of every
+# cell: its maximum SM clock, and the instructions one transition takes (one
+# add-then-max, half a 3-input min). The passes do not fill them (columns end early,
+# and from L = 17 on a cell is one binary search), so this is context, not their roof.
 MAX_SM_MHZ = 2070
 ALU_OPS_PER_TRANSITION = 1.5
 
@@ -129,8 +131,8 @@ def load_json(path):
 # the sources each first-pass kernel is built from, by the L it serves
 FIRST_PASS_SOURCES = {
     "small_dense_kernel": ("dp_small.cu", "dp_small.cuh", "gen_device.cuh", "common.cuh"),
-    "mid_kernel": ("dp_mid.cu", "common.cuh"),
-    "deep_kernel": ("dp_deep.cu", "common.cuh"),
+    "warp_kernel": ("dp_warp.cu", "chain.cuh", "common.cuh"),
+    "deep_kernel": ("dp_deep.cu", "chain.cuh", "common.cuh"),
 }
 
 
@@ -161,10 +163,11 @@ def traffic_record(workload: str, L: int):
 
 
 def first_pass_kernel(L: int) -> str:
-    """The kernel of a direction's first pass over the batch."""
+    """The kernel of a direction's first pass over a large batch (a small one of L <= 64
+    takes solo_kernel, a large one of L <= 19 mid_kernel)."""
     if L <= 16:
         return "small_dense_kernel"
-    return "mid_kernel" if L <= 256 else "deep_kernel"
+    return "warp_kernel" if L <= 192 else "deep_kernel"
 
 
 def binding_roof(*roofs, **extra):
@@ -639,7 +642,7 @@ def run_ours(args):
     ms = graph_ms if graph_ms is not None else eager_ms
     del sg
 
-    # ---- ALU roof: the DP's transition op mix, register-only, all SMs
+    # ---- the listings' transition op mix, register-only, all SMs
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     roof_threads, roof_blocks, roof_iters = 512, sms * 4, 20_000
     sink = torch.empty(roof_blocks * roof_threads, dtype=torch.int32, device=dev)
@@ -681,46 +684,45 @@ def run_ours(args):
     # launches; its work is the instances it solved (the listed ones are left
     # to the work-list pass)
     first_s = (fwd_k_ms + bwd_k_ms) * 1e-3
-    first_trans = transitions(L) * (2 * B - listed[0] - listed[1])
-    achieved = first_trans / first_s / 1e9
-    # ALU roof from unit counts: 4 x 16 integer-ALU lanes per SM per clock, the
-    # 32-bit passes spend 1.5 ALU instructions per transition
-    peak = sms * 64 * MAX_SM_MHZ * 1e6 / ALU_OPS_PER_TRANSITION / 1e9
+    fill_peak = sms * 64 * MAX_SM_MHZ * 1e6 / ALU_OPS_PER_TRANSITION
     traffic = traffic_record(args.workload, L)
     hbm_peak = (load_json(PEAKS_PATH) or {}).get("hbm_gbs", 6800.0)
     dp_gbs = dp_bytes(L) * (2 * B - listed[0] - listed[1]) / first_s / 1e9
-    # kernels of this library per step: the generator; per direction the first
-    # pass (split into several launches for long deep-chain batches) and the
-    # pass over its work list; the two timeline replays
-    launches_per_step = 1 + 2 * dc.dc_schedule_kernel_launches(B, L) + 2
-    # both roofs of the DP pass; the one it comes closer to (the larger minimal
-    # time at peak) binds and is reported, the other rides along
-    alu_roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gtransitions/s",
-                "frac": achieved / peak,
-                "peak_source": f"{sms} SMs x 64 integer-ALU lanes x {MAX_SM_MHZ} MHz / "
-                               f"{ALU_OPS_PER_TRANSITION} ALU instructions per transition",
-                "peak_probe": roof[0] / 1e9,
-                "peak_probe_source": "register-only loop of the 32-bit passes' op mix, "
-                                     "all SMs, measured in this run",
-                "peak_u64_probe": roof[1] / 1e9}
+    # kernels of this library per step: the generator and, per direction, the first pass
+    # (one or several launches) and the pass over its work list; as separate calls also
+    # the two timeline replays, which the graph's passes evaluate themselves. The graph of
+    # a large batch of short rows is the one pass of dc_step_batch: its table copy, the
+    # pair kernel and the two list passes.
+    kernels = 1 + 2 * dc.dc_schedule_kernel_launches(B, L)
+    if graph_ms is None:
+        launches_per_step = kernels + 2
+    else:
+        launches_per_step = 4 if dc.fused_step(B, L) else kernels
     hbm_roof = {"bound": "hbm", "achieved": dp_gbs, "peak": hbm_peak, "unit": "GB/s",
                 "frac": dp_gbs / hbm_peak,
                 "bytes_per_instance_direction": dp_bytes(L),
-                "peak_source": "MEASURED_PEAKS.json hbm_gbs (copy, burst)"}
+                "peak_source": "MEASURED_PEAKS.json hbm_gbs (copy, burst), 6,800 without it"}
     # the whole library call per direction (counter reset, first pass, work-list
-    # pass), against the same roofs
-    call_gtps = trans / dp_s / 1e9
+    # pass), against the same roof
     call_gbs = 2 * dp_bytes(L) * B / dp_s / 1e9
-    dp_call = {"ms_forward": fwd_ms, "ms_backward": bwd_ms,
-               "alu_frac": call_gtps / peak, "hbm_frac": call_gbs / hbm_peak,
+    dp_call = {"ms_forward": fwd_ms, "ms_backward": bwd_ms, "hbm_frac": call_gbs / hbm_peak,
                "note": "the whole dc_schedule_* call per direction: counter reset, "
                        "first pass and work-list pass, all instances"}
-    roofline = binding_roof(alu_roof, hbm_roof,
+    # the listings' transitions over the same time, against the rate of a pass that
+    # computes each of them
+    table = {"transitions_per_s": trans / dp_s, "fill_rate_at_peak": fill_peak,
+             "ratio": trans / dp_s / fill_peak,
+             "fill_rate_source": f"{sms} SMs x 64 integer-ALU lanes x {MAX_SM_MHZ} MHz / "
+                                 f"{ALU_OPS_PER_TRANSITION} ALU instructions per transition",
+             "probe": roof[0], "probe_u64": roof[1],
+             "note": "the passes leave most of the tables out (columns end early, cells by "
+                     "search), so a ratio above 1 is a better algorithm and no roof"}
+    roofline = binding_roof(hbm_roof,
                             kernel=("first DP pass, forward + backward "
                                     f"({first_pass_kernel(L)}), timed on its own launches"),
                             kernel_ms={"forward": fwd_k_ms, "backward": bwd_k_ms},
                             listed_to_work_list={"forward": listed[0], "backward": listed[1]},
-                            traffic=traffic, dp_call=dp_call)
+                            traffic=traffic, dp_call=dp_call, table=table)
     if traffic is None:
         roofline["traffic_note"] = ("no DRAM record in profiles/dp_traffic.json matches this "
                                     "workload and the current sources of its first-pass kernel")

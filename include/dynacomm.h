@@ -112,11 +112,10 @@ dc_status dc_profile_gen(const dc_profile_cfg *cfg, int64_t *fc, int64_t *pt, in
 /* ------------------------------------------------------------------------
  * dc_schedule_workspace_bytes -- device scratch a schedule call needs for
  * (batch, L): a work list for instances that the first pass leaves to a
- * second (values beyond its 32-bit forms, or an optimum with more segments
- * than it keeps traceback columns for); traceback slots of the
- * thread-per-instance kernel (17 <= L <= 256) or, for L > 256, the per-CTA
- * slots of the warp-per-instance kernel with their flags and per-launch
- * counters; for L > 64, per-CTA DP tables of the second pass. Pure host
+ * second (values that its kept columns cannot hold in 32 bits, or an optimum
+ * with more segments than it keeps columns for); from L = 17 on the kept columns
+ * of its resident threads, warps or CTAs, and for L > 192 their flags and the
+ * per-launch counters; for L > 64, per-CTA tables of the second pass. Pure host
  * function, no CUDA call.
  * ---------------------------------------------------------------------- */
 size_t dc_schedule_workspace_bytes(int64_t batch, int32_t L);

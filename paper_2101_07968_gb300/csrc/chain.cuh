@@ -1,7 +1,7 @@
 // One instance of the DynaComm DP (Eq. 8 / Algorithm 3 and Eq. 9 / Algorithm 4)
 // solved by a warp or a CTA in O(L log L) per segment count: the device code shared
-// by the warp-per-instance pass (dp_mid.cu), the CTA-per-instance pass (dp_deep.cu)
-// and the work-list pass (dp_group.cu).
+// by the warp-per-instance pass (dp_warp.cu), the CTA-per-instance pass (dp_deep.cu),
+// the work-list pass (dp_group.cu) and its drawing form (dp_fused.cu).
 //
 // With the layers in processing order, P the prefix of the transfer costs and C
 // that of the compute costs, put

@@ -48,8 +48,7 @@ size_t warp_scratch_bytes(int64_t batch, int L);  // dp_warp.cu
 size_t deep_slot_bytes(int L);                   // dp_deep.cu
 int64_t deep_slots_bound(int L);                 // dp_deep.cu
 
-// CTA-per-instance tables for the instances the deep-chain kernel lists (L >
-// kMidLMax): a few, within ~1 GiB.
+// Tables of the work-list pass for L > kMidLMax: a few instances, within ~1 GiB.
 inline int64_t list_table_slots(int L)
 {
     const int64_t per = tri_cells(L) * 8;
@@ -61,11 +60,11 @@ inline int64_t list_table_slots(int L)
 
 struct Workspace {
     // Layout: [0, 256) header (work-list counter, tile ticket), [256, 256 +
-    // 4*batch) work list, then, 256-aligned, the looped kernel's traceback slots
-    // (17 <= L <= kMidLMax) or, for L > kMidLMax, the deep-chain kernel's slot
-    // flags and per-launch tickets (4 bytes each) and, 256-aligned, its per-CTA
-    // slots; then, 256-aligned, the per-CTA DP tables of the group kernel for
-    // the listed instances (L > kSmemTableLMax).
+    // 4*batch) work list, then, 256-aligned, the kept columns of the looped kernel's
+    // threads or of the warp kernel's warps (17 <= L <= kMidLMax) or, for L > kMidLMax,
+    // the deep kernel's slot flags and per-launch tickets (4 bytes each) and,
+    // 256-aligned, the kept columns of its CTAs; then, 256-aligned, the per-CTA
+    // tables of the work-list pass (L > kSmemTableLMax).
     static size_t list_bytes(int64_t batch, int) { return size_t(batch) * 4; }
     static size_t table_offset(int64_t batch, int L)
     {

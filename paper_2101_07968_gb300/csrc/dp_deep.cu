@@ -27,8 +27,8 @@
 //    programmatic dependent launch: each may fill the SMs as the one before drains.
 //    A CTA claims a free slot from a bitmap for as long as it lives.
 //
-// Measured, both directions together: 16,384 instances of L = 1024 in 1.08 ms, and
-// 383 of L = 1023 in 0.16 ms (1.65 and 0.21 ms with 64-bit values only, eight rows
+// Measured, both directions together: 16,384 instances of L = 1024 in 0.92 ms, and
+// 383 of L = 1023 in 0.117 ms (1.65 and 0.21 ms with 64-bit values only, eight rows
 // per thread and two key buffers; 532 and 20.5 ms for the fill of all L columns over
 // every candidate).
 #include "chain.cuh"

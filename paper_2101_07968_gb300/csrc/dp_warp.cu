@@ -174,9 +174,11 @@ cudaError_t launch_solo(bool forward, int64_t batch, int L, const int64_t *comp,
 }
 
 // Slots of the kept columns past shared memory: one per warp of the largest grid, and
-// no more than the batch has instances (rounded up to whole CTAs of 8).
+// no more than the batch has instances (rounded up to whole CTAs of 8). The solo kernel
+// keeps its columns on chip.
 size_t warp_scratch_bytes(int64_t batch, int L)
 {
+    if (use_solo(batch, L)) return 0;
     int64_t n = kSlotWarps;
     const int64_t need = (batch + 7) / 8 * 8;
     if (need < n) n = need;

@@ -27,7 +27,7 @@ cudaError_t launch_schedule(bool forward, int64_t batch, int L, const int64_t *c
                             void *workspace, const PassEvents &pe, cudaStream_t stream)
 {
     unsigned char *ws = static_cast<unsigned char *>(workspace);
-    // events around the first pass of a looped or deep-chain solve
+    // events around the first pass (launch_small records its own)
     auto mark = [&](cudaEvent_t ev) { return ev ? cudaEventRecord(ev, stream) : cudaSuccess; };
     if (use_solo(batch, L)) {  // one pass, nothing listed
         cudaError_t e = mark(pe.start);
@@ -47,8 +47,8 @@ cudaError_t launch_schedule(bool forward, int64_t batch, int L, const int64_t *c
                             count, list, pe, stream);
     }
     if (L <= kMidLMax) {
-        // looped 32-bit pass (tile ticket + work list in the header), then the
-        // CTA-per-instance kernel over the listed 64-bit / deep instances
+        // warp-per-instance or looped pass (ticket and work list in the header), then
+        // the work-list pass over the instances it listed
         uint32_t *count = reinterpret_cast<uint32_t *>(ws);
         uint32_t *ticket = count + 1;
         uint32_t *list = reinterpret_cast<uint32_t *>(ws + 256);
@@ -71,8 +71,8 @@ cudaError_t launch_schedule(bool forward, int64_t batch, int L, const int64_t *c
                             count, list, ws + Workspace::group_tables_offset(batch, L),
                             int64_t(Workspace::slots(batch, L)), stream);
     }
-    // warp-per-instance pass over the batch (three shifted 32-bit forms), then
-    // the CTA-per-instance kernel over the instances it listed
+    // CTA-per-instance pass over the batch, its columns kept as 32-bit words, then the
+    // work-list pass over the instances it listed, every column in 64 bits
     uint32_t *count = reinterpret_cast<uint32_t *>(ws);
     uint32_t *list = reinterpret_cast<uint32_t *>(ws + 256);
     const int64_t nslots = Workspace::deep_slots(batch, L);

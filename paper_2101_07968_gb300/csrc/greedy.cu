@@ -1,6 +1,6 @@
 // The paper's competing schedulers as batched kernels (Sec. II-C): greedy
 // parameter scheduling of iBatch (Algorithm 1, forward) and greedy gradient
-// scheduling of iPart (Algorithm 2, backward), one instance per thread.
+// scheduling of iPart (Algorithm 2, backward).
 //
 // Readings where the listings leave a choice open (the same as the oracle's):
 //  * ties in "choose the one with minimum ..." keep the first candidate of the
