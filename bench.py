@@ -690,14 +690,15 @@ def run_ours(args):
     dp_gbs = dp_bytes(L) * (2 * B - listed[0] - listed[1]) / first_s / 1e9
     # kernels of this library per step: the generator and, per direction, the first pass
     # (one or several launches) and the pass over its work list; as separate calls also
-    # the two timeline replays, which the graph's passes evaluate themselves. The graph of
-    # a large batch of short rows is the one pass of dc_step_batch: its table copy, the
-    # pair kernel and the two list passes.
+    # the two timeline replays, which the graph's passes evaluate themselves. Where the
+    # graph is the one pass of dc_step_batch it launches that call's kernels.
     kernels = 1 + 2 * dc.dc_schedule_kernel_launches(B, L)
     if graph_ms is None:
         launches_per_step = kernels + 2
     else:
-        launches_per_step = 4 if dc.fused_step(B, L) else kernels
+        mode = int(cfg["layer_mode"])
+        launches_per_step = (dc.dc_step_kernel_launches(B, L, mode) if dc.fused_step(B, L, mode)
+                             else kernels)
     hbm_roof = {"bound": "hbm", "achieved": dp_gbs, "peak": hbm_peak, "unit": "GB/s",
                 "frac": dp_gbs / hbm_peak,
                 "bytes_per_instance_direction": dp_bytes(L),

@@ -173,9 +173,10 @@ dc_status dc_schedule_backward_batch(int64_t batch, int32_t L, const int64_t *bc
  * bit for bit. Outputs, forward first then backward: makespan [2][batch],
  * bits [2][batch][W], nseg [2][batch] and status [2][batch] (both nullable).
  * workspace: device, >= dc_schedule_generated_workspace_bytes(batch, L) bytes
- * (the two work lists and a copy of the generator's tables). Errors: those of dc_profile_gen (config), DC_ERR_BAD_SHAPE
- * for L > 16, DC_ERR_NULL, DC_ERR_WORKSPACE, DC_ERR_CUDA. There is no counterpart
- * in the paper, whose profiler produces the profiles (Sec. IV-A).
+ * (the two work lists and a copy of the generator's tables). Errors: those of
+ * dc_profile_gen (config), DC_ERR_BAD_SHAPE for L > 16, DC_ERR_NULL,
+ * DC_ERR_WORKSPACE, DC_ERR_CUDA. There is no counterpart in the paper, whose
+ * profiler produces the profiles (Sec. IV-A).
  * ---------------------------------------------------------------------- */
 size_t dc_schedule_generated_workspace_bytes(int64_t batch, int32_t L);
 dc_status dc_schedule_generated_batch(const dc_profile_cfg *cfg, int64_t *makespan, uint32_t *bits,
@@ -194,6 +195,15 @@ dc_status dc_step_batch(const dc_profile_cfg *cfg, int64_t *fc, int64_t *pt, int
                         int64_t *gt, int64_t *dt, int64_t *makespan, uint32_t *bits, int32_t *nseg,
                         int32_t *status, int64_t *replay, void *workspace, size_t workspace_bytes,
                         cudaStream_t stream);
+
+/* ------------------------------------------------------------------------
+ * dc_step_kernel_launches -- how many kernels one dc_step_batch or
+ * dc_schedule_generated_batch call launches: one for a small batch, otherwise a
+ * copy of the generator's tables, the pass over the batch and a list pass per
+ * direction. For counting only. Returns 0 for batch <= 0 or L outside [1, 16]. Pure
+ * host function, no CUDA call.
+ * ---------------------------------------------------------------------- */
+int32_t dc_step_kernel_launches(int64_t batch, int32_t L, int32_t layer_mode);
 
 /* ------------------------------------------------------------------------
  * dc_greedy_forward_batch, dc_greedy_backward_batch -- the paper's competing

@@ -1,6 +1,7 @@
-// Generate-and-solve for 1 <= L <= 16 (dc_schedule_generated_batch): the short-L
-// passes of dp_small.cu with each tile's rows drawn inside the kernel by the
-// profile generator's device functions instead of being read from memory.
+// Generate-and-solve for 1 <= L <= 16 (dc_schedule_generated_batch, dc_step_batch): the
+// short-L passes of dp_small.cu with each tile's rows drawn inside the kernel by the
+// profile generator's device functions instead of being read from memory; small batches
+// take one launch of the chain solver on drawn rows (fused_solo_kernel).
 #include "chain.cuh"
 #include "dp_small.cuh"
 
@@ -211,7 +212,7 @@ __global__ void __launch_bounds__(32, DC_SMALL_MINB)
 template <bool FWD>
 struct DrawLoader {
     const GenParams &g;
-    const GenTables *t;
+    const LayerRow *layer;
     const InstanceDraws &d;
     int64_t gi;
     __device__ __forceinline__ void row(int r, uint64_t &c, uint64_t &x) const
@@ -219,7 +220,7 @@ struct DrawLoader {
         c = x = 0;
         if (r > g.L) return;
         int64_t wire, flops, f, b, v;
-        layer_numerators(g, t->layer, gi, FWD ? r - 1 : g.L - r, wire, flops);
+        layer_numerators(g, layer, gi, FWD ? r - 1 : g.L - r, wire, flops);
         wire_costs(g, d, uint64_t(wire), uint64_t(flops), f, b, v);
         c = uint64_t(FWD ? f : b);
         x = uint64_t(v);
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(32)
         const int64_t gi = g.inst0 + i;
         const InstanceDraws d = instance_draws(g, t->rate, t->bw, gi);
         const int L = g.L;
-        chain_solve_warp<FWD, 1>(0, i, L, DrawLoader<FWD>{g, t, d, gi}, d.dt, o.out[dir],
+        chain_solve_warp<FWD, 1>(0, i, L, DrawLoader<FWD>{g, t->layer, d, gi}, d.dt, o.out[dir],
                                  KeptValues{table, L});
         __syncwarp();  // shared memory is read
     }
@@ -271,6 +272,89 @@ cudaError_t launch_fused_list(const GenParams &g, const GenTables *t, const Fuse
     lc.attrs = at;
     lc.numAttrs = 1;
     return cudaLaunchKernelEx(&lc, fused_list_kernel<FWD>, g, t, o);
+}
+
+// Small batches, one launch: warp 0 of a CTA draws two instances' rows, one layer to a
+// lane, and writes them out (STORE); then each of the four warps solves one instance in
+// one direction with every column on chip, as solo_kernel does. The tables are read from
+// the parameter block, where only the layers' lookups diverge. Bound by integer issue
+// (drawn by each warp for itself, two layers to a lane, the kernel took twice as long).
+constexpr int kSoloInstances = 2;
+__host__ __device__ inline int fused_solo_bytes(int L)
+{
+    return chain_pair_bytes(64) + (int(tri_cells(L)) * 8 + 15) / 16 * 16;
+}
+
+// The costs of one instance's drawn rows in processing order (see RowLoader).
+template <bool FWD>
+struct DrawnLoader {
+    const int64_t *comp, *xfer;  // shared memory, layer order
+    int L;
+    __device__ __forceinline__ void operator()(int r, uint64_t &c0, uint64_t &c1, uint64_t &x0,
+                                               uint64_t &x1) const
+    {
+        c0 = c1 = x0 = x1 = 0;
+        if (r > L) return;
+        const int at = FWD ? r - 1 : L - r, next = FWD ? at + 1 : at - 1;
+        c0 = uint64_t(comp[at]);
+        x0 = uint64_t(xfer[at]);
+        if (r < L) {
+            c1 = uint64_t(comp[next]);
+            x1 = uint64_t(xfer[next]);
+        }
+    }
+};
+
+template <bool STORE>
+__global__ void __launch_bounds__(64 * kSoloInstances)
+    fused_solo_kernel(const __grid_constant__ GenParams g, const FusedOut o)
+{
+    static_assert(kSoloInstances == 2 && kSmallLMax == 16, "a half warp draws an instance");
+    __shared__ int64_t rows[kSoloInstances][3][kSmallLMax], dts[kSoloInstances];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, L = g.L;
+    const int64_t i0 = int64_t(blockIdx.x) * kSoloInstances;
+    if (warp == 0) {
+        const int h = lane >> 4, l = lane & 15;
+        const bool there = i0 + h < g.batch;
+        const int64_t i = there ? i0 + h : i0, gi = g.inst0 + i;
+        int64_t rate, bw;
+        InstanceDraws d;
+        base_draws(g, g.rate_knots, g.bw_knots, gi, rate, bw, d.dt);
+        d.rate = uint64_t(rate);
+        d.bw = uint64_t(bw);
+        const uint64_t inv = ~uint64_t(0) / ((lane & 1) ? d.bw : d.rate);  // one division, not two
+        d.mrate = __shfl_sync(0xffffffffu, inv, 16 * h);
+        d.mbw = __shfl_sync(0xffffffffu, inv, 16 * h + 1);
+        if (there && l < L) {
+            int64_t wire, flops, f, b, x;
+            layer_numerators(g, g.layer, gi, l, wire, flops);
+            wire_costs(g, d, uint64_t(wire), uint64_t(flops), f, b, x);
+            rows[h][0][l] = f;
+            rows[h][1][l] = b;
+            rows[h][2][l] = x;
+            if (l == 0) dts[h] = d.dt;
+            if constexpr (STORE) {
+                const int64_t at = i * L + l;
+                o.fc[at] = f;
+                o.bc[at] = b;
+                o.pt[at] = x;
+                o.gt[at] = x;
+                if (l == 0) o.dt[i] = d.dt;
+            }
+        }
+        if (i0 == 0 && lane < 2) *(lane == 0 ? o.wide_count[0] : o.wide_count[1]) = 0u;  // nothing listed
+    }
+    const int kb = warp * fused_solo_bytes(L), h = warp >> 1;
+    const KeptValues kept{&sh<int64_t>(kb + chain_pair_bytes(64)), L};
+    if (lane == 0) zero_row(kb, 64);
+    __syncthreads();
+    if (i0 + h >= g.batch) return;
+    if ((warp & 1) == 0)
+        chain_solve_warp<true, 1>(kb, i0 + h, L, DrawnLoader<true>{rows[h][0], rows[h][2], L}, dts[h],
+                                  o.out[0], kept);
+    else
+        chain_solve_warp<false, 1>(kb, i0 + h, L, DrawnLoader<false>{rows[h][1], rows[h][2], L}, dts[h],
+                                   o.out[1], kept);
 }
 
 template <int L, bool STORE>
@@ -303,6 +387,18 @@ cudaError_t launch_fused_L(const GenParams &g, const GenTables *t, const FusedOu
 
 size_t fused_workspace_bytes(int64_t batch) { return fused_tables_offset(batch) + sizeof(GenTables); }
 
+// Whether one launch of fused_solo_kernel takes the batch. The pair kernel's path is five
+// launches, and a thread per instance is slow to finish; but the solo kernel takes 1.5 us
+// per 1,000 instances, 3.5 to 5 where the layers' knots are looked up. Whole steps from a
+// graph, solo against pair: one instance 6.2 us against 12-22; 4,096 x 8 (tiny) 10.3
+// against 16.4, 4,096 x 16 (VGG-16) 12.3 against 20.8; 8,000 x 8 15.3 against 16.5, 8,000 x
+// 16 18.5 against 28.8; 12,000 x 8 20.6 against 16.5. Log-uniform layers: 6,000 x 8 22.6
+// against 24.5, x 16 34 against 45; 8,000 x 8 27.4 against 24.6.
+bool use_fused_solo(int64_t batch, int layer_mode)
+{
+    return batch <= (layer_mode == DC_LAYERS_LOGUNIFORM ? 6000 : 8000);
+}
+
 // Generate-and-solve for 1 <= L <= 16; rows: where the profiles go, or null.
 cudaError_t launch_fused(const GenParams &g, const SolveOut (&out)[2], const StepRows *rows,
                          void *workspace, cudaStream_t stream)
@@ -324,6 +420,15 @@ cudaError_t launch_fused(const GenParams &g, const SolveOut (&out)[2], const Ste
         o.dt = rows->dt;
         o.pairs = ((reinterpret_cast<uintptr_t>(o.fc) | reinterpret_cast<uintptr_t>(o.pt) |
                     reinterpret_cast<uintptr_t>(o.bc) | reinterpret_cast<uintptr_t>(o.gt)) & 15u) == 0;
+    }
+    if (use_fused_solo(B, g.layer_mode)) {
+        const unsigned grid = unsigned((B + kSoloInstances - 1) / kSoloInstances);
+        const size_t smem = size_t(2 * kSoloInstances) * fused_solo_bytes(g.L);  // 8.5 KB at L = 16
+        if (rows)
+            fused_solo_kernel<true><<<grid, 64 * kSoloInstances, smem, stream>>>(g, o);
+        else
+            fused_solo_kernel<false><<<grid, 64 * kSoloInstances, smem, stream>>>(g, o);
+        return cudaGetLastError();
     }
     cudaError_t e = cudaMemsetAsync(ws, 0, 3 * sizeof(uint32_t), stream);
     if (e != cudaSuccess) return e;

@@ -179,6 +179,12 @@ dc_status dc_step_batch(const dc_profile_cfg *cfg, int64_t *fc, int64_t *pt, int
                      stream);
 }
 
+int32_t dc_step_kernel_launches(int64_t batch, int32_t L, int32_t layer_mode)
+{
+    if (batch <= 0 || L < 1 || L > dc::kSmallLMax) return 0;
+    return dc::use_fused_solo(batch, layer_mode) ? 1 : 4;
+}
+
 int32_t dc_schedule_kernel_launches(int64_t batch, int32_t L)
 {
     if (batch <= 0 || L < 1 || L > DC_L_MAX) return 0;

@@ -126,6 +126,7 @@ void fill_gen_params(const dc_profile_cfg *c, GenParams &g);
 // Generate-and-solve for 1 <= L <= 16 (dp_fused.cu), forward first, the profiles to
 // `rows` unless it is null; workspace: fused_workspace_bytes(batch).
 size_t fused_workspace_bytes(int64_t batch);
+bool use_fused_solo(int64_t batch, int layer_mode);  // one launch takes the batch
 struct StepRows {
     int64_t *fc, *pt, *bc, *gt, *dt;
 };

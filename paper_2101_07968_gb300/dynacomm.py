@@ -60,6 +60,7 @@ _SIGNATURES = {
     "dc_profile_gen": (_I32, [ctypes.POINTER(dc_profile_cfg), _VP, _VP, _VP, _VP, _VP, _VP]),
     "dc_schedule_workspace_bytes": (_SZ, [_I64, _I32]),
     "dc_schedule_kernel_launches": (_I32, [_I64, _I32]),
+    "dc_step_kernel_launches": (_I32, [_I64, _I32, _I32]),
     "dc_schedule_forward_batch": (_I32, [_I64, _I32, _VP, _VP, _VP, _VP, _VP, _VP, _VP, _VP,
                                          _SZ, _VP]),
     "dc_schedule_backward_batch": (_I32, [_I64, _I32, _VP, _VP, _VP, _VP, _VP, _VP, _VP, _VP,
@@ -169,6 +170,10 @@ def dc_status_string(status: int) -> str:
 
 def dc_schedule_kernel_launches(batch: int, L: int) -> int:
     return int(lib().dc_schedule_kernel_launches(int(batch), int(L)))
+
+
+def dc_step_kernel_launches(batch: int, L: int, layer_mode: int) -> int:
+    return int(lib().dc_step_kernel_launches(int(batch), int(L), int(layer_mode)))
 
 
 def dc_schedule_workspace_bytes(batch: int, L: int) -> int:
@@ -398,10 +403,15 @@ def greedy(direction: int, comp, xfer, dt, stream=None) -> dict:
     return out
 
 
-def fused_step(batch: int, L: int) -> bool:
-    """Whether StepGraph takes dc_step_batch: where the step is bound by memory more than
-    by the solve. 1,000,000 x 8 (AlexNet) 99 us against 115 with separate passes, 65,536
-    x 8 22 against 23; but 1,000,000 x 16 log-uniform 324 against 307, VGG-16 equal."""
+def fused_step(batch: int, L: int, layer_mode: int = 0) -> bool:
+    """Whether StepGraph takes dc_step_batch. Small batches, in one launch: 4,096 x 8
+    (tiny) 10.3 us against 12.4 with separate passes, 8,000 x 16 18.5 against 20.6; with
+    log-uniform layers (layer_mode 2) 2,000 x 8 12.4 against 14.4, but 4,096 x 8 18.5
+    against 17.1. Large batches where the step is bound by memory more than by the solve:
+    1,000,000 x 8 (AlexNet) 99 us against 115, 65,536 x 8 22 against 23; but 1,000,000 x 16
+    log-uniform 324 against 307, VGG-16 equal."""
+    if dc_step_kernel_launches(batch, L, layer_mode) == 1:
+        return layer_mode != 2 or batch <= 2000
     return L <= 11 and batch >= 65536
 
 
@@ -409,11 +419,11 @@ class StepGraph:
     """One whole step for a fixed config -- dc_profile_gen, the forward and backward
     DPs and the f_m replay of both decisions -- captured once as a CUDA graph and
     replayed. For small batches the host cost of the step's launches exceeds the
-    kernels' own time; replay() issues them as one graph launch. Large batches of
-    short rows (fused_step) take the one pass of dc_step_batch, which writes the
-    profiles out while it solves them. Otherwise the two directions are independent, so after the generator they run on two branches
-    of the graph (each with its own workspace): one direction's kernels start on
-    the SMs the other's tail leaves free. Each DP pass evaluates f_m itself
+    kernels' own time; replay() issues them as one graph launch. Small batches and large
+    ones of short rows (fused_step) take the one pass of dc_step_batch, which writes the
+    profiles out while it solves them. Otherwise, after the generator, the two independent
+    directions run on two branches of the graph (each with its own workspace): one
+    direction's kernels start on the SMs the other's tail leaves free. Each DP pass evaluates f_m itself
     (dc_schedule_replay_batch), so the profiles are read once per direction. After each
     replay():
     prof (fc, pt, bc, gt, dt), sched.out[d] and replay_out[d] for d in (FWD, BWD)
@@ -429,7 +439,7 @@ class StepGraph:
                      for k in ("fc", "pt", "bc", "gt")}
         self.prof["dt"] = torch.empty(B, dtype=torch.int64, device=device)
         self.sched = Scheduler(B, L, device=device)
-        self.fused = fused_step(B, L)
+        self.fused = fused_step(B, L, int(cfg["layer_mode"]))
         if self.fused:  # one [2, B] buffer per output, the directions' views of it
             W = max(words(L), 1)
             self.both = {

@@ -24,7 +24,10 @@ def dc():
     ("vgg16", 16, 70_003, {}), ("alexnet", 8, 65_537, {}), ("deepchain", 11, 65_600, {}), ("tiny", 8, 33, {}),
     ("deepchain", 1, 100, {}), ("deepchain", 2, 70, {}), ("deepchain", 5, 999, {}),
     ("deepchain", 11, 3001, {}), ("deepchain", 12, 3001, {}), ("deepchain", 15, 40_001, {}),
-    ("vgg16", 16, 5000, dict(bw_lo=1, bw_hi=50, dt_hi=2**33)), ("alexnet", 8, 1, {})])
+    ("vgg16", 16, 5000, dict(bw_lo=1, bw_hi=50, dt_hi=2**33)), ("alexnet", 8, 1, {}),
+    ("tiny", 8, 7999, {}), ("tiny", 8, 8001, {}), ("tiny", 16, 8000, {}), ("deepchain", 16, 6000, {}),
+    ("deepchain", 16, 6001, {}), ("deepchain", 7, 2, {}), ("tiny", 3, 4097, dict(bw_hi=2000, dt_hi=2**40)),
+    ("vgg16", 16, 9001, dict(bw_lo=1, bw_hi=50, dt_hi=2**33))])
 def test_one_pass_step(dc, name, L, batch, kw, offset):
     import torch
     cfg = wl.with_batch(wl.config(name), batch, inst0=7)
@@ -56,7 +59,7 @@ def test_one_pass_step(dc, name, L, batch, kw, offset):
             assert torch.equal(o[k][d], exp[k]), (k, d)
         rep = dc.eval_timeline(d, ref[c], ref[x], ref["dt"], exp["bits"])
         assert torch.equal(o["replay"][d], rep), d
-    if dc.fused_step(batch, L) and not offset:
+    if dc.fused_step(batch, L, cfg["layer_mode"]) and not offset:
         g = dc.StepGraph(cfg)
         for _ in range(2):
             g.replay()
