@@ -39,12 +39,12 @@
 //  * persistent single-warp CTAs walk 32-instance tiles. A tile's rows arrive by
 //    cp.async (coalesced 16-byte copies of cost pairs for even L) at a row
 //    stride at which every lane reads its own row without bank conflicts
-//    (stage_stride); the prefix sums then leave them in registers. Short rows
-//    (L < kSplitMinL) stage in the warp's table area, which keeps a warp small
-//    (many resident warps) while the next tile is prefetched into L2; longer
-//    rows stage beside the table, so that the next tile's copies are in flight
-//    while this one is solved, and take their tiles from a ticket (see the
-//    kernel).
+//    (stage_stride); the prefix sums then leave them in registers. Rows of 7
+//    to 11 layers stage in the warp's table area, which keeps a warp small
+//    (many resident warps) while the next tile is prefetched into L2; the others
+//    stage beside the table, so that the next tile's copies are in flight while
+//    this one is solved (staged_beside), and take their tiles from a ticket from
+//    kSplitMinL on (see the kernel).
 #include "dp_small.cuh"
 
 namespace dc {
@@ -55,15 +55,15 @@ namespace {
 __host__ __device__ constexpr int dense_min_ctas(int L) { return L >= kSplitMinL ? 12 : DC_SMALL_MINB; }
 
 // 32-bit pass over the whole batch; persistent single-warp CTAs.
-//  * shared design (L < kSplitMinL): a tile's rows are staged in the warp's table
+//  * shared design (7 <= L < kSplitMinL): a tile's rows are staged in the warp's table
 //    area, so a warp holds only max(rows, table) of shared memory and many warps
 //    fit an SM; while a tile is solved its successor is prefetched into L2. Tiles
 //    are dealt statically (warp w takes w, w + grid, ...): short tiles, for which
 //    one atomic per tile on a shared ticket would cost more than the balance gains.
-//  * split design (L >= kSplitMinL): the staging lies beside the table, and the
+//  * split design (staged_beside): the staging lies beside the table, and the
 //    copies of the warp's next tile (rows and dt) are issued as soon as this
-//    tile's rows are read, so they land while it is solved. Tiles come from an
-//    atomic ticket, claimed one tile ahead: warps on a crowded sub-partition
+//    tile's rows are read, so they land while it is solved. From kSplitMinL on tiles
+//    come from an atomic ticket, claimed one tile ahead: warps on a crowded sub-partition
 //    progress more slowly than others, and a static deal would leave the SMs
 //    emptying out behind the slowest warps.
 template <int L, bool FWD, bool REPLAY>
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
 {
     using K = Tab32<L>;
     constexpr int W = (L - 1 + 31) / 32;
-    constexpr bool kSplit = L >= kSplitMinL;
+    constexpr bool kSplit = staged_beside(L), kTicket = L >= kSplitMinL;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x;
     int32_t *lw = reinterpret_cast<int32_t *>(smem) + lane;
@@ -113,10 +113,10 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
             if (lane < r) cp_async8(stD + lane, dt + b + lane);
             stage_tile<L>(stC, stX, comp, xfer, b, r, lane, pairs);  // commits the group
         };
-        int64_t tile = int64_t(__shfl_sync(0xffffffffu, claim(), 0));
+        int64_t tile = kTicket ? int64_t(__shfl_sync(0xffffffffu, claim(), 0)) : int64_t(blockIdx.x);
         if (tile >= tiles) return;
         stage(tile);
-        uint32_t next_raw = claim();  // claimed a tile ahead: its copies go out mid-tile
+        uint32_t next_raw = kTicket ? claim() : 0u;  // claimed a tile ahead: its copies go out mid-tile
         while (tile < tiles) {
             const int64_t i = tile * 32 + lane;
             const bool active = lane < rows_of(tile);
@@ -130,10 +130,11 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
             row_uv<L, FWD>(stC + lane * K::kStride, stX + lane * K::kStride, dti, U, V, xraw,
                            wide, st);
             __syncwarp();  // the staging is read: the next tile's copies may land there
-            const int64_t next = int64_t(__shfl_sync(0xffffffffu, next_raw, 0));
+            const int64_t next =
+                kTicket ? int64_t(__shfl_sync(0xffffffffu, next_raw, 0)) : tile + gridDim.x;
             if (next < tiles) {
                 stage(next);
-                next_raw = claim();
+                if (kTicket) next_raw = claim();
             }
             tile = next;
             finish(i, active, U, V, dti, xraw, wide, st);
@@ -192,7 +193,7 @@ cudaError_t launch_dir(int64_t batch, const int64_t *comp, const int64_t *xfer,
                        const int64_t *dt, const SolveOut &o, uint32_t *wide_count,
                        uint32_t *wide_list, const PassEvents &pe, cudaStream_t stream)
 {
-    constexpr int kSmem = L >= kSplitMinL ? Tab32<L>::kSplitBytes : Tab32<L>::kSharedBytes;
+    constexpr int kSmem = staged_beside(L) ? Tab32<L>::kSplitBytes : Tab32<L>::kSharedBytes;
     static DeviceCache resident;  // single-warp CTAs of the dense kernel per SM
     int per_sm = 0;
     cudaError_t le = resident.get(per_sm, [](int &n) {

@@ -19,10 +19,15 @@ namespace {
 #define DC_SMALL_MINB 16  // resident single-warp CTAs per SM the registers must allow
 #endif
 // From this L on the dense and fused passes take their tiles from an atomic
-// ticket (and the dense pass stages each tile beside its table); shorter rows
-// take every grid-th tile, for which one atomic per tile costs more than the
-// balance gains.
+// ticket; shorter rows take every grid-th tile, for which one atomic per tile costs
+// more than the balance gains.
 constexpr int kSplitMinL = 12;
+// Whether the dense pass stages a tile beside its table, where the next one lands while
+// this one is solved, or in the table's place: from kSplitMinL on, where a long solve
+// hides the copies, and up to L = 6, where both are small enough for as many warps as the
+// registers allow (1,000,000 instances per direction: L = 4 21.2 us against 23.5, 6 28.1
+// against 30.8; but 7 39.7 against 36.0 and 8 37.7 against 33.9, with fewer warps).
+__host__ __device__ constexpr bool staged_beside(int L) { return L <= 6 || L >= kSplitMinL; }
 constexpr int kKeepCols = DC_KEEP_COLS;  // the 32-bit pass stores columns 2..kKeepCols
 
 // index of stored cell (m, n), 2 <= n <= L-1, n <= m <= L

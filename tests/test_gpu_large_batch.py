@@ -55,3 +55,19 @@ def test_hard_instances_repeated(dc, L):
             assert (got == exp[k][None]).all(), (L, d, k)
         got = out["bits"].cpu().numpy().view(np.uint32)[:, :W].reshape(copies, len(dt), W)
         assert (got == exp["bits"].reshape(1, len(dt), W)).all(), (L, d)
+
+
+@pytest.mark.parametrize("L", [1, 2, 3, 4, 5, 6, 7])
+def test_short_rows_many_tiles(dc, L):
+    """Several tiles to a warp, a ragged last one, odd rows copied by 8 bytes."""
+    cfg = wl.lsweep_config(L, 400_017)
+    prof = dc.profile_gen(cfg)
+    W = dc.words(L)
+    for d, (c, x) in ((0, ("fc", "pt")), (1, ("bc", "gt"))):
+        out = dc.schedule(d, prof[c], prof[x], prof["dt"])
+        exp = oracle.schedule_batch(d, *(prof[k].cpu().numpy() for k in (c, x, "dt")),
+                                    nthreads=os.cpu_count() or 1)
+        for k in ("status", "makespan", "nseg"):
+            assert (out[k].cpu().numpy() == exp[k]).all(), (L, d, k)
+        got = out["bits"].cpu().numpy().view(np.uint32)[:, :W]
+        assert (got == exp["bits"].reshape(len(got), W)).all(), (L, d)
