@@ -131,6 +131,7 @@ def load_json(path):
 # the sources each first-pass kernel is built from, by the L it serves
 FIRST_PASS_SOURCES = {
     "small_dense_kernel": ("dp_small.cu", "dp_small.cuh", "gen_device.cuh", "common.cuh"),
+    "solo_kernel": ("dp_warp.cu", "chain.cuh", "common.cuh"),
     "warp_kernel": ("dp_warp.cu", "chain.cuh", "common.cuh"),
     "deep_kernel": ("dp_deep.cu", "chain.cuh", "common.cuh"),
 }
@@ -162,9 +163,11 @@ def traffic_record(workload: str, L: int):
     return None
 
 
-def first_pass_kernel(L: int) -> str:
-    """The kernel of a direction's first pass over a large batch (a small one of L <= 64
-    takes solo_kernel, a large one of L <= 19 mid_kernel)."""
+def first_pass_kernel(L: int, launches: int = 2) -> str:
+    """The kernel of a direction's first pass; launches: the call's kernels, one where
+    solo_kernel solves a small batch (a large one of 17 <= L <= 19 takes mid_kernel)."""
+    if launches == 1:
+        return "solo_kernel"
     if L <= 16:
         return "small_dense_kernel"
     return "warp_kernel" if L <= 192 else "deep_kernel"
@@ -720,7 +723,8 @@ def run_ours(args):
                      "search), so a ratio above 1 is a better algorithm and no roof"}
     roofline = binding_roof(hbm_roof,
                             kernel=("first DP pass, forward + backward "
-                                    f"({first_pass_kernel(L)}), timed on its own launches"),
+                                    f"({first_pass_kernel(L, dc.dc_schedule_kernel_launches(B, L))}), "
+                                    "timed on its own launches"),
                             kernel_ms={"forward": fwd_k_ms, "backward": bwd_k_ms},
                             listed_to_work_list={"forward": listed[0], "backward": listed[1]},
                             traffic=traffic, dp_call=dp_call, table=table)
