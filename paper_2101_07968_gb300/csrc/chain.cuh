@@ -198,9 +198,10 @@ __device__ __forceinline__ int warp_first(int lo, int len, Pred pred)
 // past L hold the totals). WARP: one warp solves it (NT = 32), else the CTA. kb: byte
 // of K; D: bytes from K to b, both arrays with room for 2 NJ NT rows. word: shared
 // memory, W decision words, pub: two values that the CTA's last row publishes (both
-// CTA only). Returns false, having written nothing, when the optimum needs columns
+// CTA only). WINDOW: keys that a search looks at first, from where it ended in the column
+// before (0: none). Returns false, having written nothing, when the optimum needs columns
 // that `kept` does not hold.
-template <bool FWD, typename T, int NJ, bool WARP, typename Kept>
+template <bool FWD, typename T, int NJ, bool WARP, int WINDOW, typename Kept>
 __device__ __forceinline__ bool chain_columns(int kb, int D, uint32_t *word, T *pub, int tid, int NT,
                                               int64_t i, int L, T dt, const T (&a)[NJ][2],
                                               const T (&b)[NJ][2], T aL, T bL, const Kept &kept,
@@ -210,6 +211,7 @@ __device__ __forceinline__ bool chain_columns(int kb, int D, uint32_t *word, T *
     using Two = typename P2::type;
     constexpr unsigned kAll = 0xffffffffu;
     constexpr int S = int(sizeof(T));
+    static_assert(!WARP || WINDOW == 0, "a warp searches the whole range");
     constexpr bool kDrop = S == 8 && !Kept::kWhole;  // kept words are H[m][1] - H[m][n]
     const int lane = tid & 31, W = words_for(L);
     const T e = FWD ? T(0) : dt, h1 = FWD ? dt : T(0);  // H[m][1] = h1 + a[m]
@@ -236,6 +238,11 @@ __device__ __forceinline__ bool chain_columns(int kb, int D, uint32_t *word, T *
     const int P = 1 << (31 - __clz(N | 1));
     const T tail = N > 0 ? aL - sh<T>(kb + D + (N - 1) * S) : aL;  // a[L] - b[L-1]
     T c = FWD ? dt : T(0);
+    // Where a row's search ended never moves back from one column to the next: its keys
+    // fall or stay, and c does not fall. So from the third column on it starts there, and
+    // the whole range is searched only when some lane has moved past the window.
+    const int lim = kb + (2 * NJ * NT - WINDOW) * S;  // keys from row L on are the largest value
+    int q[NJ][2];
     for (int n = 2; n <= L; ++n) {
         if (FWD) c += dt;
         if (c + tail >= hL) break;
@@ -245,10 +252,30 @@ __device__ __forceinline__ bool chain_columns(int kb, int D, uint32_t *word, T *
             const int r = 2 * (j * NT + tid) + 1;
             const T t0 = c + a[j][0], t1 = c + a[j][1];
             int q0 = kb, q1 = kb;
+            bool search = true;
+            if constexpr (WINDOW > 0) {
+                if (n > 2) {
+                    q0 = q[j][0];
+                    q1 = q[j][1];
+                    // backward, two in five warps have not moved at all
+                    if (!FWD) search = __any_sync(kAll, sh<T>(q0) < t0 || sh<T>(q1) < t1);
+                    if (search) {
+                        q0 = min(q0, lim);
+                        q1 = min(q1, lim);
+                        search = __any_sync(kAll, sh<T>(q0 + (WINDOW - 1) * S) < t0 ||
+                                                      sh<T>(q1 + (WINDOW - 1) * S) < t1);
+                        if (!search) halve_from<T, WINDOW / 2>(t0, t1, q0, q1);
+                    }
+                }
+            }
             if constexpr (WARP)
                 halve_from<T, NJ == 1 ? 32 : NJ == 2 ? 64 : 128>(t0, t1, q0, q1);
-            else
+            else if (search)
                 search_below<T>(kb, N, P, t0, t1, q0, q1);
+            if constexpr (WINDOW > 0) {
+                q[j][0] = q0;
+                q[j][1] = q1;
+            }
             // k = p + 1, at q, is the first with H + e + b >= t, k = p the last below it
             // (p = 0 gives t, which lowers nothing)
             v[j][0] = min(min(h[j][0], sh<T>(q0) - sh<T>(q0 + D)), t0 - sh<T>(q0 + D - S));
@@ -526,7 +553,7 @@ __device__ __forceinline__ bool chain_solve_warp(int kb, int64_t i, int L, const
             if (sizeof(T) == 8 && !Kept::kWhole &&
                 !words_hold(uint64_t(aL), uint64_t(bL), uint64_t(FWD ? dt : 0)))
                 return false;
-            return chain_columns<FWD, T, NJ, true>(kb, D, static_cast<uint32_t *>(nullptr),
+            return chain_columns<FWD, T, NJ, true, 0>(kb, D, static_cast<uint32_t *>(nullptr),
                                                    static_cast<T *>(nullptr), lane, 32, i, L, T(dt),
                                                    a, b, aL, bL, kept, o);
         },
@@ -614,7 +641,8 @@ __device__ __forceinline__ int cta_prefix(uint64_t *tot, uint32_t *orw, int L, c
 // Solves instance i with the whole CTA, NJ row pairs per thread, keeping columns in
 // `kept`. Returns false, having written nothing, when the instance is left to the work
 // list: its values do not fit there, or its optimum needs a column it does not hold.
-template <bool FWD, int NJ, typename Load, typename Kept>
+// WINDOW: see chain_columns.
+template <bool FWD, int NJ, int WINDOW = 0, typename Load, typename Kept>
 __device__ bool chain_solve(int64_t i, int L, const Load &load, int64_t dt, const SolveOut &o,
                             const Kept &kept)
 {
@@ -642,7 +670,7 @@ __device__ bool chain_solve(int64_t i, int L, const Load &load, int64_t dt, cons
                 a32[j][u] = int32_t(a[j][u]);
                 b32[j][u] = int32_t(b[j][u]);
             }
-        return chain_columns<FWD, int32_t, NJ, false>(0, D, word, reinterpret_cast<int32_t *>(pub), tid,
+        return chain_columns<FWD, int32_t, NJ, false, WINDOW>(0, D, word, reinterpret_cast<int32_t *>(pub), tid,
                                                       NT, i, L, int32_t(dt), a32, b32, int32_t(aL),
                                                       int32_t(bL), kept, o);
     }
@@ -655,7 +683,7 @@ __device__ bool chain_solve(int64_t i, int L, const Load &load, int64_t dt, cons
             b64[j][u] = int64_t(b[j][u]);
         }
     if (!Kept::kWhole && !words_hold(aL, bL, uint64_t(FWD ? dt : 0))) return false;
-    return chain_columns<FWD, int64_t, NJ, false>(0, D, word, reinterpret_cast<int64_t *>(pub), tid, NT,
+    return chain_columns<FWD, int64_t, NJ, false, WINDOW>(0, D, word, reinterpret_cast<int64_t *>(pub), tid, NT,
                                                   i, L, dt, a64, b64, int64_t(aL), int64_t(bL), kept, o);
 }
 

@@ -8,7 +8,7 @@
 //    (deep_threads): a column is one independent binary search per row in shared
 //    memory, so every thread works in every column; a thread's searches run two at
 //    a time to overlap their shared-memory latency, and the other CTAs of the SM
-//    hide the rest;
+//    hide the rest; from 640 layers on it starts where the last column's ended;
 //  * what bounds it: integer issue in the searches (L log2 L steps of 3 to 4
 //    instructions a column) and the two CTA barriers of a column; the profiles are
 //    read once (16 L bytes per instance and direction) and the columns kept for the
@@ -27,8 +27,8 @@
 //    programmatic dependent launch: each may fill the SMs as the one before drains.
 //    A CTA claims a free slot from a bitmap for as long as it lives.
 //
-// Measured, both directions together: 16,384 instances of L = 1024 in 0.92 ms, and
-// 383 of L = 1023 in 0.117 ms (1.65 and 0.21 ms with 64-bit values only, eight rows
+// Measured, both directions together: 16,384 instances of L = 1024 in 0.88 ms, and
+// 383 of L = 1023 in 0.102 ms (1.65 and 0.21 ms with 64-bit values only, eight rows
 // per thread and two key buffers; 532 and 20.5 ms for the fill of all L columns over
 // every candidate).
 #include "chain.cuh"
@@ -39,6 +39,11 @@ int sm_count();  // SMs of the current device (dp_small.cu)
 
 namespace {
 
+// From this depth on a search first looks at the 32 keys from where it ended in the column
+// before: 83 to 90 in 100 end there on the deep chain, in 6 steps instead of 10. Both
+// directions: 5,000 x 2,047 824 us -> 754, 16,384 x 1,024 924 -> 880, 10,000 x 700 428 ->
+// 417; but 24,000 x 512 564 -> 573, whose searches are 9 steps, and nothing at 300.
+constexpr int kWindowMinL = 640;
 constexpr int kSplitLMin = 256;  // longer batches are split into launches above this depth
 constexpr int kSmemPerSm = 227 * 1024;
 constexpr int kKeep = 64;  // columns 1..kKeep kept for the traceback
@@ -85,7 +90,7 @@ __device__ int claim_slot(uint32_t *busy, int nslots)
     return -1;
 }
 
-template <bool FWD, int NJ>
+template <bool FWD, int NJ, int WINDOW>
 __global__ void __launch_bounds__(kChainThreads, 1) deep_kernel(DeepArgs a)
 {
     __shared__ int s_slot;
@@ -110,7 +115,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) deep_kernel(DeepArgs a)
         const uint32_t taken = s_taken;
         if (int64_t(taken) >= a.count) break;
         const int64_t i = a.lo + int64_t(taken);
-        const bool solved = chain_solve<FWD, NJ>(
+        const bool solved = chain_solve<FWD, NJ, WINDOW>(
             i, L, RowLoader<FWD>{a.comp + i * L, a.xfer + i * L, L, a.vec != 0}, __ldg(a.dt + i),
             a.out, kept);
         if (!solved && tid == 0) {
@@ -157,14 +162,14 @@ int deep_threads(int64_t count, int L, int sms)
     return L <= 384 || count * (nt1 / 32) <= int64_t(sms) * 256 ? nt1 : nt2;
 }
 
-template <bool FWD, int NJ>
+template <bool FWD, int NJ, int WINDOW>
 cudaError_t launch_deep_nj(DeepArgs a, int nt, bool pdl, cudaStream_t stream)
 {
     static DeviceCache attr;
     int done = 0;
     cudaError_t e = attr.get(done, [](int &v) {
         v = 1;
-        return cudaFuncSetAttribute(deep_kernel<FWD, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        return cudaFuncSetAttribute(deep_kernel<FWD, NJ, WINDOW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     kSmemPerSm - 1024);
     });
     if (e != cudaSuccess) return e;
@@ -179,7 +184,7 @@ cudaError_t launch_deep_nj(DeepArgs a, int nt, bool pdl, cudaStream_t stream)
     if (a.shared > kKeep) a.shared = kKeep;
     const size_t smem = fixed + a.shared * col;
     int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, deep_kernel<FWD, NJ>, nt, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, deep_kernel<FWD, NJ, WINDOW>, nt, smem);
     if (e != cudaSuccess) return e;
     int64_t grid = int64_t(nb < 1 ? 1 : nb) * sm_count();
     if (grid > a.nslots) grid = a.nslots;
@@ -194,7 +199,7 @@ cudaError_t launch_deep_nj(DeepArgs a, int nt, bool pdl, cudaStream_t stream)
     at[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = at;
     lc.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&lc, deep_kernel<FWD, NJ>, a);
+    return cudaLaunchKernelEx(&lc, deep_kernel<FWD, NJ, WINDOW>, a);
 }
 
 template <bool FWD>
@@ -203,8 +208,11 @@ cudaError_t launch_deep_dir(const DeepArgs &a, bool pdl, cudaStream_t stream)
     int nt = deep_threads(a.count, a.L, sm_count());
     // the test hook's warps, where four rows per thread cover the instance
     if (const int f = forced_warps(); f && a.L <= 128 * f) nt = 32 * f;
-    return a.L <= 2 * nt ? launch_deep_nj<FWD, 1>(a, nt, pdl, stream)
-                         : launch_deep_nj<FWD, 2>(a, nt, pdl, stream);
+    if (a.L < kWindowMinL)
+        return a.L <= 2 * nt ? launch_deep_nj<FWD, 1, 0>(a, nt, pdl, stream)
+                             : launch_deep_nj<FWD, 2, 0>(a, nt, pdl, stream);
+    return a.L <= 2 * nt ? launch_deep_nj<FWD, 1, 32>(a, nt, pdl, stream)
+                         : launch_deep_nj<FWD, 2, 32>(a, nt, pdl, stream);
 }
 
 // Instances per launch: four resident waves above L = 256, the whole batch below.

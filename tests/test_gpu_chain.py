@@ -80,3 +80,25 @@ def test_ties_everywhere(dc, L, zero):
         if zero in (name, "all"):
             a[:] = 0
     _same(dc, comp, xfer, dt, (L, zero))
+
+
+@pytest.mark.parametrize("L", [639, 640, 641, 1023, 1024, 1025])
+def test_searches_from_the_last_columns_end(dc, L):
+    """From 640 layers on a search starts where the last column's ended: crossings that
+    stay, that move a little, and that jump (one layer as long as hundreds), near both
+    ends of the keys, with many columns and values beyond 32 bits among them."""
+    parts = [wl.skewed_instances(L, 10, L), wl.tie_heavy_instances(L + 1, 6, L)]
+    rng = np.random.default_rng(L)
+    comp = rng.integers(1, 2000, (16, L))
+    xfer = rng.integers(1, 2000, (16, L))
+    for i in range(16):
+        comp[i, rng.integers(0, L, 4)] *= 10 ** (i % 4)
+        xfer[i, rng.integers(0, L, 4)] *= 10 ** (i // 4)
+    comp[:4, : L // 2] = 0
+    xfer[4:8, L // 2:] = 0
+    comp[8:12] <<= 22
+    xfer[8:12] <<= 22
+    dt = rng.integers(0, 4000, 16)
+    dt[8:12] <<= 22
+    parts.append((comp.astype(np.int64), xfer.astype(np.int64), dt.astype(np.int64)))
+    _same(dc, *(np.concatenate([p[q] for p in parts]) for q in range(3)), L)
