@@ -17,8 +17,9 @@
 // replays its lane's row. Warps are persistent (one resident wave) and prefetch
 // their next tile into L2 while the current one is copied. For L <= 16 the
 // replay is unrolled at compile time and inputs are screened on their high
-// words. Longer rows are read by each thread directly.
-#include "common.cuh"
+// words. Longer rows take one warp per instance (eval_warp_kernel), up to 95 and large
+// batches one thread (launch_eval).
+#include "chain.cuh"
 
 namespace dc {
 
@@ -70,6 +71,7 @@ struct Replay {
     }
 };
 
+// One instance per thread, its rows read where they are.
 template <bool FWD>
 __global__ void __launch_bounds__(256)
     eval_kernel(int64_t batch, int L, const int64_t *__restrict__ comp,
@@ -92,6 +94,76 @@ __global__ void __launch_bounds__(256)
             rp.step<FWD>(__ldg(crow + col), __ldg(xrow + col), uint64_t(d), cut);
         }
         makespan[i] = rp.result(L, d);
+    }
+}
+
+// One instance per warp, 64 rows at a time, two to a lane. In the prefixes a, b and the
+// costs e, c_j of chain.cuh the replay is the largest, over the segments j of the
+// decision, of c_j + a[end] - b[start] + (s - j) e, plus e + b[L]; so a segment needs only
+// its number and the b of the break before it, which ballots give. Bound by the reads
+// (and, with a 64-bit scan per 64 rows, close to integer issue). Per direction against one
+// thread per instance, whose reads are uncoalesced (forward): 16,384 x 1,024 73 us against
+// 276, 2,048 x 1,024 14.7 against 267, 120,000 x 128 81 against 137, 1,000 x 129 9.4
+// against 18 (a call from the host).
+template <bool FWD>
+__global__ void __launch_bounds__(256)
+    eval_warp_kernel(int64_t batch, int L, const int64_t *__restrict__ comp,
+                     const int64_t *__restrict__ xfer, const int64_t *__restrict__ dt,
+                     const uint32_t *__restrict__ bits, int64_t *__restrict__ makespan, bool vec)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, W = words_for(L);
+    const unsigned lower = (1u << lane) - 1u;
+    const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
+    for (int64_t i = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); i < batch; i += warps) {
+        const RowLoader<FWD> load{comp + i * L, xfer + i * L, L, vec};
+        const uint32_t *brow = bits + i * W;
+        const uint64_t d = uint64_t(__ldg(dt + i));
+        // unsigned arithmetic: garbage from rejected inputs wraps instead of overflowing
+        uint64_t any = d, aL = 0, bL = 0, start = 0;  // start: b of the last break
+        int64_t best = INT64_MIN;
+        int cnt = 0;  // breaks so far
+        for (int r0 = 1; r0 <= L; r0 += 64) {
+            const int r = r0 + 2 * lane;
+            uint64_t a0, a1, b0, b1;
+            if (FWD)
+                load(r, b0, b1, a0, a1);
+            else
+                load(r, a0, a1, b0, b1);
+            const uint32_t word = r < L ? __ldg(brow + ((r - 1) >> 5)) : 0u;
+            const bool k0 = (word >> ((r - 1) & 31)) & 1u, k1 = r + 1 < L && ((word >> (r & 31)) & 1u);
+            any |= a0 | a1 | b0 | b1;
+            uint64_t sa = a0 + a1, sb = b0 + b1;
+            scan2(sa, sb, lane);
+            const uint64_t ar1 = aL + sa, br1 = bL + sb, ar0 = ar1 - a1, br0 = br1 - b1;
+            const unsigned e0 = __ballot_sync(kAll, k0), e1 = __ballot_sync(kAll, k1), e = e0 | e1;
+            const uint64_t last = k1 ? br1 : br0;
+            const unsigned below = e & lower;
+            const uint64_t prev = __shfl_sync(kAll, last, below ? 31 - __clz(int(below)) : 0);
+            const uint64_t s0 = below ? prev : start, s1 = k0 ? br0 : s0;
+            const uint64_t n0 = uint64_t(cnt + __popc(e0 & lower) + __popc(e1 & lower));
+            const uint64_t c0 = FWD ? (n0 + 1) * d : 0 - n0 * d;
+            const uint64_t c1 = k0 ? (FWD ? c0 + d : c0 - d) : c0;
+            if (k0 || r == L) best = max(best, int64_t(c0 + ar0 - s0));
+            if (k1 || r + 1 == L) best = max(best, int64_t(c1 + ar1 - s1));
+            const uint64_t top = __shfl_sync(kAll, last, e ? 31 - __clz(int(e)) : 0);
+            if (e) start = top;
+            cnt += __popc(e0) + __popc(e1);
+            aL += __shfl_sync(kAll, sa, 31);
+            bL += __shfl_sync(kAll, sb, 31);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(kAll, best, o));
+        const uint32_t all = __reduce_or_sync(kAll, uint32_t(any >> 32));
+        if (lane == 0) {
+            int64_t f = int64_t(uint64_t(best) + bL + (FWD ? 0 : uint64_t(cnt + 1) * d));
+            if (all >> 31)
+                f = -int64_t(DC_ERR_NEGATIVE);
+            else if (all >> 20 || exceeds_range(L, int64_t(d), FWD ? bL : aL, FWD ? aL : bL))
+                f = -int64_t(DC_ERR_RANGE);
+            makespan[i] = f;
+        }
+        __syncwarp();  // see the end of chain_columns
     }
 }
 
@@ -397,14 +469,30 @@ cudaError_t launch_eval(bool forward, int64_t batch, int L, const int64_t *comp,
                 batch, L, comp, xfer, dt, bits, makespan, pairs);
         return cudaGetLastError();
     }
-    int64_t blocks = (batch + 255) / 256;
+    // Below 96 rows half of a warp's second 64 are past the end, and many threads hide their
+    // uncoalesced reads: 240,000 x 65 68 us forward and 110 backward against 144, 200,000 x 88
+    // 109 and 123 against 127; but 20,000 x 72 19 against 16, 160,000 x 96 130 against 104.
+    if (L < 96 && batch >= 50000) {
+        int64_t blocks = (batch + 255) / 256;
+        if (blocks > 152 * 64) blocks = 152 * 64;
+        if (forward)
+            eval_kernel<true><<<unsigned(blocks), 256, 0, stream>>>(batch, L, comp, xfer, dt, bits,
+                                                                   makespan);
+        else
+            eval_kernel<false><<<unsigned(blocks), 256, 0, stream>>>(batch, L, comp, xfer, dt, bits,
+                                                                    makespan);
+        return cudaGetLastError();
+    }
+    const bool vec = (L % 2 == 0) &&
+                     ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0;
+    int64_t blocks = (batch + 7) / 8;
     if (blocks > 152 * 64) blocks = 152 * 64;
     if (forward)
-        eval_kernel<true><<<unsigned(blocks), 256, 0, stream>>>(batch, L, comp, xfer, dt, bits,
-                                                               makespan);
+        eval_warp_kernel<true><<<unsigned(blocks), 256, 0, stream>>>(batch, L, comp, xfer, dt, bits,
+                                                                    makespan, vec);
     else
-        eval_kernel<false><<<unsigned(blocks), 256, 0, stream>>>(batch, L, comp, xfer, dt,
-                                                                bits, makespan);
+        eval_warp_kernel<false><<<unsigned(blocks), 256, 0, stream>>>(batch, L, comp, xfer, dt, bits,
+                                                                     makespan, vec);
     return cudaGetLastError();
 }
 
