@@ -24,7 +24,7 @@ struct GenParams {
     int64_t batch, inst0;
     uint64_t seed;
     int32_t L, layer_mode, rate_dist, bw_dist, bwd_mult, bits;
-    int32_t words;  // every quotient is below 2^32 (WordDiv)
+    int32_t words;  // every cost is below 2^32 (word_costs)
     int64_t rate_lo, rate_hi, bw_lo, bw_hi, dt_lo, dt_hi;
     int64_t params_lo, params_hi, flops_lo, flops_hi;
     int64_t rate_knots[kKnots + 1], bw_knots[kKnots + 1];
@@ -230,7 +230,8 @@ __device__ __forceinline__ void wire_costs(const GenParams &g, const InstanceDra
     }
 }
 
-// The same costs where every quotient is below 2^32: `wire` is bits * 1000 * params.
+// The same costs where each of them is below 2^32 (with bwd_mult 2 the forward ones and
+// the transfers): `wire` is bits * 1000 * params.
 __device__ __forceinline__ void word_costs(const GenParams &g, const WordDiv &rate, const WordDiv &bw,
                                            uint64_t wire, uint64_t flops, uint32_t &fc,
                                            uint64_t &bc, uint32_t &xfer)

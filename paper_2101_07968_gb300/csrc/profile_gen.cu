@@ -21,12 +21,12 @@ namespace {
 // at a time, so the output rows are written coalesced. Only __syncwarp between the
 // phases.
 //
-// WORDS: every quotient is below 2^32 (all configurations here): divisions in 32-bit
-// steps (WordDiv), an instance's divisors in one 16-byte and one 4-byte load, a layer's
-// numerators in one 16-byte load. SHARED: the knots and layer tables in shared memory;
-// without it (small batches) lanes read the few entries they need from the parameters,
-// which beats copying the tables in every CTA. Bound by the HBM writes on large batches
-// (1,000,000 x 16, 520 MB: 84 us, 6.2 TB/s, with either division), by integer issue on
+// WORDS: every cost is below 2^32 (all configurations here; see fill_gen_params):
+// divisions in 32-bit steps (WordDiv), an instance's divisors in one 16-byte and one 4-byte
+// load, a layer's numerators in one 16-byte load. SHARED: the knots and layer tables in
+// shared memory; without it (small batches) lanes read the few entries they need from the
+// parameters, which beats copying the tables in every CTA. Bound by the HBM writes on large
+// batches (1,000,000 x 16, 520 MB: 84 us, 6.2 TB/s, with either division), by integer issue on
 // short rows (1,000,000 x 8: 48 us, 53 with 64-bit divisions) and on log-uniform layers
 // (16,384 x 1,024: 127 us, 376 with 64-bit divisions in tiles of 32).
 constexpr int kGenWarps = 8;
@@ -165,7 +165,9 @@ void fill_gen_params(const dc_profile_cfg *c, GenParams &g)
     g.params_hi = c->params_hi;
     g.flops_lo = c->flops_lo;
     g.flops_hi = c->flops_hi;
-    // the largest numerators, and whether their quotients all fit 32 bits
+    // the largest numerators, and whether their costs, the quotients rounded up, all fit
+    // 32 bits (word_costs rounds up in 32 bits: a quotient of 2^32 - 1 with a remainder
+    // would come out 0)
     int64_t most_p = c->params_hi, most_f = c->flops_hi;
     if (c->layer_mode == DC_LAYERS_FIXED) {
         most_p = most_f = 0;
@@ -174,7 +176,7 @@ void fill_gen_params(const dc_profile_cfg *c, GenParams &g)
             most_f = std::max(most_f, c->fixed_flops[l]);
         }
     }
-    auto fits = [](int64_t num, int64_t d) { return num / d < (int64_t(1) << 32); };
+    auto fits = [](int64_t num, int64_t d) { return (num + d - 1) / d < (int64_t(1) << 32); };
     g.words = fits(int64_t(c->bits_per_param) * 1000 * most_p, c->bw_lo) &&
               fits(int64_t(c->bwd_flops_mult == 2 ? 1 : c->bwd_flops_mult) * most_f, c->rate_lo);
     if (c->rate_dist == DC_DIST_LOGUNIFORM) knots(c->rate_lo, c->rate_hi, g.rate_knots);

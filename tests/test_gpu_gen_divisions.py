@@ -56,3 +56,46 @@ def test_every_value(dc, name, kw, batch):
             ref = dc.schedule(d, got[c], got[x], got["dt"])
             for k in ("makespan", "bits", "nseg", "status"):
                 assert torch.equal(out[k][d], ref[k]), (k, d)
+
+
+# Numerators at the 32-bit steps' upper edge, d * 2^32 - 1 and its neighbours: the largest
+# cost is the QUOTIENT ROUNDED UP, 2^32 - 1 (in 32 bits) or 2^32 (not in 32 bits).
+def _edge(rate, flops, mult=2, bits=32, params=(1, 2, 3, 4), bw=1000):
+    cfg = wl.config("vgg16")
+    cfg.update(L=len(flops), fixed_flops=list(flops), fixed_params=list(params),
+               rate_lo=rate, rate_hi=rate, bw_lo=bw, bw_hi=bw, bits_per_param=bits,
+               bwd_flops_mult=mult)
+    return cfg
+
+
+K = 2**32
+EDGES = [_edge(d, (f, 1, 0, d), mult)
+         for d in (2, 3, 255) for mult in (1, 2)
+         for f in ((K - 1) * d, (K - 1) * d + 1, K * d - 1, K * d)]
+EDGES += [_edge(d, (f, 1, 0, d), 3)
+          for d in (2, 3, 255) for f in ((K - 1) * d // 3, (K - 1) * d // 3 + 1, K * d // 3)]
+EDGES += [_edge(1000, (1, 2, 3, 4), 2, bits, (p, 1, 0, 2), bw)
+          for bits, p, bw in ((32, 35_030_827, 261), (1, 4_299_262_263, 1001),
+                              (1, 4_299_262_262, 1001), (1, 4_299_262_264, 1001))]
+
+
+@pytest.mark.parametrize("edge", range(len(EDGES)))
+@pytest.mark.parametrize("batch", [37, 9000, 70_001])  # every generator and generate-and-solve kernel
+def test_costs_at_two_to_the_32(dc, edge, batch):
+    import torch
+    cfg = wl.with_batch(EDGES[edge], batch)
+    got = dc.profile_gen(cfg)
+    exp = oracle.profile_gen(cfg)
+    for k in ("fc", "pt", "bc", "gt", "dt"):
+        assert np.array_equal(got[k].cpu().numpy(), exp[k]), k
+    ref = {d: dc.schedule(d, got[c], got[x], got["dt"])
+           for d, c, x in ((0, "fc", "pt"), (1, "bc", "gt"))}
+    out = dc.GeneratedScheduler(cfg).run()
+    for d in (0, 1):
+        for k in ("makespan", "bits", "nseg", "status"):
+            assert torch.equal(out[k][d], ref[d][k]), (k, d)
+    g = dc.StepGraph(cfg)
+    g.replay()
+    torch.cuda.synchronize()
+    for k in ("fc", "pt", "bc", "gt", "dt"):
+        assert np.array_equal(g.prof[k].cpu().numpy(), exp[k]), k
