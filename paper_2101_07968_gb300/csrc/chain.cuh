@@ -138,15 +138,16 @@ struct Pair<int64_t> {
 // q = the byte offset of key p + 1, with p the number of keys below t.
 //
 // halve_from<STEP>: the count lies in [0, 2 STEP - 1] past q; keys that the caller
-// padded with the largest value end it earlier.
-template <typename T, int STEP>
+// padded with the largest value end it earlier. UPTO: p counts the keys up to t (the
+// padding too where t is the largest value: t + 1, to search below it, would not exist).
+template <typename T, int STEP, bool UPTO = false>
 __device__ __forceinline__ void halve_from(T t0, T t1, int &q0, int &q1)
 {
     constexpr int S = int(sizeof(T));
     const T k0 = sh<T>(q0 + (STEP - 1) * S), k1 = sh<T>(q1 + (STEP - 1) * S);
-    if (k0 < t0) q0 += STEP * S;
-    if (k1 < t1) q1 += STEP * S;
-    if constexpr (STEP > 1) halve_from<T, STEP / 2>(t0, t1, q0, q1);
+    if (UPTO ? k0 <= t0 : k0 < t0) q0 += STEP * S;
+    if (UPTO ? k1 <= t1 : k1 < t1) q1 += STEP * S;
+    if constexpr (STEP > 1) halve_from<T, STEP / 2, UPTO>(t0, t1, q0, q1);
 }
 // search_below: N keys from byte kb, P the largest power of two <= N: the first probe
 // splits [0, N] into two ranges of at most P values, the rest halve it.

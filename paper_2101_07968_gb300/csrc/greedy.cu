@@ -492,7 +492,7 @@ __device__ __forceinline__ T greedy_backward_rows(int kb, int D, int L, T dt, T 
     T sent = dt;
     // a chain advances by a row or more each step, so L steps end them all
     for (int step = 1; step < L && __any_sync(kAll, q[0] < end || q[1] < end); ++step) {
-        T t[2];
+        T lim[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const bool on = q[u] < end;
@@ -500,14 +500,15 @@ __device__ __forceinline__ T greedy_backward_rows(int kb, int D, int L, T dt, T 
             mask[u] |= on ? uint64_t(1) << (p - 1) : uint64_t(0);
             // the longest segment whose compute the link estimate covers, else one layer
             // and the zero-compute layers after it; a finished chain stays at L
-            t[u] = (on ? max(A[u] + sent + B[u], next[u]) : aL) + 1;
+            lim[u] = on ? max(A[u] + sent + B[u], next[u]) : aL;
         }
         int n0 = kb, n1 = kb;
-        halve_from<T, 32>(t[0], t[1], n0, n1);
+        halve_from<T, 32, true>(lim[0], lim[1], n0, n1);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const bool on = q[u] < end;
-            q[u] = aL < t[u] ? end : (u == 0 ? n0 : n1);  // the search counts to 63 rows
+            // the search counts to 63 rows, and past L where the limit is the padding's value
+            q[u] = aL <= lim[u] ? end : (u == 0 ? n0 : n1);
             const T a = sh<T>(q[u] - S), b = sh<T>(q[u] + D - S);
             next[u] = sh<T>(q[u]);
             link[u] = on ? max(link[u], a) + dt + (b - B[u]) : link[u];

@@ -87,3 +87,35 @@ def test_deep(dc, L):
         for q in cuts:
             word[(q - 1) // 32] |= np.uint32(1 << ((q - 1) % 32))
         assert mk[i] == t and np.array_equal(bits[i], word), (L, i)
+
+
+def _edge_instances(L, total):
+    """Sums of a[L] + b[L] + (L + 1) dt = total, with and without a zero-cost tail in
+    processing order of either direction, concentrated in a layer or spread."""
+    rng = np.random.default_rng(L)
+    comp, xfer, dt = [], [], []
+    for d in (0, 1, 1 << 20):
+        rest = total - (L + 1) * d
+        for j in (0, 1, L // 2, L - 1):  # layers below j (or above L - 1 - j) cost nothing
+            for x in (0, 1, rest // 2, rest):
+                c, t = np.zeros(L, np.int64), np.zeros(L, np.int64)
+                c[j], t[j] = rest - x, x
+                spread = np.diff(np.r_[0, np.sort(rng.integers(0, rest + 1, 2 * (L - j) - 1)), rest])
+                cs, ts = np.zeros(L, np.int64), np.zeros(L, np.int64)
+                cs[j:], ts[j:] = spread[::2], spread[1::2]
+                for a, b in ((c, t), (c, t[::-1]), (cs, ts)):
+                    comp += [a, a[::-1]]
+                    xfer += [b, b[::-1]]
+                    dt += [d, d]
+    return np.array(comp), np.array(xfer), np.array(dt, np.int64)
+
+
+@pytest.mark.parametrize("total", [2**31 - 2, 2**31 - 1, 2**31])
+@pytest.mark.parametrize("L", [8, 9, 16, 22, 23, 33, 63, 64, 65, 129])
+def test_sums_at_two_to_the_31(dc, L, total):
+    """The 32-bit forms end at a sum of 2^31 - 1, where no value may grow by one more."""
+    comp, xfer, dt = _edge_instances(L, total)
+    for d in (0, 1):
+        mk, bits = _run(dc, d, comp, xfer, dt)
+        exp = oracle.greedy_batch(d, comp, xfer, dt, nthreads=os.cpu_count() or 1)
+        assert np.array_equal(mk, exp["makespan"]) and np.array_equal(bits, exp["bits"]), (L, d)
