@@ -579,11 +579,12 @@ class HostPipeline:
         results go back in two groups: those of all pieces but the last, beside the
         last one's input copies, then the last one's."""
         import torch
+        if not self.batch:
+            return
         canon = self._canonical(host_in)
         cur = torch.cuda.current_stream()
         self.s_in.wait_stream(cur)
-        pieces = [(c, lo, hi) for c, (lo, hi) in enumerate(zip(self.bounds, self.bounds[1:]))
-                  if hi > lo]
+        pieces = [(c, lo, hi) for c, (lo, hi) in enumerate(zip(self.bounds, self.bounds[1:]))]
         with torch.cuda.stream(self.s_in):
             for c, lo, hi in pieces:
                 for k in self.IN_KEYS:

@@ -63,3 +63,16 @@ def test_host_pipeline_shared_transfer_buffer(dc):
     h_sep, _ = pipe.bytes_per_run(sep)
     h_shared, _ = pipe.bytes_per_run(shared)
     assert h_sep - h_shared == ref["gt"].nbytes
+
+
+def test_empty_batch(dc):
+    """No profiles: nothing to do, as in every call of the library."""
+    import torch
+    pipe = dc.HostPipeline(0, 16)
+    host = {k: torch.empty((0, 16), dtype=torch.int64).pin_memory() for k in ("fc", "pt", "bc", "gt")}
+    host["dt"] = torch.empty(0, dtype=torch.int64).pin_memory()
+    out = pipe.host_buffers()
+    pipe.run(host, out)
+    torch.cuda.synchronize()
+    assert all(v.numel() == 0 for v in out.values())
+    assert pipe.bytes_per_run(host) == (0, 0)
