@@ -289,8 +289,9 @@ __device__ __forceinline__ bool chain_columns(int kb, int D, uint32_t *word, T *
         T hn;
         if (WARP) {
             // the last row that a lane holds is row L or past it (then it has row L's a, and
-            // comes out the same); every lane has read column n-1 here
+            // comes out the same)
             hn = __shfl_sync(kAll, v[NJ - 1][1], 31);
+            __syncwarp();  // every lane has read column n-1 (a shuffle orders no memory)
         } else {
             __syncthreads();
             hn = pub[n & 1];
