@@ -1,7 +1,7 @@
 // One instance of the DynaComm DP (Eq. 8 / Algorithm 3 and Eq. 9 / Algorithm 4)
 // solved by a warp or a CTA in O(L log L) per segment count: the device code shared
-// by the warp-per-instance pass (dp_warp.cu), the CTA-per-instance pass (dp_deep.cu),
-// the work-list pass (dp_group.cu) and its drawing form (dp_fused.cu).
+// by the warp-per-instance pass (dp_warp.cu), the CTA-per-instance pass (dp_deep.cu) and
+// the work-list passes (dp_group.cu, dp_small.cu, the drawing one in dp_fused.cu).
 //
 // With the layers in processing order, P the prefix of the transfer costs and C
 // that of the compute costs, put
@@ -59,8 +59,8 @@ __device__ __forceinline__ T &sh(int off)
 // Arrays of the solver: K (the newest column's keys H + e + b) and b of rows 1, 2, ..,
 // 8 bytes a row (the 32-bit form uses the first half of each array), with 16 bytes
 // between them whose last 8 are zero: b of row 0.
-__host__ __device__ inline int chain_rows_bytes(int rows) { return rows * 8; }
-__host__ __device__ inline int chain_pair_bytes(int rows) { return 2 * chain_rows_bytes(rows) + 16; }
+__host__ __device__ constexpr int chain_rows_bytes(int rows) { return rows * 8; }
+__host__ __device__ constexpr int chain_pair_bytes(int rows) { return 2 * chain_rows_bytes(rows) + 16; }
 
 // The columns kept for the traceback, 1..last, as 32-bit words at a stride of
 // chain_stride(L) cells; columns 1..shared in shared memory (from byte `sm`) and the

@@ -23,7 +23,7 @@ constexpr uint64_t kShiftedLimit = 0x7FFFFFFFull;
 
 // Triangle of DP cells (m, n), 1 <= n <= m <= L, stored column by column:
 // column n holds rows n..L contiguously.
-__host__ __device__ inline int64_t tri_cells(int L) { return int64_t(L) * (L + 1) / 2; }
+__host__ __device__ constexpr int64_t tri_cells(int L) { return int64_t(L) * (L + 1) / 2; }
 __host__ __device__ inline int64_t tri_col(int L, int n)
 {
     return int64_t(n - 1) * L - int64_t(n - 1) * (n - 2) / 2;
@@ -210,6 +210,24 @@ __host__ __device__ inline bool exceeds_range(int L, int64_t dt, uint64_t sc, ui
 // start launching before the earlier one's CTAs exit.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Host: a launch with that attribute.
+template <typename... Params, typename... Args>
+cudaError_t launch_early(void (*kernel)(Params...), int64_t grid, int nt, size_t smem,
+                         cudaStream_t stream, const Args &...args)
+{
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(unsigned(grid));
+    lc.blockDim = dim3(unsigned(nt));
+    lc.dynamicSmemBytes = smem;
+    lc.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kernel, args...);
+}
 
 template <typename T>
 __device__ __forceinline__ T dmax(T a, T b) { return a > b ? a : b; }

@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(32, DC_SMALL_MINB)
             const bool wd = fwd ? wide[0] : wide[1];
             const uint64_t xd = fwd ? xraw[0] : xraw[1];
             const SolveOut od = fwd ? o.out[0] : o.out[1];
-            const bool done = solve_uv<L, STORE>(fwd, active && std == DC_OK && !wd, U, V, int32_t(dti),
+            const bool done = solve_uv<L, STORE, kKeepCols>(fwd, active && std == DC_OK && !wd, U, V, int32_t(dti),
                                                  xd, lw, i, od);
             if (active && std != DC_OK) {
                 write_failure(std, i, W, od);
@@ -233,45 +233,51 @@ struct DrawLoader {
     }
 };
 
-// Pass over one direction's list, rows regenerated: one warp per instance, every value
-// and every column (chain.cuh).
-template <bool FWD>
-__global__ void __launch_bounds__(32)
+// Pass over one direction's list, rows regenerated (see small_list_kernel).
+template <int L, bool FWD>
+__global__ void __launch_bounds__(32 * List64<L, true>::kWarps)
     fused_list_kernel(const __grid_constant__ GenParams g, const GenTables *t, const FusedOut o)
 {
+    static_assert(Table<L, int64_t, L>::kWords >= 2 * L, "a lane's rows lie where its table will");
     constexpr int dir = FWD ? 0 : 1;
-    int64_t *table = &sh<int64_t>(chain_pair_bytes(64));
-    if (threadIdx.x == 0) zero_row(0, 64);
     pdl_wait();  // the passes ahead of this one have finished
-    const int64_t count = int64_t(*o.wide_count[dir]);
-    for (int64_t j = blockIdx.x; j < count; j += gridDim.x) {
-        const int64_t i = int64_t(o.wide_list[dir][j]);
-        if (!DC_CHECK(i < g.batch)) continue;
-        const int64_t gi = g.inst0 + i;
-        const InstanceDraws d = instance_draws(g, t->rate, t->bw, gi);
-        const int L = g.L;
-        chain_solve_warp<FWD, 1>(0, i, L, DrawLoader<FWD>{g, t->layer, d, gi}, d.dt, o.out[dir],
-                                 KeptValues{table, L});
-        __syncwarp();  // shared memory is read
-    }
+    list_pass<L, true>(
+        g.batch, int64_t(*o.wide_count[dir]), o.wide_list[dir],
+        [&](int kb, int64_t i, const KeptValues &kept) {
+            const InstanceDraws d = instance_draws(g, t->rate, t->bw, g.inst0 + i);
+            chain_solve_warp<FWD, 1>(kb, i, L, DrawLoader<FWD>{g, t->layer, d, g.inst0 + i}, d.dt,
+                                     o.out[dir], kept);
+        },
+        [&](bool active, int64_t i) {
+            int64_t *row = &sh<int64_t>(8 * int(threadIdx.x)), dti = 0;
+            if (active) {
+                const InstanceDraws d = instance_draws(g, t->rate, t->bw, g.inst0 + i);
+                dti = d.dt;
+#pragma unroll 1
+                for (int l = 0; l < L; ++l) {
+                    int64_t wire, flops, f, b, x;
+                    layer_numerators(g, t->layer, g.inst0 + i, l, wire, flops);
+                    wire_costs(g, d, uint64_t(wire), uint64_t(flops), f, b, x);
+                    row[32 * l] = FWD ? f : b;
+                    row[32 * (L + l)] = x;
+                }
+            }
+            list_solve_lane<L, FWD>(
+                active, i, dti,
+                [&](int col, int64_t &cv, int64_t &xv) {
+                    cv = row[32 * col];
+                    xv = row[32 * (L + col)];
+                },
+                o.out[dir]);
+        });
 }
 
-template <bool FWD>
+template <int L, bool FWD>
 cudaError_t launch_fused_list(const GenParams &g, const GenTables *t, const FusedOut &o,
                               cudaStream_t stream)
 {
-    const int64_t lgrid = g.batch < int64_t(sm_count()) * 16 ? g.batch : int64_t(sm_count()) * 16;
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(unsigned(lgrid));
-    lc.blockDim = dim3(32);
-    lc.dynamicSmemBytes = chain_pair_bytes(64) + size_t(tri_cells(g.L)) * 8;
-    lc.stream = stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, fused_list_kernel<FWD>, g, t, o);
+    static DeviceCache listers;
+    return launch_list<L, true>(listers, g.batch, stream, fused_list_kernel<L, FWD>, g, t, o);
 }
 
 // Small batches, one launch: warp 0 of a CTA draws two instances' rows, one layer to a
@@ -378,9 +384,9 @@ cudaError_t launch_fused_L(const GenParams &g, const GenTables *t, const FusedOu
     fused_pair_kernel<L, STORE><<<unsigned(grid), 32, Pair32<L>::kBytes, stream>>>(g, t, o);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = launch_fused_list<true>(g, t, o, stream);
+    e = launch_fused_list<L, true>(g, t, o, stream);
     if (e != cudaSuccess) return e;
-    return launch_fused_list<false>(g, t, o, stream);
+    return launch_fused_list<L, false>(g, t, o, stream);
 }
 
 }  // namespace

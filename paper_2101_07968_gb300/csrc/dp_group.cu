@@ -1,7 +1,7 @@
-// DynaComm DP of listed instances, any 1 <= L <= 4096 (Eq. 8 / Algorithm 3 and
-// Eq. 9 / Algorithm 4): the pass over the first passes' work lists (dp_small.cu,
-// dp_mid.cu, dp_warp.cu, dp_deep.cu), whose instances have values
-// beyond the first pass's range or an optimum deeper than its kept columns. The
+// DynaComm DP of listed instances, 17 <= L <= 4096 (Eq. 8 / Algorithm 3 and
+// Eq. 9 / Algorithm 4): the pass over the first passes' work lists (dp_mid.cu,
+// dp_warp.cu, dp_deep.cu; the lists of L <= 16 are dp_small.cu's own), whose instances
+// have values beyond the first pass's range or an optimum deeper than its kept columns. The
 // method is in chain.cuh; this pass takes every value (64 bits) and keeps every
 // column: one warp per instance with the table in shared memory up to L = 64, otherwise
 // one CTA per instance with a table in the caller's workspace.
@@ -38,9 +38,9 @@ __global__ void __launch_bounds__(kChainThreads, 1) group_kernel(GroupArgs a)
     }
 }
 
-// L <= 64: one warp per instance, the table in shared memory. The CTA form's barriers and
-// 64-bit scan cost it ten times the time there: 1,000,000 x 16 with some 6,000 instances
-// listed took 121 us a direction with it, 103 with this kernel (70 of it the first pass).
+// L <= 64: one warp per instance, the table in shared memory, without the CTA form's
+// barriers (some 6,000 listed instances of L = 16 took 51 us with that, 33 with this kernel
+// on 4 warps per SM).
 template <bool FWD>
 __global__ void __launch_bounds__(32) list_warp_kernel(GroupArgs a)
 {
@@ -59,25 +59,6 @@ __global__ void __launch_bounds__(32) list_warp_kernel(GroupArgs a)
     }
 }
 
-// Launched early (programmatic dependent launch): the CTAs wait in hardware until the
-// first pass completes, so the launch overlaps that pass's tail.
-template <typename Kernel>
-cudaError_t launch_list(Kernel kernel, const GroupArgs &a, int64_t grid, int nt, size_t smem,
-                        cudaStream_t stream)
-{
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(unsigned(grid));
-    lc.blockDim = dim3(unsigned(nt));
-    lc.dynamicSmemBytes = smem;
-    lc.stream = stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, kernel, a);
-}
-
 template <bool FWD, int NJ>
 cudaError_t launch_group_nj(const GroupArgs &a, int nt, int64_t grid, cudaStream_t stream)
 {
@@ -89,15 +70,17 @@ cudaError_t launch_group_nj(const GroupArgs &a, int nt, int64_t grid, cudaStream
                                     int(chain_smem_most(DC_L_MAX)));
     });
     if (e != cudaSuccess) return e;
-    return launch_list(group_kernel<FWD, NJ>, a, grid, nt, chain_smem_bytes(a.L, 2 * NJ * nt), stream);
+    // launched early: the CTAs wait in hardware until the first pass completes, so the
+    // launch overlaps that pass's tail
+    return launch_early(group_kernel<FWD, NJ>, grid, nt, chain_smem_bytes(a.L, 2 * NJ * nt), stream, a);
 }
 
 template <bool FWD>
 cudaError_t launch_group_dir(const GroupArgs &a, int64_t grid, cudaStream_t stream)
 {
     if (a.L <= kSmemTableLMax)
-        return launch_list(list_warp_kernel<FWD>, a, grid, 32,
-                           chain_pair_bytes(64) + size_t(tri_cells(a.L)) * 8, stream);
+        return launch_early(list_warp_kernel<FWD>, grid, 32,
+                            chain_pair_bytes(64) + size_t(tri_cells(a.L)) * 8, stream, a);
     // lists are short: two rows per thread, for the shortest column
     int nt = 32 * ((a.L + 63) / 64);
     if (nt > kChainThreads) nt = 32 * ((a.L + 127) / 128);

@@ -30,9 +30,11 @@
 //  * transfer costs are first capped at the instance's total compute, which
 //    changes no decision (see row_prefix); the shifted 32-bit form is exact
 //    whenever the capped bound L*dt + sum(capped xfer) + sum(comp) is below
-//    2^31. Other instances (and the deep ones above) are appended to a work list
-//    that the CTA-per-instance pass solves afterwards (dp_group.cu); it is launched
-//    early and waits in hardware for this one (programmatic dependent launch);
+//    2^31. Other instances (and the deep ones above) are appended to a work list,
+//    which small_list_kernel solves afterwards in 64 bits, with the same fill for an
+//    instance per lane or by the chain solver for an instance per warp (see List64 in
+//    dp_small.cuh); it is launched early and waits in hardware for this one
+//    (programmatic dependent launch);
 //  * with REPLAY the traceback also evaluates f_m of the decision, segment by segment
 //    (a select chain and two instructions a step), in place of a kernel that reads the
 //    rows again: the 1,000,000-instance VGG-16 step takes 208 us instead of 291;
@@ -85,7 +87,11 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
     uint32_t *ticket = wide_count + 1;     // tiles handed out (zero before the launch)
 
     const int64_t tiles = (batch + 31) / 32;
-    pdl_trigger();  // the list pass may be scheduled as soon as CTAs of this one exit
+    // The list pass may be scheduled as CTAs of this one exit: from the start, which hides
+    // its launch (1,000,000 x 8, both directions: 67.5 us against 69.1 with the last tiles);
+    // on long tiles only with the last ones, because its waiting CTAs would take the places
+    // that the other direction's pass is to fill (the VGG-16 step: 205.5 us against 209.5)
+    if (!kTicket) pdl_trigger();
     auto rows_of = [&](int64_t t) { return int(batch - t * 32 < 32 ? batch - t * 32 : 32); };
     auto claim = [&]() {
         uint32_t v = 0;
@@ -96,7 +102,7 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
     auto finish = [&](int64_t i, bool active, const int32_t (&U)[L + 1], const int32_t (&V)[L + 1],
                       int64_t dti, uint64_t xraw, bool wide, int st) {
         const bool run = active && st == DC_OK && !wide;
-        const bool done = solve_uv<L, REPLAY>(FWD, run, U, V, int32_t(dti), xraw, lw, i, o);
+        const bool done = solve_uv<L, REPLAY, kKeepCols>(FWD, run, U, V, int32_t(dti), xraw, lw, i, o);
         if (active && st != DC_OK) {
             write_failure(st, i, W, o);
         } else if (active && (wide || !done)) {
@@ -137,6 +143,7 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
                 if (kTicket) next_raw = claim();
             }
             tile = next;
+            if (kTicket && tile >= tiles) pdl_trigger();
             finish(i, active, U, V, dti, xraw, wide, st);
         }
     } else {
@@ -169,6 +176,34 @@ __global__ void __launch_bounds__(32, dense_min_ctas(L))
             finish(i, active, U, V, dti, xraw, wide, st);
         }
     }
+}
+
+// The pass over the dense pass's list.
+template <int L, bool FWD>
+__global__ void __launch_bounds__(32 * List64<L, false>::kWarps)
+    small_list_kernel(const int64_t *__restrict__ comp, const int64_t *__restrict__ xfer,
+                      const int64_t *__restrict__ dt, const SolveOut o, int64_t batch,
+                      const uint32_t *__restrict__ wide_count, const uint32_t *__restrict__ wide_list,
+                      bool pairs)
+{
+    pdl_wait();  // the dense pass has finished its list
+    list_pass<L, false>(
+        batch, int64_t(*wide_count), wide_list,
+        [&](int kb, int64_t i, const KeptValues &kept) {
+            chain_solve_warp<FWD, 1>(
+                kb, i, L, RowLoader<FWD>{comp + i * L, xfer + i * L, L, L % 2 == 0 && pairs}, __ldg(dt + i),
+                o, kept);
+        },
+        [&](bool active, int64_t i) {
+            const int64_t *crow = comp + i * L, *xrow = xfer + i * L;
+            list_solve_lane<L, FWD>(
+                active, i, active ? __ldg(dt + i) : 0,
+                [&](int col, int64_t &cv, int64_t &xv) {
+                    cv = __ldg(crow + col);
+                    xv = __ldg(xrow + col);
+                },
+                o);
+        });
 }
 
 }  // namespace
@@ -211,20 +246,19 @@ cudaError_t launch_dir(int64_t batch, const int64_t *comp, const int64_t *xfer,
         const cudaError_t re = cudaEventRecord(pe.start, stream);
         if (re != cudaSuccess) return re;
     }
+    const bool pairs = ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0;
     small_dense_kernel<L, FWD, REPLAY><<<unsigned(grid), 32, kSmem, stream>>>(
-        batch, comp, xfer, dt, o, wide_count, wide_list,
-        ((reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(xfer)) & 15u) == 0);
+        batch, comp, xfer, dt, o, wide_count, wide_list, pairs);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (pe.stop) {
         e = cudaEventRecord(pe.stop, stream);
         if (e != cudaSuccess) return e;
     }
-    // the list length is known on the device only: one-warp CTAs (up to 4 per SM) walk
-    // it, and the surplus exits at once
-    const int64_t lgrid = batch < int64_t(sm_count()) * 4 ? batch : int64_t(sm_count()) * 4;
-    return launch_group(FWD, batch, L, comp, xfer, dt, o, wide_count, wide_list, nullptr, lgrid,
-                        stream);
+    static DeviceCache listers;
+    return launch_list<L, false>(listers, batch, stream, small_list_kernel<L, FWD>, comp, xfer, dt, o,
+                                 batch, static_cast<const uint32_t *>(wide_count),
+                                 static_cast<const uint32_t *>(wide_list), pairs);
 }
 
 template <int L, bool REPLAY>

@@ -3,6 +3,7 @@
 // (dp_fused.cu). The design notes are at the top of dp_small.cu.
 #pragma once
 
+#include "chain.cuh"
 #include "gen_device.cuh"
 
 namespace dc {
@@ -46,20 +47,26 @@ __host__ __device__ constexpr int stage_stride(int L)
     return (L % 2 == 1) ? L : (L % 4 == 2 ? L : L + 2);
 }
 
-// Shared memory of a warp of the 32-bit pass. Its table, per lane (32-bit words,
-// lane-interleaved): word 0 unused, the kept cells of columns 2..kLast at
-// 1 + cell2 (a traceback step loads one word below a column's first cell, which
-// stays inside the table), then U[0..L]; column 1 is not stored, being U shifted
-// by a constant. The tile's staging (comp and xfer rows at a padded stride, then
-// dt) either shares the table's area (kSharedBytes) or lies beside it
-// (kSplitBytes), so that the next tile can land while this one is solved.
-template <int L>
-struct Tab32 {
-    static constexpr int kLast = kKeepCols < L - 1 ? kKeepCols : L - 1;  // last stored column
+// A warp's table, per lane (values of type T, lane-interleaved): value 0 unused, the kept
+// cells of columns 2..kLast at 1 + cell2 (a traceback step loads one value below a
+// column's first cell, which stays inside the table), then U[0..L]; column 1 is not
+// stored, being U shifted by a constant. KEEP: the last column kept, if there are as many.
+template <int L, typename T, int KEEP>
+struct Table {
+    static constexpr int kLast = KEEP < L - 1 ? KEEP : L - 1;  // last stored column
     static constexpr int kCells = kLast >= 2 ? cell2(L, L, kLast) + 1 : 0;
     static constexpr int kOffU = 1 + kCells;
     static constexpr int kWords = kOffU + L + 1;
-    static constexpr int kBytes = 32 * kWords * 4;
+    static constexpr int kBytes = 32 * kWords * int(sizeof(T));
+};
+
+// Shared memory of a warp of the 32-bit pass: its table, and the tile's staging (comp and
+// xfer rows at a padded stride, then dt), which either shares the table's area
+// (kSharedBytes) or lies beside it (kSplitBytes), so that the next tile can land while
+// this one is solved.
+template <int L>
+struct Tab32 : Table<L, int32_t, kKeepCols> {
+    using Table<L, int32_t, kKeepCols>::kBytes;
     static constexpr int kStride = stage_stride(L);               // staging row stride (int64)
     static constexpr int kRowsBytes = 2 * 32 * kStride * 8;        // comp + xfer rows of a tile
     static constexpr int kSharedBytes = kRowsBytes > kBytes ? kRowsBytes : kBytes;
@@ -91,28 +98,38 @@ __device__ __forceinline__ T lds(const T *lane_base, int v) { return lane_base[3
 // column, and the previous column C in the max operand. Each candidate differs from Eq. 8/9's by a
 // constant of its row, so every argmin is the same. All values and sums lie in
 // [-2^31, 2^31) when the capped bound L*dt + sum(comp) + sum(capped xfer) is
-// below 2^31; other instances take the work-list pass. The table stores A (forward)
+// below 2^31; other instances take the work-list pass, which has the same form in 64
+// bits (T). The table stores A (forward)
 // or F (backward) for columns 1..kKeepCols and the row U (Q forward, BC - dt
 // backward); V (G forward, NGT backward) stays in registers.
+
+__device__ __forceinline__ int32_t add_max(int32_t a, int32_t b, int32_t c) { return __viaddmax_s32(a, b, c); }
+__device__ __forceinline__ int64_t add_max(int64_t a, int64_t b, int64_t c) { return dmax(a + b, c); }
+__device__ __forceinline__ int32_t add_min(int32_t a, int32_t b, int32_t c) { return __viaddmin_s32(a, b, c); }
+__device__ __forceinline__ int64_t add_min(int64_t a, int64_t b, int64_t c) { return dmin(a + b, c); }
+__device__ __forceinline__ int32_t min3(int32_t a, int32_t b, int32_t c) { return __vimin3_s32(a, b, c); }
+__device__ __forceinline__ int64_t min3(int64_t a, int64_t b, int64_t c) { return dmin(dmin(a, b), c); }
+template <typename T>
+constexpr T kLeast = sizeof(T) == 4 ? T(INT32_MIN) : T(INT64_MIN);
 
 // Minimum of c[0..cnt-1] (cnt a compile-time constant after unrolling): two
 // chains of 3-input mins, so that each row has two independent dependency chains
 // and the rows of a column interleave.
-template <int N>
-__device__ __forceinline__ int32_t min_fold3(const int32_t (&c)[N], int cnt)
+template <int N, typename T>
+__device__ __forceinline__ T min_fold3(const T (&c)[N], int cnt)
 {
     if (cnt == 1) return c[0];
-    if (cnt == 2) return min(c[0], c[1]);
-    int32_t a = c[0], b = c[1];
+    if (cnt == 2) return dmin(c[0], c[1]);
+    T a = c[0], b = c[1];
     int j = 2;
 #pragma unroll
     for (; j + 3 < cnt; j += 4) {
-        a = __vimin3_s32(a, c[j], c[j + 1]);
-        b = __vimin3_s32(b, c[j + 2], c[j + 3]);
+        a = min3(a, c[j], c[j + 1]);
+        b = min3(b, c[j + 2], c[j + 3]);
     }
-    if (j + 1 < cnt) return __vimin3_s32(__vimin3_s32(a, b, c[j]), c[j + 1], cnt > j + 2 ? c[j + 2] : c[j + 1]);
-    if (j < cnt) return __vimin3_s32(a, b, c[j]);
-    return min(a, b);
+    if (j + 1 < cnt) return min3(min3(a, b, c[j]), c[j + 1], cnt > j + 2 ? c[j + 2] : c[j + 1]);
+    if (j < cnt) return min3(a, b, c[j]);
+    return dmin(a, b);
 }
 
 // The fill also keeps a cell's value of the column before when that is lower (fewer
@@ -129,40 +146,39 @@ __device__ __forceinline__ int32_t min_fold3(const int32_t (&c)[N], int cnt)
 // constant, which folds every choice below away; the fused pass solves both
 // directions with one copy of this code. Every lane of the warp calls it; `run` is
 // false for lanes without a 32-bit instance, whose values are not used.
-template <int L>
-__device__ __forceinline__ void fill_e(const bool fwd, const bool run, const int32_t (&U)[L + 1],
-                                       const int32_t (&V)[L + 1], int32_t dt, int32_t fcL,
-                                       int32_t *lw, int32_t &bestV, int &best_s)
+template <int L, int KEEP, typename T>
+__device__ __forceinline__ void fill_e(const bool fwd, const bool run, const T (&U)[L + 1],
+                                       const T (&V)[L + 1], T dt, T fcL, T *lw, T &bestV, int &best_s)
 {
-    using K = Tab32<L>;
+    using K = Table<L, T, KEEP>;
     // forward: U = Q, V = G, col = A; backward: U = BC - dt, V = NGT, col = F
-    const int32_t dt2 = 2 * dt;
-    const int32_t c1 = fwd ? fcL - dt : dt;  // column 1 is U + c1
-    const int32_t sdt = fwd ? -dt : dt;      // column n is its minimum + sdt
-    const int32_t sold = fwd ? -dt : 0;      // column n - 1 in column n's terms, less column n - 1
-    const int32_t slim = fwd ? 0 : -dt;      // a cell of column n helps only below col[L] + slim
-    const int32_t uL = fwd ? U[L] : 0;       // row L's minimum less uL: B[L][n] or F[L][n] - dt
-    const int32_t step = fwd ? dt : 0, base = fwd ? 0 : dt2;
-    const int32_t tail = L > 1 ? U[L] + V[L - 1] : 0;  // no later minimum of row L is below it
-    int32_t col[L + 1];
+    const T dt2 = 2 * dt;
+    const T c1 = fwd ? fcL - dt : dt;  // column 1 is U + c1
+    const T sdt = fwd ? -dt : dt;      // column n is its minimum + sdt
+    const T sold = fwd ? -dt : 0;      // column n - 1 in column n's terms, less column n - 1
+    const T slim = fwd ? 0 : -dt;      // a cell of column n helps only below col[L] + slim
+    const T uL = fwd ? U[L] : 0;       // row L's minimum less uL: B[L][n] or F[L][n] - dt
+    const T step = fwd ? dt : 0, base = fwd ? 0 : dt2;
+    const T tail = L > 1 ? U[L] + V[L - 1] : 0;  // no later minimum of row L is below it
+    T col[L + 1];
 #pragma unroll
     for (int m = 1; m <= L; ++m) col[m] = U[m] + c1;
     bestV = fwd ? fcL + dt : U[L] + dt2;
     best_s = 1;
 #pragma unroll
     for (int n = 2; n <= L; ++n) {
-        int32_t lim = 0;
+        T lim = 0;
         bool more = false;
 #pragma unroll
         for (int m = L; m >= n; --m) {  // descending: column n overwrites column n-1 in place
             const int cnt = m - n + 1;  // k = n-1 .. m-1
-            const int32_t u = U[m];
-            int32_t c[L];
+            const T u = U[m];
+            T c[L];
 #pragma unroll
-            for (int j = 0; j < cnt; ++j) c[j] = __viaddmax_s32(u, V[n - 1 + j], col[n - 1 + j]);
-            const int32_t b = min_fold3<L>(c, cnt);
-            const int32_t old = col[m] + sold;
-            col[m] = __viaddmin_s32(b, sdt, old);
+            for (int j = 0; j < cnt; ++j) c[j] = add_max(u, V[n - 1 + j], col[n - 1 + j]);
+            const T b = min_fold3<L>(c, cnt);
+            const T old = col[m] + sold;
+            col[m] = add_min(b, sdt, old);
             if (m == L) {
                 if (col[m] < old) {  // strict: the lowest n wins ties
                     bestV = b - uL + n * step + base;  // X[L][n] - P[L] or X[L][n] - S[L]
@@ -170,7 +186,7 @@ __device__ __forceinline__ void fill_e(const bool fwd, const bool run, const int
                 }
                 lim = col[m] + slim;
             } else {
-                more |= col[m] < min(old, lim);
+                more |= col[m] < dmin(old, lim);
             }
             if (n <= K::kLast) lw[32 * (1 + cell2(L, m, n))] = col[m];
         }
@@ -180,8 +196,8 @@ __device__ __forceinline__ void fill_e(const bool fwd, const bool run, const int
 
 // Number of v[0..N-1] (non-increasing) above t: N a power of two, halved by selects.
 // next: the first value that is not above, if any.
-template <int N>
-__device__ __forceinline__ int count_above(const int32_t (&v)[N], int32_t t, int32_t &next)
+template <int N, typename T>
+__device__ __forceinline__ int count_above(const T (&v)[N], T t, T &next)
 {
     if constexpr (N == 1) {
         if (v[0] <= t) next = v[0];
@@ -189,7 +205,7 @@ __device__ __forceinline__ int count_above(const int32_t (&v)[N], int32_t t, int
     } else {
         constexpr int H = N / 2;
         const bool up = v[H - 1] > t;  // the first half lies above t
-        int32_t w[H];
+        T w[H];
 #pragma unroll
         for (int j = 0; j < H; ++j) w[j] = up ? v[H + j] : v[j];
         if (!up) next = v[H - 1];
@@ -205,19 +221,19 @@ __host__ __device__ constexpr int ceil_log2(int x) { return x <= 1 ? 0 : 1 + cei
 // transfer sum. Every lane of the warp calls it; lanes with `run` false write nothing
 // but their slice. REPLAY: o.replay takes f_m of the decision. Returns false (having
 // written nothing) when the traceback needs a column the pass did not keep.
-template <int L, bool REPLAY>
-__device__ __forceinline__ bool solve_uv(const bool fwd, const bool run, const int32_t (&U)[L + 1],
-                                         const int32_t (&V)[L + 1], int32_t dt, uint64_t xraw,
-                                         int32_t *lw, int64_t i, const SolveOut &o)
+template <int L, bool REPLAY, int KEEP, typename T>
+__device__ __forceinline__ bool solve_uv(const bool fwd, const bool run, const T (&U)[L + 1],
+                                         const T (&V)[L + 1], T dt, uint64_t xraw, T *lw, int64_t i,
+                                         const SolveOut &o)
 {
-    using K = Tab32<L>;
+    using K = Table<L, T, KEEP>;
     constexpr int W = (L - 1 + 31) / 32;
-    const int32_t fcL = V[0];  // forward: FC[L]
+    const T fcL = V[0];  // forward: FC[L]
 #pragma unroll
     for (int m = 0; m <= L; ++m) lw[32 * (K::kOffU + m)] = U[m];  // the traceback reads U[m]
-    int32_t bestV;
+    T bestV;
     int s;
-    fill_e<L>(fwd, run, U, V, dt, fcL, lw, bestV, s);
+    fill_e<L, KEEP>(fwd, run, U, V, dt, fcL, lw, bestV, s);
     if (!run) return true;
     if (s - 1 > K::kLast && s - 1 >= 2) return false;
 
@@ -225,66 +241,69 @@ __device__ __forceinline__ bool solve_uv(const bool fwd, const bool run, const i
     // at (k, n-1). That k is the first with U[m] + V[k] <= the cell (chain.cuh), found
     // by a binary search over V in registers.
     constexpr int kPad = 1 << ceil_log2(L > 2 ? L - 1 : 1);
-    int32_t vs[kPad];
+    T vs[kPad];
 #pragma unroll
-    for (int j = 0; j < kPad; ++j) vs[j] = j + 1 < L ? V[j + 1] : INT32_MIN;
+    for (int j = 0; j < kPad; ++j) vs[j] = j + 1 < L ? V[j + 1] : kLeast<T>;
     uint32_t word = 0;
     int err = 0;
     int m = L, n = s;
-    int32_t target = fwd ? bestV - s * dt + U[L] : bestV - 2 * dt;  // B[L][s] + Q[L] or F[L][s] - dt
-    const int32_t off1 = fwd ? fcL - dt : dt;  // column 1 is U + off1 (not stored)
+    T target = fwd ? bestV - s * dt + U[L] : bestV - 2 * dt;  // B[L][s] + Q[L] or F[L][s] - dt
+    const T off1 = fwd ? fcL - dt : dt;  // column 1 is U + off1 (not stored)
     // f_m of the decision from its own segments, in the cells' shifted terms: the
     // largest over its segments of U[end] + V[start] and the shift since, then the
     // first segment's U
-    int32_t span = INT32_MIN, later = 0;
+    T span = kLeast<T>, later = 0;
     while (n > 1) {
         const int nm1 = n - 1;
-        const int32_t u = lds(lw, K::kOffU + m);
-        int32_t vk = INT32_MIN;
+        const T u = lds(lw, K::kOffU + m);
+        T vk = kLeast<T>;
         const int k = 1 + count_above<kPad>(vs, target - u, vk);
         // cell (k, n-1) of a kept column is word base + k
         const int base = nm1 == 1 ? K::kOffU : 1 + cell2(L, 0, nm1);
         const int at = k < m ? k : m;  // inside the column
-        const int32_t fk = lds(lw, base + at) + (nm1 == 1 ? off1 : 0);
+        const T fk = lds(lw, base + at) + (nm1 == 1 ? off1 : 0);
         if (k < nm1 || k >= m || fk > target) {  // cannot happen: the fill took this minimum
             err = 1;
             break;
         }
         word |= 1u << ((k - 1) & 31);
         if constexpr (REPLAY) {
-            span = max(span, u + vk + later);
+            span = dmax(span, u + vk + later);
             later += fwd ? -dt : dt;
         }
         target = fwd ? fk + dt : fk - dt;  // the cell (k, n-1): B + Q[k] = A + dt, or F - dt
         m = k;
         n = nm1;
     }
-    o.makespan[i] = int64_t(uint64_t(uint32_t(bestV)) + xraw);
+    auto absolute = [&](T v) {  // both are at least 0
+        return int64_t((sizeof(T) == 4 ? uint64_t(uint32_t(v)) : uint64_t(v)) + xraw);
+    };
+    o.makespan[i] = absolute(bestV);
     if (o.nseg) o.nseg[i] = s;
     if (o.status) o.status[i] = err ? DC_ERR_INTERNAL : DC_OK;
     if constexpr (REPLAY) {
-        int32_t f = bestV;  // s = 1: the one segment, dt + FC[L] or dt + BC[L]
+        T f = bestV;  // s = 1: the one segment, dt + FC[L] or dt + BC[L]
         if (s > 1) {
-            span = max(span, lds(lw, K::kOffU + m) + off1 + later - (fwd ? -dt : dt));
+            span = dmax(span, lds(lw, K::kOffU + m) + off1 + later - (fwd ? -dt : dt));
             f = fwd ? span - U[L] + s * dt : span + 2 * dt;
         }
-        o.replay[i] = err ? -int64_t(DC_ERR_INTERNAL) : int64_t(uint64_t(uint32_t(f)) + xraw);
+        if (sizeof(T) == 4 || o.replay) o.replay[i] = err ? -int64_t(DC_ERR_INTERNAL) : absolute(f);
     }
     if (W > 0) o.bits[i * W] = word;
     return true;
 }
 
-// U and V from 64-bit prefix sums (the caller has checked the 32-bit range).
-template <int L, bool FWD>
+// U and V from 64-bit prefix sums (the caller has checked T's range).
+template <int L, bool FWD, typename T>
 __device__ __forceinline__ void shifted_uv(const uint64_t (&Pc)[L + 1], const uint64_t (&Px)[L + 1],
-                                           int64_t dti, int32_t (&U)[L + 1], int32_t (&V)[L + 1])
+                                           int64_t dti, T (&U)[L + 1], T (&V)[L + 1])
 {
-    const int32_t dt = int32_t(dti);
-    const int32_t fcL = int32_t(Pc[L]);
+    const T dt = T(dti);
+    const T fcL = T(Pc[L]);
 #pragma unroll
     for (int m = 0; m <= L; ++m) {
-        U[m] = FWD ? dt + int32_t(Px[m]) : int32_t(Pc[m]) - dt;
-        V[m] = FWD ? fcL - int32_t(Pc[m]) : -int32_t(Px[m]);
+        U[m] = FWD ? dt + T(Px[m]) : T(Pc[m]) - dt;
+        V[m] = FWD ? fcL - T(Pc[m]) : -T(Px[m]);
     }
 }
 
@@ -458,6 +477,104 @@ __device__ __forceinline__ void row_uv(const int64_t *rc, const int64_t *rx, int
         st = DC_ERR_RANGE;
     wide = uint64_t(L) * uint64_t(dti) + Pc[L] + Px[L] > kShiftedLimit;  // capped bound
     shifted_uv<L, FWD>(Pc, Px, dti, U, V);
+}
+
+// ---------------------------------------------------------------------------
+// The pass over a first pass's list, every value in 64 bits and every column kept:
+// instances with values past the shifted form's range or optima deeper than kKeepCols.
+// A short list takes a warp per instance (chain.cuh), whose lanes share the work: it ends
+// soonest. A longer one takes a lane per instance with the fill above, several times
+// faster on a full GPU, up to the depth at which the unrolled 64-bit fill no longer fits
+// the instruction cache; beyond it warps at a higher occupancy. DRAWN: the rows are drawn
+// again, one layer after the other in the lane form.
+// Measured, one direction of 1,000,000 log-uniform instances that all lie past 2^31, one
+// warp per instance on 4 warps per SM (alone) / an unrolled fill of every column, a lane
+// per instance / these rules: L = 4 3,430 us / 159 / 136, L = 8 5,150 / 424 / 340, L = 12
+// 4,040 / 689 / 437, L = 15 4,150 / 1,001 / 986, L = 16 3,700 / 1,220 / 870-960; generated
+// and solved at L = 12 with costs in nanoseconds, both directions, 3,270 / 2,434 / 690.
+// Where the lines lie, 400,000 instances of which a part is listed, by warp against by lane:
+// 608 of L = 12 25 us against 26, of L = 8 17 against 17-23; 1,500 27 against 27 and 20
+// against 18-23; 3,000 30 against 28 and 22 against 19-24; of L = 6 14.2 against 13.6, 16.8
+// against 13.6 and 19 against 14.3; at L = 2 and 4 never faster.
+// All of L = 16: lanes 1,300 us, warps 870. All of L = 15: 990 against 900-1,050, but 580
+// against 880-1,030 at L = 14. Drawn lists, 1,000,000 plain log-uniform instances (some
+// thousand listed): L = 12 210 us by warp and 218 by lane, L = 15 261 and 277.
+// Four single-warp CTAs per SM hold up the short calls least (L = 8, nothing listed: 15.2
+// us against 16.4 with sixteen).
+template <int L, bool DRAWN>
+struct List64 {
+    static constexpr bool kLanes = L <= (DRAWN ? 12 : 15);  // whether a list may take a lane per instance
+    // lists up to here go by warp
+    static constexpr int kByWarp = L <= 4 ? 0 : DRAWN ? 4864 : L <= 6 ? 1200 : 2432;
+    static constexpr int kWarps = kLanes ? 1 : 4;               // warps per CTA
+    static constexpr int kCtas = !kLanes ? 8 : DRAWN ? 16 : 4;  // CTAs per SM, at most
+    static constexpr int kChainBytes = (chain_pair_bytes(64) + int(tri_cells(L)) * 8 + 15) / 16 * 16;
+    static constexpr int kLaneBytes = kLanes ? Table<L, int64_t, L>::kBytes : 0;
+    static constexpr int kSlice = kLaneBytes > kChainBytes ? kLaneBytes : kChainBytes;  // a warp's
+    static constexpr int kBytes = kWarps * kSlice;
+};
+
+// Walks a list: by_warp(kb, i, kept) solves instance i with the warp, kb: byte of the warp's
+// slice of shared memory; by_lane(active, i), called by every lane of the warp, an instance
+// per lane where `active`.
+template <int L, bool DRAWN, typename ByWarp, typename ByLane>
+__device__ __forceinline__ void list_pass(int64_t batch, int64_t count, const uint32_t *list,
+                                          ByWarp by_warp, ByLane by_lane)
+{
+    using K = List64<L, DRAWN>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, kb = warp * K::kSlice;
+    if (K::kByWarp > 0 && (!K::kLanes || count <= K::kByWarp)) {
+        if (lane == 0) zero_row(kb, 64);
+        const KeptValues kept{&sh<int64_t>(kb + chain_pair_bytes(64)), L};
+        for (int64_t j = int64_t(blockIdx.x) * K::kWarps + warp; j < count;
+             j += int64_t(gridDim.x) * K::kWarps) {
+            const int64_t i = int64_t(list[j]);
+            if (!DC_CHECK(i < batch)) continue;
+            by_warp(kb, i, kept);
+            __syncwarp();  // shared memory is read
+        }
+        return;
+    }
+    if constexpr (K::kLanes) {
+        for (int64_t j0 = int64_t(blockIdx.x) * 32; j0 < count; j0 += int64_t(gridDim.x) * 32) {
+            const bool listed = j0 + lane < count;
+            const int64_t i = listed ? int64_t(list[j0 + lane]) : 0;
+            by_lane(listed && DC_CHECK(i < batch), i);
+        }
+    }
+}
+
+// Host: launches a list kernel. The list's length is known on the device only; its CTAs
+// are launched early and the surplus exits at once.
+template <int L, bool DRAWN, typename... Params, typename... Args>
+cudaError_t launch_list(DeviceCache &resident, int64_t batch, cudaStream_t stream,
+                        void (*kernel)(Params...), const Args &...args)
+{
+    using K = List64<L, DRAWN>;
+    int n = 0;
+    const cudaError_t e = resident.get(n, [&](int &v) {
+        const cudaError_t q =
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kernel, 32 * K::kWarps, K::kBytes);
+        if (v > K::kCtas) v = K::kCtas;
+        return q;
+    });
+    if (e != cudaSuccess) return e;
+    const int64_t most = int64_t(sm_count()) * n, need = (batch + K::kWarps - 1) / K::kWarps;
+    return launch_early(kernel, need < most ? need : most, 32 * K::kWarps, K::kBytes, stream, args...);
+}
+
+// One instance per lane: rows(col, comp, xfer) gives the costs of the lane's instance i, of
+// latency dti, in layer order. Every lane of the warp calls it.
+template <int L, bool FWD, typename Rows>
+__device__ __forceinline__ void list_solve_lane(bool active, int64_t i, int64_t dti, Rows rows,
+                                                const SolveOut &o)
+{
+    uint64_t Pc[L + 1] = {}, Px[L + 1] = {}, xraw = 0;
+    bool neg = false, big = false;  // checked by the first pass
+    if (active) row_prefix<L, FWD>(rows, Pc, Px, xraw, neg, big);
+    int64_t U[L + 1], V[L + 1];
+    shifted_uv<L, FWD>(Pc, Px, dti, U, V);
+    solve_uv<L, true, L>(FWD, active, U, V, dti, xraw, &sh<int64_t>(8 * int(threadIdx.x)), i, o);
 }
 
 }  // namespace
