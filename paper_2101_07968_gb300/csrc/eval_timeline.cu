@@ -17,8 +17,8 @@
 // replays its lane's row. Warps are persistent (one resident wave) and prefetch
 // their next tile into L2 while the current one is copied. For L <= 16 the
 // replay is unrolled at compile time and inputs are screened on their high
-// words. Longer rows take one warp per instance (eval_warp_kernel), up to 95 and large
-// batches one thread (launch_eval).
+// words. Longer rows take one warp per instance (eval_warp_kernel) or, in large batches of
+// up to 257 layers, one thread (eval_per_thread).
 #include "chain.cuh"
 
 namespace dc {
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(256)
 // (and, with a 64-bit scan per 64 rows, close to integer issue). Per direction against one
 // thread per instance, whose reads are uncoalesced (forward): 16,384 x 1,024 73 us against
 // 276, 2,048 x 1,024 14.7 against 267, 120,000 x 128 81 against 137, 1,000 x 129 9.4
-// against 18 (a call from the host).
+// against 18 (a call from the host); where threads are faster, see eval_per_thread.
 template <bool FWD>
 __global__ void __launch_bounds__(256)
     eval_warp_kernel(int64_t batch, int L, const int64_t *__restrict__ comp,
@@ -410,6 +410,26 @@ cudaError_t launch_small_eval(int64_t batch, const int64_t *comp, const int64_t 
 
 }  // namespace
 
+// Above 64 layers: whether an instance takes a thread. Many threads hide their uncoalesced
+// reads, better in rows that start all over a 128-byte line (odd L most) and not where
+// they start at the same place (L a multiple of 16); a warp's last 64 rows are partly past
+// the end. Thread against warp, forward: 20,000 x 65 12.3 us against 15.5, x 97 16.5 against
+// 16.9, x 72 19.3 against 15.6; 60,000 x 129 40 against 57, x 257 73 against 85, x 140 50
+// against 56, x 80 46 against 40; 100,000 x 100 54 against 69, x 112 93 against 69; 200,000 x
+// 161 147 against 173, x 200 237 against 213. Backward: 40,000 x 97 24.5 against 27.8, 60,000
+// x 129 68 against 57; 100,000 x 129 73 against 89, x 140 72 against 87, x 161 90 against 95;
+// 200,000 x 104 141 against 128.
+static bool eval_per_thread(bool forward, int64_t batch, int L)
+{
+    const bool odd = L % 2 == 1;
+    if (L % 16 == 0) return false;
+    if (batch < 50000)
+        return (odd || L <= 70) && batch >= (forward ? 20000 : 40000) && L <= (forward ? 129 : 100);
+    if (L < 96) return true;
+    if (forward) return L <= (odd ? 257 : 140);
+    return L <= (batch >= 80000 ? 140 : 104) && batch <= 150000;
+}
+
 cudaError_t launch_eval(bool forward, int64_t batch, int L, const int64_t *comp,
                         const int64_t *xfer, const int64_t *dt, const uint32_t *bits,
                         int64_t *makespan, cudaStream_t stream)
@@ -469,10 +489,7 @@ cudaError_t launch_eval(bool forward, int64_t batch, int L, const int64_t *comp,
                 batch, L, comp, xfer, dt, bits, makespan, pairs);
         return cudaGetLastError();
     }
-    // Below 96 rows half of a warp's second 64 are past the end, and many threads hide their
-    // uncoalesced reads: 240,000 x 65 68 us forward and 110 backward against 144, 200,000 x 88
-    // 109 and 123 against 127; but 20,000 x 72 19 against 16, 160,000 x 96 130 against 104.
-    if (L < 96 && batch >= 50000) {
+    if (eval_per_thread(forward, batch, L)) {
         int64_t blocks = (batch + 255) / 256;
         if (blocks > 152 * 64) blocks = 152 * 64;
         if (forward)

@@ -1,5 +1,5 @@
 """dc_eval_timeline_batch above 64 layers (one warp per instance, 64 rows at a time; one
-thread below 96 layers and on large batches) against the oracle's event replay: odd and even
+thread on large batches of up to 257) against the oracle's event replay: odd and even
 depths around the chunks, rows off a 16-byte boundary, no break, every break, ties, values
 beyond 32 bits and faulty inputs."""
 import os
@@ -54,3 +54,24 @@ def test_replays_of_any_decision(dc, L, copies):
             got = dc.eval_timeline(d, dev(comp), dev(xfer), dev(dt), dev(bits.view(np.int32)))
             exp = oracle.replay_batch(d, comp, xfer, dt, bits, nthreads=os.cpu_count() or 1)
             assert (got.cpu().numpy().reshape(copies, B) == exp[None]).all(), (L, d, offset)
+
+
+@pytest.mark.parametrize("batch", [20_000, 40_000, 50_000, 80_000, 150_001])
+@pytest.mark.parametrize("L", [65, 70, 72, 97, 100, 101, 112, 129, 131, 140, 142, 257, 259])
+def test_where_a_thread_takes_an_instance(dc, L, batch):
+    """Batches and depths on both sides of every line between a warp and a thread per
+    instance."""
+    import torch
+    B = 125
+    comp, xfer, dt = wl.skewed_instances(L, B, L)
+    comp[:30] <<= 20
+    xfer[50, L - 1], dt[51] = -1, 1 << 52
+    bits = np.concatenate([wl.random_decisions(L, 60, L, density=0.1), wl.random_decisions(L, 65, L, density=0.9)])
+    t = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (comp, xfer, dt, bits.view(np.int32))]
+    copies = -(-batch // B)
+    for n in (batch - 1, batch):
+        dev = [a.repeat((copies,) + (1,) * (a.dim() - 1))[:n].contiguous() for a in t]
+        for d in (0, 1):
+            exp = oracle.replay_batch(d, comp, xfer, dt, bits, nthreads=os.cpu_count() or 1)
+            got = dc.eval_timeline(d, *dev).cpu().numpy()
+            assert np.array_equal(got, np.tile(exp, copies)[:n]), (L, n, d)
