@@ -641,15 +641,21 @@ cudaError_t launch_greedy_cta(const GreedyArgs &g, int nt, cudaStream_t stream)
 }
 
 // One instance per thread where a warp's lanes are better used on 32 instances than on
-// one short row. Forward: up to L = 22 (100,000 x 20: 38 us against 44 per warp, 500,000
-// x 24 equal, 100,000 x 32 72 against 45), and above the warp kernel's rows up to 128
-// on large batches (100,000 x 100: 139 against 152 per CTA; but 10,000 x 100: 50 against
-// 39). Backward, quadratic in L per thread: up to L = 8, and up to 12 on large batches
-// (500,000 x 12: 208 us against 284; 100,000 x 12 76 against 73).
+// one short row. Forward: up to L = 22 (100,000 x 20: 38 us against 44 per warp; but 100,000
+// x 24 38 against 32, x 32 61 against 32), at odd L, whose rows start all over a line, up to
+// 25 on large batches (100,000 x 23 30.5 against 32.4, 200,000 x 25 58.0 against 58.8, but
+// 60,000 x 25 25 against 22, 200,000 x 27 65 against 60), and above the warp kernel's rows up
+// to 128 on large batches (100,000 x 100: 139 against 152 per CTA; but 10,000 x 100: 50
+// against 39). Backward, quadratic in L per thread: up to L = 8, and up to 12 on large
+// batches (500,000 x 12: 208 us against 284; 100,000 x 12 76 against 73). The warp kernel is
+// slower on values past 32 bits, which the host cannot see: 200,000 x 28 forward 90 us, 70
+// per thread (60 in 32 bits); 200,000 x 13 backward 159, 120 (117 in 32 bits).
 template <bool FWD>
 bool per_thread(int64_t batch, int L)
 {
-    if (FWD) return L <= 22 || (L > 64 && L <= 128 && batch >= 50000);
+    if (FWD)
+        return L <= 22 || (L <= 25 && L % 2 == 1 && batch >= 100000) ||
+               (L > 64 && L <= 128 && batch >= 50000);
     return L <= 8 || (L <= 12 && batch >= 50000);
 }
 

@@ -1,6 +1,7 @@
-"""The CTA-per-instance greedy schedulers at depths around their warp, row-pair and
-search boundaries, in 32 and in 64 bits, against the oracle; above L = 600, where the
-oracle's backward enumeration is too slow, against the same rule by bisection."""
+"""The greedy schedulers of one instance per warp (L <= 64) and per CTA at depths around
+their warp, row-pair and search boundaries, in 32 and in 64 bits, and on both sides of the
+lines to the kernel of one instance per thread, against the oracle; above L = 600, where
+the oracle's backward enumeration is too slow, against the same rule by bisection."""
 import bisect
 import os
 
@@ -42,7 +43,7 @@ def _instances(L, B, wide):
 
 
 @pytest.mark.parametrize("wide", [False, True])
-@pytest.mark.parametrize("L", [17, 18, 33, 34, 63, 64, 65, 66, 127, 128, 129, 257])
+@pytest.mark.parametrize("L", list(range(9, 19)) + [33, 34, 63, 64, 65, 66, 127, 128, 129, 257])
 def test_depths(dc, L, wide):
     comp, xfer, dt = _instances(L, 21, wide)
     for d in (0, 1):
@@ -119,3 +120,24 @@ def test_sums_at_two_to_the_31(dc, L, total):
         mk, bits = _run(dc, d, comp, xfer, dt)
         exp = oracle.greedy_batch(d, comp, xfer, dt, nthreads=os.cpu_count() or 1)
         assert np.array_equal(mk, exp["makespan"]) and np.array_equal(bits, exp["bits"]), (L, d)
+
+
+# 5,001: four warps to a CTA, several instances to a warp; from 50,000 and 100,000 on some
+# depths take a thread per instance
+@pytest.mark.parametrize("batch", [5_001, 49_999, 50_000, 99_999, 100_000])
+@pytest.mark.parametrize("L", [8, 9, 12, 13, 16, 22, 23, 24, 25, 27, 54, 64, 65, 128, 129])
+def test_large_batches(dc, L, batch):
+    import torch
+    comp, xfer, dt = _instances(L, 41, False)
+    comp[20:31] <<= 22  # mixed widths within a warp's and a CTA's instances
+    xfer[25:36] <<= 20
+    comp[37, L - 1], xfer[38, 0], dt[39] = -1, 1 << 52, -4  # faults between good ones
+    copies = -(-batch // len(dt))
+    t = [torch.from_numpy(np.ascontiguousarray(a)).cuda().repeat((copies,) + (1,) * (a.ndim - 1))[:batch]
+         .contiguous() for a in (comp, xfer, dt)]
+    for d in (0, 1):
+        out = dc.greedy(d, *t)
+        exp = oracle.greedy_batch(d, comp, xfer, dt, nthreads=os.cpu_count() or 1)
+        assert np.array_equal(out["makespan"].cpu().numpy(), np.tile(exp["makespan"], copies)[:batch]), (L, d)
+        assert np.array_equal(out["bits"].cpu().numpy().view(np.uint32),
+                              np.tile(exp["bits"], (copies, 1))[:batch]), (L, d)
