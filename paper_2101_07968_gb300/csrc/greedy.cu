@@ -330,7 +330,15 @@ __device__ __forceinline__ T greedy_chain(const T *A, const T *B, int L, int P, 
     return link;
 }
 
-// Algorithm 2 by the CTA; the result in thread 0.
+// The chain again, for its decision. Not inlined: a second copy beside the loop over the
+// chains takes registers from it (20,000 x 128 91 us with it inlined, 73 so).
+template <typename T>
+__device__ __noinline__ void mark_chain(const T *A, const T *B, int L, int P, T dt, int p, uint32_t *word)
+{
+    greedy_chain(A, B, L, P, dt, p, [&](int q) { set_bit(word, q); });
+}
+
+// Algorithm 2 by the CTA, two warps or more; the result in thread 0.
 template <typename T>
 __device__ T greedy_backward_cta(const T *A, const T *B, int L, T dt, uint32_t *word, longlong2 *best_of)
 {
@@ -339,14 +347,11 @@ __device__ T greedy_backward_cta(const T *A, const T *B, int L, T dt, uint32_t *
     while (2 * P < L) P *= 2;
     T best = T(0);
     int at = 0;  // ties keep the longest first push (the lowest second position)
-    uint64_t mask = 0;
     for (int p = 1 + tid; p < L; p += int(blockDim.x)) {
-        uint64_t breaks = 0;
-        const T t = greedy_chain(A, B, L, P, dt, p, [&](int q) { breaks |= uint64_t(1) << ((q - 1) & 63); });
+        const T t = greedy_chain(A, B, L, P, dt, p, [](int) {});
         if (at == 0 || t <= best) {
             best = t;
             at = p;
-            mask = breaks;
         }
     }
     int64_t key = at ? int64_t(best) : INT64_MAX;
@@ -360,25 +365,16 @@ __device__ T greedy_backward_cta(const T *A, const T *B, int L, T dt, uint32_t *
             from = f;
         }
     }
-    if (NW > 1) {
-        if (lane == 0) best_of[warp] = make_longlong2(key, from);
-        __syncthreads();
-        for (int w = 0; w < NW; ++w) {
-            const longlong2 o = best_of[w];
-            if (o.x < key || (o.x == key && int(o.y) > from)) {
-                key = o.x;
-                from = int(o.y);
-            }
+    if (lane == 0) best_of[warp] = make_longlong2(key, from);
+    __syncthreads();
+    for (int w = 0; w < NW; ++w) {
+        const longlong2 o = best_of[w];
+        if (o.x < key || (o.x == key && int(o.y) > from)) {
+            key = o.x;
+            from = int(o.y);
         }
     }
-    if (L <= 64) {  // one warp or two: the chain's own breaks
-        if (at == from) {
-            word[0] = uint32_t(mask);
-            if (L > 33) word[1] = uint32_t(mask >> 32);
-        }
-    } else if (tid == 0) {
-        greedy_chain(A, B, L, P, dt, from, [&](int q) { set_bit(word, q); });
-    }
+    if (tid == 0) mark_chain(A, B, L, P, dt, from, word);
     __syncthreads();
     return T(key);
 }
@@ -386,7 +382,7 @@ __device__ T greedy_backward_cta(const T *A, const T *B, int L, T dt, uint32_t *
 template <bool FWD, typename T, int NJ>
 __device__ void greedy_solve(unsigned char *smem, uint32_t *word, longlong2 *best_of, int64_t i,
                              const GreedyArgs &g, T dt, const uint64_t (&a)[NJ][2],
-                             const uint64_t (&b)[NJ][2], uint64_t aL, uint64_t bL)
+                             const uint64_t (&b)[NJ][2])
 {
     const int L = g.L, tid = threadIdx.x, NT = blockDim.x, W = words_for(L);
     T *A = reinterpret_cast<T *>(smem), *B = reinterpret_cast<T *>(smem + greedy_row_bytes(L));
@@ -405,14 +401,12 @@ __device__ void greedy_solve(unsigned char *smem, uint32_t *word, longlong2 *bes
         B[0] = T(0);
     }
     __syncthreads();
-    T t = T(aL) + T(bL) + dt;  // L = 1: one segment
-    if (L > 1) {
-        if (!FWD)
-            t = greedy_backward_cta(A, B, L, dt, word, best_of);
-        else if (tid < 32)
-            t = greedy_forward_warp(A, B, L, dt, word);
-        if (FWD) __syncwarp();
-    }
+    T t = T(0);
+    if (!FWD)
+        t = greedy_backward_cta(A, B, L, dt, word, best_of);
+    else if (tid < 32)
+        t = greedy_forward_warp(A, B, L, dt, word);
+    if (FWD) __syncwarp();
     if (tid < 32) {
         if (tid == 0) g.makespan[i] = int64_t(t);
         for (int w = tid; w < W; w += 32) g.bits[i * W + w] = word[w];
@@ -564,17 +558,15 @@ __global__ void __launch_bounds__(256, 5) greedy_warp_kernel(GreedyArgs g)
                 sh<Two>(kb + D + 2 * lane * S) = P2::make(b[0][0], b[0][1]);
                 __syncwarp();
                 uint32_t mine = 0u;
-                T t = aL + bL + T(dt);  // L = 1: one segment
-                if (L > 1) {
-                    if (FWD) {
-                        t = greedy_forward_rows<T>(kb, D, L, T(dt), a, b, aL, mine);
-                    } else {
-                        uint64_t breaks = 0;
-                        int owner = 0;
-                        t = greedy_backward_rows<T>(kb, D, L, T(dt), aL, breaks, owner);
-                        breaks = __shfl_sync(0xffffffffu, breaks, owner);
-                        mine = lane == 0 ? uint32_t(breaks) : uint32_t(breaks >> 32);
-                    }
+                T t;
+                if (FWD) {
+                    t = greedy_forward_rows<T>(kb, D, L, T(dt), a, b, aL, mine);
+                } else {
+                    uint64_t breaks = 0;
+                    int owner = 0;
+                    t = greedy_backward_rows<T>(kb, D, L, T(dt), aL, breaks, owner);
+                    breaks = __shfl_sync(0xffffffffu, breaks, owner);
+                    mine = lane == 0 ? uint32_t(breaks) : uint32_t(breaks >> 32);
                 }
                 if (lane == 0) g.makespan[i] = int64_t(t);
                 if (lane < W) g.bits[i * W + lane] = mine;
@@ -609,9 +601,9 @@ __global__ void __launch_bounds__(kChainThreads, 1) greedy_cta_kernel(GreedyArgs
             if (tid == 0) g.makespan[i] = -int64_t(st);
             for (int w = tid; w < W; w += NT) g.bits[i * W + w] = 0u;
         } else if (aL + bL + uint64_t(L + 1) * uint64_t(dt) < (uint64_t(1) << 31)) {
-            greedy_solve<FWD, int32_t, NJ>(smem, word, best_of, i, g, int32_t(dt), a, b, aL, bL);
+            greedy_solve<FWD, int32_t, NJ>(smem, word, best_of, i, g, int32_t(dt), a, b);
         } else {
-            greedy_solve<FWD, int64_t, NJ>(smem, word, best_of, i, g, dt, a, b, aL, bL);
+            greedy_solve<FWD, int64_t, NJ>(smem, word, best_of, i, g, dt, a, b);
         }
         __syncthreads();  // shared memory is read
     }
