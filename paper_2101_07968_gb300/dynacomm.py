@@ -457,9 +457,9 @@ class StepGraph:
         else:
             self.sched_b = Scheduler(B, L, device=device)  # the backward branch's workspace
             self.sched.out[BWD] = self.sched_b.out[BWD]
+            self._branch = torch.cuda.Stream(device=device)
             self.replay_out = {d: torch.empty(B, dtype=torch.int64, device=device)
                                for d in (FWD, BWD)}
-        self._branch = torch.cuda.Stream(device=device)
         # one eager step first: one-time setup (function attributes, occupancy
         # queries) happens outside the capture
         side = torch.cuda.Stream(device=device)
