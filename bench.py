@@ -814,8 +814,8 @@ def run_e2e(dc, torch, prof, sched, B, L, W, dev, args, barrier, world):
             "ms_step_min_max": [min(per_step), max(per_step)],
             "path": f"pinned host profiles -> dynacomm.HostPipeline ({pipe.chunks} "
                     f"piece{'s' if pipe.chunks != 1 else ''}, "
-                    "copies overlapped with dc_schedule_forward/backward_batch and "
-                    "dc_eval_timeline_batch) -> pinned host results",
+                    "copies overlapped with dc_schedule_replay_batch of both directions) "
+                    "-> pinned host results",
             "inputs": "fc, pt, bc, dt; gt is the pt host buffer (equal transfer costs), "
                       "copied once" if shared_xfer else "fc, pt, bc, gt, dt"}
 

@@ -302,7 +302,7 @@ const char *dc_status_string(dc_status s);
  * dc_schedule_forward_batch, dc_schedule_backward_batch or
  * dc_schedule_batch_static call made by the calling thread records `start` on
  * its stream right before it launches its first pass over the batch (the
- * dense, looped or deep-chain kernel, all of that pass's launches) and `stop`
+ * dense, looped, warp- or CTA-per-instance kernel, all of its launches) and `stop`
  * right after them, before its work-list pass; cudaEventElapsedTime(start,
  * stop) is then that pass's time on the GPU. start, stop: events created by
  * the caller on the current device, both non-NULL (DC_ERR_NULL if only one

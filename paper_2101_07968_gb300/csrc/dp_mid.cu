@@ -38,7 +38,7 @@
 //    workspace (coalesced across the warp) and the traceback re-derives each
 //    Path[m][n] as the lowest k whose candidate equals the cell. Instances whose
 //    optimum needs a deeper column, or whose values need more than 31 bits, are
-//    put on a work list that the CTA-per-instance kernel solves afterwards;
+//    put on a work list that list_warp_kernel solves afterwards (dp_group.cu);
 //  * persistent single-warp CTAs claim 32-instance tiles from an atomic ticket, so
 //    the long, uneven per-tile work balances across the GPU;
 //  * the traceback skips the candidates that cannot match: U[m] + V[k] is
@@ -79,7 +79,7 @@ inline bool use_looped(int64_t batch, int L) { return L <= kLoopedLMax && batch 
 // (column, V) pairs with column 1 in .x and V (G forward, NGT backward) in .y.
 // Checks the input; returns false when this kernel does not solve the instance
 // (an input error, whose outputs it writes, or values beyond 31 bits, which it
-// lists for the CTA-per-instance kernel).
+// lists for the second pass).
 template <bool FWD>
 __device__ __forceinline__ bool mid_prefix(int64_t batch, int64_t i, int L, const int64_t *__restrict__ comp,
                                            const int64_t *__restrict__ xfer, int64_t dti,

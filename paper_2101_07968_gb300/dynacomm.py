@@ -519,9 +519,10 @@ class HostPipeline:
     """End-to-end scheduling of profiles that live in pinned host memory.
 
     The batch is cut into `chunks` contiguous pieces. Three CUDA streams overlap
-    the host->device copy of piece c+1 with the forward DP, backward DP and
-    timeline replay of piece c (all through the C ABI on slices of the device
-    buffers), and with the device->host copy of piece c-1's results. Inputs and
+    the host->device copies of later pieces with the forward and backward DP of
+    piece c, each of which also evaluates f_m of its decisions (through the C ABI,
+    on slices of the device buffers), and the results' copies back, in two groups
+    (see run), with the last piece's inputs. Inputs and
     outputs are dicts of pinned CPU tensors: inputs fc, pt, bc, gt [batch, L] and
     dt [batch]; outputs, per direction d in (FWD, BWD), (d, "makespan"),
     (d, "bits"), (d, "nseg"), (d, "replay"). Inputs that are the same host

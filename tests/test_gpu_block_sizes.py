@@ -1,9 +1,9 @@
 """The barrier discipline checked by running the kernels with their block size
 permuted (compute-sanitizer's race check is closed on this machine).
 
-DC_BLOCK_WARPS=1|2|4|8 makes the looped kernel (17 <= L <= 256), the deep-chain
-kernel (L > 256) and the CTA-per-instance kernel of the work lists run with that
-many warps per CTA. A missing __syncwarp / __syncthreads, or an index that
+DC_BLOCK_WARPS=1|2|4|8 makes the warp-per-instance kernel (17 <= L <= 192), the
+CTA-per-instance kernel (above) and that of the work lists (L > 64) run with that
+many warps per CTA where they can. A missing __syncwarp / __syncthreads, or an index that
 assumes one block size, shows up as outputs that change with it: every output
 word must be identical for every block size, and equal to the oracle's.
 """
@@ -51,9 +51,9 @@ def _wide(seed, B, L):
 
 
 CASES = [
-    ("looped L=54", lambda: wl.skewed_instances(501, 700, 54)),
-    ("looped L=100 + list", lambda: _wide(502, 300, 100)),
-    ("looped L=200", lambda: wl.tie_heavy_instances(503, 200, 200)),
+    ("warp L=54", lambda: wl.skewed_instances(501, 700, 54)),
+    ("warp L=100 + list", lambda: _wide(502, 300, 100)),
+    ("deep L=200", lambda: wl.tie_heavy_instances(503, 200, 200)),
     ("deep L=300 + list", lambda: _wide(504, 120, 300)),
     ("deep L=600", lambda: wl.skewed_instances(505, 60, 600)),
 ]

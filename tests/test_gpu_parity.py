@@ -94,9 +94,8 @@ def test_dp_many_tiles_per_warp(dc, L):
 @pytest.mark.parametrize("L", [257, 258, 300, 333, 512, 600])
 @pytest.mark.parametrize("kind", ["tie", "uni", "skew"])
 def test_dp_deep_random_parity(dc, L, kind):
-    """The warp-per-instance deep-chain kernel (L > 256) and its work list:
-    several waves of instances, odd and even L (odd L stages rows with plain
-    loads), tie-heavy inputs for the traceback's lowest-k rule."""
+    """The CTA-per-instance kernel: odd and even L (odd L reads its rows by 8 bytes),
+    tie-heavy inputs for the traceback's lowest-k rule."""
     B = 45
     gen = {"tie": wl.tie_heavy_instances, "uni": wl.random_instances,
            "skew": wl.skewed_instances}[kind]
@@ -107,10 +106,9 @@ def test_dp_deep_random_parity(dc, L, kind):
 
 @pytest.mark.parametrize("B", [500, 1000, 2000])
 def test_dp_deep_warps_per_instance(dc, B):
-    """Batch sizes that give the deep-chain kernel 4, 2 and 1 warps per instance
-    (the rows of a column dealt to the warps strip by strip), full batches
-    bit-exact with the oracle; the xfer array starts 8 bytes past a 16-byte
-    boundary in one direction, which stages the rows with plain loads."""
+    """Batches of one to a few instances per CTA of the CTA-per-instance kernel, full
+    batches bit-exact with the oracle; the xfer array starts 8 bytes past a 16-byte
+    boundary in one direction, whose rows are then read by 8 bytes."""
     import torch
     L = 300
     comp, xfer, dt = wl.skewed_instances(4000 + B, B, L)

@@ -1,5 +1,5 @@
 """dc_time_next_pass on the GPU: the events it asks for bracket the first pass of
-the next schedule call (dense, looped and deep-chain kernels), inside the call's
+the next schedule call (one launch, dense, warp- and CTA-per-instance kernels), inside the call's
 own time, and leave every output as it is without the request; the request is
 used up by that one call."""
 import numpy as np
@@ -30,7 +30,7 @@ def _events(torch, n):
     return evs
 
 
-@pytest.mark.parametrize("L, B", [(8, 5000), (16, 40_013), (54, 3000), (300, 200)])
+@pytest.mark.parametrize("L, B", [(8, 5000), (16, 40_013), (54, 3000), (100, 500), (300, 200)])
 def test_first_pass_events(dc, L, B):
     import torch
     comp, xfer, dt = wl.random_instances(77 + L, B, L)

@@ -1,8 +1,7 @@
 """The checked build (-DDC_CHECKED) on the GPU: every kernel family with its
-index checks compiled in, on inputs that reach each of them (short L, looped L,
-the CTA-per-instance work list, the deep-chain kernel with 1 and 8 warps per
-instance, the forward E form, faults), gives outputs bit-identical to the
-normal build's and records no failed check. The checks count a failure and skip
+index checks compiled in, on inputs that reach each of them (one launch, the dense,
+looped, warp- and CTA-per-instance passes, their work lists by warp, by lane and by
+CTA, drawn rows, faults), gives outputs bit-identical to the normal build's and records no failed check. The checks count a failure and skip
 the access instead of trapping, so a wrong index shows up here as a count.
 
 Run the whole GPU suite against the checked build with
@@ -41,10 +40,18 @@ def _use(dc, path):
 
 
 def _cases():
-    yield "vgg16", wl.with_batch(wl.config("vgg16"), 20_000)
-    yield "resnet50", wl.with_batch(wl.config("resnet50"), 4_000)
-    yield "deep1", wl.with_batch(wl.config("deepchain"), 2_000)   # one warp per instance
-    yield "deep8", wl.with_batch(wl.config("deepchain"), 40)      # eight warps per instance
+    yield "vgg16", wl.with_batch(wl.config("vgg16"), 20_000)           # one launch
+    yield "vgg16 dense", wl.with_batch(wl.config("vgg16"), 60_000)     # a few listed: by warp
+    yield "log12", wl.lsweep_config(12, 300_000)
+    yield "wide12", wl.lsweep_config(12, 30_000)                       # all listed: by lane
+    yield "wide5", wl.lsweep_config(5, 30_000)
+    yield "log18", wl.lsweep_config(18, 170_000)                       # a thread per instance
+    yield "resnet50", wl.with_batch(wl.config("resnet50"), 4_000)      # one launch
+    yield "resnet50 warp", wl.with_batch(wl.config("resnet50"), 60_000)
+    yield "wide54", wl.with_batch(wl.config("resnet50"), 45_000)
+    yield "log100", wl.lsweep_config(100, 3_000)
+    yield "deep1", wl.with_batch(wl.config("deepchain"), 2_000)        # 1,024 rows by 256 threads
+    yield "deep8", wl.with_batch(wl.config("deepchain"), 40)           # by 512
 
 
 def _solve(dc, prof, L):
@@ -57,6 +64,20 @@ def _solve(dc, prof, L):
         torch.cuda.synchronize()
         out[d] = {k: v.cpu().numpy() for k, v in r.items()}
         out[d]["replay"] = rep.cpu().numpy()
+    return out
+
+
+def _draw(dc):
+    """Generate and solve: a short list, a list of everything, and one launch."""
+    import torch
+    out = []
+    for name, B, kw in (("vgg16", 12_007, {}), ("alexnet", 12_007, dict(rate_lo=1, rate_hi=2)),
+                        ("vgg16", 12_007, dict(rate_lo=1, rate_hi=2)), ("tiny", 500, {})):
+        cfg = wl.with_batch(wl.config(name), B)
+        cfg.update(kw)
+        r = dc.GeneratedScheduler(cfg).run()
+        torch.cuda.synchronize()
+        out.append({k: v.cpu().numpy() for k, v in r.items()})
     return out
 
 
@@ -78,7 +99,9 @@ def test_checked_build_matches_and_records_nothing(libs):
     for name, cfg in _cases():
         prof = dc.profile_gen(cfg)
         prof = {k: v.clone() for k, v in prof.items()}
-        if name in ("vgg16", "resnet50"):  # a few faults and 64-bit instances
+        if name.startswith("wide"):  # every value past 32 bits
+            prof = {k: v << 12 for k, v in prof.items()}
+        if name.startswith(("vgg16", "resnet50")):  # a few faults and 64-bit instances
             prof["pt"][5, 0] = 1 << 40
             prof["fc"][9, 1] = -1
             prof["dt"][13] = 1 << 51
@@ -89,6 +112,7 @@ def test_checked_build_matches_and_records_nothing(libs):
     inputs.append(("wide300", 300, {"fc": t(comp), "bc": t(comp), "pt": t(xfer), "gt": t(xfer),
                                      "dt": t(dt)}))
     want = {name: _solve(dc, prof, L) for name, L, prof in inputs}
+    drawn = _draw(dc)
     _use(dc, checked)
     dc.checked_failures(reset=True)
     for name, L, prof in inputs:
@@ -96,5 +120,8 @@ def test_checked_build_matches_and_records_nothing(libs):
         for d in (FWD, BWD):
             for k, v in want[name][d].items():
                 assert np.array_equal(got[d][k], v), (name, d, k)
+    for one, other in zip(drawn, _draw(dc)):
+        for k, v in one.items():
+            assert np.array_equal(other[k], v), k
     fails = dc.checked_failures()
     assert all(c == 0 for c, _ in fails.values()), fails
