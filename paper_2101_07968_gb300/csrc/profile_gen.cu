@@ -227,18 +227,26 @@ cudaError_t launch_gen(const dc_profile_cfg *c, int64_t *fc, int64_t *pt, int64_
 {
     static thread_local GenParams g;  // 25 KB: kept off the caller's stack
     fill_gen_params(c, g);
-    // tiles of 32 instances once they fill the GPU (8 warps per SM; 32 where a tile is long),
-    // else smaller ones, down to 32 elements, and for long rows several warps to an instance
+    // Few instances and elements, and tables that lanes read at a few places only: no copy
+    // of them (4,096 x 8: 3.4 us from a graph, 7.2 with the copy and tiles of 32; but the
+    // log-uniform layer tables, read at 64 places a step, serialise: 11 times slower on
+    // 16,384 x 1,024; and so do the knots, read once per instance, and fixed layers: 60,000 x
+    // 1 7.8 us against 5.6 with the copy, 30,000 x 8 (AlexNet) 9.1 against 6.8, 20,000 x 8 7.3
+    // against 6.4; but with drawn layers 20,000 x 13 7.2 against 8.3)
+    const bool shared = c->batch * c->L > (int64_t(1) << 18) ||
+                        c->batch > (c->layer_mode == DC_LAYERS_FIXED ? 16000 : 24000) ||
+                        c->layer_mode == DC_LAYERS_LOGUNIFORM;
+    // Tiles of 32 instances once they fill the GPU (8 warps per SM, 32 where a tile is long;
+    // 4 where short rows share a copy of the tables: log-uniform 10,000 x 4 8.1 us against
+    // 9.5 with 8, but 20,000 x 24 11.7 against 11.1), else smaller ones, down to 32 elements,
+    // and for long rows several warps to an instance
     int ti = 32, tw = 1;
+    const int fill = shared && c->L <= 16 ? 4 : 8;
     auto tiles_of = [&](int n) { return (c->batch + n - 1) / n; };
-    while (ti > 1 && tiles_of(ti) < 152 * (ti * c->L >= 4096 ? 32 : 8) && ti / 2 * c->L >= 32) ti /= 2;
+    while (ti > 1 && tiles_of(ti) < 152 * (ti * c->L >= 4096 ? 32 : fill) && ti / 2 * c->L >= 32) ti /= 2;
     while (ti == 1 && tw < 4 && c->batch * tw < 152 * 32 && c->L >= 128 * tw) tw *= 2;
     const int64_t warps = tiles_of(ti) * tw;
-    // few elements, and tables that lanes read at a few places only: no copy of them
-    // (4,096 x 8: 3.4 us from a graph, 7.2 with the copy and tiles of 32; but the
-    // log-uniform layer tables, read at 64 places a step, serialise: 11 times slower on
-    // 16,384 x 1,024)
-    if (c->batch * c->L <= (int64_t(1) << 18) && c->layer_mode != DC_LAYERS_LOGUNIFORM) {
+    if (!shared) {
         const unsigned blocks = unsigned((warps + 3) / 4);
         if (g.words)
             gen_kernel<false, true><<<blocks, 128, 0, stream>>>(g, ti, tw, fc, pt, bc, gt, dt);

@@ -99,3 +99,15 @@ def test_costs_at_two_to_the_32(dc, edge, batch):
     torch.cuda.synchronize()
     for k in ("fc", "pt", "bc", "gt", "dt"):
         assert np.array_equal(g.prof[k].cpu().numpy(), exp[k]), k
+
+
+@pytest.mark.parametrize("batch", [16_000, 16_001, 24_000, 24_001])
+@pytest.mark.parametrize("name,L", [("alexnet", 0), ("tiny", 1), ("tiny", 10), ("deepchain", 3), ("deepchain", 17)])
+def test_tables_in_shared_memory_or_not(dc, name, L, batch):
+    """Both sides of the line between reading the tables from the parameters and copying
+    them, and of the number of instances to a tile."""
+    cfg = wl.with_batch(wl.config(name), batch, inst0=5)
+    cfg["L"] = L or cfg["L"]
+    got, exp = dc.profile_gen(cfg), oracle.profile_gen(cfg)
+    for k in ("fc", "pt", "bc", "gt", "dt"):
+        assert np.array_equal(got[k].cpu().numpy(), exp[k]), k
